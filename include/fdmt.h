@@ -684,7 +684,12 @@ int fdmt_schedule_info(fdmt_plan_t plan, int32_t *groups, int32_t *bounds, int32
  * slack that end a block's shared memory, bytes of the warps' descriptor
  * slots before it), 7 the planner's cost
  * model per group (6 each: HBM KiB, shared-memory pipe kilo-slots, work
- * items, thousands of ops, resident blocks, modelled microseconds).  The
+ * items, thousands of ops, resident blocks, modelled microseconds), 8 runs
+ * (16 each, the ops of single and pair stages as the kernel runs them:
+ * destination, destination row bytes, first column, width, four source
+ * offsets, four source row strides, rows, two step masks, flags), 9 the
+ * stages over the runs (as kind 5 with 64 added to the kind of single and
+ * pair stages, whose offsets count runs).  The
  * fused adjoint (empty unless the plan has one): kind 10 launches in launch
  * order (15 each: top level lt, bottom level lb, 1 if the launch ends with
  * the transpose of the initialisation, tile, row-box width (0 for row

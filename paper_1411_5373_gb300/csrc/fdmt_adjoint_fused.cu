@@ -26,6 +26,105 @@ namespace fdmt {
 
 namespace {
 
+// Predicated stores (no branch): only columns below the limit are written.
+__device__ __forceinline__ void sts_if(uint32_t a, float v, bool p) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.shared.f32 [%0], %1;\n\t}"
+               ::"r"(a), "f"(v), "r"((uint32_t)p) : "memory");
+}
+__device__ __forceinline__ void stg_if(float *g, float v, bool p) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.f32 [%0], %1;\n\t}"
+               ::"l"(g), "f"(v), "r"((uint32_t)p) : "memory");
+}
+
+// A gather op's result to shared memory; a whole piece without predicates.
+__device__ __forceinline__ void st_piece_smem(uint32_t addr, const float (&v)[kLaneCols], int width, int lane) {
+  addr += (uint32_t)lane * 4u;
+  if (width >= kPieceCols) {
+#pragma unroll
+    for (int k = 0; k < kLaneCols; ++k) sts_f32(addr + 128u * (uint32_t)k, v[k]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < kLaneCols; ++k) sts_if(addr + 128u * (uint32_t)k, v[k], lane + 32 * k < width);
+  }
+}
+
+// A warp's descriptor stream through the stages of its items.  The words
+// of the stage that runs next (its kind and this warp's first and end
+// descriptor) are requested one stage ahead; during the last chunk of a
+// stage the first chunk of the next stage (or of the next item's first
+// stage) comes into `q`, so a stage starts without a round trip to L2.
+struct DescStream {
+  uint32_t slot;      // the warp's slot in shared memory (kDescSlotBytes)
+  int4 q;             // this lane's 16 bytes of the next stage's first chunk
+  int kind, i0, i1;   // the next stage (kind < 0: none)
+  bool ready;         // q holds that chunk
+};
+
+// Request the words of stage s of template tp (none if tp is null).
+__device__ __forceinline__ void ds_peek(DescStream &ds, const int32_t *__restrict__ stages,
+                                        const FusedTemplate *tp, int s, int warp) {
+  ds.ready = false;
+  if (tp == nullptr || s >= tp->n_stages) {
+    ds.kind = -1;
+    ds.i0 = ds.i1 = 0;
+    return;
+  }
+  const int32_t *p = stages + tp->stage_begin + s * kStageWords;
+  ds.kind = __ldg(p);
+  ds.i0 = __ldg(p + 1 + warp);
+  ds.i1 = __ldg(p + 2 + warp);
+}
+
+// Load the first chunk of the requested stage into q.
+__device__ __forceinline__ void ds_load_first(DescStream &ds, const FusedOp *__restrict__ ops, int lane) {
+  if (ds.ready || ds.kind < 0) return;
+  int4 q = make_int4(0, 0, 0, 0);
+  if (2 * ds.i0 + lane < 2 * ds.i1) q = __ldg(reinterpret_cast<const int4 *>(ops) + 2 * ds.i0 + lane);
+  ds.q = q;
+  ds.ready = true;
+}
+
+// The stage about to run (the one requested last) as a range of ops.
+struct OpRange {
+  int kind, i0, i1;
+};
+__device__ __forceinline__ OpRange ds_take(const DescStream &ds) { return OpRange{ds.kind, ds.i0, ds.i1}; }
+
+// A warp's descriptor slot: the template's layout ends with the slots of
+// the block's warps, then the over-read slack.
+__device__ __forceinline__ uint32_t desc_slot(uint32_t sbase, const FusedTemplate &tp, int warp) {
+  return sbase + (uint32_t)(tp.smem_bytes - kOverRead - kDescBytes + warp * kDescSlotBytes);
+}
+
+// Runs body(op) for ops i0 .. i1 - 1 of this warp, in order.  The lanes copy
+// the descriptors kDescChunk at a time (two lanes per 32-byte op) into the
+// warp's slot; the next chunk's loads are in flight while the current chunk
+// runs (for the last chunk: the next stage's first chunk), and every op is
+// read back from the slot as a broadcast.  On entry ds.q holds the first
+// chunk if ds.ready; ds's stage words are the next stage's.
+template <class F>
+__device__ __forceinline__ void for_ops(const FusedOp *__restrict__ ops, int i0, int i1, DescStream &ds, int lane,
+                                        F &&body) {
+  const int4 *src = reinterpret_cast<const int4 *>(ops);
+  int4 q = ds.q;
+  if (!ds.ready) q = (2 * i0 + lane < 2 * i1) ? __ldg(src + 2 * i0 + lane) : make_int4(0, 0, 0, 0);
+  ds.ready = false;
+  for (int base = i0; base < i1; base += kDescChunk) {
+    __syncwarp();  // every lane is done with the previous chunk
+    sts_v4(ds.slot + 16u * (uint32_t)lane, q);
+    __syncwarp();
+    const int nb = base + kDescChunk;
+    if (nb < i1) {
+      if (2 * nb + lane < 2 * i1) q = __ldg(src + 2 * nb + lane);
+    } else {
+      ds_load_first(ds, ops, lane);
+    }
+    const int n = min(kDescChunk, i1 - base);
+    for (int k = 0; k < n; ++k) body(lds_desc<FusedOp>(ds.slot + 32u * (uint32_t)k));
+  }
+  if (i0 >= i1) ds_load_first(ds, ops, lane);
+}
+
 // out_row[t] for t = t0 + lane + 32 k: written where the piece column is
 // below `width` and 0 <= t < nt (bands tile time with their own offset, so
 // t0 may be negative).
@@ -64,7 +163,7 @@ __device__ __forceinline__ void for_op_pairs(const FusedOp *__restrict__ ops, in
     if (nb < i1) {
       if (2 * nb + lane < 2 * i1) q = __ldg(src + 2 * nb + lane);
     } else {
-      ds_load_first(ds, ops, nullptr, lane);
+      ds_load_first(ds, ops, lane);
     }
     const int n = min(kDescChunk, i1 - base);
     for (int k = 0; k < n; k += 2) {
@@ -75,7 +174,7 @@ __device__ __forceinline__ void for_op_pairs(const FusedOp *__restrict__ ops, in
            FusedOp{b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w}, two);
     }
   }
-  if (i0 >= i1) ds_load_first(ds, ops, nullptr, lane);
+  if (i0 >= i1) ds_load_first(ds, ops, lane);
 }
 
 // One transposed level: each op sums its run of p2 parent rows (stride p1
@@ -84,7 +183,7 @@ template <int OUT>
 __device__ __forceinline__ void adj_gather_stage(uint32_t sbase, const FusedOp *__restrict__ ops, int i0, int i1,
                                                  DescStream &ds, int lane, float *__restrict__ out, int64_t nt,
                                                  int64_t T0) {
-  for_ops(ops, nullptr, i0, i1, ds, lane, [&](const FusedOp &op) {
+  for_ops(ops, i0, i1, ds, lane, [&](const FusedOp &op) {
     // the sum starts from the first row of the run and adds the others in
     // row order; runs of one to three rows (nearly all) are straight-line
     float v[kLaneCols];
@@ -112,7 +211,7 @@ __device__ __forceinline__ void adj_gather_stage(uint32_t sbase, const FusedOp *
       }
     }
     if constexpr (OUT == kOutSmem)
-      st_piece_smem<float, false>(sbase + (uint32_t)op.dst, v, op.width, lane);
+      st_piece_smem(sbase + (uint32_t)op.dst, v, op.width, lane);
     else
       adj_store_global(out + (int64_t)op.dst * nt, T0 + op.col, v, op.width, nt, lane);
   });
@@ -231,7 +330,7 @@ __device__ __forceinline__ void adj_init_stage(uint32_t sbase, const FusedOp *__
 // keeps two ops' input samples in flight, so it is compiled for two
 // resident blocks per SM (more registers per thread).
 template <bool INIT>
-__global__ void __launch_bounds__(kFusedThreads, INIT ? 2 : kFusedMinBlocks)
+__global__ void __launch_bounds__(kFusedThreads, INIT ? 2 : 3)
 adjoint_cone_kernel(const __grid_constant__ TmaMaps maps, float *__restrict__ out, int64_t nt, int32_t W,
                     int64_t ntiles, int64_t items, const FusedTemplate *__restrict__ tpls,
                     const FusedLoad *__restrict__ loads, const FusedOp *__restrict__ ops,
@@ -284,7 +383,7 @@ adjoint_cone_kernel(const __grid_constant__ TmaMaps maps, float *__restrict__ ou
     }
     phase ^= 1u;
     {
-      const StageRange r = ds_take(ds);
+      const OpRange r = ds_take(ds);
       if (cur.n_stages > 1) ds_peek(ds, stages, &cur, 1, warp);
       else ds_peek(ds, stages, next < items ? &tp_next : nullptr, 0, warp);
       if (!INIT && cur.n_stages == 1) adj_gather_stage<kOutGlobal>(bar, ops, r.i0, r.i1, ds, lane, out, nt, T0);
@@ -299,7 +398,7 @@ adjoint_cone_kernel(const __grid_constant__ TmaMaps maps, float *__restrict__ ou
       T0_cur = T0_next;
     }
     for (int s = 1; s < cur.n_stages; ++s) {
-      const StageRange r = ds_take(ds);
+      const OpRange r = ds_take(ds);
       if (s + 1 < cur.n_stages) ds_peek(ds, stages, &cur, s + 1, warp);
       else ds_peek(ds, stages, next < items ? &tp : nullptr, 0, warp);
       if (s == cur.n_stages - 1) {

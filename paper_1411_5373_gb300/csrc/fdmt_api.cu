@@ -111,8 +111,8 @@ void profile_release(fdmt::Profiler &pr) {
 
 void free_device(fdmt_plan_s *p) {
   DeviceTables &d = p->dev;
-  void *ptrs[] = {d.init, d.ops, d.adj, d.adj2, d.adj2_terms, d.status, d.f_tpls, d.f_loads, d.f_walks,
-                  d.f_ops, d.f_stages, d.in_shift, d.a_tpls, d.a_loads, d.a_ops, d.a_stages};
+  void *ptrs[] = {d.init, d.ops, d.adj, d.adj2, d.adj2_terms, d.status, d.f_progs, d.f_prog, d.f_loads,
+                  d.f_ops, d.in_shift, d.a_tpls, d.a_loads, d.a_ops, d.a_stages};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   d.init = nullptr;
@@ -121,11 +121,10 @@ void free_device(fdmt_plan_s *p) {
   d.adj2 = nullptr;
   d.adj2_terms = nullptr;
   d.status = nullptr;
-  d.f_tpls = nullptr;
+  d.f_progs = nullptr;
+  d.f_prog = nullptr;
   d.f_loads = nullptr;
-  d.f_walks = nullptr;
   d.f_ops = nullptr;
-  d.f_stages = nullptr;
   d.in_shift = nullptr;
   d.a_tpls = nullptr;
   d.a_loads = nullptr;
@@ -344,11 +343,10 @@ int fdmt_plan_curve(double f_min, double f_max, int32_t nf, int64_t nt, int32_t 
     if (e == cudaSuccess && p->mapped) e = upload(p->in_shift, &d.in_shift);
     if (e == cudaSuccess && p->has_fused) {
       d.fused = &p->fused;
-      e = upload(p->fused.tpls, &d.f_tpls);
+      e = upload(p->fused.progs, &d.f_progs);
+      if (e == cudaSuccess) e = upload(p->fused.prog, &d.f_prog);
       if (e == cudaSuccess) e = upload(p->fused.loads, &d.f_loads);
-      if (e == cudaSuccess) e = upload(p->fused.walks, &d.f_walks);
-      if (e == cudaSuccess) e = upload(p->fused.ops, &d.f_ops);
-      if (e == cudaSuccess) e = upload(p->fused.stages, &d.f_stages);
+      if (e == cudaSuccess && p->search_k > 0) e = upload(p->fused.ops, &d.f_ops);
     }
     if (e == cudaSuccess && p->has_adj_fused) {
       d.adj_fused = &p->adj_fused;
@@ -689,6 +687,14 @@ int fdmt_fused_tables(fdmt_plan_t plan, int32_t kind, int32_t *dst, int64_t n, i
                                 (int32_t)g.block_slots, (int32_t)(g.seconds * 1e6)};
         v.insert(v.end(), row, row + 6);
       }
+      break;
+    case 8:
+      for (const fdmt::FusedRun &x : f.runs)
+        v.insert(v.end(), {x.dst, x.dst_row, x.col, x.width, x.p0, x.p1, x.p2, x.p3, x.g0, x.g1, x.g2, x.g3, x.n,
+                           (int32_t)x.inc, (int32_t)x.sub, x.flags});
+      break;
+    case 9:
+      v = f.run_stages;
       break;
     case 10:
       // fused adjoint launches: lt, lb, init, W, box, tpl_begin, tpl_count,

@@ -76,7 +76,8 @@ __device__ __forceinline__ int find_seg(const BSeg *__restrict__ segs, int nsegs
 // (uint16 for integer levels stored narrow).
 template <class TI, class TB>
 __device__ __forceinline__ void stage_seg_item(unsigned char *smem, uint32_t bar, const BSeg *__restrict__ sg,
-                                               const CUtensorMap *__restrict__ maps, const FusedTemplate &tp,
+                                               const CUtensorMap *__restrict__ maps, const FusedProg &tp,
+                                               const int4 *__restrict__ prog, uint32_t prog_dst,
                                                const FusedLoad *__restrict__ loads, const FusedLoad &first,
                                                int64_t T0, int lane) {
   const CUtensorMap *m = maps + sg->map;
@@ -86,6 +87,7 @@ __device__ __forceinline__ void stage_seg_item(unsigned char *smem, uint32_t bar
     stage_item<uint16_t>(smem, bar, m, tp, loads, first, T0, sg->box, sg->cshift, lane);
   else
     stage_item<TB>(smem, bar, m, tp, loads, first, T0, sg->box, sg->cshift, lane);
+  if (lane == 0) stage_prog(prog_dst, tp, prog, bar);
 }
 
 // The first stage of an item with the segment's runtime types: the input
@@ -94,48 +96,46 @@ __device__ __forceinline__ void stage_seg_item(unsigned char *smem, uint32_t bar
 // GEN: some beam's plan has pass-through stages (as for the single-beam
 // kernel); the batch has no channel weights.
 template <class TI, class TB, class A, bool GEN>
-__device__ __forceinline__ void batch_first_stage(bool from_input, bool i16, bool o16, uint32_t bar,
-                                                  const int32_t *__restrict__ stages, const FusedTemplate &tp,
-                                                  const FusedWalk *__restrict__ walks, const FusedOp *__restrict__ ops,
-                                                  int warp, int lane, void *out, int64_t nt, int64_t T0, int lim,
-                                                  DescStream &ds, const FusedTemplate *next) {
+__device__ __forceinline__ void batch_first_stage(bool from_input, bool i16, bool o16, uint32_t bar, uint32_t prog,
+                                                  int n_stages, int warp, int lane, void *out, int64_t nt, int64_t T0,
+                                                  int lim) {
   TB *o = static_cast<TB *>(out);
   if constexpr (std::is_same<TB, int32_t>::value) {
     uint16_t *o_16 = static_cast<uint16_t *>(out);
     if (from_input) {
       if (o16)
-        item_first_stage<TI, TB, A, uint16_t, false, true, false, GEN, false>(
-            bar, stages, tp, walks, ops, nullptr, warp, lane, o_16, nt, T0, lim, ds, next);
+        item_first_stage<TI, TB, A, uint16_t, false, true, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane,
+                                                                              o_16, nt, T0, lim);
       else
-        item_first_stage<TI, TB, A, TB, false, true, false, GEN, false>(bar, stages, tp, walks, ops, nullptr, warp,
-                                                                        lane, o, nt, T0, lim, ds, next);
+        item_first_stage<TI, TB, A, TB, false, true, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o,
+                                                                        nt, T0, lim);
     } else if (i16 && o16) {
-      item_first_stage<TI, uint16_t, A, uint16_t, false, false, false, GEN, false>(
-          bar, stages, tp, walks, ops, nullptr, warp, lane, o_16, nt, T0, lim, ds, next);
+      item_first_stage<TI, uint16_t, A, uint16_t, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp,
+                                                                                   lane, o_16, nt, T0, lim);
     } else if (i16) {
-      item_first_stage<TI, uint16_t, A, TB, false, false, false, GEN, false>(bar, stages, tp, walks, ops, nullptr,
-                                                                             warp, lane, o, nt, T0, lim, ds, next);
+      item_first_stage<TI, uint16_t, A, TB, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane,
+                                                                             o, nt, T0, lim);
     } else {
-      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false>(bar, stages, tp, walks, ops, nullptr, warp,
-                                                                       lane, o, nt, T0, lim, ds, next);
+      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
+                                                                       T0, lim);
     }
   } else {
     if (from_input)
-      item_first_stage<TI, TB, A, TB, false, true, false, GEN, false>(bar, stages, tp, walks, ops, nullptr, warp,
-                                                                      lane, o, nt, T0, lim, ds, next);
+      item_first_stage<TI, TB, A, TB, false, true, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
+                                                                      T0, lim);
     else
-      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false>(bar, stages, tp, walks, ops, nullptr, warp,
-                                                                       lane, o, nt, T0, lim, ds, next);
+      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
+                                                                       T0, lim);
   }
 }
 
 template <class TI, class TB, class A, bool GEN>
 __global__ void __launch_bounds__(kFusedThreads, kFusedMinBlocks)
 batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, const CUtensorMap *__restrict__ maps,
-                   const FusedTemplate *__restrict__ tpls, const FusedLoad *__restrict__ loads,
-                   const FusedWalk *__restrict__ walks, const FusedOp *__restrict__ ops,
-                   const int32_t *__restrict__ stages, unsigned long long *__restrict__ counter,
-                   int *__restrict__ done, int *__restrict__ status, uint64_t wait_ns) {
+                   const FusedProg *__restrict__ tpls, const int4 *__restrict__ prog,
+                   const FusedLoad *__restrict__ loads, int prog_off, int prog_slot,
+                   unsigned long long *__restrict__ counter, int *__restrict__ done, int *__restrict__ status,
+                   uint64_t wait_ns) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar = smem_u32(smem);
@@ -159,16 +159,15 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
   int64_t next = *s_next;
   if (item >= total) return;
   int si = find_seg(segs, nsegs, item, 0);
-  FusedTemplate cur;
+  FusedProg cur;
   {
     const int32_t local = (int32_t)(item - segs[si].first);
     cur = tpls[segs[si].tpl_begin + local / segs[si].ntiles];
   }
   uint32_t phase = 0;
   bool staged = false;  // this item's copies were issued while the previous item computed
-  DescStream ds;
-  ds.slot = desc_slot(smem_u32(smem), cur, warp);
-  ds_peek(ds, stages, &cur, 0, warp);
+  uint32_t slot = 0;    // this item's programme slot
+  auto prog_at = [&](uint32_t k) { return bar + (uint32_t)(prog_off + (int)k * prog_slot); };
   // The previous item's completion, published off the critical path: by
   // thread 32 while the block waits for the next item's copies, or by
   // thread 0 before it waits for producers (so that it never waits on
@@ -186,7 +185,7 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     const int64_t T0 = (int64_t)((int32_t)(item - sg->first) % ntiles) * W;
     // The next item: its segment, template and (warp 0) copy descriptors.
     int nsi = si;
-    FusedTemplate tpn = FusedTemplate{0, 0, 0, 0, 0, 0, 0, 0};
+    FusedProg tpn = FusedProg{0, 0, 0, 0, 0, 0, 0, 0};
     int32_t nl = 0;
     if (next < total) {
       nsi = find_seg(segs, nsegs, next, si);
@@ -234,7 +233,8 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
       if (warp == 0) {
         // Rows written by other blocks with generic stores, read by TMA.
         asm volatile("fence.proxy.async.global;" ::: "memory");
-        stage_seg_item<TI, TB>(smem, bar, sg, maps, cur, loads, fetch_load(cur, loads, lane), T0, lane);
+        stage_seg_item<TI, TB>(smem, bar, sg, maps, cur, prog, prog_at(slot), loads, fetch_load(cur, loads, lane), T0,
+                               lane);
       }
     }
     long long nn = 0;  // the item after next
@@ -251,26 +251,27 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     // Integer state stored as uint16 on either side of this group.
     constexpr bool kNarrow = std::is_same<TB, int32_t>::value;
     const bool i16 = kNarrow && sg->in_size == 2, o16 = kNarrow && sg->out_size == 2;
-    const FusedTemplate tp = cur;
-    batch_first_stage<TI, TB, A, GEN>(from_input, i16, o16, bar, stages, tp, walks, ops, warp, lane, sg->out, nt, T0,
-                                 lim, ds, next < total ? &tpn : nullptr);
+    const int n_stages = cur.n_stages;
+    batch_first_stage<TI, TB, A, GEN>(from_input, i16, o16, bar, prog_at(slot), n_stages, warp, lane, sg->out, nt, T0,
+                                      lim);
     __syncthreads();  // the staged rows are no longer read; s_early is visible
     const bool early = *s_early != 0;
     if (early && warp == 0) {
       const BSeg *nsg = segs + nsi;
       // rows written by other blocks with generic stores, read by TMA
       if (nsi != si) asm volatile("fence.proxy.async.global;" ::: "memory");
-      stage_seg_item<TI, TB>(smem, bar, nsg, maps, tpn, loads, ldn, (int64_t)(nl % nsg->ntiles) * nsg->W, lane);
+      stage_seg_item<TI, TB>(smem, bar, nsg, maps, tpn, prog, prog_at(slot ^ 1u), loads, ldn,
+                             (int64_t)(nl % nsg->ntiles) * nsg->W, lane);
     }
     if (next < total) cur = tpn;
     const SearchArgs no_search{};
     if (kNarrow && o16)
-      item_later_stages<A, uint16_t, false, false, GEN>(bar, stages, tp, ops, walks, warp, lane,
-                                                        static_cast<uint16_t *>(sg->out), nt, T0, lim, 0, no_search,
-                                                        ds, next < total ? &tpn : nullptr);
+      item_later_stages<A, uint16_t, false, false, GEN>(bar, prog_at(slot), n_stages, nullptr, warp, lane,
+                                                        static_cast<uint16_t *>(sg->out), nt, T0, lim, 0, no_search);
     else
-      item_later_stages<A, TB, false, false, GEN>(bar, stages, tp, ops, walks, warp, lane, static_cast<TB *>(sg->out),
-                                                  nt, T0, lim, 0, no_search, ds, next < total ? &tpn : nullptr);
+      item_later_stages<A, TB, false, false, GEN>(bar, prog_at(slot), n_stages, nullptr, warp, lane,
+                                                  static_cast<TB *>(sg->out), nt, T0, lim, 0, no_search);
+    slot ^= 1u;
     if (threadIdx.x == 0) *s_next = nn;
     __syncthreads();  // all of this item's stores are issued; Pa / Pb are free; s_next is visible
     pending = sg->done_idx;
@@ -312,14 +313,12 @@ struct FusedBatch {
   size_t ws_bytes = 0;
   std::vector<BSeg> segs;
   int64_t total = 0;
-  int smem_bytes = 0, grid = 0;
+  int smem_bytes = 0, prog_off = 0, prog_slot = 0, grid = 0;
   bool general = false;  // some beam's plan has pass-through stages
   // device
-  FusedTemplate *d_tpls = nullptr;
+  FusedProg *d_tpls = nullptr;
+  int32_t *d_prog = nullptr;
   FusedLoad *d_loads = nullptr;
-  FusedWalk *d_walks = nullptr;
-  FusedOp *d_ops = nullptr;
-  int32_t *d_lops = nullptr;
   BSeg *d_segs = nullptr;
   CUtensorMap *d_maps = nullptr;
   unsigned long long *d_counter = nullptr;
@@ -336,7 +335,7 @@ namespace {
 void release(FusedBatch *fb) {
   if (fb->exec) cudaGraphExecDestroy(fb->exec);
   if (fb->graph) cudaGraphDestroy(fb->graph);
-  void *ptrs[] = {fb->d_tpls, fb->d_loads, fb->d_walks, fb->d_ops, fb->d_lops, fb->d_segs,
+  void *ptrs[] = {fb->d_tpls, fb->d_prog, fb->d_loads, fb->d_segs,
                   fb->d_maps, fb->d_counter, fb->d_done, fb->d_status};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -410,11 +409,9 @@ int fused_batch_create(const std::vector<fdmt_beam_desc> &desc, const std::vecto
   fpar.narrow = (dtype == FDMT_U8_I32);
   fpar.W = prm.fused_tile;
   fpar.smem_budget = prm.smem_budget > 0 ? prm.smem_budget : 72 * 1024;
-  std::vector<FusedTemplate> tpls;
+  std::vector<FusedProg> tpls;
   std::vector<FusedLoad> loads;
-  std::vector<FusedWalk> walks;
-  std::vector<FusedOp> ops;
-  std::vector<int32_t> lops;
+  std::vector<int32_t> prog;
   size_t ws = 0;
   for (int b = 0; b < fb->n; ++b) {
     FusedPlan &fp = fb->plans[b];
@@ -433,32 +430,26 @@ int fused_batch_create(const std::vector<fdmt_beam_desc> &desc, const std::vecto
     fb->level_rows[b] = tabs[b].level_rows;
     fb->general |= fp.general;
     const int32_t t_off = (int32_t)tpls.size(), l_off = (int32_t)loads.size();
-    const int32_t w_off = (int32_t)walks.size(), o_off = (int32_t)ops.size();
-    const int32_t lo_off = (int32_t)lops.size();
-    for (FusedTemplate tp : fp.tpls) {
+    const int32_t p_off = (int32_t)(prog.size() / 4);
+    for (FusedProg tp : fp.progs) {
       tp.load_begin += l_off;
-      tp.walk_begin += w_off;
-      tp.stage_begin += lo_off;
+      tp.prog += p_off;
       tpls.push_back(tp);
     }
     loads.insert(loads.end(), fp.loads.begin(), fp.loads.end());
-    walks.insert(walks.end(), fp.walks.begin(), fp.walks.end());
-    ops.insert(ops.end(), fp.ops.begin(), fp.ops.end());
-    // Stage words: the kind, then indices into the walks (kind 0) or ops.
-    for (size_t i = 0; i < fp.stages.size(); i += kStageWords) {
-      lops.push_back(fp.stages[i]);
-      const int32_t off = (fp.stages[i] & kStageKindMask) == kStageWalk ? w_off : o_off;
-      for (int32_t k = 1; k < kStageWords; ++k) lops.push_back(fp.stages[i + k] + off);
-    }
+    prog.insert(prog.end(), fp.prog.begin(), fp.prog.end());
     for (const FusedGroup &g : fp.groups) {
       fb->tpl_base[b].push_back(t_off + g.tpl_begin);
-      fb->smem_bytes = std::max(fb->smem_bytes, g.smem_bytes);
+      // the programme slots lie behind the largest group's regions
+      fb->prog_off = std::max(fb->prog_off, g.prog_off);
+      fb->prog_slot = std::max(fb->prog_slot, g.prog_slot);
     }
     fb->ws_off[b] = ws;
     ws += (size_t)rup((int64_t)fp.ws_bytes, 256);
   }
   fb->ws_bytes = ws;
-  if (tpls.size() >= ((size_t)1 << 31) || ops.size() >= ((size_t)1 << 31)) {
+  fb->smem_bytes = fb->prog_off + 2 * fb->prog_slot + kOverRead;
+  if (tpls.size() >= ((size_t)1 << 31) || prog.size() >= ((size_t)1 << 31) || fb->smem_bytes > 227 * 1024) {
     delete fb;
     return FDMT_ERR_UNSUPPORTED;
   }
@@ -481,9 +472,7 @@ int fused_batch_create(const std::vector<fdmt_beam_desc> &desc, const std::vecto
   fb->grid = per_sm * sms;
   e = upload(tpls, &fb->d_tpls);
   if (e == cudaSuccess) e = upload(loads, &fb->d_loads);
-  if (e == cudaSuccess) e = upload(walks, &fb->d_walks);
-  if (e == cudaSuccess) e = upload(ops, &fb->d_ops);
-  if (e == cudaSuccess) e = upload(lops, &fb->d_lops);
+  if (e == cudaSuccess) e = upload(prog, &fb->d_prog);
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&fb->d_counter), sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&fb->d_done), sizeof(int) * (size_t)fb->n * kMaxGroups);
   if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&fb->d_status), sizeof(int));
@@ -592,8 +581,8 @@ int fused_batch_execute(FusedBatch *fb, const void *const *in, void *const *out,
       if (le == cudaSuccess) {
         const int nsegs = (int)fb->segs.size();
         const uint64_t wait_ns = (uint64_t)fb->prm.wait_ms * 1000000ull;
-        void *args[] = {&fb->d_segs, (void *)&nsegs, &fb->total, &fb->d_maps, &fb->d_tpls, &fb->d_loads,
-                        &fb->d_walks, &fb->d_ops, &fb->d_lops, &fb->d_counter, &fb->d_done, &fb->d_status,
+        void *args[] = {&fb->d_segs, (void *)&nsegs, &fb->total, &fb->d_maps, &fb->d_tpls, &fb->d_prog,
+                        &fb->d_loads, &fb->prog_off, &fb->prog_slot, &fb->d_counter, &fb->d_done, &fb->d_status,
                         (void *)&wait_ns};
         le = cudaLaunchKernel(kernel_for(fb->dtype, fb->general), dim3(fb->grid), dim3(kFusedThreads), args,
                               (size_t)fb->smem_bytes, cap);

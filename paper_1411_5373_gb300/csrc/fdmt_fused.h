@@ -81,11 +81,12 @@ constexpr int32_t kPieceCols = 32 * kLaneCols;
 // Ops read whole pieces whatever their width: the block's shared memory
 // ends with this much slack so those reads stay inside it.
 constexpr int32_t kOverRead = kPieceCols * 4;
-// Op descriptors: each warp copies its ops kDescChunk at a time into its own
-// slot of shared memory (one round trip to L2 per chunk) and reads them back
-// as broadcasts.  The slots lie between the last region and the slack.
-constexpr int32_t kDescChunk = 16;
-constexpr int32_t kDescSlotBytes = kDescChunk * 32;  // 32-byte FusedOp
+// Descriptors of the fused adjoint: each warp copies its ops kDescChunk at a
+// time into its own slot of shared memory (one round trip to L2 per chunk)
+// and reads them back as broadcasts.  The slots lie between the last region
+// and the slack.
+constexpr int32_t kDescSlotBytes = 512;
+constexpr int32_t kDescChunk = kDescSlotBytes / 32;  // 32-byte FusedOp
 constexpr int32_t kDescBytes = kFusedBlockWarps * kDescSlotBytes;
 
 // Reuse flags of an op, valid against the previous op of the same warp's
@@ -141,6 +142,63 @@ struct FusedWalk {
   int32_t flags;    // kWalkNoUpper: a single channel, whose Option-1 rows pass up
 };
 
+// The ops of one node's rows, lowered for the kernel.  A run computes rows
+// 0 .. n - 1 of a strip of kPieceCols columns that moves with the delay: row
+// r writes columns c(r) + i, c(0) = col and c one larger after every row
+// whose lower row grows, so that the upper half's samples keep their place
+// in the strip (the upper half is read dl columns earlier, and dl grows with
+// c) and stay in registers.  Row r is (s[p0] + s[p1]) + (s[p2] + s[p3]) for a
+// pair, s[p0] + s[p2] for a single level, at byte offsets that step from row
+// to row by two bits:
+//   inc = 1 (the lower row grows): p0, p1 one column later, and
+//     sub = 1: p0 a row later (g0), p1 a column earlier (its half's dl grew),
+//     sub = 0: p1 a row later (g1);
+//   inc = 0 (the upper row grows):
+//     sub = 1: p2 a row later (g2), p3 a column earlier,
+//     sub = 0: p3 a row later (g3).
+// (single levels: p0 or p2 a row later).  The columns outside [0, width) hold
+// sums of whatever lies beside the rows; they are written only under
+// kRunWhole, where the row pitch leaves room for whole strips beside the
+// node's columns.
+struct FusedRun {
+  int32_t dst;      // byte offset of row 0 at column col; top stage: global row of row 0
+  int32_t dst_row;  // bytes from one output row to the next in shared memory
+  int32_t col;      // first column of row 0 (may be negative)
+  int32_t width;    // the node's columns
+  int32_t p0, p1, p2, p3;
+  int32_t g0, g1, g2, g3;
+  int32_t n;        // rows, at most kRunRows
+  uint32_t inc, sub;  // bit r: the step from row r to row r + 1
+  int32_t flags;    // kOpLoOne, kOpHiOne, kOpNoHi (every row of the run), kRunWhole
+};
+constexpr int32_t kRunRows = 32;
+constexpr int32_t kRunWhole = 256;
+// Columns a run's strip may move over its rows: a stored row's pitch leaves
+// at least this many columns free.
+constexpr int32_t kRunGrow = 16;
+// Bytes kept free below the staged rows: a run reads its lower rows from up
+// to kRunRows - 1 columns before their first.
+constexpr int32_t kUnderRead = 128;
+// Stages over the runs: as the stages, with single and pair stages' offsets
+// into the runs, and this bit set in their kind.
+constexpr int32_t kStageRuns = 64;
+
+// What the kernel needs of a work item besides its rows, as one block that
+// is copied to shared memory with them: per stage kProgStageBytes (the kind,
+// then the byte offsets within the block of each warp's first walk or run
+// and of the stage's end; a search stage has its first and last op instead),
+// then the walks and runs.
+struct FusedProg {
+  int32_t load_begin, load_count;  // the item's row copies
+  int32_t tx_bytes;                // bytes the copies and the block deliver
+  int32_t n_stages;
+  int32_t prog;        // first 16-byte word of the block in FusedPlan::prog
+  int32_t prog_bytes;  // a multiple of 16
+  int32_t pad0, pad1;
+};
+constexpr int32_t kProgStageBytes = 48;
+constexpr int32_t kProgMinBytes = 4096;  // the two slots for programmes are at least this large together
+
 // Per stage of a template: kind, then the first op (or walk) of each warp
 // and the end of the stage's ops.
 constexpr int32_t kStageWords = 2 + kFusedBlockWarps;
@@ -176,6 +234,8 @@ struct FusedGroup {
   bool from_input = false;
   int32_t tpl_begin = 0, tpl_count = 0;
   int32_t smem_bytes = 0;     // group-wide layout: barrier + S + Pa + Pb (+ Pt + Q with a search)
+                              //   + two programme slots + slack
+  int32_t prog_off = 0, prog_slot = 0;  // byte offset of the first programme slot, bytes of one
   int32_t s_end = 0, pa_end = 0;  // byte offsets where S and Pa end
   int32_t search_k = 0;       // boxcar widths searched in this launch (0 = none; last group only)
   int32_t hist = 0;           // history columns of the top level's window (search)
@@ -210,6 +270,10 @@ struct FusedPlan {
   std::vector<FusedWalk> walks;
   std::vector<FusedOp> ops;
   std::vector<int32_t> stages;
+  std::vector<FusedRun> runs;       // the ops as the kernel runs them
+  std::vector<int32_t> run_stages;  //   and the stages over them (kStageRuns)
+  std::vector<FusedProg> progs;     // per template: its programme
+  std::vector<int32_t> prog;        //   in here
   // Workspace: intermediate level states between launches (ping-pong).
   size_t ws_split = 0, ws_bytes = 0;
   double model_seconds = 0;

@@ -19,10 +19,7 @@ namespace fdmt {
 
 constexpr int kFusedWarps = kFusedBlockWarps;
 constexpr int kFusedThreads = 32 * kFusedWarps;
-#ifndef FDMT_MIN_BLOCKS
-#define FDMT_MIN_BLOCKS 3
-#endif
-constexpr int kFusedMinBlocks = FDMT_MIN_BLOCKS;  // resident blocks per SM the register budget allows
+constexpr int kFusedMinBlocks = 2;  // resident blocks per SM the register budget allows
 constexpr int kWaitTries = 4000;            // x the suspend hint below: a ~2 s bound
 constexpr uint32_t kSuspendHintNs = 500000;
 
@@ -44,6 +41,10 @@ __device__ __forceinline__ void fence_mbar_init() {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 // try_wait with a suspend-time hint: a waiting thread sleeps in hardware
@@ -128,51 +129,6 @@ __device__ __forceinline__ void sts_s32(uint32_t a, int32_t v) {
   asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
-// Predicated shared-memory loads (no branch): 0 where the predicate is off,
-// and no shared-memory access is made for those lanes.
-__device__ __forceinline__ float lds_f32_if(uint32_t a, bool p) {
-  float v;
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.f32 %0, 0f00000000;\n\t"
-               "@q ld.shared.f32 %0, [%1];\n\t}" : "=f"(v) : "r"(a), "r"((uint32_t)p) : "memory");
-  return v;
-}
-__device__ __forceinline__ int32_t lds_s32_if(uint32_t a, bool p) {
-  int32_t v;
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.s32 %0, 0;\n\t"
-               "@q ld.shared.s32 %0, [%1];\n\t}" : "=r"(v) : "r"(a), "r"((uint32_t)p) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint32_t lds_u16_if(uint32_t a, bool p) {
-  uint32_t v;
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t"
-               "@q ld.shared.u16 %0, [%1];\n\t}" : "=r"(v) : "r"(a), "r"((uint32_t)p) : "memory");
-  return v;
-}
-__device__ __forceinline__ uint32_t lds_u8_if(uint32_t a, bool p) {
-  uint32_t v;
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t"
-               "@q ld.shared.u8 %0, [%1];\n\t}" : "=r"(v) : "r"(a), "r"((uint32_t)p) : "memory");
-  return v;
-}
-template <class T> struct LdsIf;
-template <> struct LdsIf<float> {
-  static __device__ __forceinline__ float get(uint32_t a, bool p) { return lds_f32_if(a, p); }
-};
-template <> struct LdsIf<int32_t> {
-  static __device__ __forceinline__ int32_t get(uint32_t a, bool p) { return lds_s32_if(a, p); }
-};
-template <> struct LdsIf<__half> {
-  static __device__ __forceinline__ float get(uint32_t a, bool p) {
-    return __half2float(__ushort_as_half((unsigned short)lds_u16_if(a, p)));
-  }
-};
-template <> struct LdsIf<uint16_t> {
-  static __device__ __forceinline__ int32_t get(uint32_t a, bool p) { return (int32_t)lds_u16_if(a, p); }
-};
-template <> struct LdsIf<uint8_t> {
-  static __device__ __forceinline__ int32_t get(uint32_t a, bool p) { return (int32_t)lds_u8_if(a, p); }
-};
-
 template <class TI, class A> __device__ __forceinline__ A load_input(uint32_t a);
 template <> __device__ __forceinline__ float load_input<float, float>(uint32_t a) { return lds_f32(a); }
 template <> __device__ __forceinline__ int32_t load_input<uint8_t, int32_t>(uint32_t a) {
@@ -214,13 +170,6 @@ __device__ __forceinline__ FusedOp ld_op(const FusedOp *__restrict__ p) {
   const int4 b = __ldg(reinterpret_cast<const int4 *>(p) + 1);
   return FusedOp{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 }
-__device__ __forceinline__ FusedWalk ld_walk(const FusedWalk *__restrict__ p) {
-  const int4 a = __ldg(reinterpret_cast<const int4 *>(p));
-  const int4 b = __ldg(reinterpret_cast<const int4 *>(p) + 1);
-  const int4 c = __ldg(reinterpret_cast<const int4 *>(p) + 2);
-  return FusedWalk{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
-}
-
 __device__ __forceinline__ void sts_v4(uint32_t a, int4 v) {
   asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                : "memory");
@@ -232,117 +181,50 @@ __device__ __forceinline__ int4 lds_v4(uint32_t a) {
   return v;
 }
 
-// A warp's descriptor stream through the stages of its items.  The words
-// of the stage that runs next (its kind and this warp's first and end op or
-// walk) are requested one stage ahead; during the last chunk of a stage the
-// first chunk of the next stage (or of the next item's first stage) comes
-// into `q`, so a stage starts without a round trip to L2.
-struct DescStream {
-  uint32_t slot;      // the warp's slot in shared memory (kDescSlotBytes)
-  int4 q;             // this lane's 16 bytes of the next stage's first chunk
-  int kind, i0, i1;   // the next stage (kind < 0: none)
-  bool ready;         // q holds that chunk
-};
-
-constexpr int kWalkChunk = kDescSlotBytes / 48;  // walks per chunk (48 bytes: three lanes each)
-
-// Request the words of stage s of template tp (none if tp is null).
-__device__ __forceinline__ void ds_peek(DescStream &ds, const int32_t *__restrict__ stages,
-                                        const FusedTemplate *tp, int s, int warp) {
-  ds.ready = false;
-  if (tp == nullptr || s >= tp->n_stages) {
-    ds.kind = -1;
-    ds.i0 = ds.i1 = 0;
-    return;
-  }
-  const int32_t *p = stages + tp->stage_begin + s * kStageWords;
-  ds.kind = __ldg(p);
-  ds.i0 = __ldg(p + 1 + warp);
-  ds.i1 = __ldg(p + 2 + warp);
+// A descriptor read from shared memory as broadcasts.
+template <class D> __device__ __forceinline__ D lds_desc(uint32_t a);
+template <> __device__ __forceinline__ FusedOp lds_desc<FusedOp>(uint32_t at) {
+  const int4 a = lds_v4(at), b = lds_v4(at + 16u);
+  return FusedOp{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+}
+template <> __device__ __forceinline__ FusedRun lds_desc<FusedRun>(uint32_t at) {
+  const int4 a = lds_v4(at), b = lds_v4(at + 16u), c = lds_v4(at + 32u), d = lds_v4(at + 48u);
+  return FusedRun{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, (uint32_t)d.y, (uint32_t)d.z, d.w};
+}
+template <> __device__ __forceinline__ FusedWalk lds_desc<FusedWalk>(uint32_t at) {
+  const int4 x = lds_v4(at), y = lds_v4(at + 16u), z = lds_v4(at + 32u);
+  return FusedWalk{x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w, z.x, z.y, z.z, z.w};
 }
 
-// Load the first chunk of the requested stage into q (walk or op layout).
-__device__ __forceinline__ void ds_load_first(DescStream &ds, const FusedOp *__restrict__ ops,
-                                              const FusedWalk *__restrict__ walks, int lane) {
-  if (ds.ready || ds.kind < 0) return;
-  const int k = ds.kind & kStageKindMask;
-  int4 q = make_int4(0, 0, 0, 0);
-  if (k == kStageWalk) {
-    if (lane < 3 * kWalkChunk && 3 * ds.i0 + lane < 3 * ds.i1)
-      q = __ldg(reinterpret_cast<const int4 *>(walks) + 3 * ds.i0 + lane);
-  } else if (k != kStageSearch) {
-    if (2 * ds.i0 + lane < 2 * ds.i1) q = __ldg(reinterpret_cast<const int4 *>(ops) + 2 * ds.i0 + lane);
-  }
-  ds.q = q;
-  ds.ready = true;
-}
+// A value every lane of the warp holds, as one the compiler knows to be
+// uniform (branches on it then need no reconvergence).
+__device__ __forceinline__ int32_t warp_all(int32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ uint32_t warp_all(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
-// The stage about to run (the one requested last) as a range.
+// Stage s of the programme at shared address `prog` for one warp: its kind
+// and the addresses of the warp's first descriptor and of their end.
 struct StageRange {
-  int kind, i0, i1;
+  int kind;
+  uint32_t first, end;
 };
-__device__ __forceinline__ StageRange ds_take(const DescStream &ds) { return StageRange{ds.kind, ds.i0, ds.i1}; }
-
-// Runs body(op) for ops i0 .. i1 - 1 of this warp, in order.  The lanes
-// copy the descriptors kDescChunk at a time (two lanes per 32-byte op) into
-// the warp's slot; the next chunk's loads are in flight while the current
-// chunk runs (for the last chunk: the next stage's first chunk), and every
-// op is read back from the slot as a broadcast.  On entry ds.q holds the
-// first chunk if ds.ready; ds's stage words are the next stage's.
-template <class F>
-__device__ __forceinline__ void for_ops(const FusedOp *__restrict__ ops, const FusedWalk *__restrict__ walks,
-                                        int i0, int i1, DescStream &ds, int lane, F &&body) {
-  const int4 *src = reinterpret_cast<const int4 *>(ops);
-  int4 q = ds.q;
-  if (!ds.ready) q = (2 * i0 + lane < 2 * i1) ? __ldg(src + 2 * i0 + lane) : make_int4(0, 0, 0, 0);
-  ds.ready = false;
-  for (int base = i0; base < i1; base += kDescChunk) {
-    __syncwarp();  // every lane is done with the previous chunk
-    sts_v4(ds.slot + 16u * (uint32_t)lane, q);
-    __syncwarp();
-    const int nb = base + kDescChunk;
-    if (nb < i1) {
-      if (2 * nb + lane < 2 * i1) q = __ldg(src + 2 * nb + lane);
-    } else {
-      ds_load_first(ds, ops, walks, lane);
-    }
-    const int n = min(kDescChunk, i1 - base);
-    for (int k = 0; k < n; ++k) {
-      const int4 a = lds_v4(ds.slot + 32u * (uint32_t)k), b = lds_v4(ds.slot + 32u * (uint32_t)k + 16u);
-      body(FusedOp{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w});
-    }
-  }
-  if (i0 >= i1) ds_load_first(ds, ops, walks, lane);
+__device__ __forceinline__ StageRange prog_stage(uint32_t prog, int s, int warp) {
+  const uint32_t at = prog + (uint32_t)(s * kProgStageBytes);
+  return StageRange{warp_all(lds_s32(at)), prog + (uint32_t)warp_all(lds_s32(at + 4u + 4u * (uint32_t)warp)),
+                    prog + (uint32_t)warp_all(lds_s32(at + 8u + 4u * (uint32_t)warp))};
 }
 
-// The same for walks (48 bytes: three lanes per walk, kWalkChunk walks per
-// slot).  A walk keeps many running sums in registers, so a later chunk's
-// descriptors are fetched when it starts, and the next stage's first chunk
-// once the last walk is done.
-template <class F>
-__device__ __forceinline__ void for_walks(const FusedWalk *__restrict__ walks, const FusedOp *__restrict__ ops,
-                                          int i0, int i1, DescStream &ds, int lane, F &&body) {
-  const int4 *src = reinterpret_cast<const int4 *>(walks);
-  constexpr int kWords = 3 * kWalkChunk;  // 16-byte words per chunk
-  bool first = ds.ready;
-  int4 q0 = ds.q;
-  ds.ready = false;
-  for (int base = i0; base < i1; base += kWalkChunk) {
-    __syncwarp();
-    if (lane < kWords && 3 * base + lane < 3 * i1) sts_v4(ds.slot + 16u * (uint32_t)lane, first ? q0 : __ldg(src + 3 * base + lane));
-    first = false;
-    __syncwarp();
-    const int n = min(kWalkChunk, i1 - base);
-    for (int k = 0; k < n; ++k) {
-      const uint32_t a = ds.slot + 48u * (uint32_t)k;
-      const int4 x = lds_v4(a), y = lds_v4(a + 16u), z = lds_v4(a + 32u);
-      body(FusedWalk{x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w, z.x, z.y, z.z, z.w});
-    }
-  }
-  ds_load_first(ds, ops, walks, lane);
+// The warps that compute (kFusedThreads threads) wait for each other.  The
+// copying warp of the single-beam kernel takes no part.
+__device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kFusedThreads) : "memory"); }
+// The same, and whether `ok` held in every thread.
+__device__ __forceinline__ bool compute_sync_and(bool ok) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+               "barrier.cta.red.and.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(r) : "r"((uint32_t)ok), "n"(kFusedThreads) : "memory");
+  return r != 0;
 }
 
-// C columns of a row piece from shared memory (columns >= width read nothing).
 // kLaneCols columns of a row piece from shared memory.  The loads are
 // unconditional (no branch or predicate between them): columns at or beyond
 // the op's width read whatever lies there, which the planner keeps inside
@@ -356,287 +238,339 @@ __device__ __forceinline__ void ld_piece(A (&v)[kLaneCols], uint32_t addr, int l
   for (int k = 0; k < kLaneCols; ++k) v[k] = (A)Lds<TSrc>::get(addr + (uint32_t)(32 * k) * es);
 }
 
-// v[k] <- v at one column earlier (lane l takes lane l - 1's value; lane 0
-// of the first column group takes `first`).
-template <class A>
-__device__ __forceinline__ void shift_one(A (&v)[kLaneCols], A first, int lane) {
-  A s[kLaneCols];
+// The same of staged input samples.
+template <class TI, class A>
+__device__ __forceinline__ void ld_samples(A (&v)[kLaneCols], uint32_t addr, int lane) {
+  addr += (uint32_t)lane * (uint32_t)sizeof(TI);
 #pragma unroll
-  for (int k = 0; k < kLaneCols; ++k) s[k] = __shfl_sync(0xffffffffu, v[k], (lane + 31) & 31);
-  v[0] = lane ? s[0] : first;
-#pragma unroll
-  for (int k = 1; k < kLaneCols; ++k) v[k] = lane ? s[k] : s[k - 1];
+  for (int k = 0; k < kLaneCols; ++k) v[k] = load_input<TI, A>(addr + (uint32_t)(32 * k) * (uint32_t)sizeof(TI));
 }
 
-// Predicated stores (no branch): only columns below the limit are written.
-__device__ __forceinline__ void sts_if(uint32_t a, float v, bool p) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.shared.f32 [%0], %1;\n\t}"
-               ::"r"(a), "f"(v), "r"((uint32_t)p) : "memory");
-}
-__device__ __forceinline__ void sts_if(uint32_t a, int32_t v, bool p) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.shared.s32 [%0], %1;\n\t}"
-               ::"r"(a), "r"(v), "r"((uint32_t)p) : "memory");
-}
-__device__ __forceinline__ void stg_if(float *g, float v, bool p) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.f32 [%0], %1;\n\t}"
-               ::"l"(g), "f"(v), "r"((uint32_t)p) : "memory");
-}
-__device__ __forceinline__ void stg_if(int32_t *g, int32_t v, bool p) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.s32 [%0], %1;\n\t}"
-               ::"l"(g), "r"(v), "r"((uint32_t)p) : "memory");
-}
-__device__ __forceinline__ void stg_if(__half *g, float v, bool p) {
-  const unsigned short h = __half_as_ushort(__float2half_rn(v));
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.u16 [%0], %1;\n\t}"
-               ::"l"(g), "h"(h), "r"((uint32_t)p) : "memory");
-}
-__device__ __forceinline__ void stg_if(uint16_t *g, int32_t v, bool p) {
-  const unsigned short h = (unsigned short)v;
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.u16 [%0], %1;\n\t}"
-               ::"l"(g), "h"(h), "r"((uint32_t)p) : "memory");
-}
-
-// Store an op's result: to shared memory (a stored level, rounded in
-// fp16-state mode) or, for the top stage, to the global row at columns
-// T0 + col + tau, tau < n.  A whole piece is stored without predicates.
-template <class A, bool R16>
-__device__ __forceinline__ void st_piece_smem(uint32_t addr, const A (&v)[kLaneCols], int width, int lane) {
-  addr += (uint32_t)lane * sizeof(A);
-  if (width >= kPieceCols) {
-#pragma unroll
-    for (int k = 0; k < kLaneCols; ++k) sts(addr + (uint32_t)(32 * k) * sizeof(A), round_state<R16>(v[k]));
-  } else {
-#pragma unroll
-    for (int k = 0; k < kLaneCols; ++k)
-      sts_if(addr + (uint32_t)(32 * k) * sizeof(A), round_state<R16>(v[k]), lane + 32 * k < width);
-  }
-}
-template <class TO, class A>
-__device__ __forceinline__ void st_piece_global(TO *__restrict__ drow, const A (&v)[kLaneCols], int n, int lane) {
-  drow += lane;
-  if (n >= kPieceCols) {
-#pragma unroll
-    for (int k = 0; k < kLaneCols; ++k) drow[32 * k] = to_store<TO>(v[k]);
-  } else {
-#pragma unroll
-    for (int k = 0; k < kLaneCols; ++k) stg_if(drow + 32 * k, v[k], lane + 32 * k < n);
-  }
-}
-
-// The top level of a searched launch into Pt, in the search layout (column c
-// of a row at word c + 4 (c / 16)); it is the output level, never rounded.
-template <class A>
-__device__ __forceinline__ void st_piece_padded(uint32_t addr, const A (&v)[kLaneCols], int width, int lane) {
-  addr += (uint32_t)(lane + 4 * (lane >> 4)) * sizeof(A);
-#pragma unroll
-  for (int k = 0; k < kLaneCols; ++k) sts_if(addr + (uint32_t)(40 * k) * sizeof(A), v[k], lane + 32 * k < width);
-}
-
-// One level per op: out = lo + hi (lo reused under kOpLoSame).
 // Where a merge stage writes: shared memory (a stored level), global memory
 // (the group's top level), or shared memory in the search layout (the top
 // level of a launch that ends with the boxcar search).
 enum : int { kOutSmem = 0, kOutGlobal = 1, kOutPadded = 2 };
 
-// GEN: the stage has ops with a passed-up or one-term half (Nf not a power
-// of two); without it those tests are compiled out of the loop.
-template <class TSrc, class A, class TO, bool R16, int OUT, bool GEN>
-__device__ __forceinline__ void stage_single(uint32_t sbase, const FusedOp *__restrict__ ops,
-                                             const FusedWalk *__restrict__ walks, int i0, int i1, DescStream &ds,
-                                             int lane, TO *__restrict__ out, int64_t nt, int64_t T0, int lim) {
-  A lo[kLaneCols], hi[kLaneCols], v[kLaneCols];
-#pragma unroll
-  for (int k = 0; k < kLaneCols; ++k) lo[k] = (A)0;
-  for_ops(ops, walks, i0, i1, ds, lane, [&](const FusedOp &op) {
-    if (!(op.flags & kOpLoSame)) ld_piece<TSrc, A>(lo, sbase + op.p0, lane);
-    if (GEN && (op.flags & kOpNoHi)) {  // no upper half: the lower row passes up
-#pragma unroll
-      for (int k = 0; k < kLaneCols; ++k) v[k] = lo[k];
-    } else {
-      ld_piece<TSrc, A>(hi, sbase + op.p1, lane);
-#pragma unroll
-      for (int k = 0; k < kLaneCols; ++k) v[k] = acc_add(lo[k], hi[k]);
-    }
-    if constexpr (OUT == kOutGlobal) {
-      st_piece_global<TO, A>(out + (int64_t)op.dst * nt + T0 + op.col, v, min(op.width, lim - op.col), lane);
-    } else if constexpr (OUT == kOutPadded) {
-      st_piece_padded<A>(sbase + op.dst, v, op.width, lane);
-    } else {
-      st_piece_smem<A, R16>(sbase + op.dst, v, op.width, lane);
-    }
-  });
+// Stores that write only where column c (as unsigned, so that a negative one
+// never qualifies) lies below n.
+__device__ __forceinline__ void sts_below(uint32_t a, float v, int c, int n) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %2, %3;\n\t@q st.shared.f32 [%0], %1;\n\t}"
+               ::"r"(a), "f"(v), "r"((uint32_t)c), "r"((uint32_t)n) : "memory");
+}
+__device__ __forceinline__ void sts_below(uint32_t a, int32_t v, int c, int n) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %2, %3;\n\t@q st.shared.s32 [%0], %1;\n\t}"
+               ::"r"(a), "r"(v), "r"((uint32_t)c), "r"((uint32_t)n) : "memory");
+}
+__device__ __forceinline__ void stg_below(float *g, float v, int c, int n) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %2, %3;\n\t@q st.global.f32 [%0], %1;\n\t}"
+               ::"l"(g), "f"(v), "r"((uint32_t)c), "r"((uint32_t)n) : "memory");
+}
+__device__ __forceinline__ void stg_below(int32_t *g, int32_t v, int c, int n) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %2, %3;\n\t@q st.global.s32 [%0], %1;\n\t}"
+               ::"l"(g), "r"(v), "r"((uint32_t)c), "r"((uint32_t)n) : "memory");
+}
+__device__ __forceinline__ void stg_below(__half *g, float v, int c, int n) {
+  const unsigned short h = __half_as_ushort(__float2half_rn(v));
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %2, %3;\n\t@q st.global.u16 [%0], %1;\n\t}"
+               ::"l"(g), "h"(h), "r"((uint32_t)c), "r"((uint32_t)n) : "memory");
+}
+__device__ __forceinline__ void stg_below(uint16_t *g, int32_t v, int c, int n) {
+  const unsigned short h = (unsigned short)v;
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %2, %3;\n\t@q st.global.u16 [%0], %1;\n\t}"
+               ::"l"(g), "h"(h), "r"((uint32_t)c), "r"((uint32_t)n) : "memory");
 }
 
-// Two levels per op: out = (s[p0] + s[p1]) + (s[p2] + s[p3]); the lower
-// half sum is reused under kOpLoSame, the upper half sum is the previous
-// one moved a column later under kOpHiShift.  The half sums belong to a
-// level below the top, so fp16-state mode rounds them.
-template <class TSrc, class A, class TO, bool R16, int OUT, bool GEN>
-__device__ __forceinline__ void stage_pair(uint32_t sbase, const FusedOp *__restrict__ ops,
-                                           const FusedWalk *__restrict__ walks, int i0, int i1, DescStream &ds,
-                                           int lane, TO *__restrict__ out, int64_t nt, int64_t T0, int lim) {
+// o = a + b over a lane's columns, each sum rounded by itself; float sums
+// two at a time (add.rn.f32x2: one issue slot for two columns).
+__device__ __forceinline__ void add_piece(float (&o)[kLaneCols], const float (&a)[kLaneCols],
+                                          const float (&b)[kLaneCols]) {
+  static_assert(kLaneCols % 2 == 0, "columns are added in pairs");
+#pragma unroll
+  for (int k = 0; k < kLaneCols; k += 2)
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+        "add.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(o[k]), "=f"(o[k + 1])
+        : "f"(a[k]), "f"(a[k + 1]), "f"(b[k]), "f"(b[k + 1]));
+}
+__device__ __forceinline__ void add_piece(int32_t (&o)[kLaneCols], const int32_t (&a)[kLaneCols],
+                                          const int32_t (&b)[kLaneCols]) {
+#pragma unroll
+  for (int k = 0; k < kLaneCols; ++k) o[k] = a[k] + b[k];
+}
+__device__ __forceinline__ float no_term(float) { return -0.0f; }
+__device__ __forceinline__ int32_t no_term(int32_t) { return 0; }
+template <bool R16, class A>
+__device__ __forceinline__ void round_piece(A (&v)[kLaneCols]) {
+#pragma unroll
+  for (int k = 0; k < kLaneCols; ++k) v[k] = round_state<R16>(v[k]);
+}
+
+// The runs of a single (PAIR false) or pair stage.  A row's four (two)
+// sources and half sums stay in registers: from one row to the next the
+// strip moves with the delay (FusedRun), so one half is unchanged and of the
+// other half's two sources one (sub = 1 below, sub = 0 above) or both are
+// read again -- on average 1.5 reads and one write per output of a pair,
+// against the four reads its sum has.  The next row's reads are issued
+// before the row is stored, so their latency overlaps the stores.  The half
+// sums belong to a level below the top: fp16-state mode rounds them.  The
+// words that steer the rows are broadcast by a shuffle, which makes the
+// branches on them uniform.
+// Bound: instruction issue, then the shared-memory pipe (one 128-byte access
+// per clock and SM).
+template <class TSrc, class A, class TO, bool R16, int OUT, bool PAIR, bool GEN>
+__device__ __forceinline__ void stage_runs(uint32_t sbase, const StageRange &range, int lane, TO *__restrict__ out,
+                                           int64_t nt, int64_t T0, int lim) {
   constexpr uint32_t es = sizeof(TSrc);
-  A lp[kLaneCols], hp[kLaneCols], a[kLaneCols], b[kLaneCols];
-#pragma unroll
-  for (int k = 0; k < kLaneCols; ++k) lp[k] = hp[k] = (A)0;
-  for_ops(ops, walks, i0, i1, ds, lane, [&](const FusedOp &op) {
-    if (!(op.flags & kOpLoSame)) {
-      ld_piece<TSrc, A>(a, sbase + op.p0, lane);
-      if (GEN && (op.flags & kOpLoOne)) {
-#pragma unroll
-        for (int k = 0; k < kLaneCols; ++k) lp[k] = round_state<R16>(a[k]);
+  for (uint32_t at = range.first; at != range.end; at += (uint32_t)sizeof(FusedRun)) {
+    const FusedRun run = lds_desc<FusedRun>(at);
+    const uint32_t flags = warp_all((uint32_t)run.flags);
+    const bool lo_one = GEN && (flags & kOpLoOne) != 0, hi_one = GEN && (flags & kOpHiOne) != 0;
+    const bool no_hi = GEN && (flags & kOpNoHi) != 0;
+    const uint32_t move = no_hi ? 0u : 1u;  // columns the strip moves when the lower row grows
+    uint32_t inc = warp_all(run.inc), sub = warp_all(run.sub);
+    uint32_t p0 = sbase + (uint32_t)run.p0, p1 = sbase + (uint32_t)run.p1;
+    uint32_t p2 = sbase + (uint32_t)run.p2, p3 = sbase + (uint32_t)run.p3;
+    const uint32_t e = move * es, g0 = (uint32_t)run.g0 + e, g1 = (uint32_t)run.g1 + e;
+    int c = warp_all(run.col);
+    const int limit = OUT == kOutGlobal ? min(warp_all(run.width), lim) : warp_all(run.width);
+    uint32_t dst = sbase + (uint32_t)run.dst;
+    TO *g = nullptr;
+    if constexpr (OUT == kOutGlobal) g = out + (int64_t)run.dst * nt + T0 + c + lane;
+    if constexpr (OUT == kOutSmem) dst += (uint32_t)lane * sizeof(A);
+    A a0[kLaneCols], b1[kLaneCols], a2[kLaneCols], b3[kLaneCols], lp[kLaneCols], hp[kLaneCols], v[kLaneCols];
+    auto lower = [&]() {
+      if constexpr (PAIR) {
+        add_piece(lp, a0, b1);
+        round_piece<R16>(lp);
       } else {
-        ld_piece<TSrc, A>(b, sbase + op.p1, lane);
 #pragma unroll
-        for (int k = 0; k < kLaneCols; ++k) lp[k] = round_state<R16>(acc_add(a[k], b[k]));
+        for (int k = 0; k < kLaneCols; ++k) lp[k] = a0[k];
       }
-    }
-    A v[kLaneCols];
-    if (GEN && (op.flags & kOpNoHi)) {  // no upper half: the lower part passes up
-#pragma unroll
-      for (int k = 0; k < kLaneCols; ++k) v[k] = lp[k];
-    } else {
-      const bool one = GEN && (op.flags & kOpHiOne) != 0;
-      if (op.flags & kOpHiShift) {
-        // column 0 of the new upper half sum (every lane reads the same words)
-        const A h0 = (A)Lds<TSrc>::get(sbase + op.p2);
-        const A first = round_state<R16>(one ? h0 : acc_add(h0, (A)Lds<TSrc>::get(sbase + op.p3)));
-        shift_one<A>(hp, first, lane);
+    };
+    auto upper = [&]() {
+      if constexpr (PAIR) {
+        add_piece(hp, a2, b3);
+        round_piece<R16>(hp);
       } else {
-        ld_piece<TSrc, A>(a, sbase + op.p2, lane);
-        if (one) {
 #pragma unroll
-          for (int k = 0; k < kLaneCols; ++k) hp[k] = round_state<R16>(a[k]);
+        for (int k = 0; k < kLaneCols; ++k) hp[k] = a2[k];
+      }
+    };
+    auto sum = [&]() { add_piece(v, lp, hp); };
+    if constexpr (GEN) {
+      // a term that a band does not have is -0 (0 for integers): adding it
+      // changes no value, the sign of a zero included
+#pragma unroll
+      for (int k = 0; k < kLaneCols; ++k) b1[k] = a2[k] = b3[k] = no_term(A());
+    }
+    auto store = [&]() {
+      if constexpr (OUT == kOutGlobal) {
+        if (c >= 0 && c + kPieceCols <= limit) {
+#pragma unroll
+          for (int k = 0; k < kLaneCols; ++k) g[32 * k] = to_store<TO>(v[k]);
         } else {
-          ld_piece<TSrc, A>(b, sbase + op.p3, lane);
 #pragma unroll
-          for (int k = 0; k < kLaneCols; ++k) hp[k] = round_state<R16>(acc_add(a[k], b[k]));
+          for (int k = 0; k < kLaneCols; ++k) stg_below(g + 32 * k, v[k], c + lane + 32 * k, limit);
         }
-      }
+      } else if constexpr (OUT == kOutSmem) {
+        round_piece<R16>(v);
+        if (flags & kRunWhole) {
 #pragma unroll
-      for (int k = 0; k < kLaneCols; ++k) v[k] = acc_add(lp[k], hp[k]);
+          for (int k = 0; k < kLaneCols; ++k) sts(dst + (uint32_t)(32 * k) * sizeof(A), v[k]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < kLaneCols; ++k)
+            sts_below(dst + (uint32_t)(32 * k) * sizeof(A), v[k], c + lane + 32 * k, limit);
+        }
+      } else {
+        // the top level of a searched launch (column c of a row at word c +
+        // 4 (c / 16)); it is the output level, never rounded
+        const int cl = c + lane;
+        const uint32_t at = dst + (uint32_t)(cl + 4 * (cl >> 4)) * (uint32_t)sizeof(A);
+#pragma unroll
+        for (int k = 0; k < kLaneCols; ++k) sts_below(at + (uint32_t)(40 * k) * sizeof(A), v[k], cl + 32 * k, limit);
+      }
+    };
+    ld_piece<TSrc, A>(a0, p0, lane);
+    if (PAIR && !lo_one) ld_piece<TSrc, A>(b1, p1, lane);
+    if (!no_hi) {
+      ld_piece<TSrc, A>(a2, p2, lane);
+      if (PAIR && !hi_one) ld_piece<TSrc, A>(b3, p3, lane);
     }
-    if constexpr (OUT == kOutGlobal) {
-      st_piece_global<TO, A>(out + (int64_t)op.dst * nt + T0 + op.col, v, min(op.width, lim - op.col), lane);
-    } else if constexpr (OUT == kOutPadded) {
-      st_piece_padded<A>(sbase + op.dst, v, op.width, lane);
-    } else {
-      st_piece_smem<A, R16>(sbase + op.dst, v, op.width, lane);
+    lower();
+    upper();
+    for (int left = warp_all(run.n) - 1; left > 0; --left) {
+      sum();
+      if (inc & 1u) {
+        if (!PAIR || (sub & 1u)) {
+          p0 += g0;
+          ld_piece<TSrc, A>(a0, p0, lane);
+          if constexpr (PAIR && GEN) {
+            p1 += e - es;
+            if (no_hi && !lo_one) ld_piece<TSrc, A>(b1, p1, lane);
+          }
+        } else {
+          p0 += e;
+          p1 += g1;
+          ld_piece<TSrc, A>(a0, p0, lane);
+          ld_piece<TSrc, A>(b1, p1, lane);
+        }
+        store();
+        c += (int)move;
+        if constexpr (OUT == kOutGlobal) g += nt + move;
+        dst += (uint32_t)run.dst_row + (OUT == kOutSmem ? move * (uint32_t)sizeof(A) : 0u);
+        lower();
+      } else {
+        if (!PAIR || (sub & 1u)) {
+          p2 += (uint32_t)run.g2;
+          ld_piece<TSrc, A>(a2, p2, lane);
+          if constexpr (PAIR) {
+            p3 -= es;
+            if (!hi_one) ld_piece<TSrc, A>(b3, p3, lane);
+          }
+        } else {
+          p3 += (uint32_t)run.g3;
+          ld_piece<TSrc, A>(b3, p3, lane);
+        }
+        store();
+        if constexpr (OUT == kOutGlobal) g += nt;
+        dst += (uint32_t)run.dst_row;
+        upper();
+      }
+      inc >>= 1;
+      sub >>= 1;
     }
-  });
-  (void)es;
+    sum();
+    store();
+  }
 }
 
 // Level 1 straight from the staged input (section 4: the Option-1 partial
 // sums of level 0 and one merge).  The running sums plo = x_lo[tau] + ... +
 // x_lo[tau - dl] and phi = x_hi[tau - dl] + ... + x_hi[tau - dl - j] are
 // kept in registers in the oracle's order (each adds one earlier sample);
-// when dl grows the upper sums move one column later (its first column is
-// summed afresh by lane 0).  SCALE multiplies every sample by its channel's
-// weight first.
+// when dl grows the upper sums are read again a column earlier (j + 1 reads;
+// j is 0 or 1 on most rows, where this costs no more than moving the sums
+// between lanes).  A row's reads are issued before the row before it is
+// stored.  SCALE multiplies every sample by its channel's weight first.
+// Bound: instruction issue.
 template <class TI, class A, class TO, bool R16, bool SCALE, bool TOP, bool GEN>
-__device__ __forceinline__ void stage_walk(uint32_t sbase, const FusedWalk *__restrict__ walks,
-                                           const FusedOp *__restrict__ ops, int i0, int i1, DescStream &ds,
-                                           int lane, const float *__restrict__ w, TO *__restrict__ out, int64_t nt,
-                                           int64_t T0, int lim) {
-  constexpr int32_t es = (int32_t)sizeof(TI);
-  A plo[kLaneCols], phi[kLaneCols], v[kLaneCols];
-  for_walks(walks, ops, i0, i1, ds, lane, [&](const FusedWalk &wk) {
+__device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &range, int lane,
+                                           const float *__restrict__ w, TO *__restrict__ out, int64_t nt, int64_t T0,
+                                           int lim) {
+  constexpr uint32_t es = (uint32_t)sizeof(TI);
+  for (uint32_t at = range.first; at != range.end; at += (uint32_t)sizeof(FusedWalk)) {
+    const FusedWalk wk = lds_desc<FusedWalk>(at);
     float wl = 1.0f, wh = 1.0f;
     if constexpr (SCALE) {
       wl = __ldg(w + wk.chan);
-      wh = __ldg(w + wk.chan + 1);
+      if (!GEN || !(wk.flags & kWalkNoUpper)) wh = __ldg(w + wk.chan + 1);
     }
-    const uint32_t xl = sbase + wk.x_lo, xh = sbase + wk.x_hi;
-    // Sample of a channel `s` columns before column col (scaled).
-    auto smp = [&](uint32_t base, int col, int s, float wt) -> A {
-      A x = load_input<TI, A>(base + (uint32_t)((col - s) * es));
-      if constexpr (SCALE) x = __fmul_rn(x, wt);
-      return x;
+    const uint32_t xl = sbase + (uint32_t)wk.x_lo, xh = sbase + (uint32_t)wk.x_hi;
+    // A channel's samples s columns earlier (scaled).
+    auto samples = [&](A (&x)[kLaneCols], uint32_t base, int s, float wt) {
+      ld_samples<TI, A>(x, base - (uint32_t)s * es, lane);
+      if constexpr (SCALE) {
+#pragma unroll
+        for (int k = 0; k < kLaneCols; ++k) x[k] = __fmul_rn(x[k], wt);
+      }
     };
-    const bool upper = !GEN || !(wk.flags & kWalkNoUpper);
-    int dl = wk.dl0, j = wk.a - wk.dl0;
+    const bool upper = !GEN || !(warp_all(wk.flags) & kWalkNoUpper);
+    int dl = warp_all(wk.dl0), j = warp_all(wk.a) - dl;
+    uint32_t bits = (uint32_t)warp_all(wk.bits);
+    const bool whole = TOP ? warp_all(wk.width) >= kPieceCols && warp_all(wk.col) + kPieceCols <= lim
+                           : warp_all(wk.width) >= kPieceCols || (warp_all(wk.dst_row) & (kPieceCols * 4 - 1)) == 0;
+    const int limit = TOP ? min(wk.width, lim - wk.col) : wk.width;
+    uint32_t dst = sbase + (uint32_t)wk.dst + (uint32_t)lane * (uint32_t)sizeof(A);
+    TO *g = nullptr;
+    if constexpr (TOP) g = out + (int64_t)wk.dst * nt + T0 + wk.col + lane;
+    A plo[kLaneCols], phi[kLaneCols], v[kLaneCols], t[kLaneCols];
+    auto store = [&]() {
+      if constexpr (TOP) {
+        if (whole) {
 #pragma unroll
-    for (int k = 0; k < kLaneCols; ++k) {
-      const int col = lane + 32 * k;
-      A s0 = smp(xl, col, 0, wl);
-      for (int t = 1; t <= dl; ++t) s0 = acc_add(s0, smp(xl, col, t, wl));
-      A s1 = A(0);
-      if (upper) {
-        s1 = smp(xh, col, dl, wh);
-        for (int t = 1; t <= j; ++t) s1 = acc_add(s1, smp(xh, col, dl + t, wh));
-      }
-      plo[k] = s0;
-      phi[k] = s1;
-    }
-    for (int r = wk.a; r <= wk.e; ++r) {
-      if (r > wk.a && !upper) {
-        // a single channel: row r is its Option-1 row r (dl = r)
-        ++dl;
-#pragma unroll
-        for (int k = 0; k < kLaneCols; ++k) plo[k] = acc_add(plo[k], smp(xl, lane + 32 * k, dl, wl));
-      } else if (r > wk.a) {
-        if ((wk.bits >> (r - wk.a - 1)) & 1) {
-          ++dl;
-          // every lane sums column 0 (the same addresses: broadcast reads)
-          A first = smp(xh, 0, dl, wh);
-          for (int t = 1; t <= j; ++t) first = acc_add(first, smp(xh, 0, dl + t, wh));
-#pragma unroll
-          for (int k = 0; k < kLaneCols; ++k) plo[k] = acc_add(plo[k], smp(xl, lane + 32 * k, dl, wl));
-          shift_one<A>(phi, first, lane);
+          for (int k = 0; k < kLaneCols; ++k) g[32 * k] = to_store<TO>(v[k]);
         } else {
-          ++j;
 #pragma unroll
-          for (int k = 0; k < kLaneCols; ++k) phi[k] = acc_add(phi[k], smp(xh, lane + 32 * k, dl + j, wh));
+          for (int k = 0; k < kLaneCols; ++k) stg_below(g + 32 * k, v[k], lane + 32 * k, max(limit, 0));
         }
+        g += nt;
+      } else {
+        round_piece<R16>(v);
+        if (whole) {
+#pragma unroll
+          for (int k = 0; k < kLaneCols; ++k) sts(dst + (uint32_t)(32 * k) * sizeof(A), v[k]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < kLaneCols; ++k)
+            sts_below(dst + (uint32_t)(32 * k) * sizeof(A), v[k], lane + 32 * k, limit);
+        }
+        dst += (uint32_t)wk.dst_row;
       }
-      if (upper) {
+    };
+    auto sum = [&]() {
+      if constexpr (R16) {
 #pragma unroll
         for (int k = 0; k < kLaneCols; ++k) v[k] = acc_add(round_state<R16>(plo[k]), round_state<R16>(phi[k]));
       } else {
+        add_piece(v, plo, phi);
+      }
+    };
+    samples(plo, xl, 0, wl);
+    if constexpr (GEN) {
 #pragma unroll
-        for (int k = 0; k < kLaneCols; ++k) v[k] = round_state<R16>(plo[k]);
-      }
-      if constexpr (TOP) {
-        st_piece_global<TO, A>(out + (int64_t)(wk.dst + r - wk.a) * nt + T0 + wk.col, v,
-                               min(wk.width, lim - wk.col), lane);
-      } else {
-        st_piece_smem<A, R16>(sbase + wk.dst + (uint32_t)((r - wk.a) * wk.dst_row), v, wk.width, lane);
-      }
+      for (int k = 0; k < kLaneCols; ++k) phi[k] = no_term(A());
     }
-  });
+    if (upper) samples(phi, xh, dl, wh);
+    for (int i = 1; i <= dl; ++i) {
+      samples(t, xl, i, wl);
+      add_piece(plo, plo, t);
+    }
+    if (upper)
+      for (int i = 1; i <= j; ++i) {
+        samples(t, xh, dl + i, wh);
+        add_piece(phi, phi, t);
+      }
+    for (int left = warp_all(wk.e - wk.a); left > 0; --left) {
+      sum();
+      if (!upper || (bits & 1u)) {  // (a single channel: row r is its Option-1 row r, dl = r)
+        ++dl;
+        samples(t, xl, dl, wl);
+        if (upper) samples(phi, xh, dl, wh);
+        store();
+        add_piece(plo, plo, t);
+        if (upper)
+          for (int i = 1; i <= j; ++i) {
+            samples(t, xh, dl + i, wh);
+            add_piece(phi, phi, t);
+          }
+      } else {
+        ++j;
+        samples(t, xh, dl + j, wh);
+        store();
+        add_piece(phi, phi, t);
+      }
+      bits >>= 1;
+    }
+    sum();
+    store();
+  }
 }
 
-// A warp's descriptor slot: the template's layout ends with the slots of
-// the block's warps, then the over-read slack.
-__device__ __forceinline__ uint32_t desc_slot(uint32_t sbase, const FusedTemplate &tp, int warp) {
-  return sbase + (uint32_t)(tp.smem_bytes - kOverRead - kDescBytes + warp * kDescSlotBytes);
-}
-
-// Stage words of stage s of a template: kind, first op of warp w, first op
-// of warp w + 1.
-__device__ __forceinline__ StageRange stage_range(const int32_t *__restrict__ stages, int stage_begin, int s,
-                                                  int warp) {
-  const int32_t *p = stages + stage_begin + s * kStageWords;
-  return StageRange{__ldg(p), __ldg(p + 1 + warp), __ldg(p + 2 + warp)};
-}
-
-// Stage s of an item; TSrc is the type of the stage's source rows (the
-// staged base level for the first stage, the accumulator type after it).
-// ds: this warp's descriptor stream (its next stage already requested).
-// GEN: the plan may hold stages with passed-up or one-term halves (else
-// only the code without those tests is compiled in).
+// A single or pair stage of an item; TSrc is the type of the stage's source
+// rows (the staged base level for the first stage, the accumulator type
+// after it).  GEN: the plan may hold stages with passed-up or one-term
+// halves (else only the code without those tests is compiled in).
 template <class TSrc, class A, class TO, bool R16, int OUT, bool GEN = true>
-__device__ __forceinline__ void run_merge_stage(const StageRange &r, uint32_t sbase, DescStream &ds,
-                                                const FusedOp *__restrict__ ops, const FusedWalk *__restrict__ walks,
-                                                int lane, TO *__restrict__ out, int64_t nt, int64_t T0, int lim) {
+__device__ __forceinline__ void run_merge_stage(const StageRange &r, uint32_t sbase, int lane, TO *__restrict__ out,
+                                                int64_t nt, int64_t T0, int lim) {
   const bool gen = GEN && (r.kind & kStageGeneral) != 0;
   if ((r.kind & kStageKindMask) == kStagePair) {
-    if (gen) stage_pair<TSrc, A, TO, R16, OUT, true>(sbase, ops, walks, r.i0, r.i1, ds, lane, out, nt, T0, lim);
-    else stage_pair<TSrc, A, TO, R16, OUT, false>(sbase, ops, walks, r.i0, r.i1, ds, lane, out, nt, T0, lim);
+    if (gen) stage_runs<TSrc, A, TO, R16, OUT, true, true>(sbase, r, lane, out, nt, T0, lim);
+    else stage_runs<TSrc, A, TO, R16, OUT, true, false>(sbase, r, lane, out, nt, T0, lim);
   } else {
-    if (gen) stage_single<TSrc, A, TO, R16, OUT, true>(sbase, ops, walks, r.i0, r.i1, ds, lane, out, nt, T0, lim);
-    else stage_single<TSrc, A, TO, R16, OUT, false>(sbase, ops, walks, r.i0, r.i1, ds, lane, out, nt, T0, lim);
+    if (gen) stage_runs<TSrc, A, TO, R16, OUT, false, true>(sbase, r, lane, out, nt, T0, lim);
+    else stage_runs<TSrc, A, TO, R16, OUT, false, false>(sbase, r, lane, out, nt, T0, lim);
   }
 }
 
@@ -755,7 +689,7 @@ __device__ __forceinline__ void stage_search_block(uint32_t sbase, const FusedOp
   const int hist = op_first.col, n = op_first.width + hist, own_hi = hist + lim, runs = n >> 4;
   const int32_t t0 = (int32_t)(T0 - hist);  // time of window column 0
   const int per_wave = kFusedThreads / runs;  // whole rows per wave (runs <= kFusedThreads)
-  __syncthreads();
+  compute_sync();
   const int lane = tid & 31;
   for (int row0 = 0; row0 < R; row0 += per_wave) {
     const int ri = row0 + tid / runs, r = tid % runs;
@@ -782,7 +716,7 @@ __device__ __forceinline__ void stage_search_block(uint32_t sbase, const FusedOp
 #pragma unroll
       for (int j = 0; j < 32; ++j) x[j] = A(0);
     }
-    __syncthreads();  // the wave's rows are all loaded before any run is overwritten
+    compute_sync();  // the wave's rows are all loaded before any run is overwritten
     const int c0 = 16 * r;
     if (valid) {
       TO *arow = out + (int64_t)op.dst * nt + T0 - hist;
@@ -821,7 +755,7 @@ __device__ __forceinline__ void stage_search_block(uint32_t sbase, const FusedOp
         sts128(cur + 16u * v, o);
       }
     }
-    __syncthreads();  // before the next wave (and phase 2) reads its rows
+    compute_sync();  // before the next wave (and phase 2) reads its rows
   }
   if (nk > 5) {
     const int groups = (n + 255) >> 8;
@@ -857,7 +791,7 @@ __device__ __forceinline__ void stage_search_block(uint32_t sbase, const FusedOp
                            lane);
       }
     }
-    __syncthreads();
+    compute_sync();
   }
   // The row bests become the tile's partials.
   for (int i = tid; i < R * nk; i += kFusedThreads) {
@@ -877,116 +811,88 @@ __device__ __forceinline__ void stage_search_block(uint32_t sbase, const FusedOp
 
 // The first stage of an item: level 1 walked from the staged input
 // (FROM_INPUT) or the first single / pair stage over the staged base rows.
-// TB is the staged base level's type and TO the type written to global
-// memory when this stage is the top.  With SEARCH the stage before the
-// search writes the top level into Pt instead.
-// ds: the warp's descriptor stream, holding this item's first stage; it
-// leaves holding the stage after it (this item's second, or the first of
-// `next`, the template of the block's next item, if any).
-// GEN as for run_merge_stage; SCALE: the input is multiplied by channel
-// weights (float input only).
+// prog: shared address of the item's programme.  TB is the staged base
+// level's type and TO the type written to global memory when this stage is
+// the top.  With SEARCH the stage before the search writes the top level
+// into Pt instead.  GEN as for run_merge_stage; SCALE: the input is
+// multiplied by channel weights (float input only).
 template <class TI, class TB, class A, class TO, bool R16, bool FROM_INPUT, bool SEARCH, bool GEN = true,
           bool SCALE = true>
-__device__ __forceinline__ void item_first_stage(uint32_t sbase, const int32_t *__restrict__ stages,
-                                                 const FusedTemplate &tp, const FusedWalk *__restrict__ walks,
-                                                 const FusedOp *__restrict__ ops, const float *__restrict__ w,
-                                                 int warp, int lane, TO *__restrict__ out, int64_t nt, int64_t T0,
-                                                 int lim, DescStream &ds, const FusedTemplate *next) {
-  ds.slot = desc_slot(sbase, tp, warp);
-  const StageRange r = ds_take(ds);
-  // (a walk keeps many sums in registers: its successor is requested after it)
-  if (FROM_INPUT) ds_peek(ds, stages, nullptr, 0, warp);
-  else if (tp.n_stages > 1) ds_peek(ds, stages, &tp, 1, warp);
-  else ds_peek(ds, stages, next, 0, warp);
-  const bool top = !SEARCH && tp.n_stages == 1;
+__device__ __forceinline__ void item_first_stage(uint32_t sbase, uint32_t prog, int n_stages,
+                                                 const float *__restrict__ w, int warp, int lane,
+                                                 TO *__restrict__ out, int64_t nt, int64_t T0, int lim) {
+  const StageRange r = prog_stage(prog, 0, warp);
+  const bool top = !SEARCH && n_stages == 1;
   if constexpr (FROM_INPUT) {
-    bool scaled = false;
     const bool gen = GEN && (r.kind & kStageGeneral) != 0;
     if constexpr (SCALE && std::is_floating_point<A>::value) {
-      if (w != nullptr) {
-        scaled = true;
-        if (gen) {
-          if (top) stage_walk<TI, A, TO, R16, true, true, true>(sbase, walks, ops, r.i0, r.i1, ds, lane, w, out, nt, T0, lim);
-          else stage_walk<TI, A, TO, R16, true, false, true>(sbase, walks, ops, r.i0, r.i1, ds, lane, w, out, nt, T0, lim);
-        } else {
-          if (top) stage_walk<TI, A, TO, R16, true, true, false>(sbase, walks, ops, r.i0, r.i1, ds, lane, w, out, nt, T0, lim);
-          else stage_walk<TI, A, TO, R16, true, false, false>(sbase, walks, ops, r.i0, r.i1, ds, lane, w, out, nt, T0, lim);
-        }
-      }
-    }
-    if (!scaled) {
       if (gen) {
-        if (top) stage_walk<TI, A, TO, R16, false, true, true>(sbase, walks, ops, r.i0, r.i1, ds, lane, w, out, nt, T0, lim);
-        else stage_walk<TI, A, TO, R16, false, false, true>(sbase, walks, ops, r.i0, r.i1, ds, lane, w, out, nt, T0, lim);
+        if (top) stage_walk<TI, A, TO, R16, true, true, true>(sbase, r, lane, w, out, nt, T0, lim);
+        else stage_walk<TI, A, TO, R16, true, false, true>(sbase, r, lane, w, out, nt, T0, lim);
       } else {
-        if (top) stage_walk<TI, A, TO, R16, false, true, false>(sbase, walks, ops, r.i0, r.i1, ds, lane, w, out, nt, T0, lim);
-        else stage_walk<TI, A, TO, R16, false, false, false>(sbase, walks, ops, r.i0, r.i1, ds, lane, w, out, nt, T0, lim);
-      }
-    }
-    if (tp.n_stages > 1) ds_peek(ds, stages, &tp, 1, warp);
-    else ds_peek(ds, stages, next, 0, warp);
-  } else if constexpr (SEARCH) {
-    if (tp.n_stages == 2) run_merge_stage<TB, A, TO, R16, kOutPadded, GEN>(r, sbase, ds, ops, walks, lane, out, nt, T0, lim);
-    else run_merge_stage<TB, A, TO, R16, kOutSmem, GEN>(r, sbase, ds, ops, walks, lane, out, nt, T0, lim);
-  } else {
-    if (top) run_merge_stage<TB, A, TO, R16, kOutGlobal, GEN>(r, sbase, ds, ops, walks, lane, out, nt, T0, lim);
-    else run_merge_stage<TB, A, TO, R16, kOutSmem, GEN>(r, sbase, ds, ops, walks, lane, out, nt, T0, lim);
-  }
-}
-
-// Stages 1 .. n - 1 of an item (sources in Pa / Pb), a block barrier after
-// each stage but the last; the last writes global memory (with SEARCH: the
-// one before it writes Pt and the last is the search).
-// ds as for item_first_stage: it enters holding stage 1 and leaves holding
-// the first stage of `next` (null: none).
-template <class A, class TO, bool R16, bool SEARCH, bool GEN = true>
-__device__ __forceinline__ void item_later_stages(uint32_t sbase, const int32_t *__restrict__ stages,
-                                                  const FusedTemplate &tp, const FusedOp *__restrict__ ops,
-                                                  const FusedWalk *__restrict__ walks, int warp, int lane,
-                                                  TO *__restrict__ out, int64_t nt, int64_t T0, int lim, int64_t tile,
-                                                  const SearchArgs &sa, DescStream &ds, const FusedTemplate *next) {
-  ds.slot = desc_slot(sbase, tp, warp);
-  for (int s = 1; s < tp.n_stages; ++s) {
-    const StageRange r = ds_take(ds);
-    if (s + 1 < tp.n_stages) ds_peek(ds, stages, &tp, s + 1, warp);
-    else ds_peek(ds, stages, next, 0, warp);
-    if constexpr (SEARCH) {
-      if (s == tp.n_stages - 1) {
-        // every thread: the whole stage's rows (warp 0's first to the end)
-        const int32_t *p = stages + tp.stage_begin + s * kStageWords;
-        stage_search_block<A, TO>(sbase, ops, __ldg(p + 1), __ldg(p + kStageWords - 1), out, nt, T0, lim, tile, sa);
-      } else {
-        if (s == tp.n_stages - 2) run_merge_stage<A, A, TO, R16, kOutPadded, GEN>(r, sbase, ds, ops, walks, lane, out, nt, T0, lim);
-        else run_merge_stage<A, A, TO, R16, kOutSmem, GEN>(r, sbase, ds, ops, walks, lane, out, nt, T0, lim);
-        __syncthreads();
+        if (top) stage_walk<TI, A, TO, R16, true, true, false>(sbase, r, lane, w, out, nt, T0, lim);
+        else stage_walk<TI, A, TO, R16, true, false, false>(sbase, r, lane, w, out, nt, T0, lim);
       }
     } else {
-      if (s == tp.n_stages - 1) {
-        run_merge_stage<A, A, TO, R16, kOutGlobal, GEN>(r, sbase, ds, ops, walks, lane, out, nt, T0, lim);
+      if (gen) {
+        if (top) stage_walk<TI, A, TO, R16, false, true, true>(sbase, r, lane, w, out, nt, T0, lim);
+        else stage_walk<TI, A, TO, R16, false, false, true>(sbase, r, lane, w, out, nt, T0, lim);
       } else {
-        run_merge_stage<A, A, TO, R16, kOutSmem, GEN>(r, sbase, ds, ops, walks, lane, out, nt, T0, lim);
-        __syncthreads();
+        if (top) stage_walk<TI, A, TO, R16, false, true, false>(sbase, r, lane, w, out, nt, T0, lim);
+        else stage_walk<TI, A, TO, R16, false, false, false>(sbase, r, lane, w, out, nt, T0, lim);
       }
     }
+  } else if constexpr (SEARCH) {
+    if (n_stages == 2) run_merge_stage<TB, A, TO, R16, kOutPadded, GEN>(r, sbase, lane, out, nt, T0, lim);
+    else run_merge_stage<TB, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lim);
+  } else {
+    if (top) run_merge_stage<TB, A, TO, R16, kOutGlobal, GEN>(r, sbase, lane, out, nt, T0, lim);
+    else run_merge_stage<TB, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lim);
   }
 }
 
-__device__ __forceinline__ FusedLoad fetch_load(const FusedTemplate &tp, const FusedLoad *__restrict__ loads,
-                                                int i) {
+// Stages 1 .. n - 1 of an item (sources in Pa / Pb), a barrier of the
+// computing warps before each; the last writes global memory (with SEARCH:
+// the one before it writes Pt and the last is the search).
+template <class A, class TO, bool R16, bool SEARCH, bool GEN = true>
+__device__ __forceinline__ void item_later_stages(uint32_t sbase, uint32_t prog, int n_stages,
+                                                  const FusedOp *__restrict__ ops, int warp, int lane,
+                                                  TO *__restrict__ out, int64_t nt, int64_t T0, int lim, int64_t tile,
+                                                  const SearchArgs &sa) {
+  for (int s = 1; s < n_stages; ++s) {
+    compute_sync();
+    if constexpr (SEARCH) {
+      if (s == n_stages - 1) {
+        // every thread: the whole stage's rows (warp 0's first to the end)
+        const uint32_t at = prog + (uint32_t)(s * kProgStageBytes);
+        stage_search_block<A, TO>(sbase, ops, lds_s32(at + 4u), lds_s32(at + 4u * (kStageWords - 1)), out, nt, T0, lim,
+                                  tile, sa);
+        return;
+      }
+    }
+    const StageRange r = prog_stage(prog, s, warp);
+    if (SEARCH && s == n_stages - 2) run_merge_stage<A, A, TO, R16, kOutPadded, GEN>(r, sbase, lane, out, nt, T0, lim);
+    else if (!SEARCH && s == n_stages - 1) run_merge_stage<A, A, TO, R16, kOutGlobal, GEN>(r, sbase, lane, out, nt, T0, lim);
+    else run_merge_stage<A, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lim);
+  }
+}
+
+// Row copies of an item: T is FusedProg, or FusedTemplate for the adjoint.
+template <class T>
+__device__ __forceinline__ FusedLoad fetch_load(const T &tp, const FusedLoad *__restrict__ loads, int i) {
   if (i < tp.load_count) return loads[tp.load_begin + i];
   return FusedLoad{0, 0, 0, 0};
 }
 
-// Stage the rows of work item `item` into region S: warp 0 only; lane 0
-// announces the bytes on the mbarrier, then the lanes issue the copies.
-// `first` is load `lane` of the template, fetched ahead of time, so the
-// copies go out without waiting on a descriptor read.  cshift > 0: row
-// blocks of 2^cshift-element chunks; else row boxes of `box` elements.
-template <class TS>
-__device__ __forceinline__ void stage_item(unsigned char *smem, uint32_t bar, const CUtensorMap *maps,
-                                           const FusedTemplate &tp, const FusedLoad *__restrict__ loads,
-                                           const FusedLoad &first, int64_t T0, int32_t box, int32_t cshift,
-                                           int lane) {
+// Stage the rows of a work item into region S: one warp; lane 0 announces
+// the bytes on the mbarrier, then the lanes issue the copies.  `first` is
+// load `lane` of the template, fetched ahead of time, so the copies go out
+// without waiting on a descriptor read.  cshift > 0: row blocks of
+// 2^cshift-element chunks; else row boxes of `box` elements.
+template <class TS, class T>
+__device__ __forceinline__ void stage_item(unsigned char *smem, uint32_t bar, const CUtensorMap *maps, const T &tp,
+                                           const FusedLoad *__restrict__ loads, const FusedLoad &first, int64_t T0,
+                                           int32_t box, int32_t cshift, int lane) {
   // Order this block's earlier generic-proxy accesses of S before the
   // async-proxy copies that overwrite it.
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1003,6 +909,15 @@ __device__ __forceinline__ void stage_item(unsigned char *smem, uint32_t bar, co
       for (int b = 0; b < ld.nbox; ++b) tma_load_row(dst + b * box_bytes, maps, x + b * box, ld.row, bar);
     }
   }
+}
+
+// Copy an item's programme to its slot at shared address dst, on the same
+// barrier phase (its bytes are part of tx_bytes); one lane.
+__device__ __forceinline__ void stage_prog(uint32_t dst, const FusedProg &pr, const int4 *__restrict__ prog,
+                                           uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(prog + pr.prog), "r"((uint32_t)pr.prog_bytes), "r"(bar)
+               : "memory");
 }
 
 }  // namespace fdmt

@@ -3,11 +3,11 @@
 // state, fdmt_fused_u8.cu for uint8).  The schedule: fdmt_fused.h; the planner: fdmt_fused_plan.cpp.
 //
 // One block computes one cone for one time tile:
-//   1. warp 0 issues TMA copies of the cone's base rows (or input channels)
-//      into shared memory; out-of-range columns arrive as zeros, which is
-//      the paper's copy rule for t < 0;
-//   2. all threads wait on the mbarrier (bounded: on timeout the block sets
-//      the plan's status word and returns instead of hanging);
+//   1. a copying warp issues TMA copies of the cone's base rows (or input
+//      channels) and of its stage programme into shared memory; out-of-range
+//      columns arrive as zeros, which is the paper's copy rule for t < 0;
+//   2. the computing warps wait on the mbarrier (bounded: on timeout the
+//      block sets the plan's status word and returns instead of hanging);
 //   3. the stages run: a cone that starts at the input walks level 1
 //      straight from the staged samples (the Option-1 partial sums of
 //      section 4 are running sums in registers); the other levels are
@@ -36,100 +36,125 @@
 namespace fdmt {
 
 // Persistent blocks: block b handles items b, b + gridDim.x, ... where item
-// = template * ntiles + tile.  Per item: wait for its staged rows, run the
-// first stage (level 1 walked from the staged input, or the first single /
-// pair stage over the staged base rows), stage the next item into S, run
-// the remaining stages in Pa / Pb; the last writes global memory.  The next
-// item's template and first copy descriptors are read while the current
-// item computes.
-// A launch that ends with the search keeps 32 sums per thread in flight in
-// its search stage: it is compiled for two resident blocks per SM (more
-// registers per thread).
+// = template * ntiles + tile.  Warps 0 .. 7 compute; warp 8 copies.  The
+// copying warp stages item i + 1 (its rows into S, its programme into one of
+// two slots, its place into one of two headers) as soon as the computing
+// warps have arrived at the `free` barrier, behind their first stage of item
+// i, the only one that reads S; its own bookkeeping is off their path.  The
+// computing warps wait for the rows (`full`), then for each other (every one
+// of them has left item i - 1, whose Pa / Pb the first stage overwrites), run
+// the first stage (level 1 walked from the staged input, or the first single
+// / pair stage over the staged base rows) and the remaining stages in Pa /
+// Pb; the last writes global memory.
 // GEN: the plan holds stages with passed-up or one-term halves (Nf not a
 // power of two); SCALE: channel weights multiply the input.  Each launch
 // takes the variant it needs, so a kernel carries only its own stage code.
-// MINB: the resident blocks per SM the register budget is set for.
-template <class TI, class TB, class TO, class A, bool FROM_INPUT, bool R16, bool SEARCH, bool GEN, bool SCALE,
-          int MINB = kFusedMinBlocks>
-__global__ void __launch_bounds__(kFusedThreads, SEARCH ? 2 : MINB)
+// The register budget is set for two resident blocks per SM (a run keeps
+// four sources and two half sums of eight columns in registers).
+// Bound: the computing warps' instruction issue and latency (without copies
+// the launches below take 0.8 .. 0.9 of their time), then HBM.  Measured on
+// a GB300, 1024 x 65536 x 1024 float32, launches [0,3] [3,7] [7,10] with a
+// 112 KiB block: 166, 137 and 121 us with ops read one by one through L2, a
+// pair's upper half moved by shuffles and warp 0 copying; 168, 136 and 109
+// us with the ops as runs; 139, 137 and 109 us with the walks' code
+// straightened as well; 105, 113 and 92 us with the programmes in shared
+// memory and a copying warp.
+constexpr int kFusedLaunchThreads = kFusedThreads + 32;
+
+template <class TI, class TB, class TO, class A, bool FROM_INPUT, bool R16, bool SEARCH, bool GEN, bool SCALE>
+__global__ void __launch_bounds__(kFusedLaunchThreads, kFusedMinBlocks)
 fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t nt, int32_t W,
-             int64_t ntiles, int64_t items, const FusedTemplate *__restrict__ tpls,
-             const FusedLoad *__restrict__ loads, const FusedWalk *__restrict__ walks,
-             const FusedOp *__restrict__ ops, const int32_t *__restrict__ stages,
-             const float *__restrict__ w, int32_t box, int32_t cshift, int *__restrict__ status,
+             int32_t ntiles, int64_t items, const FusedProg *__restrict__ progs, const int4 *__restrict__ prog,
+             const FusedLoad *__restrict__ loads, const FusedOp *__restrict__ ops, const float *__restrict__ w,
+             int32_t box, int32_t cshift, int32_t prog_off, int32_t prog_slot, int *__restrict__ status,
              const SearchArgs sa) {
   using TS = typename std::conditional<FROM_INPUT, TI, TB>::type;  // staged element type
   extern __shared__ __align__(128) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t bar = smem_u32(smem);
-
-  int64_t item = blockIdx.x;
-  if (item >= items) return;
+  const int warp = warp_all((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
+  // The barrier slot: the `full` and `free` mbarriers, then two item headers
+  // (first column, columns, stages, tile).
+  const uint32_t full = smem_u32(smem), free_bar = full + 8u, header = full + 32u;
   if (threadIdx.x == 0) {
-    mbar_init(bar, 1);
+    mbar_init(full, 1);
+    mbar_init(free_bar, kFusedWarps);
     fence_mbar_init();
   }
-  // item = tpl * ntiles + tile, advanced by gridDim.x without divisions.
-  int64_t tile = (int64_t)blockIdx.x % ntiles, tpl = (int64_t)blockIdx.x / ntiles;
-  const int64_t step_tile = (int64_t)gridDim.x % ntiles, step_tpl = (int64_t)gridDim.x / ntiles;
-  auto advance = [&]() {
-    tile += step_tile;
-    tpl += step_tpl;
-    if (tile >= ntiles) {
-      tile -= ntiles;
-      ++tpl;
-    }
-  };
-  FusedTemplate tp = tpls[tpl];
   __syncthreads();
-  int64_t T0_cur = tile * (int64_t)W;
-  if (warp == 0) stage_item<TS>(smem, bar, maps.m, tp, loads, fetch_load(tp, loads, lane), T0_cur, box, cshift, lane);
-  advance();  // (tpl, tile) of the next item from here on
-  FusedTemplate tp_next = FusedTemplate{0, 0, 0, 0, 0, 0, 0, 0};
-  if (item + gridDim.x < items) tp_next = tpls[tpl];
-  DescStream ds;
-  ds.slot = desc_slot(bar, tp, warp);
-  ds_peek(ds, stages, &tp, 0, warp);
-  uint32_t phase = 0;
-  for (; item < items; item += gridDim.x) {
-    const FusedTemplate cur = tp;
-    const int64_t T0 = T0_cur;
-    const int64_t next = item + gridDim.x;
-    const int64_t T0_next = tile * (int64_t)W;
-    FusedLoad ld_next = FusedLoad{0, 0, 0, 0};
-    if (warp == 0 && next < items) ld_next = fetch_load(tp_next, loads, lane);
-    if (!mbar_wait_bounded(bar, phase)) {
-      // The copies did not complete in time: report it, give in-flight
-      // copies one more bounded wait so none lands after the block exits.
+  if (warp == kFusedWarps) {
+    // item = tpl * ntiles + tile, advanced by gridDim.x without divisions.
+    int64_t item = blockIdx.x;
+    if (item >= items) return;
+    int32_t tile = (int32_t)(item % ntiles), tpl = (int32_t)(item / ntiles);
+    const int32_t step_tile = (int32_t)(gridDim.x % ntiles), step_tpl = (int32_t)(gridDim.x / ntiles);
+    FusedProg pr = progs[tpl];
+    FusedLoad ld = fetch_load(pr, loads, lane);
+    uint32_t slot = 0, phase = 0;
+    bool first = true;
+    for (; item < items; item += gridDim.x) {
+      if (!first) {
+        if (!mbar_wait_bounded(free_bar, phase)) {
+          // The computing warps gave up (or never arrived): let the copies in
+          // flight land before the block ends.
+          atomicExch(status, 1);
+          mbar_wait_bounded(full, phase);
+          return;
+        }
+        phase ^= 1u;
+      }
+      first = false;
+      const int64_t T0 = (int64_t)tile * W;
+      if (lane == 0) {
+        const int lim = (int)((nt - T0) < (int64_t)W ? (nt - T0) : (int64_t)W);
+        sts_v4(header + 16u * slot, make_int4(tile, lim, pr.n_stages, 0));
+      }
+      stage_item<TS>(smem, full, maps.m, pr, loads, ld, T0, box, cshift, lane);
+      if (lane == 0) stage_prog(full + (uint32_t)(prog_off + (int)slot * prog_slot), pr, prog, full);
+      slot ^= 1u;
+      tile += step_tile;
+      tpl += step_tpl;
+      if (tile >= ntiles) {
+        tile -= ntiles;
+        ++tpl;
+      }
+      if (item + gridDim.x < items) {
+        pr = progs[tpl];
+        ld = fetch_load(pr, loads, lane);
+      }
+    }
+    // The last copies land before the block ends: the computing warps wait
+    // for them (or give up, which the bounded wait covers).
+    mbar_wait_bounded(full, phase);
+    return;
+  }
+  uint32_t slot = 0, phase = 0;
+  for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const bool ok = mbar_wait_bounded(full, phase);
+    phase ^= 1u;
+    if (!compute_sync_and(ok)) {
+      // The copies did not complete in time: report it; the copying warp
+      // gives them one more bounded wait.
       atomicExch(status, 1);
-      mbar_wait_bounded(bar, phase);
       return;
     }
-    phase ^= 1u;
-    const int lim = (int)((nt - T0) < (int64_t)W ? (nt - T0) : (int64_t)W);
-    item_first_stage<TI, TB, A, TO, R16, FROM_INPUT, SEARCH, GEN, SCALE>(
-        bar, stages, cur, walks, ops, w, warp, lane, out, nt, T0, lim, ds, next < items ? &tp_next : nullptr);
-    __syncthreads();  // S is no longer read: stage the next item into it
-    if (next < items) {
-      if (warp == 0) stage_item<TS>(smem, bar, maps.m, tp_next, loads, ld_next, T0_next, box, cshift, lane);
-      tp = tp_next;
-      advance();
-      if (next + gridDim.x < items) tp_next = tpls[tpl];
-      T0_cur = T0_next;
-    }
-    item_later_stages<A, TO, R16, SEARCH, GEN>(bar, stages, cur, ops, walks, warp, lane, out, nt, T0, lim, T0 / W,
-                                               sa, ds, next < items ? &tp : nullptr);
-    __syncthreads();  // Pa / Pb are reused by the next item
+    const int4 h = lds_v4(header + 16u * slot);
+    const int lim = h.y, n_stages = warp_all(h.z);
+    const int64_t tile = h.x, T0 = tile * W;
+    const uint32_t prg = full + (uint32_t)(prog_off + (int)slot * prog_slot);
+    item_first_stage<TI, TB, A, TO, R16, FROM_INPUT, SEARCH, GEN, SCALE>(full, prg, n_stages, w, warp, lane, out, nt,
+                                                                         T0, lim);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(free_bar);  // this warp reads S no more
+    item_later_stages<A, TO, R16, SEARCH, GEN>(full, prg, n_stages, ops, warp, lane, out, nt, T0, lim, tile, sa);
+    slot ^= 1u;
   }
 }
 
 namespace {
 
-template <class TI, class TB, class TO, class A, bool FI, bool R16, bool SEARCH, bool GEN, bool SCALE,
-          int MINB = kFusedMinBlocks>
+template <class TI, class TB, class TO, class A, bool FI, bool R16, bool SEARCH, bool GEN, bool SCALE>
 cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const void *base, int64_t base_rows,
                            void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa) {
-  auto kern = fused_kernel<TI, TB, TO, A, FI, R16, SEARCH, GEN, SCALE, MINB>;
+  auto kern = fused_kernel<TI, TB, TO, A, FI, R16, SEARCH, GEN, SCALE>;
   static std::once_flag attr_once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(attr_once, [&] {
@@ -144,7 +169,7 @@ cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const vo
   const int32_t box = g.box;
   const int64_t items = (int64_t)g.tpl_count * g.ntiles;
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFusedThreads, g.smem_bytes);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFusedLaunchThreads, g.smem_bytes);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   int dev = 0, sms = 0;
@@ -152,51 +177,29 @@ cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const vo
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int64_t blocks = std::min<int64_t>(items, (int64_t)per_sm * sms);
   dt.prof->begin(s, FI ? K_FUSED_LOCAL : K_FUSED_CONE, g.lb * 100 + g.lt);
-  kern<<<(unsigned)blocks, kFusedThreads, g.smem_bytes, s>>>(
-      maps, static_cast<TO *>(dst), nt, g.W, g.ntiles, items, dt.f_tpls + g.tpl_begin, dt.f_loads,
-      dt.f_walks, dt.f_ops, dt.f_stages, w, box, cshift, dt.status, sa ? *sa : SearchArgs{});
+  kern<<<(unsigned)blocks, kFusedLaunchThreads, g.smem_bytes, s>>>(
+      maps, static_cast<TO *>(dst), nt, g.W, (int32_t)g.ntiles, items, dt.f_progs + g.tpl_begin,
+      reinterpret_cast<const int4 *>(dt.f_prog), dt.f_loads, dt.f_ops, w, box, cshift, g.prog_off, g.prog_slot,
+      dt.status, sa ? *sa : SearchArgs{});
   dt.prof->end(s);
   return cudaGetLastError();
 }
 
-// The variant with or without pass-through stage code (GEN) and weights.
-template <class TI, class TB, class TO, class A, bool FI, bool R16, bool SEARCH, int MINB>
-cudaError_t launch_gen_scale(const DeviceTables &dt, const FusedGroup &g, const void *base, int64_t base_rows,
-                             void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa) {
-  const bool gen = dt.fused->general;
-  if constexpr (FI && std::is_floating_point<A>::value) {
-    if (w != nullptr)
-      return gen ? launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, true, MINB>(dt, g, base, base_rows, dst, w,
-                                                                                    nt, s, sa)
-                 : launch_variant<TI, TB, TO, A, FI, R16, SEARCH, false, true, MINB>(dt, g, base, base_rows, dst, w,
-                                                                                     nt, s, sa);
-  }
-  return gen ? launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, false, MINB>(dt, g, base, base_rows, dst, w, nt,
-                                                                                 s, sa)
-             : launch_variant<TI, TB, TO, A, FI, R16, SEARCH, false, false, MINB>(dt, g, base, base_rows, dst, w, nt,
-                                                                                  s, sa);
-}
-
 // The launch of one group, with the kernel variant the plan and the
-// arguments need (weights only for float input from the input).  Float32
-// sums whose shared memory leaves room for at most two blocks per SM take
-// the variant compiled for two (more registers per thread: measured faster
-// there; for integer and fp16-state sums it measured slower).
+// arguments need: with or without pass-through stage code (GEN) and weights
+// (only for float input from the input).
 template <class TI, class TB, class TO, class A, bool FI, bool R16, bool SEARCH = false>
 cudaError_t launch_group(const DeviceTables &dt, const FusedGroup &g, const void *base, int64_t base_rows,
                          void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa = nullptr) {
-  if constexpr (std::is_same<A, float>::value && !R16 && !SEARCH && kFusedMinBlocks > 2) {
-    // blocks per SM that the shared memory admits
-    int dev = 0, smem_sm = 0, reserved = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-    if (e != cudaSuccess) return e;
-    if (smem_sm / (g.smem_bytes + reserved) <= 2)
-      return launch_gen_scale<TI, TB, TO, A, FI, R16, SEARCH, 2>(dt, g, base, base_rows, dst, w, nt, s, sa);
+  const bool gen = dt.fused->general;
+  if constexpr (FI && std::is_floating_point<A>::value) {
+    if (w != nullptr)
+      return gen ? launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, true>(dt, g, base, base_rows, dst, w, nt, s, sa)
+                 : launch_variant<TI, TB, TO, A, FI, R16, SEARCH, false, true>(dt, g, base, base_rows, dst, w, nt, s,
+                                                                               sa);
   }
-  return launch_gen_scale<TI, TB, TO, A, FI, R16, SEARCH, kFusedMinBlocks>(dt, g, base, base_rows, dst, w, nt, s,
-                                                                           sa);
+  return gen ? launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, false>(dt, g, base, base_rows, dst, w, nt, s, sa)
+             : launch_variant<TI, TB, TO, A, FI, R16, SEARCH, false, false>(dt, g, base, base_rows, dst, w, nt, s, sa);
 }
 
 // The launches of a float plan (A the sums' type, R16: fp16-state rounding).

@@ -17,14 +17,15 @@
 // on a chunk boundary; the input channels of a from-input cone share one
 // window (the union of theirs) so they form one block.
 //
-// The level grouping and W are chosen by a cost model (dynamic programming
-// over group boundaries).  A launch takes the larger of its HBM time (staged
-// plus written bytes) and its on-chip time: a cost per column of every
-// shared-memory op and Option-1 step, plus, per block slot of the GPU
-// (SMs x resident blocks), a latency per work item and per op.  The
-// constants are a least-squares fit to per-launch device times measured on a
-// GB300 over 907 launches of 5 shapes x 4-7 level groupings x 4 tiles x 3
-// budgets (mean absolute error 5 %).
+// The level grouping, W and, where few items would leave SMs idle, the
+// shared memory per item are chosen by a cost model (dynamic programming
+// over group boundaries).  A launch's time is the 3.3-norm of its HBM time
+// (the rows it reads and writes, each once) and its on-chip time (work items
+// per block slot of the GPU times the time of one item, a sum over its
+// stages, row strips, runs, walks and copies), plus a constant.  The
+// constants are a least-squares fit to 7710 launches measured on a GB300 (11
+// shapes from 64 x 1024 to 4096 x 65536, 3 data types, random level
+// groupings, 9 tiles, 3 budgets; mean absolute error 7 %).
 #include "fdmt_fused.h"
 
 #include <algorithm>
@@ -34,15 +35,23 @@
 namespace fdmt {
 namespace {
 
-constexpr int32_t kBarrierBytes = 128;  // mbarrier slot, keeps regions 128-byte aligned
-constexpr double kHbmRate = 6.0e12;          // bytes/s of unique rows in and out
+constexpr int32_t kBarrierBytes = 128 + kUnderRead;  // mbarrier slot and slack, keeps regions 128-byte aligned
+constexpr double kHbmRate = 6.74e12;         // bytes/s of unique rows in and out
 constexpr double kL2Rate = 14.0e12;          // bytes/s of staged rows (halos and overlaps come from L2)
-constexpr double kSlotSeconds = 7.0e-12;     // per shared-memory pipe slot (GPU-wide)
-constexpr double kItemSeconds = 0.3e-6;      // per work item, per block slot
-constexpr double kOpSeconds = 0;             // per op, per block slot
-constexpr double kLaunchSeconds = 8e-6;
+constexpr double kNorm = 3.3;
+constexpr double kLaunchSeconds = 6.6e-6;
+constexpr double kStageSeconds = 0.325e-6;   // one item, two blocks on its SM: per stage,
+constexpr double kPairSeconds = 16.9e-9;     //   row strip of a pair stage,
+constexpr double kSingleSeconds = 6.3e-9;    //   of a single stage,
+constexpr double kTopSeconds = 16.6e-9;      //   of the top stage (its stores) on top of that,
+constexpr double kRunSeconds = 6.9e-9;       //   run,
+constexpr double kWalkSeconds = 8.3e-9;      //   sample read or row written of a walk,
+constexpr double kCopySeconds = 27.3e-9;     //   copy instruction
+constexpr double kByteSeconds = 0.67e-12;    //   and byte copied
+constexpr double kAloneShare = 0.6;          // time of an item whose block has an SM to itself
+constexpr double kWaveTail = 0.7;            // a started wave counts as at most this much more than its items
 constexpr double kSms = 152;
-constexpr double kMaxBlocksPerSm = 4;        // the fused kernel's register limit
+constexpr double kMaxBlocksPerSm = 2;        // the fused kernel's register budget
 
 int64_t round_up(int64_t v, int64_t a) { return (v + a - 1) / a * a; }
 int64_t ceil_to(int64_t v, int64_t a) { return round_up(v, a); }
@@ -57,15 +66,33 @@ struct Node {
   int32_t klo = -1, khi = -1;  // the halves in the level below (khi < 0: none, rows pass up)
 };
 
+// The rows of one node of a single or pair stage: its first column piece's
+// ops, ops[op .. op + n), and what a run needs beside them.
+struct NodeRows {
+  int32_t op, n;
+  int32_t width;         // the node's columns
+  int32_t pitch;         // columns from one output row to the next (shared memory)
+  int32_t es;            // bytes per source sample
+  int32_t g[4];          // row strides of the sources
+  int32_t flags;         // kOpLoOne, kOpHiOne, kOpNoHi
+  int32_t step;          // first of n - 1 row steps (bit 0 inc, bit 1 sub; see FusedRun)
+};
+struct StageRows {
+  std::vector<NodeRows> nodes;
+  std::vector<uint8_t> steps;
+};
+
 struct ConeOut {
   FusedTemplate tpl{};
   std::vector<FusedLoad> loads;
   std::vector<FusedWalk> walks;                 // the first stage of a launch from the input
   std::vector<std::vector<FusedOp>> stage_ops;  // single / pair stages, in row order (before the warp split)
+  std::vector<StageRows> stage_rows;            // the same by node (empty for the search)
   std::vector<int32_t> kinds;                   // stage kinds
   double hbm = 0;
-  double slots = 0;  // cost model: shared-memory pipe slots of one tile (warp instructions)
-  double nops = 0;   // ops and walks of one tile
+  double slots = 0;  // shared-memory pipe slots of one tile (warp instructions), for inspection
+  double nops = 0;   // ops and walks of one tile, for inspection
+  double work = 0;   // cost model: seconds of the stages of one tile
 };
 
 // Region sizes of one cone: S = staged source rows (input channels or the
@@ -77,6 +104,7 @@ struct ConeShape {
   int64_t s_bytes = 0, pa_bytes = 0, pb_bytes = 0;
   int64_t pt_bytes = 0;  // search: the top level in the search layout
   int32_t top_rows = 0;  // rows of the top node
+  int64_t prog_bytes = 0;  // at most this much of the item's programme (walks and runs)
   std::vector<std::pair<int32_t, int32_t>> needs;  // (window elements from the aligned start, rows) per staged node
   int32_t x_o = 0;  // row blocks, from input: the channels' common window starts at T0 - x_o
 };
@@ -113,6 +141,16 @@ std::vector<int32_t> stored_levels(int32_t lb, int32_t lt) {
 }
 
 namespace {
+
+// Row pitch of a stored level's node of `cols` columns.  Rows that nearly
+// fill whole strips get the room of whole strips, so that runs store them
+// without testing columns (kRunWhole): a strip may start up to kRunGrow
+// columns before its row (in the free columns of the row before it) and
+// reaches at most the end of its row's pitch.
+int32_t stored_pitch(int32_t cols) {
+  const int32_t whole = (int32_t)round_up(cols + kRunGrow, kPieceCols);
+  return whole - cols <= cols / 6 + kRunGrow ? whole : (int32_t)round_up(cols + kRunGrow, 4);
+}
 
 void shape_cone(const Tables &t, int32_t lb, int32_t lt, int32_t band, int32_t r0, int32_t r1,
                 int32_t W, const FusedPlan &fp, const StageFmt &f, ConeShape &cs) {
@@ -164,8 +202,8 @@ void shape_cone(const Tables &t, int32_t lb, int32_t lt, int32_t band, int32_t r
   int64_t pa = 0, pb = 0;
   int32_t k = 0;  // index among stored computed levels
   for (int32_t i = 0; i < m; ++i) {
-    int64_t off = 0;
     const bool staged = (i == 0 && !from_input);
+    int64_t off = staged ? 0 : kUnderRead;
     const bool stored = !(i == 0 && from_input) &&
                         std::find(st.begin(), st.end(), lb + i) != st.end();
     for (Node &n : nodes[i]) {
@@ -180,7 +218,7 @@ void shape_cone(const Tables &t, int32_t lb, int32_t lt, int32_t band, int32_t r
         n.smem = (int32_t)off;
         off += round_up((int64_t)rows * n.stride * sB, 128);
       } else if (stored) {
-        n.stride = (int32_t)round_up(W + n.s, 4);
+        n.stride = stored_pitch(W + n.s);
         n.smem = (int32_t)off;
         off += round_up((int64_t)rows * n.stride * sA, 128);
       }
@@ -204,7 +242,7 @@ void shape_cone(const Tables &t, int32_t lb, int32_t lt, int32_t band, int32_t r
     if (i == 0 && from_input) cs.s_bytes = round_up(cs.s_bytes, 128);
     if (staged) {
       cs.s_bytes = off;
-    } else if (stored) {
+    } else if (stored) {  // (the region starts with the slack before its first row)
       if ((k & 1) == 0) pa = std::max(pa, off);
       else pb = std::max(pb, off);
       ++k;
@@ -212,6 +250,22 @@ void shape_cone(const Tables &t, int32_t lb, int32_t lt, int32_t band, int32_t r
   }
   cs.pa_bytes = pa;
   cs.pb_bytes = pb;
+  // Walks and runs of the stages' nodes: their rows are cut after 32 rows or
+  // (lower_stage) where the delay has grown by 9 .. 17 columns.
+  for (size_t si = 1; si < st.size(); ++si) {
+    const int32_t i = st[si] - lb;
+    for (const Node &n : nodes[i]) {
+      const int64_t cols = (i == m && f.search_k == 0) ? W : W + n.s, rows = n.e - n.a + 1;
+      if (from_input && si == 1) {
+        cs.prog_bytes += (rows + 31) / 32 * ((cols + kPieceCols - 1) / kPieceCols) * (int64_t)sizeof(FusedWalk);
+        continue;
+      }
+      const std::vector<int32_t> &dl = t.dl[lb + i][n.band];
+      const int64_t grow = n.khi >= 0 ? dl[n.e] - dl[n.a] : 0;
+      const int64_t strips = (cols + kRunGrow + kPieceCols - 1) / kPieceCols;
+      cs.prog_bytes += (1 + rows / kRunRows + grow / 9) * strips * (int64_t)sizeof(FusedRun);
+    }
+  }
   if (f.search_k > 0) {
     // The top rows, W + hist columns each in the search layout (region Pt).
     Node &n = nodes[m].front();
@@ -233,8 +287,17 @@ int64_t search_q_bytes(const StageFmt &f, int64_t rows) {
   return round_up(rows * f.search_k * 8, 128);
 }
 
-int64_t cone_bytes(const ConeShape &cs) {
-  return kBarrierBytes + cs.s_bytes + cs.pa_bytes + cs.pb_bytes + cs.pt_bytes + kDescBytes + kOverRead;
+// Bytes of one programme slot for items of `stages` stages and at most
+// `descs` bytes of walks and runs (a stage's split over the warps can cut a
+// run in two at each of its seven borders).
+int64_t prog_slot_bytes(int64_t stages, int64_t descs) {
+  const int64_t n = stages * (kProgStageBytes + (kFusedBlockWarps - 1) * (int64_t)sizeof(FusedRun)) + descs;
+  return std::max<int64_t>(kProgMinBytes / 2, round_up(n, 128));
+}
+
+int64_t cone_bytes(const ConeShape &cs, int64_t stages) {
+  return kBarrierBytes + cs.s_bytes + cs.pa_bytes + cs.pb_bytes + cs.pt_bytes +
+         2 * prog_slot_bytes(stages, cs.prog_bytes) + kOverRead;
 }
 
 // Emits the loads, inits and ops of a shaped cone at the given region bases.
@@ -258,6 +321,41 @@ double op_slots(int32_t kind, int32_t flags) {
   const double lo = (flags & kOpLoSame) ? 0 : ((flags & kOpLoOne) ? 1 : 2);
   const double up = (flags & kOpNoHi) ? 0 : ((flags & kOpHiShift) ? 1 : ((flags & kOpHiOne) ? 1 : 2));
   return lo + up + 1;
+}
+
+// The same of one walk: the first row's samples of both channels, then one
+// sample more per row, or, where the lower row grows, one and the upper
+// channel's j + 1 again; and the rows' stores.
+double walk_cost(const FusedWalk &wk) {
+  double n = wk.dl0 + 1 + (wk.flags & kWalkNoUpper ? 0 : wk.a - wk.dl0 + 1) + 1;
+  int32_t j = wk.a - wk.dl0;
+  for (int32_t r = 0; r < wk.e - wk.a; ++r) {
+    if (wk.flags & kWalkNoUpper) n += 2;
+    else if ((wk.bits >> r) & 1) n += 2 + j + 1;
+    else n += 2, ++j;
+  }
+  return n;
+}
+
+// Rows ra .. re of level-1 node p as a walk: its row steps.
+FusedWalk walk_rows(const Tables &t, const Node &p, bool upper, int32_t ra, int32_t re) {
+  const std::vector<int32_t> &dl = t.dl[1][p.band];
+  FusedWalk wk{};
+  wk.a = ra;
+  wk.e = re;
+  wk.dl0 = dl[ra];
+  for (int32_t r = ra + 1; r <= re; ++r)
+    if (dl[r] > dl[r - 1]) wk.bits |= 1 << (r - ra - 1);
+  wk.flags = upper ? 0 : kWalkNoUpper;
+  return wk;
+}
+
+// Cost model: the rows of one node of a single or pair stage.
+double stage_work(const Tables &t, int32_t level, const Node &p, int32_t cols, bool pair, bool to_global) {
+  const std::vector<int32_t> &dl = t.dl[level][p.band];
+  const int32_t grow = p.khi >= 0 ? std::min(kRunGrow, dl[p.e] - dl[p.a]) : 0;
+  const double strips = (cols + grow + kPieceCols - 1) / kPieceCols;
+  return strips * ((p.e - p.a + 1) * ((pair ? kPairSeconds : kSingleSeconds) + (to_global ? kTopSeconds : 0)) + kRunSeconds);
 }
 
 // Emits the loads, walks and stage ops of a shaped cone at the given region
@@ -348,27 +446,17 @@ void emit_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPl
         for (int32_t c0 = 0; c0 < wp; c0 += kPieceCols) {
           for (int32_t ra = p.a; ra <= p.e; ra += 32) {
             const int32_t re = std::min(p.e, ra + 31);
-            FusedWalk wk{};
+            FusedWalk wk = walk_rows(t, p, upper, ra, re);
             wk.dst = top ? (t.band_row0[lt][p.band] + ra) : leaf(io, p, ra, c0);
             wk.dst_row = top ? 0 : p.stride * sA;
             wk.x_lo = clo.xsmem + (clo.xdelta + c0) * sI;
             wk.x_hi = chi.xsmem + (chi.xdelta + c0 + de) * sI;
             wk.width = std::min(kPieceCols, wp - c0);
             wk.col = c0;
-            wk.a = ra;
-            wk.e = re;
-            wk.dl0 = dlv(1, p.band, ra);
-            wk.bits = 0;
-            double sl = (wk.dl0 + 1) + (ra - wk.dl0 + 1) + 1;
-            for (int32_t r = ra + 1; r <= re; ++r) {
-              const int32_t inc = dlv(1, p.band, r) - dlv(1, p.band, r - 1);
-              if (inc) wk.bits |= 1 << (r - ra - 1);
-              sl += 1 + inc + 1;
-            }
             wk.chan = clo.band;
-            wk.flags = upper ? 0 : kWalkNoUpper;
             c.walks.push_back(wk);
-            c.slots += sl * kLaneCols;
+            c.slots += walk_cost(wk) * kLaneCols;
+            c.work += walk_cost(wk) * kWalkSeconds + (top ? (re - ra + 1) * kTopSeconds : 0);
             c.nops += 1;
             if (top) c.hbm += (double)std::min(kPieceCols, W - c0) * (re - ra + 1) * fp.level_size[lt];
           }
@@ -383,6 +471,7 @@ void emit_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPl
     const bool to_global = top && !search;
     c.kinds.push_back(kind | (top && search ? kStagePadded : 0));
     std::vector<FusedOp> ops;
+    StageRows sr;
     const int32_t wmax = to_global ? W : [&] {
       int32_t v = 0;
       for (const Node &p : par) v = std::max(v, W + p.s);
@@ -398,6 +487,40 @@ void emit_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPl
         const int32_t de = dlv(l1, p.band, p.e);
         const std::vector<Node> &kid = nodes[io - 1];
         const Node &klo = kid[p.klo], &khi = upper ? kid[p.khi] : kid[p.klo];
+        if (c0 == 0) {
+          NodeRows nr{};
+          nr.op = (int32_t)ops.size();
+          nr.n = p.e - p.a + 1;
+          nr.width = wp;
+          nr.pitch = to_global ? 0 : p.stride;
+          const int32_t is = pair ? io - 2 : io - 1;  // level index of the sources
+          nr.es = (is == 0 && !from_input) ? sB : sA;
+          nr.flags = upper ? 0 : kOpNoHi;
+          if (!pair) {
+            nr.g[0] = klo.stride * nr.es;
+            nr.g[2] = khi.stride * nr.es;
+          } else {
+            const std::vector<Node> &g = nodes[io - 2];
+            nr.g[0] = g[klo.klo].stride * nr.es;
+            nr.g[2] = g[khi.klo].stride * nr.es;
+            if (klo.khi >= 0) nr.g[1] = g[klo.khi].stride * nr.es;
+            else nr.flags |= kOpLoOne;
+            if (upper) {
+              if (khi.khi >= 0) nr.g[3] = g[khi.khi].stride * nr.es;
+              else nr.flags |= kOpHiOne;
+            }
+          }
+          nr.step = (int32_t)sr.steps.size();
+          for (int32_t dt = p.a; dt < p.e; ++dt) {
+            const int32_t j = dlv(l1, p.band, dt), inc = dlv(l1, p.band, dt + 1) - j;
+            const Node &k = inc ? klo : khi;
+            const int32_t r = inc ? j : dt - j;  // the row of k that grows
+            const int32_t sub = (pair && k.khi >= 0) ? dlv(l1 - 1, k.band, r + 1) - dlv(l1 - 1, k.band, r) : 1;
+            sr.steps.push_back((uint8_t)(inc | sub << 1));
+          }
+          c.work += stage_work(t, l1, p, wp, pair, to_global);
+          sr.nodes.push_back(nr);
+        }
         int32_t pj = -1, pm = -1;
         for (int32_t dt = p.a; dt <= p.e; ++dt) {
           // (a band without an upper half has dl = dt: row dt is its lower row dt)
@@ -452,6 +575,7 @@ void emit_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPl
       }
     }
     c.stage_ops.push_back(std::move(ops));
+    c.stage_rows.push_back(std::move(sr));
   }
   if (search) {
     // One search op per top row: the row in Pt, its global row, the W
@@ -473,6 +597,50 @@ void emit_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPl
     c.stage_ops.push_back(std::move(ops));
   }
   c.tpl.n_stages = (int32_t)c.kinds.size();
+}
+
+// What emit_cone adds to the cost model, without the loads, walks and ops:
+// `work`, `hbm`, the bytes copied and the number of copies.  The search over
+// groupings and tiles compares launches by this alone.
+void count_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPlan &fp, const StageFmt &f,
+                const ConeShape &cs, ConeOut &c, int32_t &copies) {
+  const bool from_input = (lb == 0);
+  const int32_t sB = fp.level_size[lb], sI = fp.input_size;
+  const std::vector<int32_t> st = stored_levels(lb, lt);
+  int64_t tx = 0;
+  const std::vector<Node> &base = cs.nodes[0];
+  if (from_input && f.chunk > 0) {
+    row_pieces((int32_t)base.size(), f.max_p, [&](int32_t, int32_t) { ++copies; });
+    for (const Node &n : base) tx += (int64_t)n.xstride * sI;
+  } else {
+    for (const Node &n : base) {
+      const int32_t rows = from_input ? 1 : n.e - n.a + 1;
+      tx += (int64_t)rows * (from_input ? n.xstride * sI : n.stride * sB);
+      if (f.chunk > 0) row_pieces(rows, f.max_p, [&](int32_t, int32_t) { ++copies; });
+      else copies += rows;
+    }
+  }
+  c.tpl.tx_bytes = (int32_t)tx;
+  c.hbm = (double)tx;
+  for (size_t si = 0; si + 1 < st.size(); ++si) {
+    const int32_t l1 = st[si + 1], io = l1 - lb;
+    const bool top = (l1 == lt), to_global = top && f.search_k == 0;
+    for (const Node &p : cs.nodes[io]) {
+      const bool upper = p.khi >= 0;
+      const int32_t n = p.e - p.a + 1, wp = to_global ? W : W + p.s;
+      if (from_input && si == 0) {
+        const double pieces = (wp + kPieceCols - 1) / kPieceCols;
+        for (int32_t ra = p.a; ra <= p.e; ra += 32) {
+          const FusedWalk wk = walk_rows(t, p, upper, ra, std::min(p.e, ra + 31));
+          c.work += pieces * (walk_cost(wk) * kWalkSeconds + (top ? (wk.e - ra + 1) * kTopSeconds : 0));
+        }
+      } else {
+        c.work += stage_work(t, l1, p, wp, l1 - st[si] == 2, to_global);
+      }
+      if (to_global) c.hbm += (double)W * n * fp.level_size[lt];
+    }
+  }
+  if (f.search_k > 0) c.hbm += (double)W * (cs.nodes[lt - lb].front().e - cs.nodes[lt - lb].front().a + 1) * fp.level_size[lt];
 }
 
 // Splits a stage's ops (or walks) into kFusedBlockWarps contiguous runs of
@@ -501,13 +669,22 @@ struct ItemOut {
   std::vector<FusedWalk> walks;
   std::vector<FusedOp> ops;
   std::vector<int32_t> stages;  // kStageWords per stage
-  double hbm = 0, slots = 0, nops = 0;
+  std::vector<StageRows> rows;  // per stage: its nodes' rows, op indices into `ops` (empty: walk, search)
+  double hbm = 0, slots = 0, nops = 0, work = 0;
 };
+
+// Cost model: one item beside its rows.
+double item_work(int64_t stages, int32_t copies, int32_t tx_bytes) {
+  return (double)stages * (kStageSeconds + (kFusedBlockWarps - 1) * kRunSeconds) + copies * kCopySeconds +
+         tx_bytes * kByteSeconds;
+}
 
 struct GroupBuild {
   bool ok = false;
   FusedGroup g;
-  std::vector<ItemOut> cones;
+  int64_t items = 0;           // templates
+  std::vector<ItemOut> cones;  // filled when emitted
+  int32_t budget = 0;
   double seconds = 0;
 };
 
@@ -542,9 +719,10 @@ int32_t choose_box(const std::vector<std::pair<int32_t, int32_t>> &needs, int32_
 
 GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int32_t W,
                            const FusedPlan &fp, int32_t budget, const StageFmt &f,
-                           std::vector<std::pair<int32_t, int32_t>> *needs) {
+                           std::vector<std::pair<int32_t, int32_t>> *needs, bool emit) {
   GroupBuild gb;
   const int32_t nb = bands_at(t.nf, lt);
+  const int64_t nst = (int64_t)stored_levels(lb, lt).size() - 1 + (f.search_k > 0 ? 1 : 0);
   for (int32_t cone_budget = budget; cone_budget >= 4096; cone_budget = cone_budget * 7 / 8) {
     std::vector<ConeShape> shapes;
     bool ok = true;
@@ -554,7 +732,7 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
         for (int32_t r0 = 0; r0 < rows; r0 += per) {
           ConeShape cs;
           shape_cone(t, lb, lt, b, r0, std::min(rows, r0 + per) - 1, W, fp, f, cs);
-          if (cone_bytes(cs) + search_q_bytes(f, cs.top_rows) > cone_budget) return false;
+          if (cone_bytes(cs, nst) + search_q_bytes(f, cs.top_rows) > cone_budget) return false;
           if (keep) keep->push_back(std::move(cs));
         }
         return true;
@@ -584,18 +762,20 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
     const int64_t cap = std::max<int64_t>(
         1, (int64_t)shapes.size() * ntiles / (int64_t)(2 * kSms * kMaxBlocksPerSm));
     std::vector<std::vector<int32_t>> bundles;
-    int64_t bs = 0, ba = 0, bb = 0, bt = 0, br = 0;
+    int64_t bs = 0, ba = 0, bb = 0, bt = 0, br = 0, bp = 0;
     for (int32_t i = 0; i < (int32_t)shapes.size(); ++i) {
       const ConeShape &cs = shapes[i];
       if (!bundles.empty() && (int64_t)bundles.back().size() < cap &&
           kBarrierBytes + bs + cs.s_bytes + ba + cs.pa_bytes + bb + cs.pb_bytes + bt + cs.pt_bytes +
-                  search_q_bytes(f, br + cs.top_rows) + kDescBytes + kOverRead <= cone_budget) {
+                  search_q_bytes(f, br + cs.top_rows) + 2 * prog_slot_bytes(nst, bp + cs.prog_bytes) + kOverRead <=
+              cone_budget) {
         bundles.back().push_back(i);
         bs += cs.s_bytes;
         ba += cs.pa_bytes;
         bb += cs.pb_bytes;
         bt += cs.pt_bytes;
         br += cs.top_rows;
+        bp += cs.prog_bytes;
       } else {
         bundles.push_back({i});
         bs = cs.s_bytes;
@@ -603,29 +783,35 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
         bb = cs.pb_bytes;
         bt = cs.pt_bytes;
         br = cs.top_rows;
+        bp = cs.prog_bytes;
       }
     }
-    int64_t ms = 0, ma = 0, mb = 0, mt = 0, mr = 0;
+    int64_t ms = 0, ma = 0, mb = 0, mt = 0, mr = 0, mp = 0;
     for (const std::vector<int32_t> &bu : bundles) {
-      int64_t s1 = 0, a1 = 0, b1 = 0, t1 = 0, r1 = 0;
+      int64_t s1 = 0, a1 = 0, b1 = 0, t1 = 0, r1 = 0, p1 = 0;
       for (int32_t i : bu) {
         s1 += shapes[i].s_bytes;
         a1 += shapes[i].pa_bytes;
         b1 += shapes[i].pb_bytes;
         t1 += shapes[i].pt_bytes;
         r1 += shapes[i].top_rows;
+        p1 += shapes[i].prog_bytes;
       }
       ms = std::max(ms, s1);
       ma = std::max(ma, a1);
       mb = std::max(mb, b1);
       mt = std::max(mt, t1);
       mr = std::max(mr, r1);
+      mp = std::max(mp, p1);
     }
     const int64_t qb = search_q_bytes(f, mr);
-    const int64_t total = kBarrierBytes + ms + ma + mb + mt + qb + kDescBytes + kOverRead;
+    const int64_t slot = prog_slot_bytes(nst, mp);
+    const int64_t total = kBarrierBytes + ms + ma + mb + mt + qb + 2 * slot + kOverRead;
     if (total > budget && total > 227 * 1024 - 1024) continue;
     if (total > budget && cone_budget > 4096) continue;
     gb = GroupBuild();
+    gb.items = (int64_t)bundles.size();
+    gb.budget = budget;
     gb.g.lb = lb;
     gb.g.lt = lt;
     gb.g.W = W;
@@ -642,13 +828,28 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
     gb.g.q_row = (int32_t)qb;
     gb.g.ntiles = (nt + W - 1) / W;
     gb.g.smem_bytes = (int32_t)total;
+    gb.g.prog_slot = (int32_t)slot;
+    gb.g.prog_off = (int32_t)(total - kOverRead - 2 * slot);
     gb.g.s_end = (int32_t)(kBarrierBytes + ms);
     gb.g.pa_end = (int32_t)(kBarrierBytes + ms + ma);
-    double hbm = 0, sl = 0, nops = 0;
+    double hbm = 0, sl = 0, nops = 0, work = 0;
     for (const std::vector<int32_t> &bu : bundles) {
       // Each cone of the item gets its own slice of S, Pa and Pb; the item's
       // stage ops are merged stage by stage, then split over the warps.
       ItemOut item;
+      if (!emit) {
+        int32_t copies = 0;
+        for (int32_t i : bu) {
+          if (needs) needs->insert(needs->end(), shapes[i].needs.begin(), shapes[i].needs.end());
+          ConeOut c;
+          count_cone(t, lb, lt, W, fp, f, shapes[i], c, copies);
+          item.tpl.tx_bytes += c.tpl.tx_bytes;
+          hbm += c.hbm;
+          work += c.work;
+        }
+        work += item_work(nst, copies, item.tpl.tx_bytes);
+        continue;
+      }
       int64_t so = 0, ao = 0, bo = 0, to = 0;
       std::vector<ConeOut> cos;
       for (int32_t i : bu) {
@@ -666,6 +867,7 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
         item.hbm += c.hbm;
         item.slots += c.slots;
         item.nops += c.nops;
+        item.work += c.work;
         cos.push_back(std::move(c));
       }
       const std::vector<int32_t> &kinds = cos.front().kinds;
@@ -677,7 +879,7 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
           for (const ConeOut &c : cos)
             for (const FusedWalk &wk : c.walks) {
               item.walks.push_back(wk);
-              cost.push_back(3.0 * (wk.e - wk.a + 1 + wk.dl0) * kLaneCols + 2.0);
+              cost.push_back(walk_cost(wk));
             }
         } else {
           base = (int32_t)item.ops.size();
@@ -690,6 +892,22 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
               cost.push_back(kind == kStageSearch ? 1.0 : op_slots(kind, op.flags) * kLaneCols + 2.0);
             }
         }
+        StageRows rows;
+        const size_t rk = (lb == 0) ? si - 1 : si;
+        if ((kinds[si] & kStageKindMask) == kStageSingle || (kinds[si] & kStageKindMask) == kStagePair) {
+          int32_t at = base;
+          for (const ConeOut &c : cos) {
+            const int32_t s0 = (int32_t)rows.steps.size();
+            for (NodeRows nr : c.stage_rows[rk].nodes) {
+              nr.op += at;
+              nr.step += s0;
+              rows.nodes.push_back(nr);
+            }
+            rows.steps.insert(rows.steps.end(), c.stage_rows[rk].steps.begin(), c.stage_rows[rk].steps.end());
+            at += (int32_t)c.stage_ops[rk].size();
+          }
+        }
+        item.rows.push_back(std::move(rows));
         const std::vector<int32_t> b = split_warps(cost);
         bool general = false;
         if ((kinds[si] & kStageKindMask) == kStageWalk) {
@@ -711,22 +929,25 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
       hbm += item.hbm;
       sl += item.slots;
       nops += item.nops;
+      work += item.work + item_work(nst, (int32_t)item.loads.size(), item.tpl.tx_bytes);
       gb.cones.push_back(std::move(item));
     }
     gb.g.hbm_bytes = hbm * (double)gb.g.ntiles;
     gb.g.smem_traffic = sl * 128.0 * (double)gb.g.ntiles;
     const double tiles = (double)gb.g.ntiles;
-    const double items = (double)gb.cones.size() * tiles;
+    const double items = (double)gb.items * tiles;
     const double slots =
         kSms * std::min(kMaxBlocksPerSm, std::max(1.0, std::floor((228.0 * 1024) / (total + 1024.0))));
-    const double on_chip = sl * tiles * kSlotSeconds +
-                           (items * kItemSeconds + nops * tiles * kOpSeconds) / slots + kLaunchSeconds;
+    const double waves = items / slots;
+    const double on_chip = work / (double)gb.items * (items <= kSms ? kAloneShare : 1.0) *
+                           std::max(waves, std::min(std::ceil(waves), waves + kWaveTail));
     // DRAM sees each base row and each output row once (neighbouring cones'
     // halos and overlaps are L2 hits); the staged bytes go through L2.
     const double unique = (double)nt * ((lb == 0 ? (double)t.nf * fp.input_size
                                                   : (double)t.level_rows[lb] * fp.level_size[lb]) +
                                         (double)t.level_rows[lt] * fp.level_size[lt]);
-    gb.seconds = std::max({unique / kHbmRate, gb.g.hbm_bytes / kL2Rate, on_chip});
+    const double mem = std::max(unique / kHbmRate, gb.g.hbm_bytes / kL2Rate);
+    gb.seconds = kLaunchSeconds + std::pow(std::pow(on_chip, kNorm) + std::pow(mem, kNorm), 1.0 / kNorm);
     gb.g.ops = nops * tiles;
     gb.g.block_slots = slots;
     gb.g.seconds = gb.seconds;
@@ -740,7 +961,7 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
 // the group's own cones: a first build with provisional boxes measures
 // them, the second uses the chosen box or block width.
 GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int32_t W,
-                       const FusedPlan &fp, int32_t budget, int32_t staging, int32_t search_k) {
+                       const FusedPlan &fp, int32_t budget, int32_t staging, int32_t search_k, bool emit) {
   const int32_t es = (lb == 0) ? fp.input_size : fp.level_size[lb];
   const int64_t rows = (lb == 0) ? t.nf : t.level_rows[lb];
   // Row blocks: chunks of 128 bytes (64 for 1-byte samples, so that a tile
@@ -758,7 +979,7 @@ GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int3
     f.box = 128 / es;
   }
   std::vector<std::pair<int32_t, int32_t>> needs;
-  GroupBuild gb = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &needs);
+  GroupBuild gb = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &needs, false);
   if (!gb.ok) return gb;
   int32_t widest = 0;
   for (const auto &nr : needs) widest = std::max(widest, nr.first);
@@ -773,25 +994,137 @@ GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int3
       if (k > 256 || (int64_t)k * chunk > nt) break;
       f.kchunks = std::max(f.kchunks, k);
       std::vector<std::pair<int32_t, int32_t>> got;
-      GroupBuild g2 = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &got);
+      GroupBuild g2 = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &got, false);
       if (!g2.ok) break;
       widest = 0;
       for (const auto &nr : got) widest = std::max(widest, nr.first);
-      if (widest <= f.kchunks * chunk) return g2;
+      if (widest <= f.kchunks * chunk)
+        return emit ? build_group_fmt(t, nt, lb, lt, W, fp, budget, f, nullptr, true) : g2;
     }
     if (staging == 2) return GroupBuild();
     f = StageFmt();  // fall back to row boxes
     f.search_k = search_k;
     f.box = 128 / es;
     needs.clear();
-    gb = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &needs);
+    gb = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &needs, false);
     if (!gb.ok) return gb;
   }
   f.box = choose_box(needs, es);
-  return build_group_fmt(t, nt, lb, lt, W, fp, budget, f, nullptr);
+  return build_group_fmt(t, nt, lb, lt, W, fp, budget, f, nullptr, emit);
 }
 
-void append_group(FusedPlan &fp, GroupBuild &gb) {
+// Shared-memory pipe slots per 32 columns of the first row of a run (all its
+// sources, the store) and of a later row (one half's sources, on average 1.5
+// of a pair's two, the store).
+double run_first_cost(bool pair) { return pair ? 5.5 : 3.5; }
+double run_step_cost(bool pair) { return pair ? 2.75 : 2.25; }
+
+// Lowers a stage's rows to runs split over the warps at about equal cost.
+// A node's rows are first cut into chunks whose delay growth is at most
+// kRunGrow and still fits the columns left free in the node's last strip (a
+// strip moves a column with every step of the lower row, so more growth
+// would take one more strip); the strips of all chunks, in order, are then dealt to the warps, each warp
+// taking rows up to the smallest cost at which the block's warps suffice.
+// dst_moves: the rows go to plain rows of shared memory (dst at column col).
+void lower_stage(const StageRows &sr, const std::vector<FusedOp> &ops, bool pair, bool dst_moves,
+                 std::vector<FusedRun> &runs, int32_t begin[kFusedBlockWarps + 1]) {
+  struct Strip {
+    int32_t node, first, n, col;  // rows first .. first + n - 1 of the node; column of the first row
+  };
+  std::vector<Strip> strips;
+  for (size_t i = 0; i < sr.nodes.size(); ++i) {
+    const NodeRows &nr = sr.nodes[i];
+    const int32_t free_cols = (nr.width + kPieceCols - 1) / kPieceCols * kPieceCols - nr.width;
+    const bool moves = !(nr.flags & kOpNoHi);  // rows without an upper half keep their columns
+    for (int32_t r = 0; r < nr.n;) {
+      int32_t grow = 0, k = 1;
+      while (r + k < nr.n && k < kRunRows) {
+        const int32_t inc = moves ? sr.steps[nr.step + r + k - 1] & 1 : 0;
+        if (grow + inc > kRunGrow || (grow + inc > free_cols && free_cols >= 8)) break;
+        grow += inc;
+        ++k;
+      }
+      for (int32_t c = -grow; c < nr.width; c += kPieceCols) strips.push_back(Strip{(int32_t)i, r, k, c});
+      r += k;
+    }
+  }
+  auto deal = [&](double cap, std::vector<FusedRun> *out) {
+    int32_t w = 0;
+    double load = 0;
+    if (out) begin[0] = (int32_t)out->size();
+    for (const Strip &s : strips) {
+      const NodeRows &nr = sr.nodes[s.node];
+      int32_t col = s.col;
+      for (int32_t r = 0; r < s.n;) {
+        // rows this warp still takes (at least one if it has none)
+        const double room = cap - load - run_first_cost(pair);
+        int32_t k = room < 0 ? 0 : std::min<int32_t>(s.n - r, 1 + (int32_t)(room / run_step_cost(pair)));
+        if (k < 1) {
+          if (load > 0) {
+            if (++w >= kFusedBlockWarps) return false;
+            if (out) begin[w] = (int32_t)out->size();
+            load = 0;
+            continue;
+          }
+          k = 1;
+        }
+        FusedRun run{};
+        int32_t moved = 0;
+        const uint8_t *st = sr.steps.data() + nr.step + s.first + r;
+        for (int32_t i = 0; i < k; ++i) {
+          if (s.first + r + i + 1 >= nr.n) break;
+          const int32_t inc = st[i] & 1;
+          if (i + 1 < k) {
+            run.inc |= (uint32_t)inc << i;
+            run.sub |= (uint32_t)(st[i] >> 1) << i;
+          }
+          moved += nr.flags & kOpNoHi ? 0 : inc;  // columns moved by the row after this part
+        }
+        if (out) {
+          const FusedOp &op = ops[nr.op + s.first + r];
+          run.dst = dst_moves ? op.dst + col * 4 : op.dst;
+          run.dst_row = nr.pitch * 4;
+          run.col = col;
+          run.width = nr.width;
+          run.p0 = op.p0 + col * nr.es;
+          run.p1 = op.p1 + col * nr.es;
+          run.p2 = (pair ? op.p2 : op.p1) + col * nr.es;
+          run.p3 = op.p3 + col * nr.es;
+          if (!pair) run.p1 = run.p3 = 0;
+          if (nr.flags & kOpLoOne) run.p1 = 0;
+          if (nr.flags & kOpHiOne) run.p3 = 0;
+          if (nr.flags & kOpNoHi) run.p2 = run.p3 = 0;
+          run.g0 = nr.g[0];
+          run.g1 = nr.g[1];
+          run.g2 = nr.g[2];
+          run.g3 = nr.g[3];
+          run.n = k;
+          run.flags = nr.flags;
+          if (dst_moves && nr.pitch % kPieceCols == 0) run.flags |= kRunWhole;
+          out->push_back(run);
+        }
+        load += run_first_cost(pair) + (k - 1) * run_step_cost(pair);
+        col += moved;
+        r += k;
+      }
+    }
+    if (out)
+      while (w < kFusedBlockWarps) begin[++w] = (int32_t)out->size();
+    return true;
+  };
+  double total = 0;
+  for (const Strip &s : strips) total += run_first_cost(pair) + (s.n - 1) * run_step_cost(pair);
+  double lo = total / kFusedBlockWarps, hi = std::max(lo, run_first_cost(pair));
+  while (!deal(hi, nullptr)) hi *= 1.25;
+  while (hi - lo > 0.5) {
+    const double mid = 0.5 * (lo + hi);
+    if (deal(mid, nullptr)) hi = mid; else lo = mid;
+  }
+  deal(hi, &runs);
+}
+
+// False if a programme outgrows the room its group has for it.
+bool append_group(FusedPlan &fp, GroupBuild &gb) {
   FusedGroup g = gb.g;
   g.tpl_begin = (int32_t)fp.tpls.size();
   g.tpl_count = (int32_t)gb.cones.size();
@@ -808,13 +1141,50 @@ void append_group(FusedPlan &fp, GroupBuild &gb) {
       fp.general |= (c.stages[i] & kStageGeneral) != 0;
       fp.stages.push_back(c.stages[i]);
       for (int32_t w = 1; w < kStageWords; ++w) fp.stages.push_back(c.stages[i + w] + off);
+      const int32_t kind = c.stages[i] & kStageKindMask;
+      if (kind == kStageSingle || kind == kStagePair) {
+        const bool dst_moves = i + kStageWords < c.stages.size() && !(c.stages[i] & kStagePadded);
+        int32_t begin[kFusedBlockWarps + 1];
+        lower_stage(c.rows[i / kStageWords], c.ops, kind == kStagePair, dst_moves, fp.runs, begin);
+        fp.run_stages.push_back(c.stages[i] | kStageRuns);
+        fp.run_stages.insert(fp.run_stages.end(), begin, begin + kFusedBlockWarps + 1);
+      } else {
+        fp.run_stages.insert(fp.run_stages.end(), fp.stages.end() - kStageWords, fp.stages.end());
+      }
     }
+    FusedProg pr{};
+    pr.load_begin = tp.load_begin;
+    pr.load_count = tp.load_count;
+    pr.n_stages = tp.n_stages;
+    pr.prog = (int32_t)(fp.prog.size() / 4);
+    std::vector<int32_t> words((size_t)tp.n_stages * (kProgStageBytes / 4), 0);
+    for (int32_t st = 0; st < tp.n_stages; ++st) {
+      const int32_t *src = fp.run_stages.data() + tp.stage_begin + st * kStageWords;
+      const size_t at = (size_t)st * (kProgStageBytes / 4);
+      const int32_t kind = src[0] & kStageKindMask;
+      words[at] = src[0];
+      if (kind == kStageSearch) {
+        for (int32_t w = 1; w < kStageWords; ++w) words[at + w] = src[w];
+        continue;
+      }
+      const int32_t size = kind == kStageWalk ? (int32_t)sizeof(FusedWalk) : (int32_t)sizeof(FusedRun);
+      for (int32_t w = 1; w < kStageWords; ++w) words[at + w] = (int32_t)words.size() * 4 + (src[w] - src[1]) * size;
+      const int32_t *d = kind == kStageWalk ? reinterpret_cast<const int32_t *>(c.walks.data() + (src[1] - w0))
+                                            : reinterpret_cast<const int32_t *>(fp.runs.data() + src[1]);
+      words.insert(words.end(), d, d + (size_t)(src[kStageWords - 1] - src[1]) * size / 4);
+    }
+    pr.prog_bytes = (int32_t)words.size() * 4;
+    pr.tx_bytes = tp.tx_bytes + pr.prog_bytes;
+    if (pr.prog_bytes > g.prog_slot) return false;
+    fp.prog.insert(fp.prog.end(), words.begin(), words.end());
+    fp.progs.push_back(pr);
     fp.loads.insert(fp.loads.end(), c.loads.begin(), c.loads.end());
     fp.walks.insert(fp.walks.end(), c.walks.begin(), c.walks.end());
     fp.ops.insert(fp.ops.end(), c.ops.begin(), c.ops.end());
     fp.tpls.push_back(tp);
   }
   fp.groups.push_back(g);
+  return true;
 }
 
 }  // namespace
@@ -827,7 +1197,8 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
     if (p.W % 64 != 0) return "tile width must be a multiple of 64";
     widths.push_back(p.W);
   } else {
-    widths = {128, 256, 384, 448, 512, 960, 1024};
+    // (whole strips of 256 columns less the windows' growth, and small ones)
+    widths = {64, 128, 192, 256, 384, 448, 704, 960};
   }
   if (p.search_k < 0 || p.search_k > kSearchMaxWidths || (p.search_k > 0 && L < 2))
     return "the search in the last launch takes 1 .. 9 widths and at least two merge levels";
@@ -851,14 +1222,25 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
       if (255LL * ((1LL << l) + rmax - 1) <= 65535 && (nt * 2) % 16 == 0) fp.level_size[l] = 2;
     }
   }
-  // Best tile for one group (lb, lt] (optionally a given tile and budget).
-  auto best_segment = [&](int32_t lb, int32_t lt, int32_t forced_W = 0, int32_t budget = 0) {
+  // Best tile for one group (lb, lt] (optionally a given tile and budget),
+  // counted only.
+  auto best_segment = [&](int32_t lb, int32_t lt, int32_t forced_W = 0, int32_t budget = 0, bool refine = false) {
     GroupBuild best;
     const std::vector<int32_t> ws = forced_W > 0 ? std::vector<int32_t>{forced_W} : widths;
     for (int32_t W : ws) {
+      if (best.ok && W / 2 >= nt) break;  // (no wider than one tile needs)
       GroupBuild gb = build_group(t, nt, lb, lt, W, fp, budget > 0 ? budget : p.smem_budget, p.staging,
-                                  lt == L ? p.search_k : 0);
+                                  lt == L ? p.search_k : 0, false);
       if (gb.ok && (!best.ok || gb.seconds < best.seconds)) best = std::move(gb);
+    }
+    // Few items leave SMs idle: smaller ones (more row ranges) may be faster
+    // (tried once the boundaries stand).
+    for (int32_t kib = 56; refine && budget == 0 && p.smem_budget == FusedParams().smem_budget && kib >= 14; kib /= 2) {
+      if (!best.ok || best.items * best.g.ntiles >= best.g.block_slots) break;
+      for (int32_t W : ws) {
+        GroupBuild gb = build_group(t, nt, lb, lt, W, fp, kib * 1024, p.staging, lt == L ? p.search_k : 0, false);
+        if (gb.ok && gb.seconds < best.seconds) best = std::move(gb);
+      }
     }
     return best;
   };
@@ -892,10 +1274,13 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
     const int32_t gw = i < p.group_W.size() ? p.group_W[i] : 0;
     const int32_t gbud = i < p.group_budget.size() ? p.group_budget[i] : 0;
     if (gw < 0 || gw % 64 != 0 || gbud < 0 || gbud > 227 * 1024) return "bad per-group parameters";
-    GroupBuild gb = best_segment(bounds[i], bounds[i + 1], gw, gbud);
+    GroupBuild gb = best_segment(bounds[i], bounds[i + 1], gw, gbud, true);
+    if (gb.ok)
+      gb = build_group(t, nt, bounds[i], bounds[i + 1], gb.g.W, fp, gb.budget, p.staging,
+                       bounds[i + 1] == L ? p.search_k : 0, true);
     if (!gb.ok) return "a level group does not fit the shared-memory budget";
     secs += gb.seconds;
-    append_group(fp, gb);
+    if (!append_group(fp, gb)) return "a programme outgrew its slot";
   }
   fp.W = fp.groups.front().W;
   fp.model_seconds = secs;

@@ -74,11 +74,10 @@ struct DeviceTables {
   int32_t descending = 0;
   // Fused schedule (null unless the plan was made with FDMT_SCHED_FUSED).
   const FusedPlan *fused = nullptr;
-  FusedTemplate *f_tpls = nullptr;
+  FusedProg *f_progs = nullptr;
+  int32_t *f_prog = nullptr;
   FusedLoad *f_loads = nullptr;
-  FusedWalk *f_walks = nullptr;
-  FusedOp *f_ops = nullptr;
-  int32_t *f_stages = nullptr;
+  FusedOp *f_ops = nullptr;  // a search stage's rows (plans that search in the last launch)
   // Fused adjoint (null unless the plan has one).
   const AdjFusedPlan *adj_fused = nullptr;
   FusedTemplate *a_tpls = nullptr;
