@@ -11,9 +11,11 @@
 // float32 with that tree order, so every B value is bit-identical to a plain
 // evaluation of the recursion.
 //
-// Two kernels.
+// Two kernels: one that streams the rows, and the finalize step.
 //
-// search_kernel streams the rows.  Work items are (row, segment of `seg`
+// search_warp_kernel streams them for up to 9 widths with 4-byte sums (see
+// there).  search_kernel does for wider searches (a window's history is then
+// several times a warp's 1024 columns) and for int64 sums.  Work items are (row, segment of `seg`
 // samples), row-major; each persistent block takes a contiguous range of
 // items, so it walks along a few rows and the history below each segment
 // (`halo` >= 2^(K-1) - 1 samples) was read by the same block just before.
@@ -279,11 +281,10 @@ __device__ __forceinline__ void flush_row(TB (&bv)[kMaxWidths], int (&br)[kMaxWi
   // red is rewritten at the next flush, after the next item's barriers.
 }
 
-// MINB = resident blocks per SM the registers must allow: 3 for the
-// narrow windows of K <= 9 with 4-byte sums (shared memory allows more), 1
-// for K >= 10 (one block's windows fill the SM) and for int64 sums.
-template <class TA, class TB, int MINB>
-__global__ void __launch_bounds__(kSearchThreads, MINB)
+// (one resident block per SM is what the registers must allow: a block's
+// windows fill the SM for K >= 10)
+template <class TA, class TB>
+__global__ void __launch_bounds__(kSearchThreads, 1)
 search_kernel(const TA *__restrict__ A, int nt, int nk, SearchGeom g, int nseg, int items, int per_block, int vec,
               TB *__restrict__ part_v, int *__restrict__ part_r) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -484,6 +485,217 @@ search_finalize_kernel(const TA *__restrict__ A, int nt, int nk, int nseg, const
   }
 }
 
+// ---------------------------------------------------------------------------
+// K <= 9 widths with 4-byte sums: one warp per window of 1024 columns, 32
+// consecutive columns per lane in registers.  B_2w[t] = B_w[t] + B_w[t - w]:
+// for w < 32 the first w columns of a lane come from the lane below (31
+// shuffles for the widths 2 .. 32), for wider ones all 32 from the lane w /
+// 32 below.  The first `halo` >= 2^(K-1) - 1 columns of a window are the
+// history of the others.  Windows come into a warp's own two buffers by
+// cp.async, coalesced, and are read back 32 columns per lane (4 words of
+// padding per lane against bank conflicts); warps never wait for each other.
+// A warp walks kWarpWindows windows of a row, keeps per lane and width the
+// largest value and the region (16 samples up to width 16, else the lane's
+// run, a part of the 256 samples the finalize step searches from there)
+// where it first saw it, and writes one partial per width.
+// Bound: instruction issue and HBM alike (12 instructions per column for
+// eight widths, float sums two at a time, maxima three operands at a time).
+// Both kernels of a call on a 1024 x 65536 float32 output, K = 8, on a
+// GB300: 185 us with the block kernel above, 89 us with
+// this one.
+
+constexpr int kWarpCols = 1024;
+constexpr int kWarpRun = 32;                       // columns per lane
+constexpr int kWarpPitch = kWarpRun + 4;           // words per lane in a buffer
+constexpr int kWarpWindows = 8;                    // windows of one walk
+constexpr int kWarpMaxWidths = 9;
+constexpr size_t kWarpSmem = (size_t)kWarps * 2 * 32 * kWarpPitch * 4;
+
+// History columns of a warp's window: whole lanes.
+int warp_halo(int nk) { return ((1 << (nk - 1)) - 1 + kWarpRun - 1) / kWarpRun * kWarpRun; }
+int64_t warp_windows(int64_t nt, int nk) {
+  const int own = kWarpCols - warp_halo(nk);
+  return (nt + own - 1) / own;
+}
+
+__device__ __forceinline__ float vmax3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ int32_t vmax3(int32_t a, int32_t b, int32_t c) { return max(max(a, b), c); }
+
+// a += b for two neighbouring columns, each sum rounded by itself.
+__device__ __forceinline__ void add_two(float &a0, float &a1, float b0, float b1) {
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %3};\n\t"
+      "add.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void add_two(int32_t &a0, int32_t &a1, int32_t b0, int32_t b1) {
+  a0 += b0;
+  a1 += b1;
+}
+
+// The largest of v[at .. at + 15].
+template <class T>
+__device__ __forceinline__ T max16(const T (&v)[kWarpRun], int at) {
+  T a = vmax3(v[at], v[at + 1], v[at + 2]), b = vmax3(v[at + 3], v[at + 4], v[at + 5]);
+  T c = vmax3(v[at + 6], v[at + 7], v[at + 8]), d = vmax3(v[at + 9], v[at + 10], v[at + 11]);
+  a = vmax3(a, v[at + 12], v[at + 13]);
+  b = vmax3(b, v[at + 14], v[at + 15]);
+  return vmax(vmax3(a, b, c), d);
+}
+
+// B_w (v, width index k - 1, w = 2^(k-1)) -> B_2w.
+template <int W, class T>
+__device__ __forceinline__ void double_width(T (&v)[kWarpRun]) {
+  if constexpr (W < kWarpRun) {
+    T below[W];
+#pragma unroll
+    for (int j = 0; j < W; ++j) below[j] = __shfl_up_sync(0xffffffffu, v[kWarpRun - W + j], 1);
+    if constexpr (W == 1) {
+#pragma unroll
+      for (int i = kWarpRun - 1; i >= 1; --i) v[i] = add_tree(v[i], v[i - 1]);
+      v[0] = add_tree(v[0], below[0]);
+    } else {
+#pragma unroll
+      for (int i = kWarpRun - 2; i >= W; i -= 2) add_two(v[i], v[i + 1], v[i - W], v[i + 1 - W]);
+#pragma unroll
+      for (int i = 0; i < W; i += 2) add_two(v[i], v[i + 1], below[i], below[i + 1]);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < kWarpRun; i += 2) {
+      const T a = __shfl_up_sync(0xffffffffu, v[i], W / kWarpRun);
+      const T b = __shfl_up_sync(0xffffffffu, v[i + 1], W / kWarpRun);
+      add_two(v[i], v[i + 1], a, b);
+    }
+  }
+}
+
+template <class T>
+struct WarpBest {
+  T v[kWarpMaxWidths];
+  int r[kWarpMaxWidths];
+};
+
+// B_w of width index k joins the lane's best: columns [lo, hi) of its 32 are
+// the window's own; t = time of column 0.
+template <int K, class T>
+__device__ __forceinline__ void warp_track(const T (&v)[kWarpRun], int lo, int hi, int t, WarpBest<T> &best) {
+  if (lo >= hi) return;
+  T m0, m1;
+  if (lo == 0 && hi == kWarpRun) {
+    m0 = max16(v, 0);
+    m1 = max16(v, 16);
+  } else {
+    m0 = m1 = lowest<T>();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (i >= lo && i < hi) m0 = vmax(m0, v[i]);
+      if (i + 16 >= lo && i + 16 < hi) m1 = vmax(m1, v[i + 16]);
+    }
+  }
+  const T m = vmax(m0, m1);
+  if (m > best.v[K]) {
+    best.v[K] = m;
+    best.r[K] = K <= 4 && !(m0 == m) ? t + 16 : t;
+  }
+}
+
+// Widths K and on.
+template <int K, class T>
+__device__ __forceinline__ void warp_widths(T (&v)[kWarpRun], int nk, int lo, int hi, int t, WarpBest<T> &best) {
+  if constexpr (K < kWarpMaxWidths) {
+    if (K >= nk) return;
+    double_width<(1 << (K - 1))>(v);
+    warp_track<K>(v, lo, hi, t, best);
+    warp_widths<K + 1>(v, nk, lo, hi, t, best);
+  }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kSearchThreads, 3)
+search_warp_kernel(const T *__restrict__ A, int nt, int nk, int halo, int nwin, int nseg, int items, int vec,
+                   T *__restrict__ part_v, int *__restrict__ part_r) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  T *const buf = reinterpret_cast<T *>(smem) + warp * 2 * 32 * kWarpPitch;
+  const int own = kWarpCols - halo;
+  // Window w of row d into buffer b: column c at word c + 4 (c / 32).
+  auto stage = [&](int d, int w, int b) {
+    const T *row = A + (int64_t)d * nt;
+    T *dst = buf + b * 32 * kWarpPitch;
+    const int t0 = w * own - halo;
+    if (vec) {
+#pragma unroll
+      for (int i = 0; i < kWarpCols / 128; ++i) {
+        const int c = 4 * lane + 128 * i, t = t0 + c;
+        const bool in = t >= 0 && t < nt;  // nt % 4 == 0: a vector is all in or all out
+        cp_async16(dst + c + 4 * (c >> 5), in ? row + t : row, in ? 16 : 0);
+      }
+    } else {
+#pragma unroll 4
+      for (int i = 0; i < kWarpRun; ++i) {
+        const int t = t0 + lane + 32 * i;
+        dst[lane + kWarpPitch * i] = t >= 0 && t < nt ? row[t] : T(0);
+      }
+    }
+    cp_async_commit();
+  };
+  for (int item = blockIdx.x * kWarps + warp; item < items; item += gridDim.x * kWarps) {
+    const int d = item / nseg, s = item - d * nseg;
+    const int w0 = s * kWarpWindows, w1 = min(w0 + kWarpWindows, nwin);
+    WarpBest<T> best;
+#pragma unroll
+    for (int k = 0; k < kWarpMaxWidths; ++k) {
+      best.v[k] = lowest<T>();
+      best.r[k] = kNoRegion;
+    }
+    stage(d, w0, 0);
+    for (int w = w0; w < w1; ++w) {
+      const int b = (w - w0) & 1;
+      if (w + 1 < w1) {
+        stage(d, w + 1, b ^ 1);
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
+      }
+      __syncwarp();
+      T v[kWarpRun];
+      const int4 *src = reinterpret_cast<const int4 *>(buf + (b * 32 + lane) * kWarpPitch);
+#pragma unroll
+      for (int i = 0; i < kWarpRun / 4; ++i) {
+        const int4 q = src[i];
+        const T *p = reinterpret_cast<const T *>(&q);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[4 * i + e] = p[e];
+      }
+      const int t = w * own - halo + lane * kWarpRun;
+      const int lo = lane * kWarpRun >= halo ? 0 : kWarpRun;
+      const int hi = min(kWarpRun, nt - t);
+      warp_track<0>(v, lo, hi, t, best);
+      warp_widths<1>(v, nk, lo, hi, t, best);
+      __syncwarp();  // the buffer is refilled two windows on
+    }
+    // One partial per width: the largest value, then the earliest region.
+#pragma unroll
+    for (int k = 0; k < kWarpMaxWidths; ++k) {
+      if (k >= nk) break;
+      T m = best.r[k] == kNoRegion ? lowest<T>() : best.v[k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = vmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+      const int r = best.r[k] != kNoRegion && best.v[k] == m ? best.r[k] : INT32_MAX;
+      const int first = __reduce_min_sync(0xffffffffu, r);
+      if (lane == 0) {
+        const int64_t slot = ((int64_t)d * nk + k) * nseg + s;
+        part_v[slot] = m;
+        part_r[slot] = first == INT32_MAX ? kNoRegion : first;
+      }
+    }
+  }
+}
+
 int halo_of(int nk) { return ((1 << (nk - 1)) - 1 + 15) / 16 * 16; }
 
 // Columns each phase produces: what the later phases read (the rest of the
@@ -537,49 +749,18 @@ SearchGeom choose_geom(int nk, int64_t nt, size_t ta, size_t tb) {
   return best;
 }
 
-template <class TA, class TB, class TP>
-cudaError_t launch_search(const void *A, int32_t nd, int64_t nt, int32_t nk, void *peak, int32_t *time, void *ws,
-                          cudaStream_t s) {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  const SearchGeom g = choose_geom(nk, nt, sizeof(TA), sizeof(TB));
-  const size_t smem = smem_of(g, nk, sizeof(TA), sizeof(TB));
-  void (*kern)(const TA *, int, int, SearchGeom, int, int, int, int, TB *, int *) = search_kernel<TA, TB, 1>;
-  if constexpr (sizeof(TB) == 4) {
-    if (nk <= 9) kern = search_kernel<TA, TB, 3>;
-  }
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-    return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSearchThreads, smem)) != cudaSuccess)
-    return e;
-  const int nseg = (int)((nt + g.seg - 1) / g.seg);
-  const int items = nd * nseg;
-  const int grid0 = std::min(items, sms * std::max(per_sm, 1));
-  const int per_block = (items + grid0 - 1) / grid0;
-  const int grid = (items + per_block - 1) / per_block;
-  TB *part_v = static_cast<TB *>(ws);
-  int *part_r = reinterpret_cast<int *>(static_cast<char *>(ws) + (size_t)nd * nk * nseg * sizeof(int64_t));
-  const int vec = (nt % 4 == 0) && (reinterpret_cast<uintptr_t>(A) % 16 == 0);
-  kern<<<grid, kSearchThreads, smem, s>>>(static_cast<const TA *>(A), (int)nt, nk, g, nseg, items, per_block, vec,
-                                          part_v, part_r);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // Widths up to 256 need one warp each (and its slice of shared memory);
-  // wider ones the whole block and the widest region.
-  const int fwarps = nk <= 9 ? std::min(nk, kWarps) : kWarps;
-  const size_t fsmem = (nk <= 9 ? (size_t)fwarps * kFinalizeWarpElems : (size_t)kFinalizeElems) * sizeof(TB);
-  auto fin = search_finalize_kernel<TA, TB, TP>;
-  if ((e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem)) != cudaSuccess)
-    return e;
-  fin<<<nd, 32 * fwarps, fsmem, s>>>(static_cast<const TA *>(A), (int)nt, nk, nseg, part_v, part_r,
-                                        static_cast<TP *>(peak), time);
-  return cudaGetLastError();
+// Partial slots per row: a warp's walks, or the block kernel's segments.
+int64_t search_segments(bool wide, int64_t nt, int32_t nk) {
+  if (!wide && nk <= kWarpMaxWidths) return (warp_windows(nt, nk) + kWarpWindows - 1) / kWarpWindows;
+  const SearchGeom g = choose_geom(nk, nt, 4, wide ? 8 : 4);
+  return (nt + g.seg - 1) / g.seg;
 }
 
 template <class TA, class TB, class TP>
 cudaError_t launch_finalize(const void *A, int32_t nd, int64_t nt, int32_t nk, int32_t nseg, const void *part_v,
                             const int *part_r, void *peak, int32_t *time, cudaStream_t s) {
+  // Widths up to 256 need one warp each (and its slice of shared memory);
+  // wider ones the whole block and the widest region.
   const int fwarps = nk <= 9 ? std::min(nk, kWarps) : kWarps;
   const size_t fsmem = (nk <= 9 ? (size_t)fwarps * kFinalizeWarpElems : (size_t)kFinalizeElems) * sizeof(TB);
   auto fin = search_finalize_kernel<TA, TB, TP>;
@@ -590,6 +771,48 @@ cudaError_t launch_finalize(const void *A, int32_t nd, int64_t nt, int32_t nk, i
   return cudaGetLastError();
 }
 
+template <class TA, class TB, class TP>
+cudaError_t launch_search(const void *A, int32_t nd, int64_t nt, int32_t nk, void *peak, int32_t *time, void *ws,
+                          cudaStream_t s) {
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  TB *part_v = static_cast<TB *>(ws);
+  const int nseg = (int)search_segments(sizeof(TB) == 8, nt, nk);
+  int *part_r = reinterpret_cast<int *>(static_cast<char *>(ws) + (size_t)nd * nk * nseg * sizeof(int64_t));
+  const int vec = (nt % 4 == 0) && (reinterpret_cast<uintptr_t>(A) % 16 == 0);
+  const int items = nd * nseg;
+  if constexpr (sizeof(TB) == 4) {
+    if (nk <= kWarpMaxWidths) {
+      auto kern = search_warp_kernel<TB>;
+      if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWarpSmem)) != cudaSuccess)
+        return e;
+      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSearchThreads, kWarpSmem)) != cudaSuccess)
+        return e;
+      const int grid = std::min((items + kWarps - 1) / kWarps, sms * std::max(per_sm, 1));
+      kern<<<grid, kSearchThreads, kWarpSmem, s>>>(static_cast<const TB *>(A), (int)nt, nk, warp_halo(nk),
+                                                   (int)warp_windows(nt, nk), nseg, items, vec, part_v, part_r);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      return launch_finalize<TA, TB, TP>(A, nd, nt, nk, nseg, part_v, part_r, peak, time, s);
+    }
+  }
+  const SearchGeom g = choose_geom(nk, nt, sizeof(TA), sizeof(TB));
+  const size_t smem = smem_of(g, nk, sizeof(TA), sizeof(TB));
+  auto kern = search_kernel<TA, TB>;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSearchThreads, smem)) != cudaSuccess)
+    return e;
+  const int grid0 = std::min(items, sms * std::max(per_sm, 1));
+  const int per_block = (items + grid0 - 1) / grid0;
+  const int grid = (items + per_block - 1) / per_block;
+  kern<<<grid, kSearchThreads, smem, s>>>(static_cast<const TA *>(A), (int)nt, nk, g, nseg, items, per_block, vec,
+                                          part_v, part_r);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return launch_finalize<TA, TB, TP>(A, nd, nt, nk, nseg, part_v, part_r, peak, time, s);
+}
+
 }  // namespace
 
 cudaError_t search_finalize(int dtype, bool wide, const void *A, int32_t nd, int64_t nt, int32_t nk, int32_t nseg,
@@ -598,13 +821,6 @@ cudaError_t search_finalize(int dtype, bool wide, const void *A, int32_t nd, int
   if (wide)
     return launch_finalize<int32_t, int64_t, int64_t>(A, nd, nt, nk, nseg, part_v, part_r, peak, time, s);
   return launch_finalize<int32_t, int32_t, int64_t>(A, nd, nt, nk, nseg, part_v, part_r, peak, time, s);
-}
-
-// Segments per row (the launch picks the same geometry from the same
-// arguments).
-int64_t search_segments(bool wide, int64_t nt, int32_t nk) {
-  const SearchGeom g = choose_geom(nk, nt, 4, wide ? 8 : 4);
-  return (nt + g.seg - 1) / g.seg;
 }
 
 }  // namespace fdmt
