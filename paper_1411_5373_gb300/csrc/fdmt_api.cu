@@ -195,6 +195,10 @@ int fdmt_plan_curve(double f_min, double f_max, int32_t nf, int64_t nt, int32_t 
   }
   const Tables &t = p->host;
   const int L = t.levels;
+  p->d_min = d_min;
+  p->descending = descending;
+  p->mapped = d_min > 0 || descending != 0;
+  if (p->mapped) p->in_shift = fdmt::input_shifts(f_min, f_max, nf, d_min, gamma);
   pingpong_sizes(t, nt, state_elem(dtype), L - 1, &p->ws_split, &p->ws_bytes);
   adjoint_ws_sizes(t, nt, &p->adj_ws_split, &p->adj_ws_bytes);
   if (flags & FDMT_SCHED_FUSED) {
@@ -204,6 +208,8 @@ int fdmt_plan_curve(double f_min, double f_max, int32_t nf, int64_t nt, int32_t 
     }
     fdmt::FusedParams fparams;
     fparams.narrow = (dtype == FDMT_U8_I32);
+    if (p->mapped) fparams.in_shift = &p->in_shift;
+    fparams.descending = descending != 0;
     if (params != nullptr) {
       if (params->tile < 0 || params->tile % 64 != 0 || params->smem_budget < 0 ||
           params->smem_budget > 227 * 1024 || params->n_bounds < 0 || params->n_bounds > 32 ||
@@ -306,13 +312,10 @@ int fdmt_plan_curve(double f_min, double f_max, int32_t nf, int64_t nt, int32_t 
     }
   }
 
-  p->d_min = d_min;
-  p->descending = descending;
-  p->mapped = d_min > 0 || descending != 0;
   if (p->mapped) {
-    p->in_shift = fdmt::input_shifts(f_min, f_max, nf, d_min, gamma);
+    // (a fused transform reads the raw input through its first launch's copies)
     p->map_off = round_up(p->has_fused ? p->fused_ws_bytes : p->ws_bytes, kAlign);
-    p->map_bytes = round_up((size_t)nf * (size_t)nt * input_elem(dtype), kAlign);
+    p->map_bytes = p->has_fused ? 0 : round_up((size_t)nf * (size_t)nt * input_elem(dtype), kAlign);
     p->adj_map_off = round_up(p->adj_ws_bytes, kAlign);
     p->adj_map_bytes = 2 * round_up((size_t)nf * (size_t)nt * sizeof(float), kAlign);
   }
@@ -412,7 +415,7 @@ int fdmt_execute(fdmt_plan_t plan, const void *in, const float *weights, void *o
   if (in == nullptr || out == nullptr || !aligned16(in) || !aligned16(out)) return FDMT_ERR_INVALID_ARG;
   if (weights != nullptr && plan->dtype == FDMT_U8_I32) return FDMT_ERR_INVALID_ARG;
   cudaError_t e = cudaSuccess;
-  if (plan->mapped) {
+  if (plan->mapped && !plan->has_fused) {
     // The transform reads the mapped input (channels ascending, d_min pre-shift).
     void *mapped = static_cast<char *>(workspace) + plan->map_off;
     e = fdmt::map_input(plan->dev, plan->dtype, in, mapped, plan->nt, static_cast<cudaStream_t>(stream));

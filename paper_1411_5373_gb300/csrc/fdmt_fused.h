@@ -258,6 +258,10 @@ struct FusedParams {
   int32_t staging = 0;                // 0 = row blocks where nt allows, 1 = row boxes, 2 = row blocks
   bool narrow = false;                // store launch-boundary levels whose uint8 sums fit as uint16
   int32_t search_k = 0;               // boxcar widths searched by the last launch (0 = none)
+  // Input mapping (d_min, channel order): the first launch's copies read
+  // channel k at row nf - 1 - k (descending) and in_shift[k] samples earlier.
+  const std::vector<int32_t> *in_shift = nullptr;
+  bool descending = false;
 };
 
 struct FusedPlan {

@@ -117,6 +117,9 @@ struct StageFmt {
   int32_t chunk = 0, kchunks = 0;
   int32_t max_p = 0;  // copies bring at most 2^max_p rows
   int32_t search_k = 0;  // > 0: the launch ends with the boxcar search of this many widths
+  const std::vector<int32_t> *in_shift = nullptr;  // mapped input (row boxes): each channel's delay
+  bool descending = false;
+  int32_t shift(int32_t channel) const { return in_shift != nullptr ? (*in_shift)[channel] : 0; }
 };
 
 }  // namespace
@@ -230,8 +233,9 @@ void shape_cone(const Tables &t, int32_t lb, int32_t lt, int32_t band, int32_t r
           n.xsmem = (int32_t)cs.s_bytes;
           cs.s_bytes += (int64_t)n.xstride * sI;
         } else {
-          const int32_t ceil_oe = (int32_t)ceil_to(n.o + n.e, alignI);
-          n.xdelta = ceil_oe - n.o;
+          // (a mapped channel is read its delay earlier: zeros before the raw row)
+          const int32_t at = n.o + f.shift(n.band);
+          n.xdelta = (int32_t)ceil_to((int64_t)at + n.e, alignI) - at;
           n.xstride = pitch(W + n.s + n.xdelta, 0);
           n.xsmem = (int32_t)cs.s_bytes;
           cs.s_bytes += round_up((int64_t)n.xstride * sI, 128);
@@ -396,7 +400,9 @@ void emit_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPl
   if (from_input) {
     if (f.chunk == 0)
       for (const Node &n : nodes[0]) {
-        c.loads.push_back(FusedLoad{n.band, n.xsmem, -(int32_t)ceil_to(n.o + n.e, 16 / sI), n.xstride / f.box});
+        c.loads.push_back(FusedLoad{f.descending ? t.nf - 1 - n.band : n.band, n.xsmem,
+                                    -(int32_t)ceil_to((int64_t)n.o + n.e + f.shift(n.band), 16 / sI),
+                                    n.xstride / f.box});
         tx += (int64_t)n.xstride * sI;
       }
   } else {
@@ -961,16 +967,24 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
 // the group's own cones: a first build with provisional boxes measures
 // them, the second uses the chosen box or block width.
 GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int32_t W,
-                       const FusedPlan &fp, int32_t budget, int32_t staging, int32_t search_k, bool emit) {
+                       const FusedPlan &fp, int32_t budget, const FusedParams &prm, int32_t search_k, bool emit) {
+  const int32_t staging = prm.staging;
   const int32_t es = (lb == 0) ? fp.input_size : fp.level_size[lb];
   const int64_t rows = (lb == 0) ? t.nf : t.level_rows[lb];
   // Row blocks: chunks of 128 bytes (64 for 1-byte samples, so that a tile
   // start, a multiple of 64 samples, is a chunk boundary).
   const int32_t chunk = std::min(128 / es, 64);
-  const bool blocks = staging != 1 && nt % chunk == 0;
-  if (staging == 2 && !blocks) return GroupBuild();
-  StageFmt f;
-  f.search_k = search_k;
+  // (mapped channels start at their own columns: row boxes)
+  const bool mapped = lb == 0 && prm.in_shift != nullptr;
+  const bool blocks = staging != 1 && nt % chunk == 0 && !mapped;
+  if (staging == 2 && nt % chunk != 0) return GroupBuild();
+  StageFmt boxes;
+  boxes.search_k = search_k;
+  if (mapped) {
+    boxes.in_shift = prm.in_shift;
+    boxes.descending = prm.descending;
+  }
+  StageFmt f = boxes;
   if (blocks) {
     f.chunk = chunk;
     f.max_p = 0;
@@ -1002,8 +1016,7 @@ GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int3
         return emit ? build_group_fmt(t, nt, lb, lt, W, fp, budget, f, nullptr, true) : g2;
     }
     if (staging == 2) return GroupBuild();
-    f = StageFmt();  // fall back to row boxes
-    f.search_k = search_k;
+    f = boxes;  // fall back to row boxes
     f.box = 128 / es;
     needs.clear();
     gb = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &needs, false);
@@ -1229,7 +1242,7 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
     const std::vector<int32_t> ws = forced_W > 0 ? std::vector<int32_t>{forced_W} : widths;
     for (int32_t W : ws) {
       if (best.ok && W / 2 >= nt) break;  // (no wider than one tile needs)
-      GroupBuild gb = build_group(t, nt, lb, lt, W, fp, budget > 0 ? budget : p.smem_budget, p.staging,
+      GroupBuild gb = build_group(t, nt, lb, lt, W, fp, budget > 0 ? budget : p.smem_budget, p,
                                   lt == L ? p.search_k : 0, false);
       if (gb.ok && (!best.ok || gb.seconds < best.seconds)) best = std::move(gb);
     }
@@ -1238,7 +1251,7 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
     for (int32_t kib = 56; refine && budget == 0 && p.smem_budget == FusedParams().smem_budget && kib >= 14; kib /= 2) {
       if (!best.ok || best.items * best.g.ntiles >= best.g.block_slots) break;
       for (int32_t W : ws) {
-        GroupBuild gb = build_group(t, nt, lb, lt, W, fp, kib * 1024, p.staging, lt == L ? p.search_k : 0, false);
+        GroupBuild gb = build_group(t, nt, lb, lt, W, fp, kib * 1024, p, lt == L ? p.search_k : 0, false);
         if (gb.ok && gb.seconds < best.seconds) best = std::move(gb);
       }
     }
@@ -1276,7 +1289,7 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
     if (gw < 0 || gw % 64 != 0 || gbud < 0 || gbud > 227 * 1024) return "bad per-group parameters";
     GroupBuild gb = best_segment(bounds[i], bounds[i + 1], gw, gbud, true);
     if (gb.ok)
-      gb = build_group(t, nt, bounds[i], bounds[i + 1], gb.g.W, fp, gb.budget, p.staging,
+      gb = build_group(t, nt, bounds[i], bounds[i + 1], gb.g.W, fp, gb.budget, p,
                        bounds[i + 1] == L ? p.search_k : 0, true);
     if (!gb.ok) return "a level group does not fit the shared-memory budget";
     secs += gb.seconds;
