@@ -443,6 +443,26 @@ int fdmt_execute(fdmt_plan_t plan, const void *in, const float *weights, void *o
   return FDMT_OK;
 }
 
+}  // extern "C"
+
+int fdmt::execute_view(fdmt_plan_s *plan, const void *in, void *out, void *workspace, size_t ws_bytes,
+                       const OutView &view, cudaStream_t s) {
+  size_t need = 0;
+  if (plan != nullptr) fdmt_workspace_bytes(plan, &need);
+  const int st = check_exec_common(plan, workspace, ws_bytes, need);
+  if (st != FDMT_OK) return st;
+  if (in == nullptr || out == nullptr || !aligned16(in) || !plan->has_fused || plan->search_k > 0)
+    return FDMT_ERR_INVALID_ARG;
+  void *bufs[2] = {workspace, workspace ? static_cast<char *>(workspace) + plan->fused_ws_split : nullptr};
+  if (run_fused(plan->dev, plan->dtype, in, nullptr, out, bufs, plan->nt, s, nullptr, &view) != cudaSuccess) {
+    cudaGetLastError();
+    return FDMT_ERR_CUDA;
+  }
+  return FDMT_OK;
+}
+
+extern "C" {
+
 int fdmt_execute_search_workspace_bytes(fdmt_plan_t plan, int32_t n_widths, size_t *bytes) {
   if (plan == nullptr || bytes == nullptr || n_widths < 1 || n_widths > 13) return FDMT_ERR_INVALID_ARG;
   size_t ws = 0;

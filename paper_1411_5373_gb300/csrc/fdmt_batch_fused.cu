@@ -98,34 +98,34 @@ __device__ __forceinline__ void stage_seg_item(unsigned char *smem, uint32_t bar
 template <class TI, class TB, class A, bool GEN>
 __device__ __forceinline__ void batch_first_stage(bool from_input, bool i16, bool o16, uint32_t bar, uint32_t prog,
                                                   int n_stages, int warp, int lane, void *out, int64_t nt, int64_t T0,
-                                                  int lim) {
+                                                  int lo, int lim) {
   TB *o = static_cast<TB *>(out);
   if constexpr (std::is_same<TB, int32_t>::value) {
     uint16_t *o_16 = static_cast<uint16_t *>(out);
     if (from_input) {
       if (o16)
         item_first_stage<TI, TB, A, uint16_t, false, true, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane,
-                                                                              o_16, nt, T0, lim);
+                                                                              o_16, nt, T0, lo, lim);
       else
         item_first_stage<TI, TB, A, TB, false, true, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o,
-                                                                        nt, T0, lim);
+                                                                        nt, T0, lo, lim);
     } else if (i16 && o16) {
       item_first_stage<TI, uint16_t, A, uint16_t, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp,
-                                                                                   lane, o_16, nt, T0, lim);
+                                                                                   lane, o_16, nt, T0, lo, lim);
     } else if (i16) {
       item_first_stage<TI, uint16_t, A, TB, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane,
-                                                                             o, nt, T0, lim);
+                                                                             o, nt, T0, lo, lim);
     } else {
       item_first_stage<TI, TB, A, TB, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
-                                                                       T0, lim);
+                                                                       T0, lo, lim);
     }
   } else {
     if (from_input)
       item_first_stage<TI, TB, A, TB, false, true, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
-                                                                      T0, lim);
+                                                                      T0, lo, lim);
     else
       item_first_stage<TI, TB, A, TB, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
-                                                                       T0, lim);
+                                                                       T0, lo, lim);
   }
 }
 
@@ -253,7 +253,7 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     const bool i16 = kNarrow && sg->in_size == 2, o16 = kNarrow && sg->out_size == 2;
     const int n_stages = cur.n_stages;
     batch_first_stage<TI, TB, A, GEN>(from_input, i16, o16, bar, prog_at(slot), n_stages, warp, lane, sg->out, nt, T0,
-                                      lim);
+                                      0, lim);
     __syncthreads();  // the staged rows are no longer read; s_early is visible
     const bool early = *s_early != 0;
     if (early && warp == 0) {
@@ -267,10 +267,10 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     const SearchArgs no_search{};
     if (kNarrow && o16)
       item_later_stages<A, uint16_t, false, false, GEN>(bar, prog_at(slot), n_stages, nullptr, warp, lane,
-                                                        static_cast<uint16_t *>(sg->out), nt, T0, lim, 0, no_search);
+                                                        static_cast<uint16_t *>(sg->out), nt, T0, 0, lim, 0, no_search);
     else
       item_later_stages<A, TB, false, false, GEN>(bar, prog_at(slot), n_stages, nullptr, warp, lane,
-                                                  static_cast<TB *>(sg->out), nt, T0, lim, 0, no_search);
+                                                  static_cast<TB *>(sg->out), nt, T0, 0, lim, 0, no_search);
     slot ^= 1u;
     if (threadIdx.x == 0) *s_next = nn;
     __syncthreads();  // all of this item's stores are issued; Pa / Pb are free; s_next is visible

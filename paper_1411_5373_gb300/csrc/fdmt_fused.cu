@@ -71,12 +71,12 @@ bool make_group_maps(CUtensorMap *maps, const FusedGroup &g, const void *base, C
 }
 
 cudaError_t run_fused(const DeviceTables &dt, int dtype, const void *in, const float *w, void *out,
-                      void *const bufs[2], int64_t nt, cudaStream_t s, const SearchArgs *sa) {
+                      void *const bufs[2], int64_t nt, cudaStream_t s, const SearchArgs *sa, const OutView *view) {
   if (dt.fused == nullptr) return cudaErrorInvalidValue;
   switch (dtype) {
-    case 0: return run_fused_u8(dt, in, out, bufs, nt, s, sa);
-    case 1: return run_fused_f32(dt, in, w, out, bufs, nt, s, sa);
-    case 2: return run_fused_typed<float, __half, float, float, true>(dt, in, w, out, bufs, nt, s, sa);
+    case 0: return run_fused_u8(dt, in, out, bufs, nt, s, sa, view);
+    case 1: return run_fused_f32(dt, in, w, out, bufs, nt, s, sa, view);
+    case 2: return run_fused_typed<float, __half, float, float, true>(dt, in, w, out, bufs, nt, s, sa, view);
     default: return cudaErrorInvalidValue;
   }
 }

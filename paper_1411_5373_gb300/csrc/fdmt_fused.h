@@ -242,6 +242,7 @@ struct FusedGroup {
   int32_t q_off = 0;          // search: byte offset of an item's per (row, width) bests
   int32_t q_row = 0;          //   and their bytes
   int64_t ntiles = 0;
+  int32_t min_x = 0;          // earliest column a copy reads, relative to its tile's first (<= 0)
   double hbm_bytes = 0;       // model: loaded + written bytes per launch
   double smem_traffic = 0;    // model: shared-memory bytes moved per launch
   double ops = 0;             // model: ops and walks per launch
@@ -283,6 +284,19 @@ struct FusedPlan {
   double model_seconds = 0;
   bool general = false;  // some stage holds passed-up or one-term halves (kStageGeneral)
 };
+
+// Output columns a caller wants of a transform: those from `first` on,
+// column t of a row at out[row * pitch + t - first].
+struct OutView {
+  int64_t first = 0, pitch = 0;
+};
+
+// First tile of every group when only output columns from `first` on are
+// wanted: a group computes the tiles its successor's copies reach.
+struct FirstTiles {
+  int64_t tile[64];  // (a plan has at most one group per level)
+};
+void first_tiles(const FusedPlan &fp, int64_t first, FirstTiles &out);
 
 // Levels a group (lb, lt] keeps in shared memory (see fdmt_fused_plan.cpp).
 std::vector<int32_t> stored_levels(int32_t lb, int32_t lt);

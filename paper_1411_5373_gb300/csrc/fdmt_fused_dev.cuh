@@ -319,7 +319,7 @@ __device__ __forceinline__ void round_piece(A (&v)[kLaneCols]) {
 // per clock and SM).
 template <class TSrc, class A, class TO, bool R16, int OUT, bool PAIR, bool GEN>
 __device__ __forceinline__ void stage_runs(uint32_t sbase, const StageRange &range, int lane, TO *__restrict__ out,
-                                           int64_t nt, int64_t T0, int lim) {
+                                           int64_t nt, int64_t T0, int lo, int lim) {
   constexpr uint32_t es = sizeof(TSrc);
   for (uint32_t at = range.first; at != range.end; at += (uint32_t)sizeof(FusedRun)) {
     const FusedRun run = lds_desc<FusedRun>(at);
@@ -332,10 +332,14 @@ __device__ __forceinline__ void stage_runs(uint32_t sbase, const StageRange &ran
     uint32_t p2 = sbase + (uint32_t)run.p2, p3 = sbase + (uint32_t)run.p3;
     const uint32_t e = move * es, g0 = (uint32_t)run.g0 + e, g1 = (uint32_t)run.g1 + e;
     int c = warp_all(run.col);
-    const int limit = OUT == kOutGlobal ? min(warp_all(run.width), lim) : warp_all(run.width);
+    int limit = warp_all(run.width);
+    if constexpr (OUT == kOutGlobal) limit = max(min(limit, lim) - lo, 0);
     uint32_t dst = sbase + (uint32_t)run.dst;
     TO *g = nullptr;
-    if constexpr (OUT == kOutGlobal) g = out + (int64_t)run.dst * nt + T0 + c + lane;
+    if constexpr (OUT == kOutGlobal) {
+      g = out + (int64_t)run.dst * nt + T0 + c + lane;
+      c -= lo;  // columns count from the first one wanted
+    }
     if constexpr (OUT == kOutSmem) dst += (uint32_t)lane * sizeof(A);
     A a0[kLaneCols], b1[kLaneCols], a2[kLaneCols], b3[kLaneCols], lp[kLaneCols], hp[kLaneCols], v[kLaneCols];
     auto lower = [&]() {
@@ -457,7 +461,7 @@ __device__ __forceinline__ void stage_runs(uint32_t sbase, const StageRange &ran
 template <class TI, class A, class TO, bool R16, bool SCALE, bool TOP, bool GEN>
 __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &range, int lane,
                                            const float *__restrict__ w, TO *__restrict__ out, int64_t nt, int64_t T0,
-                                           int lim) {
+                                           int lo, int lim) {
   constexpr uint32_t es = (uint32_t)sizeof(TI);
   for (uint32_t at = range.first; at != range.end; at += (uint32_t)sizeof(FusedWalk)) {
     const FusedWalk wk = lds_desc<FusedWalk>(at);
@@ -478,9 +482,10 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
     const bool upper = !GEN || !(warp_all(wk.flags) & kWalkNoUpper);
     int dl = warp_all(wk.dl0), j = warp_all(wk.a) - dl;
     uint32_t bits = (uint32_t)warp_all(wk.bits);
-    const bool whole = TOP ? warp_all(wk.width) >= kPieceCols && warp_all(wk.col) + kPieceCols <= lim
+    const int skip = TOP ? max(lo - wk.col, 0) : 0;  // columns before the first one wanted
+    const bool whole = TOP ? warp_all(wk.width) >= kPieceCols && warp_all(wk.col) + kPieceCols <= lim && warp_all(skip) == 0
                            : warp_all(wk.width) >= kPieceCols || (warp_all(wk.dst_row) & (kPieceCols * 4 - 1)) == 0;
-    const int limit = TOP ? min(wk.width, lim - wk.col) : wk.width;
+    const int limit = TOP ? max(min(wk.width, lim - wk.col) - skip, 0) : wk.width;
     uint32_t dst = sbase + (uint32_t)wk.dst + (uint32_t)lane * (uint32_t)sizeof(A);
     TO *g = nullptr;
     if constexpr (TOP) g = out + (int64_t)wk.dst * nt + T0 + wk.col + lane;
@@ -492,7 +497,7 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
           for (int k = 0; k < kLaneCols; ++k) g[32 * k] = to_store<TO>(v[k]);
         } else {
 #pragma unroll
-          for (int k = 0; k < kLaneCols; ++k) stg_below(g + 32 * k, v[k], lane + 32 * k, max(limit, 0));
+          for (int k = 0; k < kLaneCols; ++k) stg_below(g + 32 * k, v[k], lane + 32 * k - skip, limit);
         }
         g += nt;
       } else {
@@ -563,14 +568,14 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
 // halves (else only the code without those tests is compiled in).
 template <class TSrc, class A, class TO, bool R16, int OUT, bool GEN = true>
 __device__ __forceinline__ void run_merge_stage(const StageRange &r, uint32_t sbase, int lane, TO *__restrict__ out,
-                                                int64_t nt, int64_t T0, int lim) {
+                                                int64_t nt, int64_t T0, int lo, int lim) {
   const bool gen = GEN && (r.kind & kStageGeneral) != 0;
   if ((r.kind & kStageKindMask) == kStagePair) {
-    if (gen) stage_runs<TSrc, A, TO, R16, OUT, true, true>(sbase, r, lane, out, nt, T0, lim);
-    else stage_runs<TSrc, A, TO, R16, OUT, true, false>(sbase, r, lane, out, nt, T0, lim);
+    if (gen) stage_runs<TSrc, A, TO, R16, OUT, true, true>(sbase, r, lane, out, nt, T0, lo, lim);
+    else stage_runs<TSrc, A, TO, R16, OUT, true, false>(sbase, r, lane, out, nt, T0, lo, lim);
   } else {
-    if (gen) stage_runs<TSrc, A, TO, R16, OUT, false, true>(sbase, r, lane, out, nt, T0, lim);
-    else stage_runs<TSrc, A, TO, R16, OUT, false, false>(sbase, r, lane, out, nt, T0, lim);
+    if (gen) stage_runs<TSrc, A, TO, R16, OUT, false, true>(sbase, r, lane, out, nt, T0, lo, lim);
+    else stage_runs<TSrc, A, TO, R16, OUT, false, false>(sbase, r, lane, out, nt, T0, lo, lim);
   }
 }
 
@@ -814,40 +819,41 @@ __device__ __forceinline__ void stage_search_block(uint32_t sbase, const FusedOp
 // prog: shared address of the item's programme.  TB is the staged base
 // level's type and TO the type written to global memory when this stage is
 // the top.  With SEARCH the stage before the search writes the top level
-// into Pt instead.  GEN as for run_merge_stage; SCALE: the input is
-// multiplied by channel weights (float input only).
+// into Pt instead.  Rows of the top level are nt apart in `out`; its columns
+// T0 + [lo, lim) are written.  GEN as for run_merge_stage; SCALE: the input
+// is multiplied by channel weights (float input only).
 template <class TI, class TB, class A, class TO, bool R16, bool FROM_INPUT, bool SEARCH, bool GEN = true,
           bool SCALE = true>
 __device__ __forceinline__ void item_first_stage(uint32_t sbase, uint32_t prog, int n_stages,
                                                  const float *__restrict__ w, int warp, int lane,
-                                                 TO *__restrict__ out, int64_t nt, int64_t T0, int lim) {
+                                                 TO *__restrict__ out, int64_t nt, int64_t T0, int lo, int lim) {
   const StageRange r = prog_stage(prog, 0, warp);
   const bool top = !SEARCH && n_stages == 1;
   if constexpr (FROM_INPUT) {
     const bool gen = GEN && (r.kind & kStageGeneral) != 0;
     if constexpr (SCALE && std::is_floating_point<A>::value) {
       if (gen) {
-        if (top) stage_walk<TI, A, TO, R16, true, true, true>(sbase, r, lane, w, out, nt, T0, lim);
-        else stage_walk<TI, A, TO, R16, true, false, true>(sbase, r, lane, w, out, nt, T0, lim);
+        if (top) stage_walk<TI, A, TO, R16, true, true, true>(sbase, r, lane, w, out, nt, T0, lo, lim);
+        else stage_walk<TI, A, TO, R16, true, false, true>(sbase, r, lane, w, out, nt, T0, lo, lim);
       } else {
-        if (top) stage_walk<TI, A, TO, R16, true, true, false>(sbase, r, lane, w, out, nt, T0, lim);
-        else stage_walk<TI, A, TO, R16, true, false, false>(sbase, r, lane, w, out, nt, T0, lim);
+        if (top) stage_walk<TI, A, TO, R16, true, true, false>(sbase, r, lane, w, out, nt, T0, lo, lim);
+        else stage_walk<TI, A, TO, R16, true, false, false>(sbase, r, lane, w, out, nt, T0, lo, lim);
       }
     } else {
       if (gen) {
-        if (top) stage_walk<TI, A, TO, R16, false, true, true>(sbase, r, lane, w, out, nt, T0, lim);
-        else stage_walk<TI, A, TO, R16, false, false, true>(sbase, r, lane, w, out, nt, T0, lim);
+        if (top) stage_walk<TI, A, TO, R16, false, true, true>(sbase, r, lane, w, out, nt, T0, lo, lim);
+        else stage_walk<TI, A, TO, R16, false, false, true>(sbase, r, lane, w, out, nt, T0, lo, lim);
       } else {
-        if (top) stage_walk<TI, A, TO, R16, false, true, false>(sbase, r, lane, w, out, nt, T0, lim);
-        else stage_walk<TI, A, TO, R16, false, false, false>(sbase, r, lane, w, out, nt, T0, lim);
+        if (top) stage_walk<TI, A, TO, R16, false, true, false>(sbase, r, lane, w, out, nt, T0, lo, lim);
+        else stage_walk<TI, A, TO, R16, false, false, false>(sbase, r, lane, w, out, nt, T0, lo, lim);
       }
     }
   } else if constexpr (SEARCH) {
-    if (n_stages == 2) run_merge_stage<TB, A, TO, R16, kOutPadded, GEN>(r, sbase, lane, out, nt, T0, lim);
-    else run_merge_stage<TB, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lim);
+    if (n_stages == 2) run_merge_stage<TB, A, TO, R16, kOutPadded, GEN>(r, sbase, lane, out, nt, T0, lo, lim);
+    else run_merge_stage<TB, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lo, lim);
   } else {
-    if (top) run_merge_stage<TB, A, TO, R16, kOutGlobal, GEN>(r, sbase, lane, out, nt, T0, lim);
-    else run_merge_stage<TB, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lim);
+    if (top) run_merge_stage<TB, A, TO, R16, kOutGlobal, GEN>(r, sbase, lane, out, nt, T0, lo, lim);
+    else run_merge_stage<TB, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lo, lim);
   }
 }
 
@@ -857,8 +863,8 @@ __device__ __forceinline__ void item_first_stage(uint32_t sbase, uint32_t prog, 
 template <class A, class TO, bool R16, bool SEARCH, bool GEN = true>
 __device__ __forceinline__ void item_later_stages(uint32_t sbase, uint32_t prog, int n_stages,
                                                   const FusedOp *__restrict__ ops, int warp, int lane,
-                                                  TO *__restrict__ out, int64_t nt, int64_t T0, int lim, int64_t tile,
-                                                  const SearchArgs &sa) {
+                                                  TO *__restrict__ out, int64_t nt, int64_t T0, int lo, int lim,
+                                                  int64_t tile, const SearchArgs &sa) {
   for (int s = 1; s < n_stages; ++s) {
     compute_sync();
     if constexpr (SEARCH) {
@@ -871,9 +877,9 @@ __device__ __forceinline__ void item_later_stages(uint32_t sbase, uint32_t prog,
       }
     }
     const StageRange r = prog_stage(prog, s, warp);
-    if (SEARCH && s == n_stages - 2) run_merge_stage<A, A, TO, R16, kOutPadded, GEN>(r, sbase, lane, out, nt, T0, lim);
-    else if (!SEARCH && s == n_stages - 1) run_merge_stage<A, A, TO, R16, kOutGlobal, GEN>(r, sbase, lane, out, nt, T0, lim);
-    else run_merge_stage<A, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lim);
+    if (SEARCH && s == n_stages - 2) run_merge_stage<A, A, TO, R16, kOutPadded, GEN>(r, sbase, lane, out, nt, T0, lo, lim);
+    else if (!SEARCH && s == n_stages - 1) run_merge_stage<A, A, TO, R16, kOutGlobal, GEN>(r, sbase, lane, out, nt, T0, lo, lim);
+    else run_merge_stage<A, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lo, lim);
   }
 }
 

@@ -5,8 +5,8 @@
 namespace fdmt {
 
 cudaError_t run_fused_f32(const DeviceTables &dt, const void *in, const float *w, void *out, void *const bufs[2],
-                          int64_t nt, cudaStream_t s, const SearchArgs *sa) {
-  return run_fused_typed<float, float, float, float, false>(dt, in, w, out, bufs, nt, s, sa);
+                          int64_t nt, cudaStream_t s, const SearchArgs *sa, const OutView *view) {
+  return run_fused_typed<float, float, float, float, false>(dt, in, w, out, bufs, nt, s, sa, view);
 }
 
 }  // namespace fdmt

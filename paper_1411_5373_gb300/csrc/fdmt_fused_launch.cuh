@@ -63,11 +63,11 @@ constexpr int kFusedLaunchThreads = kFusedThreads + 32;
 
 template <class TI, class TB, class TO, class A, bool FROM_INPUT, bool R16, bool SEARCH, bool GEN, bool SCALE>
 __global__ void __launch_bounds__(kFusedLaunchThreads, kFusedMinBlocks)
-fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t nt, int32_t W,
-             int32_t ntiles, int64_t items, const FusedProg *__restrict__ progs, const int4 *__restrict__ prog,
-             const FusedLoad *__restrict__ loads, const FusedOp *__restrict__ ops, const float *__restrict__ w,
-             int32_t box, int32_t cshift, int32_t prog_off, int32_t prog_slot, int *__restrict__ status,
-             const SearchArgs sa) {
+fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t nt, int64_t pitch, int64_t first,
+             int32_t W, int32_t tile0, int32_t ntiles, int64_t items, const FusedProg *__restrict__ progs,
+             const int4 *__restrict__ prog, const FusedLoad *__restrict__ loads, const FusedOp *__restrict__ ops,
+             const float *__restrict__ w, int32_t box, int32_t cshift, int32_t prog_off, int32_t prog_slot,
+             int *__restrict__ status, const SearchArgs sa) {
   using TS = typename std::conditional<FROM_INPUT, TI, TB>::type;  // staged element type
   extern __shared__ __align__(128) unsigned char smem[];
   const int warp = warp_all((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
@@ -81,7 +81,7 @@ fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t
   }
   __syncthreads();
   if (warp == kFusedWarps) {
-    // item = tpl * ntiles + tile, advanced by gridDim.x without divisions.
+    // item = tpl * ntiles + tile - tile0, advanced by gridDim.x without divisions.
     int64_t item = blockIdx.x;
     if (item >= items) return;
     int32_t tile = (int32_t)(item % ntiles), tpl = (int32_t)(item / ntiles);
@@ -102,10 +102,10 @@ fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t
         phase ^= 1u;
       }
       first = false;
-      const int64_t T0 = (int64_t)tile * W;
+      const int64_t T0 = (int64_t)(tile0 + tile) * W;
       if (lane == 0) {
         const int lim = (int)((nt - T0) < (int64_t)W ? (nt - T0) : (int64_t)W);
-        sts_v4(header + 16u * slot, make_int4(tile, lim, pr.n_stages, 0));
+        sts_v4(header + 16u * slot, make_int4(tile0 + tile, lim, pr.n_stages, 0));
       }
       stage_item<TS>(smem, full, maps.m, pr, loads, ld, T0, box, cshift, lane);
       if (lane == 0) stage_prog(full + (uint32_t)(prog_off + (int)slot * prog_slot), pr, prog, full);
@@ -140,11 +140,12 @@ fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t
     const int lim = h.y, n_stages = warp_all(h.z);
     const int64_t tile = h.x, T0 = tile * W;
     const uint32_t prg = full + (uint32_t)(prog_off + (int)slot * prog_slot);
-    item_first_stage<TI, TB, A, TO, R16, FROM_INPUT, SEARCH, GEN, SCALE>(full, prg, n_stages, w, warp, lane, out, nt,
-                                                                         T0, lim);
+    const int lo = first > T0 ? (int)(first - T0) : 0;
+    item_first_stage<TI, TB, A, TO, R16, FROM_INPUT, SEARCH, GEN, SCALE>(full, prg, n_stages, w, warp, lane, out,
+                                                                         pitch, T0, lo, lim);
     __syncwarp();
     if (lane == 0) mbar_arrive(free_bar);  // this warp reads S no more
-    item_later_stages<A, TO, R16, SEARCH, GEN>(full, prg, n_stages, ops, warp, lane, out, nt, T0, lim, tile, sa);
+    item_later_stages<A, TO, R16, SEARCH, GEN>(full, prg, n_stages, ops, warp, lane, out, pitch, T0, lo, lim, tile, sa);
     slot ^= 1u;
   }
 }
@@ -153,7 +154,8 @@ namespace {
 
 template <class TI, class TB, class TO, class A, bool FI, bool R16, bool SEARCH, bool GEN, bool SCALE>
 cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const void *base, int64_t base_rows,
-                           void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa) {
+                           void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa,
+                           int64_t tile0, const OutView *view) {
   auto kern = fused_kernel<TI, TB, TO, A, FI, R16, SEARCH, GEN, SCALE>;
   static std::once_flag attr_once;
   static cudaError_t attr_err = cudaSuccess;
@@ -167,7 +169,8 @@ cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const vo
   if (!make_group_maps(maps.m, g, base, map_type<TS>(), sizeof(TS), (uint64_t)base_rows, (uint64_t)nt, &cshift))
     return cudaErrorInvalidValue;
   const int32_t box = g.box;
-  const int64_t items = (int64_t)g.tpl_count * g.ntiles;
+  const int64_t ntiles = g.ntiles - tile0, items = (int64_t)g.tpl_count * ntiles;
+  const OutView v = view != nullptr ? *view : OutView{0, nt};
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFusedLaunchThreads, g.smem_bytes);
   if (e != cudaSuccess) return e;
@@ -178,9 +181,9 @@ cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const vo
   const int64_t blocks = std::min<int64_t>(items, (int64_t)per_sm * sms);
   dt.prof->begin(s, FI ? K_FUSED_LOCAL : K_FUSED_CONE, g.lb * 100 + g.lt);
   kern<<<(unsigned)blocks, kFusedLaunchThreads, g.smem_bytes, s>>>(
-      maps, static_cast<TO *>(dst), nt, g.W, (int32_t)g.ntiles, items, dt.f_progs + g.tpl_begin,
-      reinterpret_cast<const int4 *>(dt.f_prog), dt.f_loads, dt.f_ops, w, box, cshift, g.prog_off, g.prog_slot,
-      dt.status, sa ? *sa : SearchArgs{});
+      maps, static_cast<TO *>(dst) - v.first, nt, v.pitch, v.first, g.W, (int32_t)tile0, (int32_t)ntiles, items,
+      dt.f_progs + g.tpl_begin, reinterpret_cast<const int4 *>(dt.f_prog), dt.f_loads, dt.f_ops, w, box, cshift,
+      g.prog_off, g.prog_slot, dt.status, sa ? *sa : SearchArgs{});
   dt.prof->end(s);
   return cudaGetLastError();
 }
@@ -190,24 +193,31 @@ cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const vo
 // (only for float input from the input).
 template <class TI, class TB, class TO, class A, bool FI, bool R16, bool SEARCH = false>
 cudaError_t launch_group(const DeviceTables &dt, const FusedGroup &g, const void *base, int64_t base_rows,
-                         void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa = nullptr) {
+                         void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa, int64_t tile0,
+                         const OutView *view) {
   const bool gen = dt.fused->general;
   if constexpr (FI && std::is_floating_point<A>::value) {
     if (w != nullptr)
-      return gen ? launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, true>(dt, g, base, base_rows, dst, w, nt, s, sa)
+      return gen ? launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, true>(dt, g, base, base_rows, dst, w, nt, s, sa,
+                                                                              tile0, view)
                  : launch_variant<TI, TB, TO, A, FI, R16, SEARCH, false, true>(dt, g, base, base_rows, dst, w, nt, s,
-                                                                               sa);
+                                                                               sa, tile0, view);
   }
-  return gen ? launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, false>(dt, g, base, base_rows, dst, w, nt, s, sa)
-             : launch_variant<TI, TB, TO, A, FI, R16, SEARCH, false, false>(dt, g, base, base_rows, dst, w, nt, s, sa);
+  return gen ? launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, false>(dt, g, base, base_rows, dst, w, nt, s, sa,
+                                                                           tile0, view)
+             : launch_variant<TI, TB, TO, A, FI, R16, SEARCH, false, false>(dt, g, base, base_rows, dst, w, nt, s, sa,
+                                                                            tile0, view);
 }
 
 // The launches of a float plan (A the sums' type, R16: fp16-state rounding).
 template <class TI, class TB, class TO, class A, bool R16>
 cudaError_t run_fused_typed(const DeviceTables &dt, const void *in, const float *w, void *out,
-                            void *const bufs[2], int64_t nt, cudaStream_t s, const SearchArgs *sa) {
+                            void *const bufs[2], int64_t nt, cudaStream_t s, const SearchArgs *sa,
+                            const OutView *view) {
   const FusedPlan &fp = *dt.fused;
   const int G = (int)fp.groups.size();
+  FirstTiles ft;
+  first_tiles(fp, view != nullptr ? view->first : 0, ft);
   for (int g = 0; g < G; ++g) {
     const FusedGroup &gr = fp.groups[g];
     const bool last = (g == G - 1);
@@ -218,17 +228,17 @@ cudaError_t run_fused_typed(const DeviceTables &dt, const void *in, const float 
       // least two merge levels, so a launch from the input walks level 1
       // into Pa before its top level goes to Pt).
       if (sa == nullptr) return cudaErrorInvalidValue;
-      e = gr.from_input ? launch_group<TI, TB, TO, A, true, R16, true>(dt, gr, in, dt.nf, dst, w, nt, s, sa)
+      e = gr.from_input ? launch_group<TI, TB, TO, A, true, R16, true>(dt, gr, in, dt.nf, dst, w, nt, s, sa, ft.tile[g], view)
                         : launch_group<TI, TB, TO, A, false, R16, true>(dt, gr, bufs[(g - 1) & 1],
-                                                                        dt.level_rows[gr.lb], dst, w, nt, s, sa);
+                                                                        dt.level_rows[gr.lb], dst, w, nt, s, sa, ft.tile[g], view);
     } else if (gr.from_input) {
-      e = last ? launch_group<TI, TB, TO, A, true, R16>(dt, gr, in, dt.nf, dst, w, nt, s)
-               : launch_group<TI, TB, TB, A, true, R16>(dt, gr, in, dt.nf, dst, w, nt, s);
+      e = last ? launch_group<TI, TB, TO, A, true, R16>(dt, gr, in, dt.nf, dst, w, nt, s, nullptr, ft.tile[g], view)
+               : launch_group<TI, TB, TB, A, true, R16>(dt, gr, in, dt.nf, dst, w, nt, s, nullptr, ft.tile[g], nullptr);
     } else {
       const void *base = bufs[(g - 1) & 1];
       const int64_t rows = dt.level_rows[gr.lb];
-      e = last ? launch_group<TI, TB, TO, A, false, R16>(dt, gr, base, rows, dst, w, nt, s)
-               : launch_group<TI, TB, TB, A, false, R16>(dt, gr, base, rows, dst, w, nt, s);
+      e = last ? launch_group<TI, TB, TO, A, false, R16>(dt, gr, base, rows, dst, w, nt, s, nullptr, ft.tile[g], view)
+               : launch_group<TI, TB, TB, A, false, R16>(dt, gr, base, rows, dst, w, nt, s, nullptr, ft.tile[g], nullptr);
     }
     if (e != cudaSuccess) return e;
   }
@@ -239,9 +249,9 @@ cudaError_t run_fused_typed(const DeviceTables &dt, const void *in, const float 
 
 // uint8 input (fdmt_fused_u8.cu).
 cudaError_t run_fused_u8(const DeviceTables &dt, const void *in, void *out, void *const bufs[2], int64_t nt,
-                         cudaStream_t s, const SearchArgs *sa);
+                         cudaStream_t s, const SearchArgs *sa, const OutView *view);
 // float32 input and state (fdmt_fused_f32.cu).
 cudaError_t run_fused_f32(const DeviceTables &dt, const void *in, const float *w, void *out, void *const bufs[2],
-                          int64_t nt, cudaStream_t s, const SearchArgs *sa);
+                          int64_t nt, cudaStream_t s, const SearchArgs *sa, const OutView *view);
 
 }  // namespace fdmt

@@ -1165,6 +1165,7 @@ bool append_group(FusedPlan &fp, GroupBuild &gb) {
         fp.run_stages.insert(fp.run_stages.end(), fp.stages.end() - kStageWords, fp.stages.end());
       }
     }
+    for (const FusedLoad &ld : c.loads) g.min_x = std::min(g.min_x, ld.xoff);
     FusedProg pr{};
     pr.load_begin = tp.load_begin;
     pr.load_count = tp.load_count;
@@ -1201,6 +1202,13 @@ bool append_group(FusedPlan &fp, GroupBuild &gb) {
 }
 
 }  // namespace
+
+void first_tiles(const FusedPlan &fp, int64_t first, FirstTiles &out) {
+  for (size_t g = fp.groups.size(); g-- > 0;) {
+    out.tile[g] = first / fp.groups[g].W;
+    first = std::max<int64_t>(0, out.tile[g] * fp.groups[g].W + fp.groups[g].min_x);
+  }
+}
 
 std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t input_size,
                        const FusedParams &p, FusedPlan &out) {

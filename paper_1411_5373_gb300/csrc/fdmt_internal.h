@@ -113,9 +113,16 @@ cudaError_t run_plain(const DeviceTables &dt, int dtype, const void *in, const f
 
 // Fused schedule: one launch per group of levels (fdmt_fused.h); bufs hold
 // the intermediate level states between groups.  A plan whose last launch
-// ends with the boxcar search needs `sa` (the partials it writes).
+// ends with the boxcar search needs `sa` (the partials it writes).  `view`:
+// only those output columns (null: all of them, rows nt apart).
 cudaError_t run_fused(const DeviceTables &dt, int dtype, const void *in, const float *w, void *out,
-                      void *const bufs[2], int64_t nt, cudaStream_t s, const SearchArgs *sa = nullptr);
+                      void *const bufs[2], int64_t nt, cudaStream_t s, const SearchArgs *sa = nullptr,
+                      const OutView *view = nullptr);
+
+// fdmt_execute of a fused plan without a search, writing only the output
+// columns of `view` (a status code; the same checks).
+int execute_view(fdmt_plan_s *plan, const void *in, void *out, void *workspace, size_t ws_bytes, const OutView &view,
+                 cudaStream_t s);
 
 // The boxcar search's finalize step (fdmt_search.cu) over partials
 // part_v / part_r laid out as (row, width, segment): per row and width the
