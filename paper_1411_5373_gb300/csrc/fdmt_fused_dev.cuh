@@ -917,6 +917,30 @@ __device__ __forceinline__ void stage_item(unsigned char *smem, uint32_t bar, co
   }
 }
 
+// Ask for the rows of a work item to be brought into L2 (the same copies as
+// stage_item, without their shared memory).
+template <class TS, class T>
+__device__ __forceinline__ void prefetch_item(const CUtensorMap *maps, const T &tp,
+                                              const FusedLoad *__restrict__ loads, const FusedLoad &first, int64_t T0,
+                                              int32_t box, int32_t cshift, int lane) {
+  for (int i = lane; i < tp.load_count; i += 32) {
+    const FusedLoad ld = (i == lane) ? first : loads[tp.load_begin + i];
+    const int32_t x = (int32_t)(T0 + ld.xoff);
+    if (cshift > 0) {
+      asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(
+                       reinterpret_cast<uint64_t>(maps + ld.nbox)),
+                   "r"(0), "r"(x >> cshift), "r"(ld.row)
+                   : "memory");
+    } else {
+      for (int b = 0; b < ld.nbox; ++b)
+        asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
+                         reinterpret_cast<uint64_t>(maps)),
+                     "r"(x + b * box), "r"(ld.row)
+                     : "memory");
+    }
+  }
+}
+
 // Copy an item's programme to its slot at shared address dst, on the same
 // barrier phase (its bytes are part of tx_bytes); one lane.
 __device__ __forceinline__ void stage_prog(uint32_t dst, const FusedProg &pr, const int4 *__restrict__ prog,
