@@ -46,6 +46,7 @@ constexpr int kMapsPerSeg = kMaxBlockP + 1;
 struct BSeg {
   int64_t first;  // first global item
   int64_t nt;
+  int64_t pitch;  // samples from one row of `out` to the next
   void *out;      // the group's top level: the beam's output or a workspace buffer
   int32_t beam, group, from_input, ntpl;
   int32_t ntiles, W, tpl_begin, box;  // tpl_begin: global template index
@@ -181,7 +182,7 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     const BSeg *sg = segs + si;
     const int32_t ntiles = sg->ntiles, W = sg->W;
     const bool from_input = sg->from_input != 0;
-    const int64_t nt = sg->nt;
+    const int64_t nt = sg->nt, pitch = sg->pitch;
     const int64_t T0 = (int64_t)((int32_t)(item - sg->first) % ntiles) * W;
     // The next item: its segment, template and (warp 0) copy descriptors.
     int nsi = si;
@@ -252,8 +253,8 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     constexpr bool kNarrow = std::is_same<TB, int32_t>::value;
     const bool i16 = kNarrow && sg->in_size == 2, o16 = kNarrow && sg->out_size == 2;
     const int n_stages = cur.n_stages;
-    batch_first_stage<TI, TB, A, GEN>(from_input, i16, o16, bar, prog_at(slot), n_stages, warp, lane, sg->out, nt, T0,
-                                      0, lim);
+    batch_first_stage<TI, TB, A, GEN>(from_input, i16, o16, bar, prog_at(slot), n_stages, warp, lane, sg->out, pitch,
+                                      T0, 0, lim);
     __syncthreads();  // the staged rows are no longer read; s_early is visible
     const bool early = *s_early != 0;
     if (early && warp == 0) {
@@ -267,10 +268,12 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     const SearchArgs no_search{};
     if (kNarrow && o16)
       item_later_stages<A, uint16_t, false, false, GEN>(bar, prog_at(slot), n_stages, nullptr, warp, lane,
-                                                        static_cast<uint16_t *>(sg->out), nt, T0, 0, lim, 0, no_search);
+                                                        static_cast<uint16_t *>(sg->out), pitch, T0, 0, lim, 0,
+                                                        no_search);
     else
       item_later_stages<A, TB, false, false, GEN>(bar, prog_at(slot), n_stages, nullptr, warp, lane,
-                                                  static_cast<TB *>(sg->out), nt, T0, 0, lim, 0, no_search);
+                                                  static_cast<TB *>(sg->out), pitch, T0, 0, lim, 0,
+                                                  no_search);
     slot ^= 1u;
     if (threadIdx.x == 0) *s_next = nn;
     __syncthreads();  // all of this item's stores are issued; Pa / Pb are free; s_next is visible
@@ -364,6 +367,7 @@ void build_segments(FusedBatch *fb, int drop_beam, int drop_group) {
       BSeg s{};
       s.first = first;
       s.nt = fb->desc[b].nt;
+      s.pitch = g + 1 == fp.groups.size() ? s.nt : fp.state_nt;
       s.beam = b;
       s.group = (int32_t)g;
       s.from_input = gr.from_input ? 1 : 0;
@@ -556,7 +560,7 @@ int fused_batch_execute(FusedBatch *fb, const void *const *in, void *const *out,
       if (!make_group_maps(&maps[k * kMapsPerSeg], gr, base,
                            g == 0 ? in_type : (narrow_in ? map_type<uint16_t>() : st_type),
                            g == 0 ? in_elem : (uint32_t)gr.in_size,
-                           rows, (uint64_t)fb->desc[b].nt, &cshift)) {
+                           rows, (uint64_t)(g == 0 ? fb->desc[b].nt : fp.state_nt), &cshift)) {
         fb->key.clear();
         return FDMT_ERR_INVALID_ARG;
       }

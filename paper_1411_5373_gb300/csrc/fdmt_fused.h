@@ -267,6 +267,7 @@ struct FusedParams {
 
 struct FusedPlan {
   int32_t W = 0;  // tile of the first group (each group has its own)
+  int64_t state_nt = 0;  // samples from one row to the next of the levels between launches (>= nt)
   int32_t state_size = 4, input_size = 4, acc_size = 4;
   std::vector<int32_t> level_size;  // [l]: bytes per stored sample of level l (level L: the output)
   std::vector<FusedGroup> groups;

@@ -180,11 +180,13 @@ cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const vo
   using TS = typename std::conditional<FI, TI, TB>::type;
   TmaMaps maps;
   int32_t cshift = 0;
-  if (!make_group_maps(maps.m, g, base, map_type<TS>(), sizeof(TS), (uint64_t)base_rows, (uint64_t)nt, &cshift))
+  // Rows of the levels between launches are state_nt apart.
+  const int64_t state_nt = dt.fused->state_nt, base_nt = FI ? nt : state_nt;
+  if (!make_group_maps(maps.m, g, base, map_type<TS>(), sizeof(TS), (uint64_t)base_rows, (uint64_t)base_nt, &cshift))
     return cudaErrorInvalidValue;
   const int32_t box = g.box;
   const int64_t ntiles = g.ntiles - tile0, items = (int64_t)g.tpl_count * ntiles;
-  const OutView v = view != nullptr ? *view : OutView{0, nt};
+  const OutView v = view != nullptr ? *view : OutView{0, g.lt == dt.levels ? nt : state_nt};
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFusedLaunchThreads, g.smem_bytes);
   if (e != cudaSuccess) return e;

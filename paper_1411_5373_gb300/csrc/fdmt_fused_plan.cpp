@@ -51,6 +51,7 @@ constexpr double kByteSeconds = 0.67e-12;    //   and byte copied
 constexpr double kAloneShare = 0.6;          // time of an item whose block has an SM to itself
 constexpr double kWaveTail = 0.7;            // a started wave counts as at most this much more than its items
 constexpr double kSms = 152;
+constexpr int64_t kPadRows = 4096;           // rows from this length on are padded between launches
 constexpr double kMaxBlocksPerSm = 2;        // the fused kernel's register budget
 
 int64_t round_up(int64_t v, int64_t a) { return (v + a - 1) / a * a; }
@@ -976,7 +977,7 @@ GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int3
   const int32_t chunk = std::min(128 / es, 64);
   // (mapped channels start at their own columns: row boxes)
   const bool mapped = lb == 0 && prm.in_shift != nullptr;
-  const bool blocks = staging != 1 && nt % chunk == 0 && !mapped;
+  const bool blocks = staging != 1 && (lb == 0 ? nt : fp.state_nt) % chunk == 0 && !mapped;
   if (staging == 2 && nt % chunk != 0) return GroupBuild();
   StageFmt boxes;
   boxes.search_k = search_k;
@@ -1228,6 +1229,12 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
   FusedPlan fp;
   fp.state_size = state_size;
   fp.input_size = input_size;
+  // Rows between launches are padded to whole chunks so that they can be
+  // staged as row blocks whatever nt (a row box takes two to four copies per
+  // row: 1000 x 50004 x 777 float32, launches [3,6] [6,10]: 87 and 88 us with
+  // boxes, 64 and 65 us with padded rows).  Columns past nt are never needed.
+  // Short rows keep their length: their launches are not bound by copies.
+  fp.state_nt = p.staging == 0 && nt >= kPadRows ? round_up(nt, 64) : nt;
   fp.acc_size = 4;
   // Stored element size of each level at a launch boundary; the output
   // (level L) is 4 bytes.  With p.narrow (integer sums of uint8 samples), a
@@ -1308,7 +1315,7 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
   // Intermediate states between groups: group g writes buffer g % 2.
   size_t even = 0, odd = 0;
   for (size_t g = 0; g + 1 < fp.groups.size(); ++g) {
-    const size_t bytes = (size_t)t.level_rows[fp.groups[g].lt] * (size_t)nt * (size_t)fp.level_size[fp.groups[g].lt];
+    const size_t bytes = (size_t)t.level_rows[fp.groups[g].lt] * (size_t)fp.state_nt * (size_t)fp.level_size[fp.groups[g].lt];
     if (g & 1) odd = std::max(odd, bytes); else even = std::max(even, bytes);
   }
   fp.ws_split = (size_t)round_up((int64_t)even, 256);
