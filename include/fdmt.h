@@ -681,7 +681,7 @@ int fdmt_schedule_info(fdmt_plan_t plan, int32_t *groups, int32_t *bounds, int32
  * 2 two levels, then the first walk or op of each of the 8 warps and the
  * end),
  * 6 constants (tile, state size, input size, acc size, bytes of over-read
- * slack that end a block's shared memory, bytes of the warps' descriptor
+ * slack that end a block's shared memory, least bytes of the programme
  * slots before it), 7 the planner's cost
  * model per group (6 each: HBM KiB, shared-memory pipe kilo-slots, work
  * items, thousands of ops, resident blocks, modelled microseconds), 8 runs

@@ -3,10 +3,10 @@
 // fdmt_adjoint_fused.h).
 //
 // One block computes one cone for one time tile, persistent over items as
-// the forward cone kernel: warp 0 stages the cone's level-lt gradient rows
-// by TMA (zeros past Nt), every thread waits on the mbarrier (bounded: on
-// timeout the block sets the plan's status word and returns), then the
-// stages run level by level, each child row summing its run of parent rows
+// the forward cone kernel: a copying warp stages the cone's level-lt gradient
+// rows by TMA (zeros past Nt) with the item's programme, the computing warps
+// wait on the mbarrier (bounded: on timeout the block sets the plan's status
+// word and returns), then the stages run level by level, each child row summing its run of parent rows
 // in increasing row order; the last stage writes the owned level-lb rows,
 // or the input gradient (the Option-1 transpose) in the launch that ends at
 // level 0.  The next item's copies go out as soon as the first stage has
@@ -15,11 +15,11 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "fdmt_adjoint_fused.h"
 #include "fdmt_fused_dev.cuh"
 #include "fdmt_internal.h"
+#include "fdmt_residency.h"
 #include "fdmt_tma.h"
 
 namespace fdmt {
@@ -48,83 +48,6 @@ __device__ __forceinline__ void st_piece_smem(uint32_t addr, const float (&v)[kL
   }
 }
 
-// A warp's descriptor stream through the stages of its items.  The words
-// of the stage that runs next (its kind and this warp's first and end
-// descriptor) are requested one stage ahead; during the last chunk of a
-// stage the first chunk of the next stage (or of the next item's first
-// stage) comes into `q`, so a stage starts without a round trip to L2.
-struct DescStream {
-  uint32_t slot;      // the warp's slot in shared memory (kDescSlotBytes)
-  int4 q;             // this lane's 16 bytes of the next stage's first chunk
-  int kind, i0, i1;   // the next stage (kind < 0: none)
-  bool ready;         // q holds that chunk
-};
-
-// Request the words of stage s of template tp (none if tp is null).
-__device__ __forceinline__ void ds_peek(DescStream &ds, const int32_t *__restrict__ stages,
-                                        const FusedTemplate *tp, int s, int warp) {
-  ds.ready = false;
-  if (tp == nullptr || s >= tp->n_stages) {
-    ds.kind = -1;
-    ds.i0 = ds.i1 = 0;
-    return;
-  }
-  const int32_t *p = stages + tp->stage_begin + s * kStageWords;
-  ds.kind = __ldg(p);
-  ds.i0 = __ldg(p + 1 + warp);
-  ds.i1 = __ldg(p + 2 + warp);
-}
-
-// Load the first chunk of the requested stage into q.
-__device__ __forceinline__ void ds_load_first(DescStream &ds, const FusedOp *__restrict__ ops, int lane) {
-  if (ds.ready || ds.kind < 0) return;
-  int4 q = make_int4(0, 0, 0, 0);
-  if (2 * ds.i0 + lane < 2 * ds.i1) q = __ldg(reinterpret_cast<const int4 *>(ops) + 2 * ds.i0 + lane);
-  ds.q = q;
-  ds.ready = true;
-}
-
-// The stage about to run (the one requested last) as a range of ops.
-struct OpRange {
-  int kind, i0, i1;
-};
-__device__ __forceinline__ OpRange ds_take(const DescStream &ds) { return OpRange{ds.kind, ds.i0, ds.i1}; }
-
-// A warp's descriptor slot: the template's layout ends with the slots of
-// the block's warps, then the over-read slack.
-__device__ __forceinline__ uint32_t desc_slot(uint32_t sbase, const FusedTemplate &tp, int warp) {
-  return sbase + (uint32_t)(tp.smem_bytes - kOverRead - kDescBytes + warp * kDescSlotBytes);
-}
-
-// Runs body(op) for ops i0 .. i1 - 1 of this warp, in order.  The lanes copy
-// the descriptors kDescChunk at a time (two lanes per 32-byte op) into the
-// warp's slot; the next chunk's loads are in flight while the current chunk
-// runs (for the last chunk: the next stage's first chunk), and every op is
-// read back from the slot as a broadcast.  On entry ds.q holds the first
-// chunk if ds.ready; ds's stage words are the next stage's.
-template <class F>
-__device__ __forceinline__ void for_ops(const FusedOp *__restrict__ ops, int i0, int i1, DescStream &ds, int lane,
-                                        F &&body) {
-  const int4 *src = reinterpret_cast<const int4 *>(ops);
-  int4 q = ds.q;
-  if (!ds.ready) q = (2 * i0 + lane < 2 * i1) ? __ldg(src + 2 * i0 + lane) : make_int4(0, 0, 0, 0);
-  ds.ready = false;
-  for (int base = i0; base < i1; base += kDescChunk) {
-    __syncwarp();  // every lane is done with the previous chunk
-    sts_v4(ds.slot + 16u * (uint32_t)lane, q);
-    __syncwarp();
-    const int nb = base + kDescChunk;
-    if (nb < i1) {
-      if (2 * nb + lane < 2 * i1) q = __ldg(src + 2 * nb + lane);
-    } else {
-      ds_load_first(ds, ops, lane);
-    }
-    const int n = min(kDescChunk, i1 - base);
-    for (int k = 0; k < n; ++k) body(lds_desc<FusedOp>(ds.slot + 32u * (uint32_t)k));
-  }
-  if (i0 >= i1) ds_load_first(ds, ops, lane);
-}
-
 // out_row[t] for t = t0 + lane + 32 k: written where the piece column is
 // below `width` and 0 <= t < nt (bands tile time with their own offset, so
 // t0 may be negative).
@@ -145,76 +68,43 @@ __device__ __forceinline__ void adj_store_global(float *__restrict__ out_row, in
   }
 }
 
-// The ops of a stage two at a time, body(a, b, two) (b = a when the stage
-// has an odd op left), so that each warp keeps the loads of two ops in
-// flight.  Descriptor chunks as in for_ops.
-template <class F>
-__device__ __forceinline__ void for_op_pairs(const FusedOp *__restrict__ ops, int i0, int i1, DescStream &ds,
-                                             int lane, F &&body) {
-  const int4 *src = reinterpret_cast<const int4 *>(ops);
-  int4 q = ds.q;
-  if (!ds.ready) q = (2 * i0 + lane < 2 * i1) ? __ldg(src + 2 * i0 + lane) : make_int4(0, 0, 0, 0);
-  ds.ready = false;
-  for (int base = i0; base < i1; base += kDescChunk) {
-    __syncwarp();  // every lane is done with the previous chunk
-    sts_v4(ds.slot + 16u * (uint32_t)lane, q);
-    __syncwarp();
-    const int nb = base + kDescChunk;
-    if (nb < i1) {
-      if (2 * nb + lane < 2 * i1) q = __ldg(src + 2 * nb + lane);
-    } else {
-      ds_load_first(ds, ops, lane);
-    }
-    const int n = min(kDescChunk, i1 - base);
-    for (int k = 0; k < n; k += 2) {
-      const bool two = k + 1 < n;
-      const uint32_t sa = ds.slot + 32u * (uint32_t)k, sb = two ? sa + 32u : sa;
-      const int4 a0 = lds_v4(sa), a1 = lds_v4(sa + 16u), b0 = lds_v4(sb), b1 = lds_v4(sb + 16u);
-      body(FusedOp{a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w},
-           FusedOp{b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w}, two);
-    }
-  }
-  if (i0 >= i1) ds_load_first(ds, ops, lane);
-}
-
 // One transposed level: each op sums its run of p2 parent rows (stride p1
 // bytes; the upper half's stride includes the one-column shift per row).
 template <int OUT>
-__device__ __forceinline__ void adj_gather_stage(uint32_t sbase, const FusedOp *__restrict__ ops, int i0, int i1,
-                                                 DescStream &ds, int lane, float *__restrict__ out, int64_t nt,
-                                                 int64_t T0) {
-  for_ops(ops, i0, i1, ds, lane, [&](const FusedOp &op) {
+__device__ __forceinline__ void adj_gather_stage(uint32_t sbase, const StageRange &range, int lane,
+                                                 float *__restrict__ out, int64_t nt, int64_t T0) {
+  for (uint32_t at = range.first; at != range.end; at += (uint32_t)sizeof(FusedOp)) {
+    const FusedOp op = prog_desc<FusedOp>(range.prog, at);
+    const int terms = warp_all(op.p2);
     // the sum starts from the first row of the run and adds the others in
     // row order; runs of one to three rows (nearly all) are straight-line
     float v[kLaneCols];
     const uint32_t a0 = sbase + (uint32_t)op.p0;
     const uint32_t step = (uint32_t)op.p1;
     ld_piece<float, float>(v, a0, lane);
-    if (op.p2 == 2) {
+    if (terms == 2) {
       float x[kLaneCols];
       ld_piece<float, float>(x, a0 + step, lane);
-#pragma unroll
-      for (int k = 0; k < kLaneCols; ++k) v[k] = __fadd_rn(v[k], x[k]);
-    } else if (op.p2 == 3) {
+      add_piece(v, v, x);
+    } else if (terms == 3) {
       float x[kLaneCols], y[kLaneCols];
       ld_piece<float, float>(x, a0 + step, lane);
       ld_piece<float, float>(y, a0 + 2 * step, lane);
-#pragma unroll
-      for (int k = 0; k < kLaneCols; ++k) v[k] = __fadd_rn(__fadd_rn(v[k], x[k]), y[k]);
-    } else if (op.p2 > 3) {
+      add_piece(v, v, x);
+      add_piece(v, v, y);
+    } else if (terms > 3) {
       uint32_t a = a0 + step;
-      for (int j = 1; j < op.p2; ++j, a += step) {
+      for (int j = 1; j < terms; ++j, a += step) {
         float x[kLaneCols];
         ld_piece<float, float>(x, a, lane);
-#pragma unroll
-        for (int k = 0; k < kLaneCols; ++k) v[k] = __fadd_rn(v[k], x[k]);
+        add_piece(v, v, x);
       }
     }
     if constexpr (OUT == kOutSmem)
       st_piece_smem(sbase + (uint32_t)op.dst, v, op.width, lane);
     else
       adj_store_global(out + (int64_t)op.dst * nt, T0 + op.col, v, op.width, nt, lane);
-  });
+  }
 }
 
 // Transpose of the Option-1 initialisation for one channel:
@@ -259,15 +149,13 @@ __device__ __forceinline__ void adj_init_op(uint32_t sbase, const FusedOp &op, c
         for (int q = 1; q < cnt; ++q) {
           float y[kLaneCols];
           ld_piece<float, float>(y, a + (uint32_t)q * step, lane);
-#pragma unroll
-          for (int k = 0; k < kLaneCols; ++k) r[k] = __fadd_rn(r[k], y[k]);
+          add_piece(r, r, y);
         }
         if (j == 0) {
 #pragma unroll
           for (int k = 0; k < kLaneCols; ++k) v[k] = r[k];
         } else {
-#pragma unroll
-          for (int k = 0; k < kLaneCols; ++k) v[k] = __fadd_rn(v[k], r[k]);
+          add_piece(v, v, r);
         }
       }
       pj += (uint32_t)cnt * step - back;
@@ -279,8 +167,7 @@ __device__ __forceinline__ void adj_init_op(uint32_t sbase, const FusedOp &op, c
       for (int ii = 0; ii <= j; ++ii) {
         float y[kLaneCols];
         ld_piece<float, float>(y, row + (uint32_t)(4 * ii), lane);
-#pragma unroll
-        for (int k = 0; k < kLaneCols; ++k) v[k] = __fadd_rn(v[k], y[k]);
+        add_piece(v, v, y);
       }
     }
   }
@@ -310,11 +197,15 @@ __device__ __forceinline__ void adj_init_op(uint32_t sbase, const FusedOp &op, c
 // (for the weight gradient) are requested before either op's sums, so the
 // two loads' latencies overlap.
 template <bool FOLD>
-__device__ __forceinline__ void adj_init_stage(uint32_t sbase, const FusedOp *__restrict__ ops, int i0, int i1,
-                                               DescStream &ds, int lane, float *__restrict__ out, int64_t nt,
-                                               int64_t T0, const float *__restrict__ w, const float *__restrict__ x,
+__device__ __forceinline__ void adj_init_stage(uint32_t sbase, const StageRange &range, int lane,
+                                               float *__restrict__ out, int64_t nt, int64_t T0,
+                                               const float *__restrict__ w, const float *__restrict__ x,
                                                float *__restrict__ part, int64_t part_row) {
-  for_op_pairs(ops, i0, i1, ds, lane, [&](const FusedOp &a, const FusedOp &b, bool two) {
+  constexpr uint32_t kOp = (uint32_t)sizeof(FusedOp);
+  for (uint32_t at = range.first; at != range.end;) {
+    const bool two = at + kOp != range.end;
+    const FusedOp a = prog_desc<FusedOp>(range.prog, at), b = prog_desc<FusedOp>(range.prog, two ? at + kOp : at);
+    at += two ? 2 * kOp : kOp;
     float xa[kLaneCols], xb[kLaneCols];
     if (part != nullptr) {
       adj_init_load_x(xa, a, x, nt, T0, lane);
@@ -322,100 +213,64 @@ __device__ __forceinline__ void adj_init_stage(uint32_t sbase, const FusedOp *__
     }
     adj_init_op<FOLD>(sbase, a, xa, lane, out, nt, T0, w, part, part_row);
     if (two) adj_init_op<FOLD>(sbase, b, xb, lane, out, nt, T0, w, part, part_row);
-  });
+  }
 }
 
-// Persistent blocks over items = template * ntiles + tile, as the forward
-// cone kernel.  INIT: the last stage is the initialisation transpose; it
-// keeps two ops' input samples in flight, so it is compiled for two
-// resident blocks per SM (more registers per thread).
+// Persistent blocks as the forward cone kernel: eight computing warps, one
+// that copies (copy_items).  INIT: the last stage is the initialisation
+// transpose.
+// Bound: latency and HBM alike.  1024 x 65536 x 1024 on a GB300, launches 10
+// -> 8 -> 6 -> 4 -> 2 -> 0 with the weight gradient: 112, 110, 116, 126 and
+// 264 us with ops read through L2 and warp 0 copying; 98, 97, 101, 104 and 248 us now.
 template <bool INIT>
-__global__ void __launch_bounds__(kFusedThreads, INIT ? 2 : 3)
+__global__ void __launch_bounds__(kFusedLaunchThreads, kFusedMinBlocks)
 adjoint_cone_kernel(const __grid_constant__ TmaMaps maps, float *__restrict__ out, int64_t nt, int32_t W,
-                    int64_t ntiles, int64_t items, const FusedTemplate *__restrict__ tpls,
-                    const FusedLoad *__restrict__ loads, const FusedOp *__restrict__ ops,
-                    const int32_t *__restrict__ stages, const float *__restrict__ w, int32_t box,
-                    int32_t cshift, int *__restrict__ status, const float *__restrict__ x,
+                    int32_t ntiles, int64_t items, const FusedProg *__restrict__ progs, const int4 *__restrict__ prog,
+                    const FusedLoad *__restrict__ loads, const float *__restrict__ w, int32_t box, int32_t cshift,
+                    int32_t prog_off, int32_t prog_slot, int *__restrict__ status, const float *__restrict__ x,
                     float *__restrict__ part, int32_t pieces) {
   extern __shared__ __align__(128) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t bar = smem_u32(smem);
-
-  int64_t item = blockIdx.x;
-  if (item >= items) return;
-  if (threadIdx.x == 0) {
-    mbar_init(bar, 1);
-    fence_mbar_init();
+  const int warp = warp_all((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
+  const uint32_t full = smem_u32(smem);
+  init_item_barriers(full);
+  if (warp == kFusedWarps) {
+    copy_items<float>(smem, maps, nt, W, 0, ntiles, items, progs, prog, loads, box, cshift, prog_off, prog_slot, status,
+                      lane);
+    return;
   }
-  int64_t tile = (int64_t)blockIdx.x % ntiles, tpl = (int64_t)blockIdx.x / ntiles;
-  const int64_t step_tile = (int64_t)gridDim.x % ntiles, step_tpl = (int64_t)gridDim.x / ntiles;
-  auto advance = [&]() {
-    tile += step_tile;
-    tpl += step_tpl;
-    if (tile >= ntiles) {
-      tile -= ntiles;
-      ++tpl;
-    }
-  };
-  FusedTemplate tp = tpls[tpl];
-  __syncthreads();
-  int64_t T0_cur = tile * (int64_t)W;
-  if (warp == 0)
-    stage_item<float>(smem, bar, maps.m, tp, loads, fetch_load(tp, loads, lane), T0_cur, box, cshift, lane);
-  advance();
-  FusedTemplate tp_next = FusedTemplate{0, 0, 0, 0, 0, 0, 0, 0};
-  if (item + gridDim.x < items) tp_next = tpls[tpl];
-  DescStream ds;
-  ds.slot = desc_slot(bar, tp, warp);
-  ds_peek(ds, stages, &tp, 0, warp);
-  uint32_t phase = 0;
-  for (; item < items; item += gridDim.x) {
-    const FusedTemplate cur = tp;
-    const int64_t T0 = T0_cur;
-    const int64_t next = item + gridDim.x;
-    const int64_t T0_next = tile * (int64_t)W;
-    FusedLoad ld_next = FusedLoad{0, 0, 0, 0};
-    if (warp == 0 && next < items) ld_next = fetch_load(tp_next, loads, lane);
-    if (!mbar_wait_bounded(bar, phase)) {
+  uint32_t slot = 0, phase = 0;
+  for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const bool ok = mbar_wait_bounded(full, phase);
+    phase ^= 1u;
+    // every computing warp has left the item before, whose regions the
+    // first stage overwrites
+    if (!compute_sync_and(ok)) {
       atomicExch(status, 1);
-      mbar_wait_bounded(bar, phase);
       return;
     }
-    phase ^= 1u;
-    {
-      const OpRange r = ds_take(ds);
-      if (cur.n_stages > 1) ds_peek(ds, stages, &cur, 1, warp);
-      else ds_peek(ds, stages, next < items ? &tp_next : nullptr, 0, warp);
-      if (!INIT && cur.n_stages == 1) adj_gather_stage<kOutGlobal>(bar, ops, r.i0, r.i1, ds, lane, out, nt, T0);
-      else adj_gather_stage<kOutSmem>(bar, ops, r.i0, r.i1, ds, lane, out, nt, T0);
-    }
-    __syncthreads();  // S is no longer read: stage the next item into it
-    if (next < items) {
-      if (warp == 0) stage_item<float>(smem, bar, maps.m, tp_next, loads, ld_next, T0_next, box, cshift, lane);
-      tp = tp_next;
-      advance();
-      if (next + gridDim.x < items) tp_next = tpls[tpl];
-      T0_cur = T0_next;
-    }
-    for (int s = 1; s < cur.n_stages; ++s) {
-      const OpRange r = ds_take(ds);
-      if (s + 1 < cur.n_stages) ds_peek(ds, stages, &cur, s + 1, warp);
-      else ds_peek(ds, stages, next < items ? &tp : nullptr, 0, warp);
-      if (s == cur.n_stages - 1) {
-        if (INIT) {
-          float *const pt = part != nullptr ? part + (T0 / W) * pieces : nullptr;
-          if (r.kind == kAdjInitF)
-            adj_init_stage<true>(bar, ops, r.i0, r.i1, ds, lane, out, nt, T0, w, x, pt, ntiles * pieces);
-          else
-            adj_init_stage<false>(bar, ops, r.i0, r.i1, ds, lane, out, nt, T0, w, x, pt, ntiles * pieces);
-        }
-        else adj_gather_stage<kOutGlobal>(bar, ops, r.i0, r.i1, ds, lane, out, nt, T0);
+    const int4 h = lds_v4(full + kItemHeader + 16u * slot);
+    const int n_stages = warp_all(h.z);
+    const int64_t T0 = (int64_t)h.x * W;
+    const Prog prg{full + (uint32_t)(prog_off + (int)slot * prog_slot), prog_slot > 0 ? nullptr : prog + h.w};
+    float *const pt = INIT && part != nullptr ? part + (int64_t)h.x * pieces : nullptr;
+    for (int s = 0; s < n_stages; ++s) {
+      if (s > 0) compute_sync();
+      const StageRange r = prog_stage(prg, s, warp);
+      if (s < n_stages - 1) {
+        adj_gather_stage<kOutSmem>(full, r, lane, out, nt, T0);
+      } else if (!INIT) {
+        adj_gather_stage<kOutGlobal>(full, r, lane, out, nt, T0);
+      } else if (r.kind == kAdjInitF) {
+        adj_init_stage<true>(full, r, lane, out, nt, T0, w, x, pt, (int64_t)ntiles * pieces);
       } else {
-        adj_gather_stage<kOutSmem>(bar, ops, r.i0, r.i1, ds, lane, out, nt, T0);
-        __syncthreads();
+        adj_init_stage<false>(full, r, lane, out, nt, T0, w, x, pt, (int64_t)ntiles * pieces);
+      }
+      if (s == 0) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full + kFreeBar);  // this warp reads S no more
       }
     }
-    __syncthreads();  // Pa / Pb are reused by the next item
+    slot ^= 1u;
   }
 }
 
@@ -437,15 +292,9 @@ adj_weights_finalize_kernel(const float *__restrict__ part, int32_t nf, int64_t 
 
 template <bool INIT>
 cudaError_t launch_adj_group(const DeviceTables &dt, const AdjGroup &g, const float *base, int64_t base_rows,
-                             float *dst, const float *w, int64_t nt, cudaStream_t s, const float *x = nullptr,
-                             float *part = nullptr) {
+                             int64_t base_nt, float *dst, const float *w, int64_t nt, cudaStream_t s,
+                             const float *x = nullptr, float *part = nullptr) {
   auto kern = adjoint_cone_kernel<INIT>;
-  static std::once_flag attr_once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(attr_once, [&] {
-    attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  });
-  if (attr_err != cudaSuccess) return attr_err;
   FusedGroup mg;  // the staged rows: row boxes of g.box samples or row blocks
   mg.box = g.box;
   mg.chunk = g.chunk;
@@ -453,24 +302,20 @@ cudaError_t launch_adj_group(const DeviceTables &dt, const AdjGroup &g, const fl
   mg.max_p = g.max_p;
   TmaMaps maps;
   int32_t cshift = 0;
-  if (!make_group_maps(maps.m, mg, base, map_type<float>(), sizeof(float), (uint64_t)base_rows, (uint64_t)nt,
+  if (!make_group_maps(maps.m, mg, base, map_type<float>(), sizeof(float), (uint64_t)base_rows, (uint64_t)base_nt,
                        &cshift))
     return cudaErrorInvalidValue;
   const int64_t items = (int64_t)g.tpl_count * g.ntiles;
   if (items == 0) return cudaSuccess;
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFusedThreads, g.smem_bytes);
+  int resident = 0;
+  const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(kern), kFusedLaunchThreads, g.smem_bytes, &resident);
   if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const int64_t blocks = std::min<int64_t>(items, (int64_t)per_sm * sms);
+  const int64_t blocks = std::min<int64_t>(items, resident);
   dt.prof->begin(s, K_ADJ_CONE, g.lb * 100 + g.lt);
-  kern<<<(unsigned)blocks, kFusedThreads, g.smem_bytes, s>>>(maps, dst, nt, g.W, g.ntiles, items,
-                                                            dt.a_tpls + g.tpl_begin, dt.a_loads, dt.a_ops,
-                                                            dt.a_stages, w, g.box, cshift, dt.status, x, part,
-                                                            g.pieces);
+  kern<<<(unsigned)blocks, kFusedLaunchThreads, g.smem_bytes, s>>>(
+      maps, dst, nt, g.W, (int32_t)g.ntiles, items, dt.a_progs + g.tpl_begin,
+      reinterpret_cast<const int4 *>(dt.a_prog), dt.a_loads, w, g.box, cshift, g.prog_off, g.prog_slot, dt.status, x,
+      part, g.pieces);
   dt.prof->end(s);
   return cudaGetLastError();
 }
@@ -488,9 +333,10 @@ cudaError_t run_adjoint_fused(const DeviceTables &dt, const float *grad_out, con
     const float *base = g == 0 ? grad_out : static_cast<const float *>(bufs[(g - 1) & 1]);
     float *dst = (g == G - 1) ? grad_in : static_cast<float *>(bufs[g & 1]);
     const int64_t rows = dt.level_rows[gr.lt];
-    const cudaError_t e = gr.init ? launch_adj_group<true>(dt, gr, base, rows, dst, w, nt, s, x,
+    const int64_t base_nt = g == 0 ? nt : ap.state_nt;
+    const cudaError_t e = gr.init ? launch_adj_group<true>(dt, gr, base, rows, base_nt, dst, w, nt, s, x,
                                                            grad_w != nullptr ? part : nullptr)
-                                  : launch_adj_group<false>(dt, gr, base, rows, dst, nullptr, nt, s);
+                                  : launch_adj_group<false>(dt, gr, base, rows, base_nt, dst, nullptr, ap.state_nt, s);
     if (e != cudaSuccess) return e;
   }
   if (grad_w == nullptr) return cudaSuccess;

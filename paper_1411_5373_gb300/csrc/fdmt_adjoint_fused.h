@@ -72,6 +72,7 @@ struct AdjGroup {
   int32_t tpl_begin = 0, tpl_count = 0;
   int32_t smem_bytes = 0;     // barrier + S + Pa + Pb + over-read slack
   int32_t s_end = 0, pa_end = 0;
+  int32_t prog_off = 0, prog_slot = 0;  // the two programme slots (FusedProg)
   int64_t ntiles = 0;         // tiles per template (time covered with the bands' offsets)
   int32_t pieces = 0;         // init launch: op pieces per channel and tile (weight-gradient partials)
   double hbm_bytes = 0;       // model: staged + written bytes per launch
@@ -90,11 +91,18 @@ struct AdjParams {
 };
 
 struct AdjFusedPlan {
+  // Samples from one row to the next of the levels between launches (>= nt):
+  // whole chunks, so that they are staged as row blocks whatever nt.  The
+  // columns past nt are written (they come out zero, as nothing reads a
+  // gradient there).
+  int64_t state_nt = 0;
   std::vector<AdjGroup> groups;   // in launch order (from level L down)
   std::vector<FusedTemplate> tpls;
   std::vector<FusedLoad> loads;
   std::vector<FusedOp> ops;
   std::vector<int32_t> stages;
+  std::vector<FusedProg> progs;  // per template: its stages and ops as one block,
+  std::vector<int32_t> prog;     //   in here
   // Workspace: the level between two launches, ping-pong (group g writes
   // buffer g % 2); bytes each buffer needs.
   size_t buf_bytes[2] = {0, 0};

@@ -13,7 +13,8 @@ namespace fdmt {
 namespace {
 
 constexpr int32_t kAdjBarrierBytes = 128;  // mbarrier slot; regions stay 128-byte aligned
-constexpr int32_t kAdjBox = 64;            // TMA box width of the staged rows (elements)
+constexpr int32_t kAdjBox = 64;            // provisional TMA box width of the staged rows (elements)
+constexpr int64_t kAdjPadRows = 4096;      // rows from this length on are padded between launches
 constexpr int64_t kAdjMaxSmem = 227 * 1024;
 constexpr int32_t kAdjChunk = 32;          // row blocks: chunks of 128 bytes
 
@@ -103,6 +104,7 @@ struct TNode {
 struct Shape {
   std::vector<std::vector<TNode>> nodes;  // [i][k] as the subtree
   int64_t s_bytes = 0, pa_bytes = 0, pb_bytes = 0;
+  int64_t n_stages = 0, n_ops = 0;  // of the item's programme
   bool any = false;  // the item owns something
 };
 
@@ -110,7 +112,7 @@ struct Shape {
 // fuse: the launch folds the level 1 -> 0 gather into the initialisation
 // transpose (level 0 is never stored).
 void shape(const Tables &t, const Subtree &st, int32_t lt, int32_t lb, bool init, bool fuse, int32_t r0,
-           int32_t r1, int32_t W, int32_t pitch, Shape &sh) {
+           int32_t r1, int32_t W, int32_t pitch, int32_t box, Shape &sh) {
   const int32_t m = lt - lb;
   sh = Shape();
   sh.nodes.resize(m + 1);
@@ -177,7 +179,7 @@ void shape(const Tables &t, const Subtree &st, int32_t lt, int32_t lb, bool init
   // than it does not fit)
   TNode &top = sh.nodes[0][0];
   if (!top.empty()) {
-    top.stride = pitch > 0 ? pitch : (int32_t)rup(top.need, kAdjBox);
+    top.stride = pitch > 0 ? pitch : (int32_t)rup(top.need, box);
     top.smem = 0;
     sh.s_bytes = top.need > top.stride ? (int64_t)1 << 40
                                        : rup((int64_t)(top.e - top.a + 1) * top.stride * 4, 128);
@@ -194,10 +196,30 @@ void shape(const Tables &t, const Subtree &st, int32_t lt, int32_t lb, bool init
     int64_t &region = ((i - 1) & 1) == 0 ? sh.pa_bytes : sh.pb_bytes;
     region = std::max(region, off);
   }
+  // The ops emit() makes of it: one per row and piece of a gather stage, one
+  // per channel and piece of the transpose.
+  const int32_t gathers = fuse ? m - 1 : m;
+  sh.n_stages = gathers + (init ? 1 : 0);
+  for (int32_t i = 1; i <= gathers; ++i)
+    for (const TNode &n : sh.nodes[i])
+      if (!n.empty())
+        sh.n_ops += (int64_t)(n.e - n.a + 1) * (((i == m && !init ? W : n.need) + kPieceCols - 1) / kPieceCols);
+  if (init)
+    for (const TNode &n : sh.nodes[m])
+      if (!n.empty()) sh.n_ops += (W + kPieceCols - 1) / kPieceCols;
 }
 
-int64_t shape_bytes(const Shape &sh) {
-  return kAdjBarrierBytes + sh.s_bytes + sh.pa_bytes + sh.pb_bytes + kDescBytes + kOverRead;
+// Bytes of one programme slot of an item (its stages' words and ops); 0
+// where the launch's programmes stay in global memory.
+int64_t prog_slot_bytes(const Shape &sh, bool far) {
+  if (far) return 0;
+  return std::max<int64_t>(kProgMinBytes / 2,
+                           rup(sh.n_stages * kProgStageBytes + sh.n_ops * (int64_t)sizeof(FusedOp), 128));
+}
+
+int64_t shape_bytes(const Shape &sh, bool far) {
+  return kAdjBarrierBytes + sh.s_bytes + sh.pa_bytes + sh.pb_bytes +
+         std::max<int64_t>(kProgMinBytes, 2 * prog_slot_bytes(sh, far)) + kOverRead;
 }
 
 // The wait of an init op for its input samples, in the cost's units
@@ -269,7 +291,7 @@ void emit(const Tables &t, const Subtree &st, int32_t lt, int32_t lb, bool init,
     }
   } else {
     for (int32_t d = top.a; d <= top.e; ++d)
-      out.loads.push_back(FusedLoad{row0 + d, top.smem + (d - top.a) * top.stride * 4, 0, top.stride / kAdjBox});
+      out.loads.push_back(FusedLoad{row0 + d, top.smem + (d - top.a) * top.stride * 4, 0, top.stride / g.box});
   }
   tp.load_count = (int32_t)out.loads.size() - tp.load_begin;
   tp.tx_bytes = (top.e - top.a + 1) * top.stride * 4;
@@ -407,7 +429,7 @@ void emit(const Tables &t, const Subtree &st, int32_t lt, int32_t lb, bool init,
 // pitch > 0: row blocks of `chunk` elements, every staged row `pitch` wide;
 // *widest receives the widest staged window of the launch's cones.
 std::string plan_group(const Tables &t, int64_t nt, int32_t lt, int32_t lb, int32_t W, int32_t budget, bool grow,
-                       int32_t pitch, int32_t chunk, AdjFusedPlan &out, AdjGroup &g, int32_t *widest) {
+                       int32_t pitch, int32_t chunk, int32_t box, bool far, AdjFusedPlan &out, AdjGroup &g, int32_t *widest) {
   const bool init = (lb == 0);
   const bool fuse = init && lt - lb >= 2 && init_fusable(t);
   g = AdjGroup();
@@ -415,7 +437,7 @@ std::string plan_group(const Tables &t, int64_t nt, int32_t lt, int32_t lb, int3
   g.lb = lb;
   g.init = init;
   g.W = W;
-  g.box = kAdjBox;
+  g.box = box;
   if (pitch > 0) {
     g.box = 0;
     g.chunk = chunk;
@@ -446,23 +468,23 @@ std::string plan_group(const Tables &t, int64_t nt, int32_t lt, int32_t lb, int3
     // range from r0 whose cone fits (binary search; the size grows with r1).
     for (int32_t r0 = 0; r0 < R;) {
       Shape sh;
-      shape(t, s, lt, lb, init, fuse, r0, r0, W, pitch, sh);
-      if (shape_bytes(sh) > budget) {
+      shape(t, s, lt, lb, init, fuse, r0, r0, W, pitch, box, sh);
+      if (shape_bytes(sh, far) > budget) {
         // One row's cone can need most of its band (a band whose upper half
         // is one channel: that channel's row reads every parent row); the
         // launch then takes the shared memory it needs, if allowed.
-        if (!grow || shape_bytes(sh) > kAdjMaxSmem)
+        if (!grow || shape_bytes(sh, far) > kAdjMaxSmem)
           return "unsupported: one row of level " + std::to_string(lt) + " does not fit";
-        budget = (int32_t)shape_bytes(sh);
+        budget = (int32_t)shape_bytes(sh, far);
       }
       int32_t lo = r0, hi = R - 1;
       while (lo < hi) {
         const int32_t mid = (lo + hi + 1) / 2;
-        shape(t, s, lt, lb, init, fuse, r0, mid, W, pitch, sh);
-        if (shape_bytes(sh) <= budget) lo = mid;
+        shape(t, s, lt, lb, init, fuse, r0, mid, W, pitch, box, sh);
+        if (shape_bytes(sh, far) <= budget) lo = mid;
         else hi = mid - 1;
       }
-      shape(t, s, lt, lb, init, fuse, r0, lo, W, pitch, sh);
+      shape(t, s, lt, lb, init, fuse, r0, lo, W, pitch, box, sh);
       if (sh.any) {
         *widest = std::max(*widest, sh.nodes[0][0].need);
         pieces.push_back(Piece{B, r0, lo, sh});
@@ -471,18 +493,21 @@ std::string plan_group(const Tables &t, int64_t nt, int32_t lt, int32_t lb, int3
     }
   }
   // Group-wide regions, tiles.
-  int64_t S = 0, Pa = 0, Pb = 0;
+  int64_t S = 0, Pa = 0, Pb = 0, slot = far ? 0 : kProgMinBytes / 2;
   int32_t omin = 0;
   for (const Piece &p : pieces) {
     S = std::max(S, p.sh.s_bytes);
     Pa = std::max(Pa, p.sh.pa_bytes);
     Pb = std::max(Pb, p.sh.pb_bytes);
+    slot = std::max(slot, prog_slot_bytes(p.sh, far));
     for (const TNode &n : p.sh.nodes.back())
       if (!n.empty()) omin = std::min(omin, n.o);
   }
-  const int64_t total = kAdjBarrierBytes + S + Pa + Pb + kDescBytes + kOverRead;
+  const int64_t total = kAdjBarrierBytes + S + Pa + Pb + std::max<int64_t>(kProgMinBytes, 2 * slot) + kOverRead;
   if (total > kAdjMaxSmem) return "unsupported: shared memory";
   g.smem_bytes = (int32_t)total;
+  g.prog_slot = (int32_t)slot;
+  g.prog_off = (int32_t)(kAdjBarrierBytes + S + Pa + Pb);
   g.s_end = (int32_t)(kAdjBarrierBytes + S);
   g.pa_end = (int32_t)(g.s_end + Pa);
   g.ntiles = (nt - omin + W - 1) / W;
@@ -499,14 +524,18 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
   if (L < 1) return "unsupported: no merge level";
   if (p.W < 64 || p.W % 64 != 0) return "tile must be a positive multiple of 64";
   if (p.smem_budget < 8 * 1024 || p.smem_budget > 227 * 1024) return "shared-memory budget out of range";
+  const int64_t state_nt = nt >= kAdjPadRows ? rup(nt, kAdjChunk) : nt;
   auto try_bounds = [&](const std::vector<int32_t> &bounds) -> std::string {
     out = AdjFusedPlan();
+    out.state_nt = state_nt;
     if (bounds.size() < 2 || bounds.front() != 0 || bounds.back() != L) return "bounds must run from 0 to L";
     for (size_t i = 1; i < bounds.size(); ++i)
       if (bounds[i] <= bounds[i - 1]) return "bounds must increase";
     for (size_t i = bounds.size() - 1; i >= 1; --i) {
       AdjGroup g;
       std::string err;
+      // Row lengths of what the launch reads and writes.
+      const int64_t in_nt = bounds[i] == L ? nt : state_nt, out_nt = bounds[i - 1] == 0 ? nt : state_nt;
       const size_t tpls = out.tpls.size(), loads = out.loads.size(), ops = out.ops.size(),
                    stages = out.stages.size();
       auto rollback = [&]() {
@@ -530,23 +559,32 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
           !p.bounds.empty() && i - 1 < p.group_budget.size() && p.group_budget[i - 1] > 0 ? p.group_budget[i - 1]
                                                                                           : p.smem_budget;
       if (W < 64 || W % 64 != 0 || budget < 8 * 1024 || budget > 227 * 1024) return "bad launch parameters";
+      // (and where an item leaves no room for its programme, the programmes
+      // stay in global memory)
+      bool far = false;
       for (;; W /= 2) {
-        err = plan_group(t, nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, out, g, &widest);
+        for (far = false;; far = true) {
+          err = plan_group(t, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, kAdjBox, far, out, g,
+                           &widest);
+          if (err.empty() || far) break;
+          rollback();
+        }
         if (err.empty() || !p.grow_budget || W / 2 < 64 || (W / 2) % 64 != 0) break;
         rollback();
       }
       if (!err.empty()) return err;
-      if (nt % kAdjChunk == 0) {
+      const int32_t measured = widest;
+      if (in_nt % kAdjChunk == 0) {
         // Row blocks: one TMA copy per 2^p staged rows, every row as wide as
         // the launch's widest window (rebuilt until the pitch covers all).
         AdjGroup gb;
         for (int iter = 0; iter < 4; ++iter) {
           const int32_t k = (widest + kAdjChunk - 1) / kAdjChunk;
-          if (k > 256 || (int64_t)k * kAdjChunk > nt) break;
+          if (k > 256 || (int64_t)k * kAdjChunk > in_nt) break;
           rollback();
           int32_t w2 = 0;
-          const std::string e2 = plan_group(t, nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget,
-                                            k * kAdjChunk, kAdjChunk, out, gb, &w2);
+          const std::string e2 = plan_group(t, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget,
+                                            k * kAdjChunk, kAdjChunk, 0, far, out, gb, &w2);
           if (!e2.empty()) break;
           if (w2 <= k * kAdjChunk) {
             g = gb;
@@ -555,11 +593,19 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
           }
           widest = w2;
         }
-        if (widest >= 0) {  // keep row boxes
+      }
+      if (widest >= 0) {
+        // Row boxes: as few of them per row as the widest window takes, of
+        // whole 128 bytes each.
+        const int32_t n = (measured + 255) / 256, box = (int32_t)rup((measured + n - 1) / n, 32);
+        rollback();
+        err = plan_group(t, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, box, far, out, g, &widest);
+        if (!err.empty()) {
           rollback();
-          err = plan_group(t, nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, out, g, &widest);
-          if (!err.empty()) return err;
+          err = plan_group(t, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, kAdjBox, far, out, g,
+                           &widest);
         }
+        if (!err.empty()) return err;
       }
       out.groups.push_back(g);
     }
@@ -598,10 +644,39 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
     gl.pieces = (gl.W + kPieceCols - 1) / kPieceCols;
     out.part_slots = (int64_t)t.nf * gl.ntiles * gl.pieces;
   }
+  // The templates' programmes.
+  for (const AdjGroup &g : out.groups)
+    for (int32_t i = g.tpl_begin; i < g.tpl_begin + g.tpl_count; ++i) {
+      const FusedTemplate &tp = out.tpls[i];
+      std::vector<int32_t> words((size_t)tp.n_stages * (kProgStageBytes / 4), 0);
+      for (int32_t s = 0; s < tp.n_stages; ++s) {
+        const int32_t *src = out.stages.data() + tp.stage_begin + s * kStageWords;
+        const size_t at = (size_t)s * (kProgStageBytes / 4);
+        words[at] = src[0];
+        for (int32_t w = 1; w < kStageWords; ++w)
+          words[at + w] = (int32_t)words.size() * 4 + (src[w] - src[1]) * (int32_t)sizeof(FusedOp);
+        const int32_t *d = reinterpret_cast<const int32_t *>(out.ops.data() + src[1]);
+        words.insert(words.end(), d, d + (size_t)(src[kStageWords - 1] - src[1]) * sizeof(FusedOp) / 4);
+      }
+      FusedProg pr{};
+      pr.load_begin = tp.load_begin;
+      pr.load_count = tp.load_count;
+      pr.n_stages = tp.n_stages;
+      pr.prog = (int32_t)(out.prog.size() / 4);
+      pr.prog_bytes = (int32_t)words.size() * 4;
+      pr.far = g.prog_slot == 0 ? 1 : 0;
+      pr.tx_bytes = tp.tx_bytes + (pr.far ? 0 : pr.prog_bytes);
+      if (!pr.far && pr.prog_bytes > g.prog_slot) {
+        out = AdjFusedPlan();
+        return "internal: a programme outgrew its slot";
+      }
+      out.prog.insert(out.prog.end(), words.begin(), words.end());
+      out.progs.push_back(pr);
+    }
   // Group k writes level lb_k into buffer k % 2 (the last writes the input
   // gradient).
   for (size_t k = 0; k + 1 < out.groups.size(); ++k) {
-    const size_t b = (size_t)t.level_rows[out.groups[k].lb] * (size_t)nt * sizeof(float);
+    const size_t b = (size_t)t.level_rows[out.groups[k].lb] * (size_t)out.state_nt * sizeof(float);
     out.buf_bytes[k & 1] = std::max(out.buf_bytes[k & 1], b);
   }
   return "";

@@ -112,7 +112,7 @@ void profile_release(fdmt::Profiler &pr) {
 void free_device(fdmt_plan_s *p) {
   DeviceTables &d = p->dev;
   void *ptrs[] = {d.init, d.ops, d.adj, d.adj2, d.adj2_terms, d.status, d.f_progs, d.f_prog, d.f_loads,
-                  d.f_ops, d.in_shift, d.a_tpls, d.a_loads, d.a_ops, d.a_stages};
+                  d.f_ops, d.in_shift, d.a_progs, d.a_prog, d.a_loads};
   for (void *q : ptrs)
     if (q) cudaFree(q);
   d.init = nullptr;
@@ -126,10 +126,9 @@ void free_device(fdmt_plan_s *p) {
   d.f_loads = nullptr;
   d.f_ops = nullptr;
   d.in_shift = nullptr;
-  d.a_tpls = nullptr;
+  d.a_progs = nullptr;
+  d.a_prog = nullptr;
   d.a_loads = nullptr;
-  d.a_ops = nullptr;
-  d.a_stages = nullptr;
 }
 
 int check_exec_common(fdmt_plan_t plan, void *workspace, size_t ws_bytes, size_t need) {
@@ -353,10 +352,9 @@ int fdmt_plan_curve(double f_min, double f_max, int32_t nf, int64_t nt, int32_t 
     }
     if (e == cudaSuccess && p->has_adj_fused) {
       d.adj_fused = &p->adj_fused;
-      e = upload(p->adj_fused.tpls, &d.a_tpls);
+      e = upload(p->adj_fused.progs, &d.a_progs);
+      if (e == cudaSuccess) e = upload(p->adj_fused.prog, &d.a_prog);
       if (e == cudaSuccess) e = upload(p->adj_fused.loads, &d.a_loads);
-      if (e == cudaSuccess) e = upload(p->adj_fused.ops, &d.a_ops);
-      if (e == cudaSuccess) e = upload(p->adj_fused.stages, &d.a_stages);
     }
     if (e != cudaSuccess) {
       free_device(p);
@@ -699,7 +697,7 @@ int fdmt_fused_tables(fdmt_plan_t plan, int32_t kind, int32_t *dst, int64_t n, i
       v = f.stages;
       break;
     case 6:
-      v = {f.W, f.state_size, f.input_size, f.acc_size, fdmt::kOverRead, fdmt::kDescBytes};
+      v = {f.W, f.state_size, f.input_size, f.acc_size, fdmt::kOverRead, fdmt::kProgMinBytes};
       break;
     case 7:
       // cost-model inputs per group: HBM KiB, shared-memory pipe kilo-slots,

@@ -88,7 +88,7 @@ __device__ __forceinline__ void stage_seg_item(unsigned char *smem, uint32_t bar
     stage_item<uint16_t>(smem, bar, m, tp, loads, first, T0, sg->box, sg->cshift, lane);
   else
     stage_item<TB>(smem, bar, m, tp, loads, first, T0, sg->box, sg->cshift, lane);
-  if (lane == 0) stage_prog(prog_dst, tp, prog, bar);
+  if (lane == 0 && !tp.far) stage_prog(prog_dst, tp, prog, bar);
 }
 
 // The first stage of an item with the segment's runtime types: the input
@@ -97,7 +97,7 @@ __device__ __forceinline__ void stage_seg_item(unsigned char *smem, uint32_t bar
 // GEN: some beam's plan has pass-through stages (as for the single-beam
 // kernel); the batch has no channel weights.
 template <class TI, class TB, class A, bool GEN>
-__device__ __forceinline__ void batch_first_stage(bool from_input, bool i16, bool o16, uint32_t bar, uint32_t prog,
+__device__ __forceinline__ void batch_first_stage(bool from_input, bool i16, bool o16, uint32_t bar, const Prog &prog,
                                                   int n_stages, int warp, int lane, void *out, int64_t nt, int64_t T0,
                                                   int lo, int lim) {
   TB *o = static_cast<TB *>(out);
@@ -253,7 +253,8 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     constexpr bool kNarrow = std::is_same<TB, int32_t>::value;
     const bool i16 = kNarrow && sg->in_size == 2, o16 = kNarrow && sg->out_size == 2;
     const int n_stages = cur.n_stages;
-    batch_first_stage<TI, TB, A, GEN>(from_input, i16, o16, bar, prog_at(slot), n_stages, warp, lane, sg->out, pitch,
+    const Prog prg{prog_at(slot), cur.far ? prog + cur.prog : nullptr};
+    batch_first_stage<TI, TB, A, GEN>(from_input, i16, o16, bar, prg, n_stages, warp, lane, sg->out, pitch,
                                       T0, 0, lim);
     __syncthreads();  // the staged rows are no longer read; s_early is visible
     const bool early = *s_early != 0;
@@ -267,11 +268,11 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     if (next < total) cur = tpn;
     const SearchArgs no_search{};
     if (kNarrow && o16)
-      item_later_stages<A, uint16_t, false, false, GEN>(bar, prog_at(slot), n_stages, nullptr, warp, lane,
+      item_later_stages<A, uint16_t, false, false, GEN>(bar, prg, n_stages, nullptr, warp, lane,
                                                         static_cast<uint16_t *>(sg->out), pitch, T0, 0, lim, 0,
                                                         no_search);
     else
-      item_later_stages<A, TB, false, false, GEN>(bar, prog_at(slot), n_stages, nullptr, warp, lane,
+      item_later_stages<A, TB, false, false, GEN>(bar, prg, n_stages, nullptr, warp, lane,
                                                   static_cast<TB *>(sg->out), pitch, T0, 0, lim, 0,
                                                   no_search);
     slot ^= 1u;

@@ -81,13 +81,10 @@ constexpr int32_t kPieceCols = 32 * kLaneCols;
 // Ops read whole pieces whatever their width: the block's shared memory
 // ends with this much slack so those reads stay inside it.
 constexpr int32_t kOverRead = kPieceCols * 4;
-// Descriptors of the fused adjoint: each warp copies its ops kDescChunk at a
-// time into its own slot of shared memory (one round trip to L2 per chunk)
-// and reads them back as broadcasts.  The slots lie between the last region
-// and the slack.
-constexpr int32_t kDescSlotBytes = 512;
-constexpr int32_t kDescChunk = kDescSlotBytes / 32;  // 32-byte FusedOp
-constexpr int32_t kDescBytes = kFusedBlockWarps * kDescSlotBytes;
+// At least this much of a block's shared memory lies between the last
+// region and the slack (the programme slots; unused where a launch's
+// programmes stay in global memory).
+constexpr int32_t kProgMinBytes = 3712;
 
 // Reuse flags of an op, valid against the previous op of the same warp's
 // list (same column piece):
@@ -187,17 +184,18 @@ constexpr int32_t kStageRuns = 64;
 // is copied to shared memory with them: per stage kProgStageBytes (the kind,
 // then the byte offsets within the block of each warp's first walk or run
 // and of the stage's end; a search stage has its first and last op instead),
-// then the walks and runs.
+// then the walks and runs.  A launch whose items leave no room for it in
+// shared memory reads it in global memory (far).
 struct FusedProg {
   int32_t load_begin, load_count;  // the item's row copies
   int32_t tx_bytes;                // bytes the copies and the block deliver
   int32_t n_stages;
   int32_t prog;        // first 16-byte word of the block in FusedPlan::prog
   int32_t prog_bytes;  // a multiple of 16
-  int32_t pad0, pad1;
+  int32_t far;         // 1: the block is not copied
+  int32_t pad;
 };
 constexpr int32_t kProgStageBytes = 48;
-constexpr int32_t kProgMinBytes = 4096;  // the two slots for programmes are at least this large together
 
 // Per stage of a template: kind, then the first op (or walk) of each warp
 // and the end of the stage's ops.
@@ -235,7 +233,7 @@ struct FusedGroup {
   int32_t tpl_begin = 0, tpl_count = 0;
   int32_t smem_bytes = 0;     // group-wide layout: barrier + S + Pa + Pb (+ Pt + Q with a search)
                               //   + two programme slots + slack
-  int32_t prog_off = 0, prog_slot = 0;  // byte offset of the first programme slot, bytes of one
+  int32_t prog_off = 0, prog_slot = 0;  // byte offset of the first programme slot, bytes of one (0: far)
   int32_t s_end = 0, pa_end = 0;  // byte offsets where S and Pa end
   int32_t search_k = 0;       // boxcar widths searched in this launch (0 = none; last group only)
   int32_t hist = 0;           // history columns of the top level's window (search)

@@ -201,16 +201,35 @@ template <> __device__ __forceinline__ FusedWalk lds_desc<FusedWalk>(uint32_t at
 __device__ __forceinline__ int32_t warp_all(int32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 __device__ __forceinline__ uint32_t warp_all(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
-// Stage s of the programme at shared address `prog` for one warp: its kind
-// and the addresses of the warp's first descriptor and of their end.
+// An item's programme: a slot of shared memory, or (far) global memory.
+struct Prog {
+  uint32_t near;
+  const int4 *far;  // null: near
+};
+__device__ __forceinline__ int32_t prog_word(const Prog &p, uint32_t off) {
+  return p.far != nullptr ? __ldg(reinterpret_cast<const int32_t *>(p.far) + (off >> 2)) : lds_s32(p.near + off);
+}
+template <class D>
+__device__ __forceinline__ D prog_desc(const Prog &p, uint32_t off) {
+  if (p.far == nullptr) return lds_desc<D>(p.near + off);
+  alignas(16) D d;
+  int4 *o = reinterpret_cast<int4 *>(&d);
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(D) / 16); ++i) o[i] = __ldg(p.far + (off >> 4) + i);
+  return d;
+}
+
+// Stage s of a programme for one warp: its kind and the offsets of the
+// warp's first descriptor and of their end.
 struct StageRange {
   int kind;
   uint32_t first, end;
+  Prog prog;
 };
-__device__ __forceinline__ StageRange prog_stage(uint32_t prog, int s, int warp) {
-  const uint32_t at = prog + (uint32_t)(s * kProgStageBytes);
-  return StageRange{warp_all(lds_s32(at)), prog + (uint32_t)warp_all(lds_s32(at + 4u + 4u * (uint32_t)warp)),
-                    prog + (uint32_t)warp_all(lds_s32(at + 8u + 4u * (uint32_t)warp))};
+__device__ __forceinline__ StageRange prog_stage(const Prog &p, int s, int warp) {
+  const uint32_t at = (uint32_t)(s * kProgStageBytes);
+  return StageRange{warp_all(prog_word(p, at)), (uint32_t)warp_all(prog_word(p, at + 4u + 4u * (uint32_t)warp)),
+                    (uint32_t)warp_all(prog_word(p, at + 8u + 4u * (uint32_t)warp)), p};
 }
 
 // The warps that compute (kFusedThreads threads) wait for each other.  The
@@ -322,7 +341,7 @@ __device__ __forceinline__ void stage_runs(uint32_t sbase, const StageRange &ran
                                            int64_t nt, int64_t T0, int lo, int lim) {
   constexpr uint32_t es = sizeof(TSrc);
   for (uint32_t at = range.first; at != range.end; at += (uint32_t)sizeof(FusedRun)) {
-    const FusedRun run = lds_desc<FusedRun>(at);
+    const FusedRun run = prog_desc<FusedRun>(range.prog, at);
     const uint32_t flags = warp_all((uint32_t)run.flags);
     const bool lo_one = GEN && (flags & kOpLoOne) != 0, hi_one = GEN && (flags & kOpHiOne) != 0;
     const bool no_hi = GEN && (flags & kOpNoHi) != 0;
@@ -464,7 +483,7 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
                                            int lo, int lim) {
   constexpr uint32_t es = (uint32_t)sizeof(TI);
   for (uint32_t at = range.first; at != range.end; at += (uint32_t)sizeof(FusedWalk)) {
-    const FusedWalk wk = lds_desc<FusedWalk>(at);
+    const FusedWalk wk = prog_desc<FusedWalk>(range.prog, at);
     float wl = 1.0f, wh = 1.0f;
     if constexpr (SCALE) {
       wl = __ldg(w + wk.chan);
@@ -816,15 +835,14 @@ __device__ __forceinline__ void stage_search_block(uint32_t sbase, const FusedOp
 
 // The first stage of an item: level 1 walked from the staged input
 // (FROM_INPUT) or the first single / pair stage over the staged base rows.
-// prog: shared address of the item's programme.  TB is the staged base
-// level's type and TO the type written to global memory when this stage is
+// TB is the staged base level's type and TO the type written to global memory when this stage is
 // the top.  With SEARCH the stage before the search writes the top level
 // into Pt instead.  Rows of the top level are nt apart in `out`; its columns
 // T0 + [lo, lim) are written.  GEN as for run_merge_stage; SCALE: the input
 // is multiplied by channel weights (float input only).
 template <class TI, class TB, class A, class TO, bool R16, bool FROM_INPUT, bool SEARCH, bool GEN = true,
           bool SCALE = true>
-__device__ __forceinline__ void item_first_stage(uint32_t sbase, uint32_t prog, int n_stages,
+__device__ __forceinline__ void item_first_stage(uint32_t sbase, const Prog &prog, int n_stages,
                                                  const float *__restrict__ w, int warp, int lane,
                                                  TO *__restrict__ out, int64_t nt, int64_t T0, int lo, int lim) {
   const StageRange r = prog_stage(prog, 0, warp);
@@ -861,7 +879,7 @@ __device__ __forceinline__ void item_first_stage(uint32_t sbase, uint32_t prog, 
 // computing warps before each; the last writes global memory (with SEARCH:
 // the one before it writes Pt and the last is the search).
 template <class A, class TO, bool R16, bool SEARCH, bool GEN = true>
-__device__ __forceinline__ void item_later_stages(uint32_t sbase, uint32_t prog, int n_stages,
+__device__ __forceinline__ void item_later_stages(uint32_t sbase, const Prog &prog, int n_stages,
                                                   const FusedOp *__restrict__ ops, int warp, int lane,
                                                   TO *__restrict__ out, int64_t nt, int64_t T0, int lo, int lim,
                                                   int64_t tile, const SearchArgs &sa) {
@@ -870,9 +888,9 @@ __device__ __forceinline__ void item_later_stages(uint32_t sbase, uint32_t prog,
     if constexpr (SEARCH) {
       if (s == n_stages - 1) {
         // every thread: the whole stage's rows (warp 0's first to the end)
-        const uint32_t at = prog + (uint32_t)(s * kProgStageBytes);
-        stage_search_block<A, TO>(sbase, ops, lds_s32(at + 4u), lds_s32(at + 4u * (kStageWords - 1)), out, nt, T0, lim,
-                                  tile, sa);
+        const uint32_t at = (uint32_t)(s * kProgStageBytes);
+        stage_search_block<A, TO>(sbase, ops, prog_word(prog, at + 4u), prog_word(prog, at + 4u * (kStageWords - 1)), out,
+                                  nt, T0, lim, tile, sa);
         return;
       }
     }
@@ -948,6 +966,92 @@ __device__ __forceinline__ void stage_prog(uint32_t dst, const FusedProg &pr, co
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                "l"(prog + pr.prog), "r"((uint32_t)pr.prog_bytes), "r"(bar)
                : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// Blocks of eight computing warps and a copying one.  The barrier slot holds
+// the `full` mbarrier (an item's rows and programme have landed), the `free`
+// mbarrier (every computing warp is done with the staged rows) and two item
+// headers (tile, columns of the tile inside [0, nt), stages, programme).
+
+constexpr int kFusedLaunchThreads = kFusedThreads + 32;
+constexpr uint32_t kFreeBar = 8, kItemHeader = 32;
+constexpr int32_t kTileChunk = 304;  // time tiles of one chunk of items
+
+__device__ __forceinline__ void init_item_barriers(uint32_t full) {
+  if (threadIdx.x == 0) {
+    mbar_init(full, 1);
+    mbar_init(full + kFreeBar, kFusedWarps);
+    fence_mbar_init();
+  }
+  __syncthreads();
+}
+
+// The copying warp: stages item i + 1 (its rows into S, its programme into
+// one of two slots, its place into one of two headers) as soon as the
+// computing warps have arrived at `free`, behind their first stage of item
+// i, the only one that reads S; its own bookkeeping is off their path.
+// Items go tile chunk by tile chunk, template by template within a chunk,
+// tile by tile within a template: neighbouring templates share staged rows,
+// and a chunk keeps their second reading within reach of L2 whatever the row
+// length.  Row blocks are also asked for one item ahead: L2 hides the HBM
+// latency that a block's single staging region cannot.  1024 x 65536 x 1024
+// float32 306 us without, 289 us with; 4096 x 2^18 x 4096, HBM-bound in its
+// cones, 5.67 ms without, 5.70 with, 6.36 with the requests but template by
+// template.  (Row boxes are bound by the rate of copies: asking twice made
+// them 5 % slower.)
+template <class TS>
+__device__ __forceinline__ void copy_items(unsigned char *smem, const TmaMaps &maps, int64_t nt, int32_t W,
+                                           int32_t tile0, int32_t ntiles, int64_t items,
+                                           const FusedProg *__restrict__ progs, const int4 *__restrict__ prog,
+                                           const FusedLoad *__restrict__ loads, int32_t box, int32_t cshift,
+                                           int32_t prog_off, int32_t prog_slot, int *__restrict__ status, int lane) {
+  const uint32_t full = smem_u32(smem), free_bar = full + kFreeBar, header = full + kItemHeader;
+  int64_t item = blockIdx.x;
+  if (item >= items) return;
+  const int32_t ntpl = (int32_t)(items / ntiles);
+  const int64_t per_chunk = (int64_t)kTileChunk * ntpl;
+  int32_t tile = 0, tpl = 0;
+  auto place = [&](int64_t i) {
+    const int64_t chunk = i / per_chunk;
+    const int32_t first_tile = (int32_t)(chunk * kTileChunk), n = min(kTileChunk, ntiles - first_tile);
+    const int32_t r = (int32_t)(i - chunk * per_chunk);
+    tpl = r / n;
+    tile = first_tile + r % n;
+  };
+  place(item);
+  FusedProg pr = progs[tpl];
+  FusedLoad ld = fetch_load(pr, loads, lane);
+  uint32_t slot = 0, phase = 0;
+  for (bool first = true; item < items; item += gridDim.x, first = false) {
+    if (!first) {
+      if (!mbar_wait_bounded(free_bar, phase)) {
+        // The computing warps gave up (or never arrived): let the copies in
+        // flight land before the block ends.
+        atomicExch(status, 1);
+        mbar_wait_bounded(full, phase);
+        return;
+      }
+      phase ^= 1u;
+    }
+    const int64_t T0 = (int64_t)(tile0 + tile) * W;
+    if (lane == 0) {
+      const int lim = (int)((nt - T0) < (int64_t)W ? (nt - T0) : (int64_t)W);
+      sts_v4(header + 16u * slot, make_int4(tile0 + tile, lim, pr.n_stages, pr.prog));
+    }
+    stage_item<TS>(smem, full, maps.m, pr, loads, ld, T0, box, cshift, lane);
+    if (lane == 0 && prog_slot > 0) stage_prog(full + (uint32_t)(prog_off + (int)slot * prog_slot), pr, prog, full);
+    slot ^= 1u;
+    if (item + gridDim.x < items) {
+      place(item + gridDim.x);
+      pr = progs[tpl];
+      ld = fetch_load(pr, loads, lane);
+      if (cshift > 0) prefetch_item<TS>(maps.m, pr, loads, ld, (int64_t)(tile0 + tile) * W, box, cshift, lane);
+    }
+  }
+  // The last copies land before the block ends: the computing warps wait
+  // for them (or give up, which the bounded wait covers).
+  mbar_wait_bounded(full, phase);
 }
 
 }  // namespace fdmt

@@ -25,24 +25,20 @@
 
 #include <algorithm>
 #include <cstring>
-#include <mutex>
 #include <type_traits>
 
 #include "fdmt_fused.h"
 #include "fdmt_fused_dev.cuh"
 #include "fdmt_internal.h"
+#include "fdmt_residency.h"
 #include "fdmt_tma.h"
 
 namespace fdmt {
 
 // Persistent blocks: block b handles items b, b + gridDim.x, ...  Warps 0 ..
-// 7 compute; warp 8 copies.  The
-// copying warp stages item i + 1 (its rows into S, its programme into one of
-// two slots, its place into one of two headers) as soon as the computing
-// warps have arrived at the `free` barrier, behind their first stage of item
-// i, the only one that reads S; its own bookkeeping is off their path.  The
-// computing warps wait for the rows (`full`), then for each other (every one
-// of them has left item i - 1, whose Pa / Pb the first stage overwrites), run
+// 7 compute; warp 8 copies (copy_items).  The computing warps wait for an
+// item's rows (`full`), then for each other (every one of them has left item
+// i - 1, whose Pa / Pb the first stage overwrites), run
 // the first stage (level 1 walked from the staged input, or the first single
 // / pair stage over the staged base rows) and the remaining stages in Pa /
 // Pb; the last writes global memory.
@@ -59,9 +55,6 @@ namespace fdmt {
 // us with the ops as runs; 139, 137 and 109 us with the walks' code
 // straightened as well; 105, 113 and 92 us with the programmes in shared
 // memory and a copying warp.
-constexpr int kFusedLaunchThreads = kFusedThreads + 32;
-constexpr int32_t kTileChunk = 304;  // time tiles of one chunk of items
-
 template <class TI, class TB, class TO, class A, bool FROM_INPUT, bool R16, bool SEARCH, bool GEN, bool SCALE>
 __global__ void __launch_bounds__(kFusedLaunchThreads, kFusedMinBlocks)
 fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t nt, int64_t pitch, int64_t first,
@@ -72,72 +65,11 @@ fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t
   using TS = typename std::conditional<FROM_INPUT, TI, TB>::type;  // staged element type
   extern __shared__ __align__(128) unsigned char smem[];
   const int warp = warp_all((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
-  // The barrier slot: the `full` and `free` mbarriers, then two item headers
-  // (first column, columns, stages, tile).
-  const uint32_t full = smem_u32(smem), free_bar = full + 8u, header = full + 32u;
-  if (threadIdx.x == 0) {
-    mbar_init(full, 1);
-    mbar_init(free_bar, kFusedWarps);
-    fence_mbar_init();
-  }
-  __syncthreads();
+  const uint32_t full = smem_u32(smem), free_bar = full + kFreeBar, header = full + kItemHeader;
+  init_item_barriers(full);
   if (warp == kFusedWarps) {
-    // Items go tile chunk by tile chunk, template by template within a
-    // chunk, tile by tile within a template: neighbouring templates share
-    // staged rows, and a chunk keeps their second reading within reach of L2
-    // whatever the row length.  Row blocks are also asked for one item ahead:
-    // L2 hides the HBM latency that a block's single staging region cannot.
-    // 1024 x 65536 x 1024 float32 306 us without, 289 us with; 4096 x 2^18 x
-    // 4096, HBM-bound in its cones, 5.67 ms without, 5.70 with, 6.36 with the
-    // requests but template by template.  (Row boxes are bound by the rate
-    // of copies: asking twice made them 5 % slower.)
-    int64_t item = blockIdx.x;
-    if (item >= items) return;
-    const int32_t ntpl = (int32_t)(items / ntiles);
-    const int64_t per_chunk = (int64_t)kTileChunk * ntpl;
-    int32_t tile = 0, tpl = 0;
-    auto place = [&](int64_t i) {
-      const int64_t chunk = i / per_chunk;
-      const int32_t first_tile = (int32_t)(chunk * kTileChunk), n = min(kTileChunk, ntiles - first_tile);
-      const int32_t r = (int32_t)(i - chunk * per_chunk);
-      tpl = r / n;
-      tile = first_tile + r % n;
-    };
-    place(item);
-    FusedProg pr = progs[tpl];
-    FusedLoad ld = fetch_load(pr, loads, lane);
-    uint32_t slot = 0, phase = 0;
-    bool first = true;
-    for (; item < items; item += gridDim.x) {
-      if (!first) {
-        if (!mbar_wait_bounded(free_bar, phase)) {
-          // The computing warps gave up (or never arrived): let the copies in
-          // flight land before the block ends.
-          atomicExch(status, 1);
-          mbar_wait_bounded(full, phase);
-          return;
-        }
-        phase ^= 1u;
-      }
-      first = false;
-      const int64_t T0 = (int64_t)(tile0 + tile) * W;
-      if (lane == 0) {
-        const int lim = (int)((nt - T0) < (int64_t)W ? (nt - T0) : (int64_t)W);
-        sts_v4(header + 16u * slot, make_int4(tile0 + tile, lim, pr.n_stages, 0));
-      }
-      stage_item<TS>(smem, full, maps.m, pr, loads, ld, T0, box, cshift, lane);
-      if (lane == 0) stage_prog(full + (uint32_t)(prog_off + (int)slot * prog_slot), pr, prog, full);
-      slot ^= 1u;
-      if (item + gridDim.x < items) {
-        place(item + gridDim.x);
-        pr = progs[tpl];
-        ld = fetch_load(pr, loads, lane);
-        if (cshift > 0) prefetch_item<TS>(maps.m, pr, loads, ld, (int64_t)(tile0 + tile) * W, box, cshift, lane);
-      }
-    }
-    // The last copies land before the block ends: the computing warps wait
-    // for them (or give up, which the bounded wait covers).
-    mbar_wait_bounded(full, phase);
+    copy_items<TS>(smem, maps, nt, W, tile0, ntiles, items, progs, prog, loads, box, cshift, prog_off, prog_slot, status,
+                   lane);
     return;
   }
   uint32_t slot = 0, phase = 0;
@@ -153,7 +85,7 @@ fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t
     const int4 h = lds_v4(header + 16u * slot);
     const int lim = h.y, n_stages = warp_all(h.z);
     const int64_t tile = h.x, T0 = tile * W;
-    const uint32_t prg = full + (uint32_t)(prog_off + (int)slot * prog_slot);
+    const Prog prg{full + (uint32_t)(prog_off + (int)slot * prog_slot), prog_slot > 0 ? nullptr : prog + h.w};
     const int lo = first > T0 ? (int)(first - T0) : 0;
     item_first_stage<TI, TB, A, TO, R16, FROM_INPUT, SEARCH, GEN, SCALE>(full, prg, n_stages, w, warp, lane, out,
                                                                          pitch, T0, lo, lim);
@@ -171,12 +103,6 @@ cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const vo
                            void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa,
                            int64_t tile0, const OutView *view) {
   auto kern = fused_kernel<TI, TB, TO, A, FI, R16, SEARCH, GEN, SCALE>;
-  static std::once_flag attr_once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(attr_once, [&] {
-    attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  });
-  if (attr_err != cudaSuccess) return attr_err;
   using TS = typename std::conditional<FI, TI, TB>::type;
   TmaMaps maps;
   int32_t cshift = 0;
@@ -187,14 +113,10 @@ cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const vo
   const int32_t box = g.box;
   const int64_t ntiles = g.ntiles - tile0, items = (int64_t)g.tpl_count * ntiles;
   const OutView v = view != nullptr ? *view : OutView{0, g.lt == dt.levels ? nt : state_nt};
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFusedLaunchThreads, g.smem_bytes);
+  int resident = 0;
+  const cudaError_t e = resident_blocks(reinterpret_cast<const void *>(kern), kFusedLaunchThreads, g.smem_bytes, &resident);
   if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const int64_t blocks = std::min<int64_t>(items, (int64_t)per_sm * sms);
+  const int64_t blocks = std::min<int64_t>(items, resident);
   dt.prof->begin(s, FI ? K_FUSED_LOCAL : K_FUSED_CONE, g.lb * 100 + g.lt);
   kern<<<(unsigned)blocks, kFusedLaunchThreads, g.smem_bytes, s>>>(
       maps, static_cast<TO *>(dst) - v.first, nt, v.pitch, v.first, g.W, (int32_t)tile0, (int32_t)ntiles, items,

@@ -118,6 +118,7 @@ struct StageFmt {
   int32_t chunk = 0, kchunks = 0;
   int32_t max_p = 0;  // copies bring at most 2^max_p rows
   int32_t search_k = 0;  // > 0: the launch ends with the boxcar search of this many widths
+  bool compact = false;  // least shared memory: tight row pitches, programmes in global memory
   const std::vector<int32_t> *in_shift = nullptr;  // mapped input (row boxes): each channel's delay
   bool descending = false;
   int32_t shift(int32_t channel) const { return in_shift != nullptr ? (*in_shift)[channel] : 0; }
@@ -151,8 +152,9 @@ namespace {
 // without testing columns (kRunWhole): a strip may start up to kRunGrow
 // columns before its row (in the free columns of the row before it) and
 // reaches at most the end of its row's pitch.
-int32_t stored_pitch(int32_t cols) {
+int32_t stored_pitch(int32_t cols, bool tight) {
   const int32_t whole = (int32_t)round_up(cols + kRunGrow, kPieceCols);
+  if (tight) return (int32_t)round_up(cols, 4);
   return whole - cols <= cols / 6 + kRunGrow ? whole : (int32_t)round_up(cols + kRunGrow, 4);
 }
 
@@ -222,7 +224,7 @@ void shape_cone(const Tables &t, int32_t lb, int32_t lt, int32_t band, int32_t r
         n.smem = (int32_t)off;
         off += round_up((int64_t)rows * n.stride * sB, 128);
       } else if (stored) {
-        n.stride = stored_pitch(W + n.s);
+        n.stride = stored_pitch(W + n.s, f.compact);
         n.smem = (int32_t)off;
         off += round_up((int64_t)rows * n.stride * sA, 128);
       }
@@ -292,17 +294,20 @@ int64_t search_q_bytes(const StageFmt &f, int64_t rows) {
   return round_up(rows * f.search_k * 8, 128);
 }
 
-// Bytes of one programme slot for items of `stages` stages and at most
+// Bytes of one programme slot (0: far) for items of `stages` stages and at most
 // `descs` bytes of walks and runs (a stage's split over the warps can cut a
 // run in two at each of its seven borders).
-int64_t prog_slot_bytes(int64_t stages, int64_t descs) {
+int64_t prog_slot_bytes(const StageFmt &f, int64_t stages, int64_t descs) {
+  if (f.compact) return 0;
   const int64_t n = stages * (kProgStageBytes + (kFusedBlockWarps - 1) * (int64_t)sizeof(FusedRun)) + descs;
   return std::max<int64_t>(kProgMinBytes / 2, round_up(n, 128));
 }
 
-int64_t cone_bytes(const ConeShape &cs, int64_t stages) {
+int64_t prog_area(int64_t slot) { return std::max<int64_t>(kProgMinBytes, 2 * slot); }
+
+int64_t cone_bytes(const StageFmt &f, const ConeShape &cs, int64_t stages) {
   return kBarrierBytes + cs.s_bytes + cs.pa_bytes + cs.pb_bytes + cs.pt_bytes +
-         2 * prog_slot_bytes(stages, cs.prog_bytes) + kOverRead;
+         prog_area(prog_slot_bytes(f, stages, cs.prog_bytes)) + kOverRead;
 }
 
 // Emits the loads, inits and ops of a shaped cone at the given region bases.
@@ -739,7 +744,7 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
         for (int32_t r0 = 0; r0 < rows; r0 += per) {
           ConeShape cs;
           shape_cone(t, lb, lt, b, r0, std::min(rows, r0 + per) - 1, W, fp, f, cs);
-          if (cone_bytes(cs, nst) + search_q_bytes(f, cs.top_rows) > cone_budget) return false;
+          if (cone_bytes(f, cs, nst) + search_q_bytes(f, cs.top_rows) > cone_budget) return false;
           if (keep) keep->push_back(std::move(cs));
         }
         return true;
@@ -774,7 +779,7 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
       const ConeShape &cs = shapes[i];
       if (!bundles.empty() && (int64_t)bundles.back().size() < cap &&
           kBarrierBytes + bs + cs.s_bytes + ba + cs.pa_bytes + bb + cs.pb_bytes + bt + cs.pt_bytes +
-                  search_q_bytes(f, br + cs.top_rows) + 2 * prog_slot_bytes(nst, bp + cs.prog_bytes) + kOverRead <=
+                  search_q_bytes(f, br + cs.top_rows) + prog_area(prog_slot_bytes(f, nst, bp + cs.prog_bytes)) + kOverRead <=
               cone_budget) {
         bundles.back().push_back(i);
         bs += cs.s_bytes;
@@ -812,8 +817,8 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
       mp = std::max(mp, p1);
     }
     const int64_t qb = search_q_bytes(f, mr);
-    const int64_t slot = prog_slot_bytes(nst, mp);
-    const int64_t total = kBarrierBytes + ms + ma + mb + mt + qb + 2 * slot + kOverRead;
+    const int64_t slot = prog_slot_bytes(f, nst, mp);
+    const int64_t total = kBarrierBytes + ms + ma + mb + mt + qb + prog_area(slot) + kOverRead;
     if (total > budget && total > 227 * 1024 - 1024) continue;
     if (total > budget && cone_budget > 4096) continue;
     gb = GroupBuild();
@@ -836,7 +841,7 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
     gb.g.ntiles = (nt + W - 1) / W;
     gb.g.smem_bytes = (int32_t)total;
     gb.g.prog_slot = (int32_t)slot;
-    gb.g.prog_off = (int32_t)(total - kOverRead - 2 * slot);
+    gb.g.prog_off = (int32_t)(total - kOverRead - prog_area(slot));
     gb.g.s_end = (int32_t)(kBarrierBytes + ms);
     gb.g.pa_end = (int32_t)(kBarrierBytes + ms + ma);
     double hbm = 0, sl = 0, nops = 0, work = 0;
@@ -967,9 +972,9 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
 // Group (lb, lt] for tile W.  The staging format follows the windows of
 // the group's own cones: a first build with provisional boxes measures
 // them, the second uses the chosen box or block width.
-GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int32_t W,
-                       const FusedPlan &fp, int32_t budget, const FusedParams &prm, int32_t search_k, bool emit) {
-  const int32_t staging = prm.staging;
+GroupBuild build_group_mode(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int32_t W,
+                       const FusedPlan &fp, int32_t budget, const FusedParams &prm, int32_t search_k, bool emit,
+                            bool compact, int32_t staging) {
   const int32_t es = (lb == 0) ? fp.input_size : fp.level_size[lb];
   const int64_t rows = (lb == 0) ? t.nf : t.level_rows[lb];
   // Row blocks: chunks of 128 bytes (64 for 1-byte samples, so that a tile
@@ -981,6 +986,7 @@ GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int3
   if (staging == 2 && nt % chunk != 0) return GroupBuild();
   StageFmt boxes;
   boxes.search_k = search_k;
+  boxes.compact = compact;
   if (mapped) {
     boxes.in_shift = prm.in_shift;
     boxes.descending = prm.descending;
@@ -1025,6 +1031,16 @@ GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int3
   }
   f.box = choose_box(needs, es);
   return build_group_fmt(t, nt, lb, lt, W, fp, budget, f, nullptr, emit);
+}
+
+// The same, in the compact layout where the roomy one does not fit, and with
+// row boxes (whose windows are not rounded to chunks) where that does not.
+GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int32_t W, const FusedPlan &fp,
+                       int32_t budget, const FusedParams &prm, int32_t search_k, bool emit) {
+  GroupBuild gb = build_group_mode(t, nt, lb, lt, W, fp, budget, prm, search_k, emit, false, prm.staging);
+  if (!gb.ok) gb = build_group_mode(t, nt, lb, lt, W, fp, budget, prm, search_k, emit, true, prm.staging);
+  if (!gb.ok && prm.staging == 0) gb = build_group_mode(t, nt, lb, lt, W, fp, budget, prm, search_k, emit, true, 1);
+  return gb;
 }
 
 // Shared-memory pipe slots per 32 columns of the first row of a run (all its
@@ -1114,7 +1130,7 @@ void lower_stage(const StageRows &sr, const std::vector<FusedOp> &ops, bool pair
           run.g3 = nr.g[3];
           run.n = k;
           run.flags = nr.flags;
-          if (dst_moves && nr.pitch % kPieceCols == 0) run.flags |= kRunWhole;
+          if (dst_moves && nr.pitch % kPieceCols == 0 && nr.pitch - nr.width >= kRunGrow) run.flags |= kRunWhole;
           out->push_back(run);
         }
         load += run_first_cost(pair) + (k - 1) * run_step_cost(pair);
@@ -1189,8 +1205,9 @@ bool append_group(FusedPlan &fp, GroupBuild &gb) {
       words.insert(words.end(), d, d + (size_t)(src[kStageWords - 1] - src[1]) * size / 4);
     }
     pr.prog_bytes = (int32_t)words.size() * 4;
-    pr.tx_bytes = tp.tx_bytes + pr.prog_bytes;
-    if (pr.prog_bytes > g.prog_slot) return false;
+    pr.far = g.prog_slot == 0 ? 1 : 0;
+    pr.tx_bytes = tp.tx_bytes + (pr.far ? 0 : pr.prog_bytes);
+    if (!pr.far && pr.prog_bytes > g.prog_slot) return false;
     fp.prog.insert(fp.prog.end(), words.begin(), words.end());
     fp.progs.push_back(pr);
     fp.loads.insert(fp.loads.end(), c.loads.begin(), c.loads.end());

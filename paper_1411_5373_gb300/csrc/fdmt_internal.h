@@ -80,10 +80,9 @@ struct DeviceTables {
   FusedOp *f_ops = nullptr;  // a search stage's rows (plans that search in the last launch)
   // Fused adjoint (null unless the plan has one).
   const AdjFusedPlan *adj_fused = nullptr;
-  FusedTemplate *a_tpls = nullptr;
+  FusedProg *a_progs = nullptr;
+  int32_t *a_prog = nullptr;
   FusedLoad *a_loads = nullptr;
-  FusedOp *a_ops = nullptr;
-  int32_t *a_stages = nullptr;
 };
 
 // What other translation units may read of a plan (see plan_view).

@@ -121,6 +121,9 @@ def _check(plan):
     (64, 960, 64, "f32", {"tile": 64, "smem_budget": 48 * 1024, "search_widths": 6}),
     (100, 960, 90, "u8", {"tile": 256, "bounds": [0, 3, 7], "search_widths": 8}),
     (256, 4096, 2048, "f32", {"gamma": 1.5}),
+    # budgets that only the compact layout fits
+    (128, 2064, 399, "f32", {"tile": 128, "smem_budget": 12288, "bounds": [0, 3, 5, 7]}),
+    (33, 448, 156, "u8", {"tile": 512, "smem_budget": 12288, "bounds": [0, 2, 4, 6], "staging": "boxes"}),
     (1024, 65536, 1024, "f32", {}),
     (1024, 65536, 1024, "u8", {"bounds": [0, 3, 6, 10]}),
 ])

@@ -1,7 +1,8 @@
-"""Rows of the levels between launches padded to whole chunks (nt from 4096 on
+"""Layouts at their limits.  Rows of the levels between launches padded to whole chunks (nt from 4096 on
 and no multiple of 64): single beams of every type and a batch in one launch,
 bit-exact to the oracle, on buffers that start as NaN bytes (the columns past
-nt are never written and must never reach an output)."""
+nt are never written and must never reach an output); and budgets that only
+the compact layout fits."""
 import numpy as np
 import pytest
 
@@ -31,6 +32,20 @@ def test_beam(nf, nt, nd, dtype):
     x = fs.random_u8(nt, nf, nt) if dtype == "u8" else fs.random_f32(nt, nf, nt)
     p = FD.Plan(1200.0, 1600.0, nf, nt, nd, dtype, schedule="fused", bounds=[0, 2, 4, p_levels(nf)])
     p.workspace().fill_(255)
+    got = p.execute(torch.from_numpy(x).cuda()).cpu().numpy()
+    p.device_status()
+    assert np.array_equal(got, oracle.fdmt(x, oracle.build_tables(1200.0, 1600.0, nf, nd), MODE[dtype]))
+
+
+@pytest.mark.parametrize("nf,nt,nd,dtype,kw", [
+    (128, 2064, 399, "f32", {"tile": 128, "smem_budget": 12288, "bounds": [0, 3, 5, 7]}),
+    (33, 448, 156, "u8", {"tile": 512, "smem_budget": 12288, "bounds": [0, 2, 4, 6], "staging": "boxes"}),
+])
+def test_compact_layout(nf, nt, nd, dtype, kw):
+    """Budgets that leave no room for the programmes in shared memory (they
+    are read in global memory) nor for whole row pitches."""
+    x = fs.random_u8(nt, nf, nt) if dtype == "u8" else fs.random_f32(nt, nf, nt)
+    p = FD.Plan(1200.0, 1600.0, nf, nt, nd, dtype, schedule="fused", **kw)
     got = p.execute(torch.from_numpy(x).cuda()).cpu().numpy()
     p.device_status()
     assert np.array_equal(got, oracle.fdmt(x, oracle.build_tables(1200.0, 1600.0, nf, nd), MODE[dtype]))
