@@ -7,65 +7,280 @@
 // with channel c in ascending frequency holding DFT bin k = (c + Nf/2) mod Nf
 // of the complex (baseband) voltages.
 //
-// One block of threads transforms the Nf-sample blocks of T output times
-// (T nbin transforms, up to 4096 complex samples) in shared memory with the
-// Stockham FFT of fdmt_stockham.cuh (radix 16 in registers, the first pass
-// reading the voltages straight from global memory), so an Nf = 1024
-// transform takes three passes and three barriers.  The squared magnitudes
-// are summed over the bin and written as an [Nf][T] tile.
+// A block of 256 threads (512 and 1024 for the largest Nf) transforms 16
+// samples per thread at a time, in registers, with Stockham passes of
+// radix 16: the first pass reads the voltages from global memory, a pass
+// reads all its values before any is stored, so one shared buffer serves
+// every exchange, and the last pass stores squared magnitudes.  Blocks are
+// persistent: the twiddle table is made once per block.
+// Bound: instruction issue, then HBM.  64 M voltages into 1024 x 65536 on a
+// GB300: 334 us with two exchange buffers (two blocks per SM), twiddles made
+// anew for every 4096 samples and the two parts of a complex sum added one
+// by one; 217 us now.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "../../include/fdmt.h"
+#include "fdmt_residency.h"
 #include "fdmt_stockham.cuh"
+#include "fdmt_tma.h"
 
 namespace fdmt {
 namespace {
 
-constexpr int kFbThreads = 256;
-constexpr int kFbSamples = 4096;  // complex samples transformed per block at once
+constexpr int kFbValues = 16;  // complex samples per thread
+// Threads of a block for 2^LN channels: larger blocks transform more times
+// at once, so that a tile's rows stay 16 bytes or wider.
+__host__ __device__ constexpr int fb_threads(int ln) { return ln <= 9 ? 256 : (ln == 10 ? 512 : 1024); }
+__host__ __device__ constexpr int fb_samples(int ln) { return kFbValues * fb_threads(ln); }
+constexpr int kFbRefSamples = 4096;  // sizes the bin that one block takes at most
 
-template <int LN>
-__global__ void __launch_bounds__(kFbThreads)
-filterbank_kernel(const float2 *__restrict__ v, int nbin, int64_t nt, int T, float *__restrict__ out) {
-  constexpr int NF = 1 << LN;
-  extern __shared__ __align__(16) float2 sm[];
-  const int F = T * nbin;      // transforms per block
-  const int padded = fft::pad16(F * NF);
-  float2 *buf0 = sm;             // [F][nf], padded
-  float2 *buf1 = sm + padded;    // [F][nf], padded
-  float2 *tw = buf1 + padded;    // [nf], padded by pad4
-  const int64_t t_first = (int64_t)blockIdx.x * T;
-  const int T_here = (int)((nt - t_first) < (int64_t)T ? (nt - t_first) : (int64_t)T);
-  const int F_here = T_here * nbin;
-  fft::twiddles<kFbThreads, LN>(tw);
-  __syncthreads();  // twiddles
-  const float2 *x =
-      fft::transform<kFbThreads, LN>(fft::GlobalSrc{v + t_first * nbin * (int64_t)NF}, buf0, buf1, tw, F_here);
-  // Consecutive threads take consecutive times of one channel row (T is a
-  // power of two; the last block may hold fewer times).
-  const int lT = 31 - __clz(T);
-  for (int i = threadIdx.x; i < NF * T; i += kFbThreads) {
-    const int c = i >> lT, tt = i & (T - 1);
-    if (tt >= T_here) continue;
-    const int k = (c + NF / 2) & (NF - 1);
-    float acc = 0.0f;
-    for (int b = 0; b < nbin; ++b) {
-      const float2 z = x[fft::pad16((tt * nbin + b) * NF + k)];
-      acc = __fadd_rn(acc, __fadd_rn(__fmul_rn(z.x, z.x), __fmul_rn(z.y, z.y)));
+// Shared-memory index of squared magnitude i: the times of a channel, a
+// multiple of Nf apart, land 32 / T banks apart when they are read back.
+__device__ __forceinline__ constexpr int pad_power(int i) { return i + (i >> 7); }
+
+// The values of pass (NS, R) in registers: work item w = threadIdx.x + it
+// threads holds elements base + r NF / R of its transform.
+template <int LN, int R>
+struct FbItem {
+  static constexpr int NF = 1 << LN, LR = fft::ilog2(R), LPER = LN - LR, PER = 1 << LPER;
+  int f, j;
+  __device__ __forceinline__ explicit FbItem(int it) {
+    const int w = (int)threadIdx.x + it * fb_threads(LN);
+    f = w >> LPER;
+    j = w & (PER - 1);
+  }
+};
+
+// pad16(i + r STEP) and pad_power(i + r STEP) for i = i0 + r STEP with i0
+// padded already: linear in r where the padding is (a step of whole runs, or
+// single steps from the start of a run), so that a pass's addresses are
+// constant offsets from one base.
+template <int STEP, bool RUN>
+__device__ __forceinline__ int step16(int i0, int p0, int r) {
+  if constexpr (STEP % 16 == 0) return p0 + r * (STEP + STEP / 16);
+  if constexpr (RUN) return p0 + r * STEP;
+  return fft::pad16(i0 + r * STEP);
+}
+template <int STEP>
+__device__ __forceinline__ int step_power(int i0, int p0, int r) {
+  if constexpr (STEP % 128 == 0) return p0 + r * (STEP + STEP / 128);
+  return pad_power(i0 + r * STEP);
+}
+
+// One pass over F transforms: `v` holds its values; the outputs go to `buf`
+// (element order), or, in the last pass (NS R = NF), their squared
+// magnitudes to `power`.
+// TILE: `power` is the [channel][time] tile of samples / NF times that a tensor
+// copy writes out, which may still be reading the last one when the first
+// pass stores.
+template <int LN, int NS, int R, bool TILE>
+__device__ __forceinline__ void fb_finish(float2 (&v)[kFbValues / R][R], float2 *buf, float *power,
+                                          const float2 *__restrict__ tw, int F) {
+  constexpr int NF = 1 << LN, LR = fft::ilog2(R), LNS = fft::ilog2(NS);
+#pragma unroll
+  for (int it = 0; it < kFbValues / R; ++it) {
+    const FbItem<LN, R> w(it);
+    const int k = w.j & (NS - 1);
+    if constexpr (NS > 1) {
+      // exp(-2 pi i r k / (NS R)) = tw[r k NF / (NS R)]
+      constexpr int SH = LN - LNS - LR;
+      const int step = k << SH;
+#pragma unroll
+      for (int r = 1; r < R; ++r)
+        v[it][r] = fft::cmul(v[it][r], tw[SH >= 2 ? r * fft::pad4(step) : fft::pad4(r * step)]);
     }
-    out[(int64_t)c * nt + t_first + tt] = acc;
+    fft::dft_regs<R>(v[it]);
+  }
+  if constexpr (TILE && NS == 1) {
+    if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    __syncthreads();
+  }
+  if constexpr (NS > 1) __syncthreads();  // every value of the pass has been read
+#pragma unroll
+  for (int it = 0; it < kFbValues / R; ++it) {
+    const FbItem<LN, R> w(it);
+    if (w.f >= F) continue;
+    const int out0 = w.f * NF + (w.j >> LNS) * NS * R + (w.j & (NS - 1));
+    const int at = NS * R == NF ? pad_power(out0) : fft::pad16(out0);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float2 z = v[it][fft::bitrev_small(r, LR)];
+      if constexpr (NS * R == NF && TILE) {
+        constexpr int kT = fb_samples(LN) / NF;
+        const int k = out0 - w.f * NF + r * NS;
+        power[((k + NF / 2) & (NF - 1)) * kT + w.f] = __fadd_rn(__fmul_rn(z.x, z.x), __fmul_rn(z.y, z.y));
+      } else if constexpr (NS * R == NF)
+        power[step_power<NS>(out0, at, r)] = __fadd_rn(__fmul_rn(z.x, z.x), __fmul_rn(z.y, z.y));
+      else  // (the first pass stores whole runs of 16)
+        buf[step16<NS, NS == 1 && R == 16>(out0, at, r)] = z;
+    }
+  }
+  if constexpr (TILE && NS * R == NF) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+}
+
+// The passes after transforms of size NS.
+template <int LN, int NS, bool TILE>
+__device__ __forceinline__ void fb_rest(float2 *buf, float *power, const float2 *__restrict__ tw, int F) {
+  constexpr int NF = 1 << LN;
+  if constexpr (NS < NF) {
+    constexpr int R = NF / NS >= 16 ? 16 : NF / NS, PER = NF / R;
+    float2 v[kFbValues / R][R];
+#pragma unroll
+    for (int it = 0; it < kFbValues / R; ++it) {
+      const FbItem<LN, R> w(it);
+      const int i0 = w.f * NF + w.j, at = fft::pad16(i0);
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[it][r] = buf[step16<PER, false>(i0, at, r)];
+    }
+    fb_finish<LN, NS, R, TILE>(v, buf, power, tw, F);
+    fb_rest<LN, NS * R, TILE>(buf, power, tw, F);
   }
 }
 
+// Squared magnitudes of F <= samples / NF transforms of the voltages at x, in
+// `power` (element f NF + k at pad_power); a barrier at the end.
+template <int LN, bool TILE>
+__device__ __forceinline__ void fb_transform(const float2 *__restrict__ x, float2 *buf, float *power,
+                                             const float2 *__restrict__ tw, int F) {
+  constexpr int NF = 1 << LN, R = NF >= 16 ? 16 : NF;
+  float2 v[kFbValues / R][R];
+#pragma unroll
+  for (int it = 0; it < kFbValues / R; ++it) {
+    const FbItem<LN, R> w(it);
+    const float2 *from = x + (w.f < F ? w.f * NF + w.j : 0);  // (a work item past the last transform stores nothing)
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[it][r] = __ldg(from + r * FbItem<LN, R>::PER);
+  }
+  fb_finish<LN, 1, R, TILE>(v, buf, power, tw, F);
+  fb_rest<LN, R, TILE>(buf, power, tw, F);
+}
+
 template <int LN>
-cudaError_t launch_filterbank(const float2 *v, int nbin, int64_t nt, int T, float *out, size_t smem,
-                              cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(filterbank_kernel<LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const int64_t blocks = (nt + T - 1) / T;
-  filterbank_kernel<LN><<<(unsigned)blocks, kFbThreads, smem, s>>>(v, nbin, nt, T, out);
+__global__ void __launch_bounds__(fb_threads(LN), 1024 / fb_threads(LN))
+filterbank_kernel(const float2 *__restrict__ v, int nbin, int64_t nt, int T, float *__restrict__ out) {
+  constexpr int NF = 1 << LN;
+  extern __shared__ __align__(16) float2 sm[];
+  float2 *buf = sm;                                // samples, padded
+  float *power = reinterpret_cast<float *>(sm);    // the same memory, after the last pass
+  float2 *tw = sm + fft::pad16(fb_samples(LN));        // [nf], padded by pad4
+  fft::twiddles<fb_threads(LN), LN>(tw);
+  __syncthreads();
+  const int lT = 31 - __clz(T);
+  constexpr int kRound = fb_samples(LN) / NF, kThreads = fb_threads(LN);  // transforms at once
+  for (int64_t t_first = (int64_t)blockIdx.x * T; t_first < nt; t_first += (int64_t)gridDim.x * T) {
+    const float2 *x = v + t_first * nbin * (int64_t)NF;
+    if (T * nbin <= kRound) {
+      const int T_here = (int)((nt - t_first) < (int64_t)T ? (nt - t_first) : (int64_t)T);
+      fb_transform<LN, false>(x, buf, power, tw, T_here * nbin);
+      // Consecutive threads take consecutive times of one channel row (T is
+      // a power of two; the last tile may hold fewer times): thread i time i
+      // mod T of channels i / T, i / T + threads / T, ...  (T can exceed the
+      // block only for Nf < 16.)
+      for (int tt = threadIdx.x & (T - 1); tt < T_here; tt += kThreads) {
+        const int dc = T < kThreads ? kThreads >> lT : 1;
+        float *o = out + (int64_t)((int)threadIdx.x >> lT) * nt + t_first + tt;
+        for (int c = (int)threadIdx.x >> lT; c < NF; c += dc, o += (int64_t)dc * nt) {
+          const int k = (c + NF / 2) & (NF - 1);
+          float acc = 0.0f;
+          for (int b = 0; b < nbin; ++b) acc = __fadd_rn(acc, power[pad_power((tt * nbin + b) * NF + k)]);
+          *o = acc;
+        }
+      }
+      __syncthreads();  // before the next tile's first pass stores
+    } else {
+      // One time (T = 1) whose bin takes more than one round: every thread
+      // keeps the sums of its channels.
+      constexpr int kOwn = (NF + kThreads - 1) / kThreads;
+      float acc[kOwn];
+#pragma unroll
+      for (int q = 0; q < kOwn; ++q) acc[q] = 0.0f;
+      for (int b0 = 0; b0 < nbin; b0 += kRound) {
+        const int F = min(kRound, nbin - b0);
+        fb_transform<LN, false>(x + (int64_t)b0 * NF, buf, power, tw, F);
+#pragma unroll
+        for (int q = 0; q < kOwn; ++q) {
+          const int c = (int)threadIdx.x + q * kThreads, k = (c + NF / 2) & (NF - 1);
+          if (c < NF)
+            for (int b = 0; b < F; ++b) acc[q] = __fadd_rn(acc[q], power[pad_power(b * NF + k)]);
+        }
+        __syncthreads();
+      }
+#pragma unroll
+      for (int q = 0; q < kOwn; ++q) {
+        const int c = (int)threadIdx.x + q * kThreads;
+        if (c < NF) out[(int64_t)c * nt + t_first] = acc[q];
+      }
+    }
+  }
+}
+
+// The same without binning where the output takes tensor copies (16-byte
+// aligned, nt a multiple of 4): the last pass stores its powers as an
+// [Nf][T] tile, which one thread writes out by copies of [256][T], off the
+// other threads' path and behind the next tile's first pass.  Taken for T
+// <= 16 times per tile, where the threads write only a part of a row's 128
+// bytes at a time, and for Nf = 16; between them whole segments cost less
+// than the tile's bank conflicts.  64 M voltages, tile against threads, us:
+// Nf = 16 251 / 292, 32 272 / 229, 64 242 / 193, 256 169 / 176, 512 192 / 205,
+// 1024 217 / 226, 2048 295 / 307, 4096 360 / 415 (before: 391, 315, 255, 385,
+// 321, 335, 447, 690).
+template <int LN>
+__global__ void __launch_bounds__(fb_threads(LN), 1024 / fb_threads(LN))
+filterbank_tile_kernel(const __grid_constant__ CUtensorMap map, const float2 *__restrict__ v, int64_t nt) {
+  constexpr int NF = 1 << LN, T = fb_samples(LN) / NF, kRows = NF < 256 ? NF : 256;
+  extern __shared__ __align__(128) float2 sm[];
+  float2 *buf = sm;
+  float *power = reinterpret_cast<float *>(sm);
+  float2 *tw = sm + fft::pad16(fb_samples(LN));
+  fft::twiddles<fb_threads(LN), LN>(tw);
+  __syncthreads();
+  for (int64_t t_first = (int64_t)blockIdx.x * T; t_first < nt; t_first += (int64_t)gridDim.x * T) {
+    const int F = (int)((nt - t_first) < (int64_t)T ? (nt - t_first) : (int64_t)T);
+    // (ends with a barrier; columns past nt of the last tile are clipped)
+    fb_transform<LN, true>(v + t_first * (int64_t)NF, buf, power, tw, F);
+    if (threadIdx.x == 0) {
+      const uint32_t src = static_cast<uint32_t>(__cvta_generic_to_shared(power));
+      for (int c = 0; c < NF; c += kRows)
+        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                         reinterpret_cast<uint64_t>(&map)),
+                     "r"((int)t_first), "r"(c), "r"(src + (uint32_t)(c * T * 4))
+                     : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+  }
+  if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
+template <int LN>
+cudaError_t launch_filterbank(const float2 *v, int nbin, int64_t nt, int T, float *out, cudaStream_t s) {
+  constexpr size_t smem = ((size_t)fft::pad16(fb_samples(LN)) + (size_t)fft::pad4(1 << LN)) * sizeof(float2);
+  cudaError_t e;
+  int resident = 0;
+  constexpr int kTile = fb_samples(LN) >> LN;
+  if constexpr (LN >= 4 && (kTile <= 16 || kTile >= 256)) {
+    constexpr int kT = kTile, kRows = LN < 8 ? 1 << LN : 256;
+    if (nbin == 1 && T == kT && nt % 4 == 0 && nt < ((int64_t)1 << 31) - kT &&
+        (reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
+      auto kern = filterbank_tile_kernel<LN>;
+      if ((e = resident_blocks(reinterpret_cast<const void *>(kern), fb_threads(LN), smem, &resident)) != cudaSuccess)
+        return e;
+      CUtensorMap map;
+      if (!make_store_map(&map, out, 1u << LN, (uint64_t)nt, kT, kRows)) return cudaErrorInvalidValue;
+      const int64_t tiles = std::min<int64_t>((nt + kT - 1) / kT, resident);
+      kern<<<(unsigned)tiles, fb_threads(LN), smem, s>>>(map, v, nt);
+      return cudaGetLastError();
+    }
+  }
+  auto kern = filterbank_kernel<LN>;
+  if ((e = resident_blocks(reinterpret_cast<const void *>(kern), fb_threads(LN), smem, &resident)) != cudaSuccess)
+    return e;
+  const int64_t blocks = std::min<int64_t>((nt + T - 1) / T, resident);
+  kern<<<(unsigned)blocks, fb_threads(LN), smem, s>>>(v, nbin, nt, T, out);
   return cudaGetLastError();
 }
 
@@ -81,31 +296,36 @@ extern "C" int fdmt_filterbank(const void *volts, int64_t n, int32_t nf, int32_t
   if (nt < 1 || n < 0 || nt > n / ((int64_t)nf * nbin)) return FDMT_ERR_INVALID_ARG;
   int log2nf = 0;
   while ((1 << log2nf) < nf) ++log2nf;
-  // Output times per block: a power of two, as many transforms as fit
-  // kFbSamples (at least one time's bin).
-  int T = fdmt::kFbSamples / (nf * nbin);
-  if (T < 1) T = 1;
-  while (T & (T - 1)) T &= T - 1;  // a power of two
-  const size_t padded = (size_t)T * nbin * nf + ((size_t)T * nbin * nf >> 4);
-  const size_t smem = (2 * padded + (size_t)nf + (size_t)nf / 4) * sizeof(float2);
-  if (smem > 200 * 1024) return FDMT_ERR_UNSUPPORTED;
+  // Output times per block: a power of two, as many transforms as a block
+  // takes at once (at least one time's bin).
+  auto times = [&](int samples) {
+    int n = std::max(1, samples / (nf * nbin));
+    while (n & (n - 1)) n &= n - 1;
+    return n;
+  };
+  const int T = times(fdmt::fb_samples(log2nf));
+  // (one time's bin: at most as many samples as two padded buffers and the
+  // twiddles held in 200 KiB)
+  const int ref = times(fdmt::kFbRefSamples);
+  const size_t padded = (size_t)ref * nbin * nf + ((size_t)ref * nbin * nf >> 4);
+  if ((2 * padded + (size_t)nf + (size_t)nf / 4) * sizeof(float2) > 200 * 1024) return FDMT_ERR_UNSUPPORTED;
   if ((nt + T - 1) / T > INT32_MAX) return FDMT_ERR_UNSUPPORTED;
   const float2 *vv = static_cast<const float2 *>(volts);
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   cudaError_t e;
   switch (log2nf) {
-    case 1: e = fdmt::launch_filterbank<1>(vv, nbin, nt, T, out, smem, cs); break;
-    case 2: e = fdmt::launch_filterbank<2>(vv, nbin, nt, T, out, smem, cs); break;
-    case 3: e = fdmt::launch_filterbank<3>(vv, nbin, nt, T, out, smem, cs); break;
-    case 4: e = fdmt::launch_filterbank<4>(vv, nbin, nt, T, out, smem, cs); break;
-    case 5: e = fdmt::launch_filterbank<5>(vv, nbin, nt, T, out, smem, cs); break;
-    case 6: e = fdmt::launch_filterbank<6>(vv, nbin, nt, T, out, smem, cs); break;
-    case 7: e = fdmt::launch_filterbank<7>(vv, nbin, nt, T, out, smem, cs); break;
-    case 8: e = fdmt::launch_filterbank<8>(vv, nbin, nt, T, out, smem, cs); break;
-    case 9: e = fdmt::launch_filterbank<9>(vv, nbin, nt, T, out, smem, cs); break;
-    case 10: e = fdmt::launch_filterbank<10>(vv, nbin, nt, T, out, smem, cs); break;
-    case 11: e = fdmt::launch_filterbank<11>(vv, nbin, nt, T, out, smem, cs); break;
-    default: e = fdmt::launch_filterbank<12>(vv, nbin, nt, T, out, smem, cs); break;
+    case 1: e = fdmt::launch_filterbank<1>(vv, nbin, nt, T, out, cs); break;
+    case 2: e = fdmt::launch_filterbank<2>(vv, nbin, nt, T, out, cs); break;
+    case 3: e = fdmt::launch_filterbank<3>(vv, nbin, nt, T, out, cs); break;
+    case 4: e = fdmt::launch_filterbank<4>(vv, nbin, nt, T, out, cs); break;
+    case 5: e = fdmt::launch_filterbank<5>(vv, nbin, nt, T, out, cs); break;
+    case 6: e = fdmt::launch_filterbank<6>(vv, nbin, nt, T, out, cs); break;
+    case 7: e = fdmt::launch_filterbank<7>(vv, nbin, nt, T, out, cs); break;
+    case 8: e = fdmt::launch_filterbank<8>(vv, nbin, nt, T, out, cs); break;
+    case 9: e = fdmt::launch_filterbank<9>(vv, nbin, nt, T, out, cs); break;
+    case 10: e = fdmt::launch_filterbank<10>(vv, nbin, nt, T, out, cs); break;
+    case 11: e = fdmt::launch_filterbank<11>(vv, nbin, nt, T, out, cs); break;
+    default: e = fdmt::launch_filterbank<12>(vv, nbin, nt, T, out, cs); break;
   }
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -2,6 +2,8 @@
 // plans and the dispatch over the input types (the kernel and the launch
 // logic: fdmt_fused_launch.cuh; float32 launches: fdmt_fused_f32.cu; uint8
 // launches: fdmt_fused_u8.cu).
+#include <mutex>
+
 #include "fdmt_fused_launch.cuh"
 
 namespace fdmt {
@@ -55,6 +57,18 @@ bool make_block_map(CUtensorMap *m, const void *base, CUtensorMapDataType type, 
 }
 
 }  // namespace
+
+bool make_store_map(CUtensorMap *map, void *base, uint64_t rows, uint64_t nt, uint32_t cols, uint32_t brows) {
+  PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
+  if (fn == nullptr) return false;
+  cuuint64_t dims[2] = {nt, rows};
+  cuuint64_t strides[1] = {nt * 4};
+  cuuint32_t boxd[2] = {cols, brows};
+  cuuint32_t es[2] = {1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, boxd, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 bool make_group_maps(CUtensorMap *maps, const FusedGroup &g, const void *base, CUtensorMapDataType type,
                      uint32_t elem, uint64_t rows, uint64_t nt, int32_t *cshift) {

@@ -23,8 +23,22 @@
 namespace fdmt {
 namespace fft {
 
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y)); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y)); }
+// Complex sums and differences: both parts in one instruction, each rounded
+// by itself.
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) {
+  float2 o;
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+      "add.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(o.x), "=f"(o.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return o;
+}
+__device__ __forceinline__ float2 csub(float2 a, float2 b) {
+  float2 o;
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+      "sub.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(o.x), "=f"(o.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return o;
+}
 // Complex product with fused multiply-adds (the transforms are compared
 // within an error bound, not bit for bit).
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {

@@ -25,4 +25,8 @@ template <> inline CUtensorMapDataType map_type<uint16_t>() { return CU_TENSOR_M
 bool make_group_maps(CUtensorMap *maps, const FusedGroup &g, const void *base, CUtensorMapDataType type,
                      uint32_t elem, uint64_t rows, uint64_t nt, int32_t *cshift);
 
+// Map over a float32 [rows][nt] matrix for copies of [brows][cols] out of
+// shared memory (nt and cols multiples of 4, the base 16-byte aligned).
+bool make_store_map(CUtensorMap *map, void *base, uint64_t rows, uint64_t nt, uint32_t cols, uint32_t brows);
+
 }  // namespace fdmt
