@@ -43,6 +43,7 @@
 
 #include "../../include/fdmt.h"
 #include "fdmt_internal.h"
+#include "fdmt_residency.h"
 
 namespace fdmt {
 namespace {
@@ -764,8 +765,10 @@ cudaError_t launch_finalize(const void *A, int32_t nd, int64_t nt, int32_t nk, i
   const int fwarps = nk <= 9 ? std::min(nk, kWarps) : kWarps;
   const size_t fsmem = (nk <= 9 ? (size_t)fwarps * kFinalizeWarpElems : (size_t)kFinalizeElems) * sizeof(TB);
   auto fin = search_finalize_kernel<TA, TB, TP>;
-  cudaError_t e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
-  if (e != cudaSuccess) return e;
+  if (fsmem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
+    if (e != cudaSuccess) return e;
+  }
   fin<<<nd, 32 * fwarps, fsmem, s>>>(static_cast<const TA *>(A), (int)nt, nk, nseg, static_cast<const TB *>(part_v),
                                         part_r, static_cast<TP *>(peak), time);
   return cudaGetLastError();
@@ -774,10 +777,8 @@ cudaError_t launch_finalize(const void *A, int32_t nd, int64_t nt, int32_t nk, i
 template <class TA, class TB, class TP>
 cudaError_t launch_search(const void *A, int32_t nd, int64_t nt, int32_t nk, void *peak, int32_t *time, void *ws,
                           cudaStream_t s) {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
+  int resident = 0;
+  cudaError_t e;
   TB *part_v = static_cast<TB *>(ws);
   const int nseg = (int)search_segments(sizeof(TB) == 8, nt, nk);
   int *part_r = reinterpret_cast<int *>(static_cast<char *>(ws) + (size_t)nd * nk * nseg * sizeof(int64_t));
@@ -786,11 +787,9 @@ cudaError_t launch_search(const void *A, int32_t nd, int64_t nt, int32_t nk, voi
   if constexpr (sizeof(TB) == 4) {
     if (nk <= kWarpMaxWidths) {
       auto kern = search_warp_kernel<TB>;
-      if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWarpSmem)) != cudaSuccess)
+      if ((e = resident_blocks(reinterpret_cast<const void *>(kern), kSearchThreads, kWarpSmem, &resident)) != cudaSuccess)
         return e;
-      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSearchThreads, kWarpSmem)) != cudaSuccess)
-        return e;
-      const int grid = std::min((items + kWarps - 1) / kWarps, sms * std::max(per_sm, 1));
+      const int grid = std::min((items + kWarps - 1) / kWarps, resident);
       kern<<<grid, kSearchThreads, kWarpSmem, s>>>(static_cast<const TB *>(A), (int)nt, nk, warp_halo(nk),
                                                    (int)warp_windows(nt, nk), nseg, items, vec, part_v, part_r);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -800,11 +799,9 @@ cudaError_t launch_search(const void *A, int32_t nd, int64_t nt, int32_t nk, voi
   const SearchGeom g = choose_geom(nk, nt, sizeof(TA), sizeof(TB));
   const size_t smem = smem_of(g, nk, sizeof(TA), sizeof(TB));
   auto kern = search_kernel<TA, TB>;
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+  if ((e = resident_blocks(reinterpret_cast<const void *>(kern), kSearchThreads, smem, &resident)) != cudaSuccess)
     return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSearchThreads, smem)) != cudaSuccess)
-    return e;
-  const int grid0 = std::min(items, sms * std::max(per_sm, 1));
+  const int grid0 = std::min(items, resident);
   const int per_block = (items + grid0 - 1) / grid0;
   const int grid = (items + per_block - 1) / per_block;
   kern<<<grid, kSearchThreads, smem, s>>>(static_cast<const TA *>(A), (int)nt, nk, g, nseg, items, per_block, vec,

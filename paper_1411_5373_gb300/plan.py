@@ -19,13 +19,14 @@ _STAGING = {"auto": 0, "boxes": 1, "blocks": 2}
 
 
 def _ptr(t):
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+    # (an integer: the entry points' argument types are declared)
+    return None if t is None else t.data_ptr()
 
 
 def _stream_handle(stream):
     import torch
     s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return s.cuda_stream
 
 
 class Plan:
@@ -111,6 +112,7 @@ class Plan:
         self._h = h
         self._ws = None
         self._adj_ws = None
+        self._ws_need = self._adj_ws_need = None  # workspace sizes, asked once
 
     # -- lifetime -----------------------------------------------------------
     def close(self):
@@ -211,14 +213,18 @@ class Plan:
     def workspace(self, device=None):
         """A cached device workspace of workspace_bytes (allocated by torch)."""
         import torch
-        need = self.workspace_bytes
+        if self._ws_need is None:
+            self._ws_need = self.workspace_bytes
+        need = self._ws_need
         if self._ws is None or self._ws.numel() < need:
             self._ws = torch.empty(max(need, 256), dtype=torch.uint8, device=device or "cuda")
         return self._ws
 
     def adjoint_workspace(self, device=None):
         import torch
-        need = self.adjoint_workspace_bytes
+        if self._adj_ws_need is None:
+            self._adj_ws_need = self.adjoint_workspace_bytes
+        need = self._adj_ws_need
         if self._adj_ws is None or self._adj_ws.numel() < need:
             self._adj_ws = torch.empty(max(need, 256), dtype=torch.uint8, device=device or "cuda")
         return self._adj_ws
