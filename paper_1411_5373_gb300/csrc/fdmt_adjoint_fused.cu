@@ -68,6 +68,17 @@ __device__ __forceinline__ void adj_store_global(float *__restrict__ out_row, in
   }
 }
 
+// The columns [first, end) of an init op's piece that lie below its width and
+// inside [0, nt).
+struct Inside {
+  int first, end;
+  __device__ __forceinline__ Inside(int64_t t0, int width, int64_t nt)
+      : first(t0 < 0 ? (int)max(t0, (int64_t)-kPieceCols) * -1 : 0),
+        end(nt - t0 < width ? (int)max(nt - t0, (int64_t)0) : width) {}
+  __device__ __forceinline__ bool whole() const { return first == 0 && end == kPieceCols; }
+  __device__ __forceinline__ bool holds(int col) const { return col >= first && col < end; }
+};
+
 // One transposed level: each op sums its run of p2 parent rows (stride p1
 // bytes; the upper half's stride includes the one-column shift per row).
 template <int OUT>
@@ -116,13 +127,33 @@ __device__ __forceinline__ void adj_gather_stage(uint32_t sbase, const StageRang
 // piece).
 __device__ __forceinline__ void adj_init_load_x(float (&xv)[kLaneCols], const FusedOp &op,
                                                 const float *__restrict__ x, int64_t nt, int64_t T0, int lane) {
-  const float *xrow = x + (int64_t)op.dst * nt;
   const int64_t t0 = T0 + op.col;
+  const Inside in(t0, op.width, nt);
+  const float *p = x + (int64_t)op.dst * nt + t0 + lane;
+  if (in.whole()) {
 #pragma unroll
-  for (int k = 0; k < kLaneCols; ++k) {
-    const int tau = lane + 32 * k;
-    const int64_t t = t0 + tau;
-    xv[k] = (tau < op.width && t >= 0 && t < nt) ? __ldg(xrow + t) : 0.f;
+    for (int k = 0; k < kLaneCols; ++k) xv[k] = __ldg(p + 32 * k);
+  } else {
+#pragma unroll
+    for (int k = 0; k < kLaneCols; ++k) xv[k] = in.holds(lane + 32 * k) ? __ldg(p + 32 * k) : 0.f;
+  }
+}
+
+// Asks L2 for the input samples that an item's init ops will read (whole 16
+// bytes inside [0, nt); the ragged ends come with their first reader).
+__device__ __forceinline__ void adj_init_ahead(const FusedProg &pr, const int4 *__restrict__ prog,
+                                               const float *__restrict__ x, int64_t nt, int64_t T0, int lane) {
+  const char *words = reinterpret_cast<const char *>(prog + pr.prog);
+  const int32_t *stage = reinterpret_cast<const int32_t *>(words + (pr.n_stages - 1) * kProgStageBytes);
+  const int32_t first = stage[1], n = (stage[kStageWords - 1] - first) / (int32_t)sizeof(FusedOp);
+  const FusedOp *ops = reinterpret_cast<const FusedOp *>(words + first);
+  for (int32_t i = lane; i < n; i += 32) {
+    const int64_t t = T0 + ops[i].col, a = t < 0 ? 0 : t, b = t + ops[i].width < nt ? t + ops[i].width : nt;
+    const float *row = x + (int64_t)ops[i].dst * nt;
+    const uint64_t from = (reinterpret_cast<uint64_t>(row + a) + 15) & ~15ull;
+    const uint64_t to = reinterpret_cast<uint64_t>(row + b) & ~15ull;
+    if (a < b && from < to)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(from), "r"((uint32_t)(to - from)) : "memory");
   }
 }
 
@@ -136,29 +167,35 @@ __device__ __forceinline__ void adj_init_op(uint32_t sbase, const FusedOp &op, c
   float v[kLaneCols];
   if constexpr (FOLD) {
     // term (j, i) is level-0 row j at column tau + i: its run of level-1
-    // rows summed in row order, as the gather would have stored it
+    // rows summed in row order, as the gather would have stored it (runs of
+    // one or two rows, nearly all, without a loop)
     uint32_t pj = sbase + (uint32_t)op.p0;
     const uint32_t step = (uint32_t)op.p1, back = 4u * (uint32_t)(op.flags & 1);
-    uint32_t runs = (uint32_t)op.flags >> 1;
-    for (int j = 0; j < op.p2; ++j, runs >>= 4) {
-      const int cnt = (int)(runs & 15u);
-      for (int ii = 0; ii <= j; ++ii) {
-        float r[kLaneCols];
-        const uint32_t a = pj + 4u * (uint32_t)ii;
-        ld_piece<float, float>(r, a, lane);
-        for (int q = 1; q < cnt; ++q) {
-          float y[kLaneCols];
+    uint32_t runs = (uint32_t)warp_all(op.flags) >> 1;
+    const int rows = warp_all(op.p2);
+    auto term = [&](float (&r)[kLaneCols], uint32_t a, int cnt) {
+      ld_piece<float, float>(r, a, lane);
+      if (cnt > 1) {
+        float y[kLaneCols];
+        ld_piece<float, float>(y, a + step, lane);
+        add_piece(r, r, y);
+        for (int q = 2; q < cnt; ++q) {
           ld_piece<float, float>(y, a + (uint32_t)q * step, lane);
           add_piece(r, r, y);
         }
-        if (j == 0) {
-#pragma unroll
-          for (int k = 0; k < kLaneCols; ++k) v[k] = r[k];
-        } else {
-          add_piece(v, v, r);
-        }
       }
+    };
+    int cnt = (int)(runs & 15u);
+    term(v, pj, cnt);
+    for (int j = 1; j < rows; ++j) {
       pj += (uint32_t)cnt * step - back;
+      runs >>= 4;
+      cnt = (int)(runs & 15u);
+      for (int ii = 0; ii <= j; ++ii) {
+        float r[kLaneCols];
+        term(r, pj + 4u * (uint32_t)ii, cnt);
+        add_piece(v, v, r);
+      }
     }
   } else {
     ld_piece<float, float>(v, sbase + (uint32_t)op.p0, lane);
@@ -171,15 +208,16 @@ __device__ __forceinline__ void adj_init_op(uint32_t sbase, const FusedOp &op, c
       }
     }
   }
+  const Inside in(T0 + op.col, op.width, nt);
   if (part != nullptr) {
-    const int64_t t0 = T0 + op.col;
     float d = 0.f;
+    if (in.whole()) {
 #pragma unroll
-    for (int k = 0; k < kLaneCols; ++k) {
-      const int tau = lane + 32 * k;
-      const int64_t t = t0 + tau;
-      const bool ok = tau < op.width && t >= 0 && t < nt;
-      d = __fadd_rn(d, ok ? __fmul_rn(xv[k], v[k]) : 0.f);
+      for (int k = 0; k < kLaneCols; ++k) d = __fadd_rn(d, __fmul_rn(xv[k], v[k]));
+    } else {
+#pragma unroll
+      for (int k = 0; k < kLaneCols; ++k)
+        d = __fadd_rn(d, in.holds(lane + 32 * k) ? __fmul_rn(xv[k], v[k]) : 0.f);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) d = __fadd_rn(d, __shfl_xor_sync(0xffffffffu, d, off));
@@ -190,7 +228,15 @@ __device__ __forceinline__ void adj_init_op(uint32_t sbase, const FusedOp &op, c
 #pragma unroll
     for (int k = 0; k < kLaneCols; ++k) v[k] = __fmul_rn(v[k], wk);
   }
-  adj_store_global(out + (int64_t)op.dst * nt, T0 + op.col, v, op.width, nt, lane);
+  float *p = out + (int64_t)op.dst * nt + T0 + op.col + lane;
+  if (in.whole()) {
+#pragma unroll
+    for (int k = 0; k < kLaneCols; ++k) p[32 * k] = v[k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < kLaneCols; ++k)
+      if (in.holds(lane + 32 * k)) p[32 * k] = v[k];
+  }
 }
 
 // The init stage takes its ops two at a time: the input samples of both
@@ -221,7 +267,10 @@ __device__ __forceinline__ void adj_init_stage(uint32_t sbase, const StageRange 
 // transpose.
 // Bound: latency and HBM alike.  1024 x 65536 x 1024 on a GB300, launches 10
 // -> 8 -> 6 -> 4 -> 2 -> 0 with the weight gradient: 112, 110, 116, 126 and
-// 264 us with ops read through L2 and warp 0 copying; 98, 97, 101, 104 and 248 us now.
+// 264 us with ops read through L2 and warp 0 copying; 98, 97, 101, 104 and
+// 248 us with programmes and a copying warp.  The last launch reads a second
+// input: 237 us with it asked for ahead, 195 with the init stage's columns
+// tested once per piece and its runs straight-line (instruction issue).
 template <bool INIT>
 __global__ void __launch_bounds__(kFusedLaunchThreads, kFusedMinBlocks)
 adjoint_cone_kernel(const __grid_constant__ TmaMaps maps, float *__restrict__ out, int64_t nt, int32_t W,
@@ -235,7 +284,9 @@ adjoint_cone_kernel(const __grid_constant__ TmaMaps maps, float *__restrict__ ou
   init_item_barriers(full);
   if (warp == kFusedWarps) {
     copy_items<float>(smem, maps, nt, W, 0, ntiles, items, progs, prog, loads, box, cshift, prog_off, prog_slot, status,
-                      lane);
+                      lane, [&](const FusedProg &pr, int64_t T0) {
+                        if (INIT && part != nullptr) adj_init_ahead(pr, prog, x, nt, T0, lane);
+                      });
     return;
   }
   uint32_t slot = 0, phase = 0;

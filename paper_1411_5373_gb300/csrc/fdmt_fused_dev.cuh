@@ -999,13 +999,15 @@ __device__ __forceinline__ void init_item_barriers(uint32_t full) {
 // float32 306 us without, 289 us with; 4096 x 2^18 x 4096, HBM-bound in its
 // cones, 5.67 ms without, 5.70 with, 6.36 with the requests but template by
 // template.  (Row boxes are bound by the rate of copies: asking twice made
-// them 5 % slower.)
-template <class TS>
+// them 5 % slower.)  also_ahead(programme, T0) asks for whatever else the next
+// item reads.
+template <class TS, class Ahead>
 __device__ __forceinline__ void copy_items(unsigned char *smem, const TmaMaps &maps, int64_t nt, int32_t W,
                                            int32_t tile0, int32_t ntiles, int64_t items,
                                            const FusedProg *__restrict__ progs, const int4 *__restrict__ prog,
                                            const FusedLoad *__restrict__ loads, int32_t box, int32_t cshift,
-                                           int32_t prog_off, int32_t prog_slot, int *__restrict__ status, int lane) {
+                                           int32_t prog_off, int32_t prog_slot, int *__restrict__ status, int lane,
+                                           Ahead also_ahead) {
   const uint32_t full = smem_u32(smem), free_bar = full + kFreeBar, header = full + kItemHeader;
   int64_t item = blockIdx.x;
   if (item >= items) return;
@@ -1046,7 +1048,9 @@ __device__ __forceinline__ void copy_items(unsigned char *smem, const TmaMaps &m
       place(item + gridDim.x);
       pr = progs[tpl];
       ld = fetch_load(pr, loads, lane);
-      if (cshift > 0) prefetch_item<TS>(maps.m, pr, loads, ld, (int64_t)(tile0 + tile) * W, box, cshift, lane);
+      const int64_t T1 = (int64_t)(tile0 + tile) * W;
+      if (cshift > 0) prefetch_item<TS>(maps.m, pr, loads, ld, T1, box, cshift, lane);
+      also_ahead(pr, T1);
     }
   }
   // The last copies land before the block ends: the computing warps wait

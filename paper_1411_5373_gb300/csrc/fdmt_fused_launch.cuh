@@ -69,7 +69,7 @@ fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t
   init_item_barriers(full);
   if (warp == kFusedWarps) {
     copy_items<TS>(smem, maps, nt, W, tile0, ntiles, items, progs, prog, loads, box, cshift, prog_off, prog_slot, status,
-                   lane);
+                   lane, [](const FusedProg &, int64_t) {});
     return;
   }
   uint32_t slot = 0, phase = 0;
