@@ -729,9 +729,13 @@ int32_t choose_box(const std::vector<std::pair<int32_t, int32_t>> &needs, int32_
   return best;
 }
 
+// What a build of a group is for: the windows of its cones (`needs`), its
+// cost as well, or its descriptors as well.
+enum class Build { kMeasure, kCount, kEmit };
+
 GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int32_t W,
                            const FusedPlan &fp, int32_t budget, const StageFmt &f,
-                           std::vector<std::pair<int32_t, int32_t>> *needs, bool emit) {
+                           std::vector<std::pair<int32_t, int32_t>> *needs, Build what) {
   GroupBuild gb;
   const int32_t nb = bands_at(t.nf, lt);
   const int64_t nst = (int64_t)stored_levels(lb, lt).size() - 1 + (f.search_k > 0 ? 1 : 0);
@@ -849,10 +853,11 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
       // Each cone of the item gets its own slice of S, Pa and Pb; the item's
       // stage ops are merged stage by stage, then split over the warps.
       ItemOut item;
-      if (!emit) {
+      if (what != Build::kEmit) {
         int32_t copies = 0;
         for (int32_t i : bu) {
           if (needs) needs->insert(needs->end(), shapes[i].needs.begin(), shapes[i].needs.end());
+          if (what == Build::kMeasure) continue;
           ConeOut c;
           count_cone(t, lb, lt, W, fp, f, shapes[i], c, copies);
           item.tpl.tx_bytes += c.tpl.tx_bytes;
@@ -1000,7 +1005,7 @@ GroupBuild build_group_mode(const Tables &t, int64_t nt, int32_t lb, int32_t lt,
     f.box = 128 / es;
   }
   std::vector<std::pair<int32_t, int32_t>> needs;
-  GroupBuild gb = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &needs, false);
+  GroupBuild gb = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &needs, Build::kMeasure);
   if (!gb.ok) return gb;
   int32_t widest = 0;
   for (const auto &nr : needs) widest = std::max(widest, nr.first);
@@ -1015,32 +1020,33 @@ GroupBuild build_group_mode(const Tables &t, int64_t nt, int32_t lb, int32_t lt,
       if (k > 256 || (int64_t)k * chunk > nt) break;
       f.kchunks = std::max(f.kchunks, k);
       std::vector<std::pair<int32_t, int32_t>> got;
-      GroupBuild g2 = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &got, false);
+      GroupBuild g2 = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &got, Build::kCount);
       if (!g2.ok) break;
       widest = 0;
       for (const auto &nr : got) widest = std::max(widest, nr.first);
       if (widest <= f.kchunks * chunk)
-        return emit ? build_group_fmt(t, nt, lb, lt, W, fp, budget, f, nullptr, true) : g2;
+        return emit ? build_group_fmt(t, nt, lb, lt, W, fp, budget, f, nullptr, Build::kEmit) : g2;
     }
     if (staging == 2) return GroupBuild();
     f = boxes;  // fall back to row boxes
     f.box = 128 / es;
     needs.clear();
-    gb = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &needs, false);
+    gb = build_group_fmt(t, nt, lb, lt, W, fp, budget, f, &needs, Build::kMeasure);
     if (!gb.ok) return gb;
   }
   f.box = choose_box(needs, es);
-  return build_group_fmt(t, nt, lb, lt, W, fp, budget, f, nullptr, emit);
+  return build_group_fmt(t, nt, lb, lt, W, fp, budget, f, nullptr, emit ? Build::kEmit : Build::kCount);
 }
 
-// The same, in the compact layout where the roomy one does not fit, and with
-// row boxes (whose windows are not rounded to chunks) where that does not.
+// The same in a layout: roomy; compact, where a budget fits no roomy one; and
+// compact with row boxes (whose windows are not rounded to chunks), where it
+// fits neither.
+enum : int32_t { kRoomy = 0, kCompact = 1, kCompactBoxes = 2 };
 GroupBuild build_group(const Tables &t, int64_t nt, int32_t lb, int32_t lt, int32_t W, const FusedPlan &fp,
-                       int32_t budget, const FusedParams &prm, int32_t search_k, bool emit) {
-  GroupBuild gb = build_group_mode(t, nt, lb, lt, W, fp, budget, prm, search_k, emit, false, prm.staging);
-  if (!gb.ok) gb = build_group_mode(t, nt, lb, lt, W, fp, budget, prm, search_k, emit, true, prm.staging);
-  if (!gb.ok && prm.staging == 0) gb = build_group_mode(t, nt, lb, lt, W, fp, budget, prm, search_k, emit, true, 1);
-  return gb;
+                       int32_t budget, const FusedParams &prm, int32_t search_k, bool emit, int32_t layout) {
+  if (layout == kCompactBoxes && prm.staging != 0) return GroupBuild();
+  return build_group_mode(t, nt, lb, lt, W, fp, budget, prm, search_k, emit, layout != kRoomy,
+                          layout == kCompactBoxes ? 1 : prm.staging);
 }
 
 // Shared-memory pipe slots per 32 columns of the first row of a run (all its
@@ -1268,28 +1274,42 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
     }
   }
   // Best tile for one group (lb, lt] (optionally a given tile and budget),
-  // counted only.
-  auto best_segment = [&](int32_t lb, int32_t lt, int32_t forced_W = 0, int32_t budget = 0, bool refine = false) {
-    GroupBuild best;
+  // counted only.  `known`: the tile that was best before.
+  struct Segment {
+    GroupBuild gb;
+    int32_t layout = kRoomy;
+  };
+  auto best_segment = [&](int32_t lb, int32_t lt, int32_t forced_W = 0, int32_t budget = 0, bool refine = false,
+                          int32_t known = 0) {
+    Segment best;
     const std::vector<int32_t> ws = forced_W > 0 ? std::vector<int32_t>{forced_W} : widths;
-    for (int32_t W : ws) {
-      if (best.ok && W / 2 >= nt) break;  // (no wider than one tile needs)
-      GroupBuild gb = build_group(t, nt, lb, lt, W, fp, budget > 0 ? budget : p.smem_budget, p,
-                                  lt == L ? p.search_k : 0, false);
-      if (gb.ok && (!best.ok || gb.seconds < best.seconds)) best = std::move(gb);
-    }
+    auto tries = [&](int32_t W, int32_t layout, int32_t bytes) {
+      GroupBuild gb = build_group(t, nt, lb, lt, W, fp, bytes, p, lt == L ? p.search_k : 0, false, layout);
+      const bool ok = gb.ok;
+      if (ok && (!best.gb.ok || gb.seconds < best.gb.seconds)) best = Segment{std::move(gb), layout};
+      return ok;
+    };
+    // Long rows take the other layouts only where no tile fits the roomy one
+    // (planning 1000 x 50004 x 777: 218 ms, 364 ms with all of them tried
+    // tile by tile); short calls are bound by launches and latency, where a
+    // lesser layout that saves a launch can win.
+    const bool all = nt < kPadRows;
+    for (int32_t layout = kRoomy; layout <= kCompactBoxes && !best.gb.ok; ++layout)
+      for (int32_t W : ws) {
+        if (known > 0 && W != known) continue;
+        if (best.gb.ok && W / 2 >= nt) break;  // (no wider than one tile needs)
+        for (int32_t l = layout; !tries(W, l, budget > 0 ? budget : p.smem_budget) && all && l < kCompactBoxes;) ++l;
+      }
     // Few items leave SMs idle: smaller ones (more row ranges) may be faster
     // (tried once the boundaries stand).
     for (int32_t kib = 56; refine && budget == 0 && p.smem_budget == FusedParams().smem_budget && kib >= 14; kib /= 2) {
-      if (!best.ok || best.items * best.g.ntiles >= best.g.block_slots) break;
-      for (int32_t W : ws) {
-        GroupBuild gb = build_group(t, nt, lb, lt, W, fp, kib * 1024, p, lt == L ? p.search_k : 0, false);
-        if (gb.ok && gb.seconds < best.seconds) best = std::move(gb);
-      }
+      if (!best.gb.ok || best.gb.items * best.gb.g.ntiles >= best.gb.g.block_slots) break;
+      for (int32_t W : ws)
+        for (int32_t l = kRoomy; !tries(W, l, kib * 1024) && all && l < kCompactBoxes;) ++l;
     }
     return best;
   };
-  std::vector<int32_t> bounds = p.bounds;
+  std::vector<int32_t> bounds = p.bounds, tile(L + 1, 0);  // tile[j]: of the group that ends at level j, if searched
   if (bounds.empty()) {
     // Dynamic programming over boundaries: cost[j] = best time to reach level j.
     std::vector<double> cost(L + 1, std::numeric_limits<double>::infinity());
@@ -1298,11 +1318,12 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
     for (int32_t j = 1; j <= L; ++j)
       for (int32_t i = std::max(0, j - 6); i < j; ++i) {
         if (!std::isfinite(cost[i])) continue;
-        GroupBuild gb = best_segment(i, j);
+        const GroupBuild gb = best_segment(i, j).gb;
         if (!gb.ok) continue;
         if (cost[i] + gb.seconds < cost[j]) {
           cost[j] = cost[i] + gb.seconds;
           from[j] = i;
+          tile[j] = gb.g.W;
         }
       }
     if (!std::isfinite(cost[L])) return "no fused schedule fits the shared-memory budget";
@@ -1319,10 +1340,12 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
     const int32_t gw = i < p.group_W.size() ? p.group_W[i] : 0;
     const int32_t gbud = i < p.group_budget.size() ? p.group_budget[i] : 0;
     if (gw < 0 || gw % 64 != 0 || gbud < 0 || gbud > 227 * 1024) return "bad per-group parameters";
-    GroupBuild gb = best_segment(bounds[i], bounds[i + 1], gw, gbud, true);
-    if (gb.ok)
-      gb = build_group(t, nt, bounds[i], bounds[i + 1], gb.g.W, fp, gb.budget, p,
-                       bounds[i + 1] == L ? p.search_k : 0, true);
+    const Segment seg = best_segment(bounds[i], bounds[i + 1], gw, gbud, true,
+                                     gw == 0 && gbud == 0 ? tile[bounds[i + 1]] : 0);
+    GroupBuild gb;
+    if (seg.gb.ok)
+      gb = build_group(t, nt, bounds[i], bounds[i + 1], seg.gb.g.W, fp, seg.gb.budget, p,
+                       bounds[i + 1] == L ? p.search_k : 0, true, seg.layout);
     if (!gb.ok) return "a level group does not fit the shared-memory budget";
     secs += gb.seconds;
     if (!append_group(fp, gb)) return "a programme outgrew its slot";
