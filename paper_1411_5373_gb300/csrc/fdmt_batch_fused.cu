@@ -413,7 +413,11 @@ int fused_batch_create(const std::vector<fdmt_beam_desc> &desc, const std::vecto
   FusedParams fpar;
   fpar.narrow = (dtype == FDMT_U8_I32);
   fpar.W = prm.fused_tile;
-  fpar.smem_budget = prm.smem_budget > 0 ? prm.smem_budget : 72 * 1024;
+  // Two blocks per SM with room to spare: 8 beams 512 x 32768 x 512 uint8 /
+  // float32 838 / 1117 us with 72 KiB (three blocks fitted it when the kernel
+  // had 80 registers: 731 / 998), 671 / 969 with 104 KiB, 775 / 906 with 112;
+  // three small beams 76 / 87, 68 / 77 and 75 / 94.
+  fpar.smem_budget = prm.smem_budget > 0 ? prm.smem_budget : 104 * 1024;
   std::vector<FusedProg> tpls;
   std::vector<FusedLoad> loads;
   std::vector<int32_t> prog;
