@@ -33,7 +33,6 @@ struct fdmt_stream_s {
   void *win[2] = {nullptr, nullptr};  // input windows [nf][window], ping-pong
   void *wout = nullptr;               // plain plans: window output [nd][window]
   bool fused = false;
-  bool fresh = true;                  // no chunk yet: the carry is zero
   void *ws = nullptr;
   size_t ws_bytes = 0;
   int cur = 0;                        // window holding the latest chunk
@@ -45,17 +44,14 @@ size_t in_size(int32_t dtype) { return dtype == FDMT_U8_I32 ? 1 : 4; }
 
 constexpr int kWindowThreads = 256;
 
-// Row blockIdx.y of a window: `carry` 16-byte words from `prev` (zeros when
-// null), then `chunk` words of the new chunk.
+// Row blockIdx.y of a window: the last `carry` 16-byte words of `prev`, then
+// `chunk` words of the new chunk.
 __global__ void __launch_bounds__(kWindowThreads)
 window_kernel(const int4 *__restrict__ prev, const int4 *__restrict__ in, int4 *__restrict__ win, int64_t carry,
               int64_t chunk) {
   const int64_t i = (int64_t)blockIdx.x * kWindowThreads + threadIdx.x, row = blockIdx.y, pitch = carry + chunk;
   if (i >= pitch) return;
-  int4 v = make_int4(0, 0, 0, 0);
-  if (i >= carry) v = __ldg(in + row * chunk + (i - carry));
-  else if (prev != nullptr) v = __ldg(prev + row * pitch + chunk + i);
-  win[row * pitch + i] = v;
+  win[row * pitch + i] = i >= carry ? __ldg(in + row * chunk + (i - carry)) : __ldg(prev + row * pitch + chunk + i);
 }
 
 void release(fdmt_stream_s *s) {
@@ -113,6 +109,13 @@ int fdmt_stream_create(double f_min, double f_max, int32_t nf, int64_t chunk, in
     release(s);
     return FDMT_ERR_NO_MEMORY;
   }
+  // The carry before the first chunk is zero (the copy rule).
+  if (s->carry > 0 && cudaMemset2D(static_cast<char *>(s->win[0]) + (size_t)chunk * s->in_es, (size_t)window * s->in_es, 0,
+                                   (size_t)carry * s->in_es, (size_t)nf) != cudaSuccess) {
+    cudaGetLastError();
+    release(s);
+    return FDMT_ERR_CUDA;
+  }
   *out = s;
   return FDMT_OK;
 }
@@ -137,7 +140,7 @@ int fdmt_stream_push(fdmt_stream_t s, const void *in, void *out, void *stream) {
     const dim3 grid((unsigned)((carry + chunk + kWindowThreads - 1) / kWindowThreads),
                     (unsigned)std::min<int32_t>(65535, s->nf - row));
     window_kernel<<<grid, kWindowThreads, 0, cs>>>(
-        s->fresh ? nullptr : static_cast<const int4 *>(s->win[s->cur]) + off,
+        static_cast<const int4 *>(s->win[s->cur]) + off,
         static_cast<const int4 *>(in) + (int64_t)row * chunk, static_cast<int4 *>(dst) + off, carry, chunk);
   }
   if (cudaGetLastError() != cudaSuccess) return FDMT_ERR_CUDA;
@@ -155,15 +158,21 @@ int fdmt_stream_push(fdmt_stream_t s, const void *in, void *out, void *stream) {
       return FDMT_ERR_CUDA;
     }
   }
-  s->fresh = false;
   s->cur = nxt;
   return FDMT_OK;
 }
 
 int fdmt_stream_reset(fdmt_stream_t s, void *stream) {
   if (s == nullptr) return FDMT_ERR_INVALID_ARG;
-  (void)stream;  // the next window is laid out with a carry of zeros
-  s->fresh = true;
+  // The carry of zeros, in stream order (a captured reset or push replays
+  // as it ran): the last columns of the window that the next push reads.
+  const size_t pitch = (size_t)s->window * s->in_es;
+  if (s->carry > 0 && cudaMemset2DAsync(static_cast<char *>(s->win[0]) + (size_t)s->chunk * s->in_es, pitch, 0,
+                                        (size_t)s->carry * s->in_es, (size_t)s->nf,
+                                        static_cast<cudaStream_t>(stream)) != cudaSuccess) {
+    cudaGetLastError();
+    return FDMT_ERR_CUDA;
+  }
   s->cur = 0;
   return FDMT_OK;
 }

@@ -38,3 +38,29 @@ def test_pushes_equal_one_transform(nf, chunk, nd, pushes, dtype):
     got = np.concatenate([st.push(p).cpu().numpy() for p in parts], axis=1)
     st.close()
     assert np.array_equal(got, want)
+
+
+def test_captured_pushes_carry_on():
+    """A reset followed by a captured pair of pushes: every replay goes on
+    from the chunks before it, the first one from zeros."""
+    nf, chunk, nd = 32, 512, 100
+    x = fs.random_u8(7, nf, 6 * chunk)
+    want = oracle.fdmt(x, oracle.build_tables(1200.0, 1600.0, nf, nd), "i64")
+    parts = [torch.from_numpy(np.ascontiguousarray(x[:, i * chunk:(i + 1) * chunk])).cuda() for i in range(6)]
+    st = FD.Stream(1200.0, 1600.0, nf, chunk, nd, "u8", "fused")
+    a, b = parts[0].clone(), parts[1].clone()
+    out = [st.push(a), st.push(b)]
+    st.reset()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        st.push(a, out[0])
+        st.push(b, out[1])
+    got = []
+    for i in range(0, 6, 2):
+        a.copy_(parts[i])
+        b.copy_(parts[i + 1])
+        graph.replay()
+        got += [o.cpu().numpy() for o in out]
+    st.close()
+    assert np.array_equal(np.concatenate(got, axis=1), want)
