@@ -121,6 +121,7 @@ class Plan:
         self._h = None
         self._ws = None
         self._adj_ws = None
+        self._ws_need = self._adj_ws_need = None  # (a closed plan has no sizes)
 
     def __del__(self):
         try:
