@@ -457,8 +457,20 @@ int fused_batch_create(const std::vector<fdmt_beam_desc> &desc, const std::vecto
     ws += (size_t)rup((int64_t)fp.ws_bytes, 256);
   }
   fb->ws_bytes = ws;
+  // One beam's regions and another's slots can exceed a block together (from
+  // budgets of 220 KiB on): programmes that the rest does not hold are then
+  // read in global memory.  (Each group by itself leaves its slots' room.)
+  const int32_t room = (227 * 1024 - kOverRead - fb->prog_off) / 2 / 128 * 128;
+  if (fb->prog_slot > room) {
+    fb->prog_slot = room;
+    for (FusedProg &tp : tpls) {
+      if (tp.far || tp.prog_bytes <= room) continue;
+      tp.far = 1;
+      tp.tx_bytes -= tp.prog_bytes;
+    }
+  }
   fb->smem_bytes = fb->prog_off + 2 * fb->prog_slot + kOverRead;
-  if (tpls.size() >= ((size_t)1 << 31) || prog.size() >= ((size_t)1 << 31) || fb->smem_bytes > 227 * 1024) {
+  if (tpls.size() >= ((size_t)1 << 31) || prog.size() >= ((size_t)1 << 31)) {
     delete fb;
     return FDMT_ERR_UNSUPPORTED;
   }
