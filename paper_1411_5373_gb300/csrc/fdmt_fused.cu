@@ -13,17 +13,33 @@ namespace fdmt {
 
 namespace {
 
+template <class F>
+F driver_entry(const char *name, int version) {
+  void *p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion(name, &p, version, cudaEnableDefault, &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess)
+    return nullptr;
+  return reinterpret_cast<F>(p);
+}
+
+// The driver's map encoder, or null.  It needs a context that is current in
+// the calling thread, and a thread that has made no runtime call that binds
+// one has none (autograd's worker, whose small allocations come from a
+// cache): the current device's is then made current.  A context that is
+// current already stays.
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+  static PFN_cuCtxGetCurrent_v4000 current = nullptr;
   static std::once_flag once;
   std::call_once(once, [] {
-    void *p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+    fn = driver_entry<PFN_cuTensorMapEncodeTiled_v12000>("cuTensorMapEncodeTiled", 12000);
+    current = driver_entry<PFN_cuCtxGetCurrent_v4000>("cuCtxGetCurrent", 4000);
   });
+  CUcontext ctx = nullptr;
+  int dev = 0;
+  if (current == nullptr || current(&ctx) != CUDA_SUCCESS) return nullptr;
+  if (ctx == nullptr && (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess)) return nullptr;
   return fn;
 }
 
