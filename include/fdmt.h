@@ -679,7 +679,8 @@ int fdmt_schedule_info(fdmt_plan_t plan, int32_t *groups, int32_t *bounds, int32
  * 4 ops (8 each: destination, four source offsets, width, reuse flags,
  * first column), 5 stages (10 words per stage: kind 0 walk / 1 one level /
  * 2 two levels, then the first walk or op of each of the 8 warps and the
- * end),
+ * end; 128 is added to the kind of a walk stage some of whose walks move
+ * their upper sums between lanes),
  * 6 constants (tile, state size, input size, acc size, bytes of over-read
  * slack that end a block's shared memory, least bytes of the programme
  * slots before it), 7 the planner's cost

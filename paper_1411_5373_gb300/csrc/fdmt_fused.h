@@ -55,6 +55,8 @@ constexpr int32_t kStageKindMask = 15;
 // (kOpLoOne, kOpHiOne, kOpNoHi; walks: kWalkNoUpper), which only Nf not a
 // power of two produces; stages without it run code without those tests.
 constexpr int32_t kStageGeneral = 32;
+// Stage word flag: some walk of the stage moves its upper sums (walk_moves).
+constexpr int32_t kStageMoves = 128;
 
 // Boxcar search in the last launch (section 4.2, pulse profile): widths
 // 2^k, k < K <= kSearchMaxWidths; the top level's time window carries
@@ -138,6 +140,19 @@ struct FusedWalk {
   int32_t chan;     // lower channel (channel weights; the upper one is chan + 1)
   int32_t flags;    // kWalkNoUpper: a single channel, whose Option-1 rows pass up
 };
+// Whether a walk moves its upper sums between lanes where the delay grows (9
+// shuffles and 8 selections for 8 columns per lane) or reads them again (j + 1
+// reads and j sums of 8): the two cost alike at j = 1, and j only grows along
+// a walk, by one with every step that is not in `bits`.
+constexpr int32_t kWalkMoves = 2;
+FDMT_HOST_DEVICE inline bool walk_moves(const FusedWalk &wk) {
+#ifdef __CUDA_ARCH__
+  const int32_t grows = __popc((uint32_t)wk.bits);
+#else
+  const int32_t grows = __builtin_popcount((uint32_t)wk.bits);
+#endif
+  return (wk.flags & kWalkNoUpper) == 0 && wk.e - wk.dl0 - grows >= kWalkMoves;
+}
 
 // The ops of one node's rows, lowered for the kernel.  A run computes rows
 // 0 .. n - 1 of a strip of kPieceCols columns that moves with the delay: row
@@ -174,7 +189,8 @@ constexpr int32_t kRunWhole = 256;
 // at least this many columns free.
 constexpr int32_t kRunGrow = 16;
 // Bytes kept free below the staged rows: a run reads its lower rows from up
-// to kRunRows - 1 columns before their first.
+// to kRunRows - 1 columns before their first, a walk that moves its upper sums
+// up to 32 samples before them.
 constexpr int32_t kUnderRead = 128;
 // Stages over the runs: as the stages, with single and pair stages' offsets
 // into the runs, and this bit set in their kind.

@@ -472,12 +472,18 @@ __device__ __forceinline__ void stage_runs(uint32_t sbase, const StageRange &ran
 // sums of level 0 and one merge).  The running sums plo = x_lo[tau] + ... +
 // x_lo[tau - dl] and phi = x_hi[tau - dl] + ... + x_hi[tau - dl - j] are
 // kept in registers in the oracle's order (each adds one earlier sample);
-// when dl grows the upper sums are read again a column earlier (j + 1 reads;
-// j is 0 or 1 on most rows, where this costs no more than moving the sums
-// between lanes).  A row's reads are issued before the row before it is
-// stored.  SCALE multiplies every sample by its channel's weight first.
-// Bound: instruction issue.
-template <class TI, class A, class TO, bool R16, bool SCALE, bool TOP, bool GEN>
+// when dl grows the upper sums move a column.  A walk whose j stays below
+// kWalkMoves reads them again a column earlier (j + 1 reads); a longer one
+// moves them between lanes, the first column coming from 32 more columns of
+// sums that are kept before the piece (`before`; each move uses up one, and
+// a walk makes at most 31).  A row's reads are issued before the row before it
+// is stored.  SCALE multiplies every sample by its channel's weight first.
+// MOVES: the stage has walks that move their sums (the code alone costs the
+// others 2 to 4 % of the launch).
+// Bound: instruction issue.  Launch [0,1] of 32 x 159808 x 2738 with fp16
+// state, 86 level-0 rows per channel: 1648 us with every upper sum read again,
+// 386 us with the moves.
+template <class TI, class A, class TO, bool R16, bool SCALE, bool TOP, bool GEN, bool MOVES>
 __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &range, int lane,
                                            const float *__restrict__ w, TO *__restrict__ out, int64_t nt, int64_t T0,
                                            int lo, int lim) {
@@ -501,6 +507,7 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
     const bool upper = !GEN || !(warp_all(wk.flags) & kWalkNoUpper);
     int dl = warp_all(wk.dl0), j = warp_all(wk.a) - dl;
     uint32_t bits = (uint32_t)warp_all(wk.bits);
+    const bool moves = MOVES && upper && warp_all((int)walk_moves(wk)) != 0;
     const int skip = TOP ? max(lo - wk.col, 0) : 0;  // columns before the first one wanted
     const bool whole = TOP ? warp_all(wk.width) >= kPieceCols && warp_all(wk.col) + kPieceCols <= lim && warp_all(skip) == 0
                            : warp_all(wk.width) >= kPieceCols || (warp_all(wk.dst_row) & (kPieceCols * 4 - 1)) == 0;
@@ -508,7 +515,26 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
     uint32_t dst = sbase + (uint32_t)wk.dst + (uint32_t)lane * (uint32_t)sizeof(A);
     TO *g = nullptr;
     if constexpr (TOP) g = out + (int64_t)wk.dst * nt + T0 + wk.col + lane;
-    A plo[kLaneCols], phi[kLaneCols], v[kLaneCols], t[kLaneCols];
+    A plo[kLaneCols], phi[kLaneCols], v[kLaneCols], t[kLaneCols], before = A(0);
+    // The upper channel's sample s columns before column lane - 32 (scaled);
+    // those that no move brings into the piece may lie up to 32 samples before
+    // the staged rows, in the slack below them (kUnderRead).
+    auto sample_before = [&](int s) -> A {
+      A x = load_input<TI, A>(xh + (uint32_t)(lane - 32 - s) * es);
+      if constexpr (SCALE) x = __fmul_rn(x, wh);
+      return x;
+    };
+    auto move_upper = [&]() {
+      const int from = (lane + 31) & 31;
+      A in = __shfl_sync(0xffffffffu, before, from);
+      before = in;
+#pragma unroll
+      for (int k = 0; k < kLaneCols; ++k) {
+        const A x = __shfl_sync(0xffffffffu, phi[k], from);
+        phi[k] = lane == 0 ? in : x;
+        in = x;
+      }
+    };
     auto store = [&]() {
       if constexpr (TOP) {
         if (whole) {
@@ -555,15 +581,20 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
         samples(t, xh, dl + i, wh);
         add_piece(phi, phi, t);
       }
+    if (moves) {
+      before = sample_before(dl);
+      for (int i = 1; i <= j; ++i) before = acc_add(before, sample_before(dl + i));
+    }
     for (int left = warp_all(wk.e - wk.a); left > 0; --left) {
       sum();
       if (!upper || (bits & 1u)) {  // (a single channel: row r is its Option-1 row r, dl = r)
         ++dl;
         samples(t, xl, dl, wl);
-        if (upper) samples(phi, xh, dl, wh);
+        if (moves) move_upper();
+        else if (upper) samples(phi, xh, dl, wh);
         store();
         add_piece(plo, plo, t);
-        if (upper)
+        if (upper && !moves)
           for (int i = 1; i <= j; ++i) {
             samples(t, xh, dl + i, wh);
             add_piece(phi, phi, t);
@@ -571,6 +602,7 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
       } else {
         ++j;
         samples(t, xh, dl + j, wh);
+        if (moves) before = acc_add(before, sample_before(dl + j));
         store();
         add_piece(phi, phi, t);
       }
@@ -579,6 +611,15 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
     sum();
     store();
   }
+}
+
+// The walk stage writing the top level (global memory) or a stored one.
+template <class TI, class A, class TO, bool R16, bool SCALE, bool GEN, bool MOVES>
+__device__ __forceinline__ void walk_out(bool top, uint32_t sbase, const StageRange &r, int lane,
+                                         const float *__restrict__ w, TO *__restrict__ out, int64_t nt, int64_t T0,
+                                         int lo, int lim) {
+  if (top) stage_walk<TI, A, TO, R16, SCALE, true, GEN, MOVES>(sbase, r, lane, w, out, nt, T0, lo, lim);
+  else stage_walk<TI, A, TO, R16, SCALE, false, GEN, MOVES>(sbase, r, lane, w, out, nt, T0, lo, lim);
 }
 
 // A single or pair stage of an item; TSrc is the type of the stage's source
@@ -848,24 +889,11 @@ __device__ __forceinline__ void item_first_stage(uint32_t sbase, const Prog &pro
   const StageRange r = prog_stage(prog, 0, warp);
   const bool top = !SEARCH && n_stages == 1;
   if constexpr (FROM_INPUT) {
-    const bool gen = GEN && (r.kind & kStageGeneral) != 0;
-    if constexpr (SCALE && std::is_floating_point<A>::value) {
-      if (gen) {
-        if (top) stage_walk<TI, A, TO, R16, true, true, true>(sbase, r, lane, w, out, nt, T0, lo, lim);
-        else stage_walk<TI, A, TO, R16, true, false, true>(sbase, r, lane, w, out, nt, T0, lo, lim);
-      } else {
-        if (top) stage_walk<TI, A, TO, R16, true, true, false>(sbase, r, lane, w, out, nt, T0, lo, lim);
-        else stage_walk<TI, A, TO, R16, true, false, false>(sbase, r, lane, w, out, nt, T0, lo, lim);
-      }
-    } else {
-      if (gen) {
-        if (top) stage_walk<TI, A, TO, R16, false, true, true>(sbase, r, lane, w, out, nt, T0, lo, lim);
-        else stage_walk<TI, A, TO, R16, false, false, true>(sbase, r, lane, w, out, nt, T0, lo, lim);
-      } else {
-        if (top) stage_walk<TI, A, TO, R16, false, true, false>(sbase, r, lane, w, out, nt, T0, lo, lim);
-        else stage_walk<TI, A, TO, R16, false, false, false>(sbase, r, lane, w, out, nt, T0, lo, lim);
-      }
-    }
+    constexpr bool kScale = SCALE && std::is_floating_point<A>::value;
+    const bool gen = GEN && (r.kind & kStageGeneral) != 0, moves = (r.kind & kStageMoves) != 0;
+    if (moves) walk_out<TI, A, TO, R16, kScale, GEN, true>(top, sbase, r, lane, w, out, nt, T0, lo, lim);
+    else if (gen) walk_out<TI, A, TO, R16, kScale, GEN, false>(top, sbase, r, lane, w, out, nt, T0, lo, lim);
+    else walk_out<TI, A, TO, R16, kScale, false, false>(top, sbase, r, lane, w, out, nt, T0, lo, lim);
   } else if constexpr (SEARCH) {
     if (n_stages == 2) run_merge_stage<TB, A, TO, R16, kOutPadded, GEN>(r, sbase, lane, out, nt, T0, lo, lim);
     else run_merge_stage<TB, A, TO, R16, kOutSmem, GEN>(r, sbase, lane, out, nt, T0, lo, lim);

@@ -335,13 +335,14 @@ double op_slots(int32_t kind, int32_t flags) {
 
 // The same of one walk: the first row's samples of both channels, then one
 // sample more per row, or, where the lower row grows, one and the upper
-// channel's j + 1 again; and the rows' stores.
+// channel's j + 1 again or moved (walk_moves); and the rows' stores.
 double walk_cost(const FusedWalk &wk) {
   double n = wk.dl0 + 1 + (wk.flags & kWalkNoUpper ? 0 : wk.a - wk.dl0 + 1) + 1;
   int32_t j = wk.a - wk.dl0;
+  const bool moves = walk_moves(wk);
   for (int32_t r = 0; r < wk.e - wk.a; ++r) {
     if (wk.flags & kWalkNoUpper) n += 2;
-    else if ((wk.bits >> r) & 1) n += 2 + j + 1;
+    else if ((wk.bits >> r) & 1) n += 2 + (moves ? std::min(j + 1, 2) : j + 1);
     else n += 2, ++j;
   }
   return n;
@@ -926,14 +927,17 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
         }
         item.rows.push_back(std::move(rows));
         const std::vector<int32_t> b = split_warps(cost);
-        bool general = false;
+        bool general = false, moves = false;
         if ((kinds[si] & kStageKindMask) == kStageWalk) {
-          for (size_t i = (size_t)base; i < item.walks.size(); ++i) general |= (item.walks[i].flags & kWalkNoUpper) != 0;
+          for (size_t i = (size_t)base; i < item.walks.size(); ++i) {
+            general |= (item.walks[i].flags & kWalkNoUpper) != 0;
+            moves |= walk_moves(item.walks[i]);
+          }
         } else {
           for (size_t i = (size_t)base; i < item.ops.size(); ++i)
             general |= (item.ops[i].flags & (kOpLoOne | kOpHiOne | kOpNoHi)) != 0;
         }
-        item.stages.push_back(kinds[si] | (general ? kStageGeneral : 0));
+        item.stages.push_back(kinds[si] | (general ? kStageGeneral : 0) | (moves ? kStageMoves : 0));
         for (int32_t w = 0; w <= kFusedBlockWarps; ++w) {
           item.stages.push_back(base + b[w]);
           // A warp's first op has nothing earlier to reuse.
