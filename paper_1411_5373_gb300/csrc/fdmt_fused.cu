@@ -2,8 +2,6 @@
 // plans and the dispatch over the input types (the kernel and the launch
 // logic: fdmt_fused_launch.cuh; float32 launches: fdmt_fused_f32.cu; uint8
 // launches: fdmt_fused_u8.cu).
-#include <mutex>
-
 #include "fdmt_fused_launch.cuh"
 
 namespace fdmt {
@@ -23,24 +21,21 @@ F driver_entry(const char *name, int version) {
   return reinterpret_cast<F>(p);
 }
 
-// The driver's map encoder, or null.  It needs a context that is current in
-// the calling thread, and a thread that has made no runtime call that binds
-// one has none (autograd's worker, whose small allocations come from a
-// cache): the current device's is then made current.  A context that is
-// current already stays.
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static PFN_cuCtxGetCurrent_v4000 current = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    fn = driver_entry<PFN_cuTensorMapEncodeTiled_v12000>("cuTensorMapEncodeTiled", 12000);
-    current = driver_entry<PFN_cuCtxGetCurrent_v4000>("cuCtxGetCurrent", 4000);
-  });
+  static const auto fn = driver_entry<PFN_cuTensorMapEncodeTiled_v12000>("cuTensorMapEncodeTiled", 12000);
+  return fn;
+}
+
+// Maps are encoded in the context that is current in the calling thread, and a
+// thread that has made no runtime call that binds one has none (autograd's
+// worker, whose small allocations come from a cache): the current device's is
+// then made current.  A context that is current already stays.
+bool bind_context() {
+  static const auto current = driver_entry<PFN_cuCtxGetCurrent_v4000>("cuCtxGetCurrent", 4000);
   CUcontext ctx = nullptr;
   int dev = 0;
-  if (current == nullptr || current(&ctx) != CUDA_SUCCESS) return nullptr;
-  if (ctx == nullptr && (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess)) return nullptr;
-  return fn;
+  if (current == nullptr || current(&ctx) != CUDA_SUCCESS) return false;
+  return ctx != nullptr || (cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess);
 }
 
 // Row-window map over a [rows][nt] matrix: boxes of `box` columns x 1 row.
@@ -76,7 +71,7 @@ bool make_block_map(CUtensorMap *m, const void *base, CUtensorMapDataType type, 
 
 bool make_store_map(CUtensorMap *map, void *base, uint64_t rows, uint64_t nt, uint32_t cols, uint32_t brows) {
   PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
-  if (fn == nullptr) return false;
+  if (fn == nullptr || !bind_context()) return false;
   cuuint64_t dims[2] = {nt, rows};
   cuuint64_t strides[1] = {nt * 4};
   cuuint32_t boxd[2] = {cols, brows};
@@ -88,6 +83,7 @@ bool make_store_map(CUtensorMap *map, void *base, uint64_t rows, uint64_t nt, ui
 
 bool make_group_maps(CUtensorMap *maps, const FusedGroup &g, const void *base, CUtensorMapDataType type,
                      uint32_t elem, uint64_t rows, uint64_t nt, int32_t *cshift) {
+  if (!bind_context()) return false;
   std::memset(maps, 0, sizeof(CUtensorMap) * (kMaxBlockP + 1));
   *cshift = 0;
   if (g.chunk > 0) {
