@@ -94,9 +94,9 @@ __device__ __forceinline__ void stage_seg_item(unsigned char *smem, uint32_t bar
 // The first stage of an item with the segment's runtime types: the input
 // or the staged base level (uint16 for narrow integer state) in, the
 // group's top type out when it is the only stage.
-// GEN: some beam's plan has pass-through stages (as for the single-beam
-// kernel); the batch has no channel weights.
-template <class TI, class TB, class A, bool GEN>
+// GEN: some beam's plan has pass-through stages, MOVES: walks that move their
+// upper sums (as for the single-beam kernel); the batch has no channel weights.
+template <class TI, class TB, class A, bool GEN, bool MOVES>
 __device__ __forceinline__ void batch_first_stage(bool from_input, bool i16, bool o16, uint32_t bar, const Prog &prog,
                                                   int n_stages, int warp, int lane, void *out, int64_t nt, int64_t T0,
                                                   int lo, int lim) {
@@ -105,32 +105,32 @@ __device__ __forceinline__ void batch_first_stage(bool from_input, bool i16, boo
     uint16_t *o_16 = static_cast<uint16_t *>(out);
     if (from_input) {
       if (o16)
-        item_first_stage<TI, TB, A, uint16_t, false, true, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane,
+        item_first_stage<TI, TB, A, uint16_t, false, true, false, GEN, false, MOVES>(bar, prog, n_stages, nullptr, warp, lane,
                                                                               o_16, nt, T0, lo, lim);
       else
-        item_first_stage<TI, TB, A, TB, false, true, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o,
+        item_first_stage<TI, TB, A, TB, false, true, false, GEN, false, MOVES>(bar, prog, n_stages, nullptr, warp, lane, o,
                                                                         nt, T0, lo, lim);
     } else if (i16 && o16) {
-      item_first_stage<TI, uint16_t, A, uint16_t, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp,
+      item_first_stage<TI, uint16_t, A, uint16_t, false, false, false, GEN, false, false>(bar, prog, n_stages, nullptr, warp,
                                                                                    lane, o_16, nt, T0, lo, lim);
     } else if (i16) {
-      item_first_stage<TI, uint16_t, A, TB, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane,
+      item_first_stage<TI, uint16_t, A, TB, false, false, false, GEN, false, false>(bar, prog, n_stages, nullptr, warp, lane,
                                                                              o, nt, T0, lo, lim);
     } else {
-      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
+      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
                                                                        T0, lo, lim);
     }
   } else {
     if (from_input)
-      item_first_stage<TI, TB, A, TB, false, true, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
+      item_first_stage<TI, TB, A, TB, false, true, false, GEN, false, MOVES>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
                                                                       T0, lo, lim);
     else
-      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
+      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
                                                                        T0, lo, lim);
   }
 }
 
-template <class TI, class TB, class A, bool GEN>
+template <class TI, class TB, class A, bool GEN, bool MOVES>
 __global__ void __launch_bounds__(kFusedThreads, kFusedMinBlocks)
 batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, const CUtensorMap *__restrict__ maps,
                    const FusedProg *__restrict__ tpls, const int4 *__restrict__ prog,
@@ -254,7 +254,7 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     const bool i16 = kNarrow && sg->in_size == 2, o16 = kNarrow && sg->out_size == 2;
     const int n_stages = cur.n_stages;
     const Prog prg{prog_at(slot), cur.far ? prog + cur.prog : nullptr};
-    batch_first_stage<TI, TB, A, GEN>(from_input, i16, o16, bar, prg, n_stages, warp, lane, sg->out, pitch,
+    batch_first_stage<TI, TB, A, GEN, MOVES>(from_input, i16, o16, bar, prg, n_stages, warp, lane, sg->out, pitch,
                                       T0, 0, lim);
     __syncthreads();  // the staged rows are no longer read; s_early is visible
     const bool early = *s_early != 0;
@@ -291,15 +291,17 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
 }
 
 template <class TI, class TB, class A>
-void *kernel_ptr(bool gen) {
-  return gen ? reinterpret_cast<void *>(batch_fused_kernel<TI, TB, A, true>)
-             : reinterpret_cast<void *>(batch_fused_kernel<TI, TB, A, false>);
+void *kernel_ptr(bool gen, bool moves) {
+  if (moves) return reinterpret_cast<void *>(batch_fused_kernel<TI, TB, A, true, true>);
+  return gen ? reinterpret_cast<void *>(batch_fused_kernel<TI, TB, A, true, false>)
+             : reinterpret_cast<void *>(batch_fused_kernel<TI, TB, A, false, false>);
 }
 
 // The kernel variant of a batch: its input type, and whether any beam's plan
-// has pass-through stages.
-void *kernel_for(int dtype, bool gen) {
-  return dtype == FDMT_U8_I32 ? kernel_ptr<uint8_t, int32_t, int32_t>(gen) : kernel_ptr<float, float, float>(gen);
+// has pass-through stages or walks that move their upper sums.
+void *kernel_for(int dtype, bool gen, bool moves) {
+  return dtype == FDMT_U8_I32 ? kernel_ptr<uint8_t, int32_t, int32_t>(gen, moves)
+                              : kernel_ptr<float, float, float>(gen, moves);
 }
 
 int64_t rup(int64_t v, int64_t a) { return (v + a - 1) / a * a; }
@@ -319,6 +321,7 @@ struct FusedBatch {
   int64_t total = 0;
   int smem_bytes = 0, prog_off = 0, prog_slot = 0, grid = 0;
   bool general = false;  // some beam's plan has pass-through stages
+  bool moves = false;    // or walks that move their upper sums
   // device
   FusedProg *d_tpls = nullptr;
   int32_t *d_prog = nullptr;
@@ -449,6 +452,7 @@ int fused_batch_create(const std::vector<fdmt_beam_desc> &desc, const std::vecto
     prog.insert(prog.end(), fp.prog.begin(), fp.prog.end());
     for (const FusedGroup &g : fp.groups) {
       fb->tpl_base[b].push_back(t_off + g.tpl_begin);
+      fb->moves |= g.moves;
       // the programme slots lie behind the largest group's regions
       fb->prog_off = std::max(fb->prog_off, g.prog_off);
       fb->prog_slot = std::max(fb->prog_slot, g.prog_slot);
@@ -477,11 +481,11 @@ int fused_batch_create(const std::vector<fdmt_beam_desc> &desc, const std::vecto
   build_segments(fb, -1, -1);
   cudaError_t e = cudaGetDevice(&fb->device);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kernel_for(dtype, fb->general), cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(kernel_for(dtype, fb->general, fb->moves), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              fb->smem_bytes);
   int per_sm = 0, sms = 0;
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel_for(dtype, fb->general), kFusedThreads,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel_for(dtype, fb->general, fb->moves), kFusedThreads,
                                                       fb->smem_bytes);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, fb->device);
   if (e != cudaSuccess || per_sm < 1) {
@@ -605,7 +609,7 @@ int fused_batch_execute(FusedBatch *fb, const void *const *in, void *const *out,
         void *args[] = {&fb->d_segs, (void *)&nsegs, &fb->total, &fb->d_maps, &fb->d_tpls, &fb->d_prog,
                         &fb->d_loads, &fb->prog_off, &fb->prog_slot, &fb->d_counter, &fb->d_done, &fb->d_status,
                         (void *)&wait_ns};
-        le = cudaLaunchKernel(kernel_for(fb->dtype, fb->general), dim3(fb->grid), dim3(kFusedThreads), args,
+        le = cudaLaunchKernel(kernel_for(fb->dtype, fb->general, fb->moves), dim3(fb->grid), dim3(kFusedThreads), args,
                               (size_t)fb->smem_bytes, cap);
       }
       e = cudaStreamEndCapture(cap, &fb->graph);

@@ -55,7 +55,7 @@ constexpr int32_t kStageKindMask = 15;
 // (kOpLoOne, kOpHiOne, kOpNoHi; walks: kWalkNoUpper), which only Nf not a
 // power of two produces; stages without it run code without those tests.
 constexpr int32_t kStageGeneral = 32;
-// Stage word flag: some walk of the stage moves its upper sums (walk_moves).
+// Stage word flag: some walk of the stage is kWalkMoves.
 constexpr int32_t kStageMoves = 128;
 
 // Boxcar search in the last launch (section 4.2, pulse profile): widths
@@ -105,8 +105,11 @@ constexpr int32_t kOpHiShift = 2;
 constexpr int32_t kOpLoOne = 4;
 constexpr int32_t kOpHiOne = 8;
 constexpr int32_t kOpNoHi = 16;
-// Walk flag: the band has a single channel (no upper channel).
+// Walk flags: the band has a single channel (no upper channel); where the
+// delay grows, the walk moves its upper sums between lanes instead of reading
+// them again.
 constexpr int32_t kWalkNoUpper = 1;
+constexpr int32_t kWalkMoves = 2;
 
 // One output row piece of a single or pair stage.  Columns tau in
 // [0, width) of the piece:
@@ -138,22 +141,8 @@ struct FusedWalk {
   int32_t a, e, dl0;
   int32_t bits;
   int32_t chan;     // lower channel (channel weights; the upper one is chan + 1)
-  int32_t flags;    // kWalkNoUpper: a single channel, whose Option-1 rows pass up
+  int32_t flags;    // kWalkNoUpper (a single channel, whose Option-1 rows pass up), kWalkMoves
 };
-// Whether a walk moves its upper sums between lanes where the delay grows (9
-// shuffles and 8 selections for 8 columns per lane) or reads them again (j + 1
-// reads and j sums of 8): the two cost alike at j = 1, and j only grows along
-// a walk, by one with every step that is not in `bits`.
-constexpr int32_t kWalkMoves = 2;
-FDMT_HOST_DEVICE inline bool walk_moves(const FusedWalk &wk) {
-#ifdef __CUDA_ARCH__
-  const int32_t grows = __popc((uint32_t)wk.bits);
-#else
-  const int32_t grows = __builtin_popcount((uint32_t)wk.bits);
-#endif
-  return (wk.flags & kWalkNoUpper) == 0 && wk.e - wk.dl0 - grows >= kWalkMoves;
-}
-
 // The ops of one node's rows, lowered for the kernel.  A run computes rows
 // 0 .. n - 1 of a strip of kPieceCols columns that moves with the delay: row
 // r writes columns c(r) + i, c(0) = col and c one larger after every row
@@ -246,6 +235,7 @@ struct FusedGroup {
   int32_t kchunks = 0;        //   and the largest copy (2^max_p rows)
   int32_t max_p = 0;
   bool from_input = false;
+  bool moves = false;         // some walk is kWalkMoves
   int32_t tpl_begin = 0, tpl_count = 0;
   int32_t smem_bytes = 0;     // group-wide layout: barrier + S + Pa + Pb (+ Pt + Q with a search)
                               //   + two programme slots + slack
@@ -297,6 +287,7 @@ struct FusedPlan {
   // Workspace: intermediate level states between launches (ping-pong).
   size_t ws_split = 0, ws_bytes = 0;
   double model_seconds = 0;
+  bool moves = false;    // walks move their upper sums where that is less work
   bool general = false;  // some stage holds passed-up or one-term halves (kStageGeneral)
 };
 

@@ -472,14 +472,13 @@ __device__ __forceinline__ void stage_runs(uint32_t sbase, const StageRange &ran
 // sums of level 0 and one merge).  The running sums plo = x_lo[tau] + ... +
 // x_lo[tau - dl] and phi = x_hi[tau - dl] + ... + x_hi[tau - dl - j] are
 // kept in registers in the oracle's order (each adds one earlier sample);
-// when dl grows the upper sums move a column.  A walk whose j stays below
-// kWalkMoves reads them again a column earlier (j + 1 reads); a longer one
-// moves them between lanes, the first column coming from 32 more columns of
-// sums that are kept before the piece (`before`; each move uses up one, and
-// a walk makes at most 31).  A row's reads are issued before the row before it
+// when dl grows the upper sums move a column.  A walk reads them again a
+// column earlier (j + 1 reads; j is 0 or 1 on most rows) or, with many delays
+// per channel (kWalkMoves), moves them between lanes, the first column coming
+// from 32 more columns of sums that are kept before the piece (`before`; each
+// move uses up one, and a walk makes at most 31).  A row's reads are issued before the row before it
 // is stored.  SCALE multiplies every sample by its channel's weight first.
-// MOVES: the stage has walks that move their sums (the code alone costs the
-// others 2 to 4 % of the launch).
+// MOVES: the stage has walks that move their sums.
 // Bound: instruction issue.  Launch [0,1] of 32 x 159808 x 2738 with fp16
 // state, 86 level-0 rows per channel: 1648 us with every upper sum read again,
 // 386 us with the moves.
@@ -507,7 +506,7 @@ __device__ __forceinline__ void stage_walk(uint32_t sbase, const StageRange &ran
     const bool upper = !GEN || !(warp_all(wk.flags) & kWalkNoUpper);
     int dl = warp_all(wk.dl0), j = warp_all(wk.a) - dl;
     uint32_t bits = (uint32_t)warp_all(wk.bits);
-    const bool moves = MOVES && upper && warp_all((int)walk_moves(wk)) != 0;
+    const bool moves = MOVES && (warp_all(wk.flags) & kWalkMoves) != 0;
     const int skip = TOP ? max(lo - wk.col, 0) : 0;  // columns before the first one wanted
     const bool whole = TOP ? warp_all(wk.width) >= kPieceCols && warp_all(wk.col) + kPieceCols <= lim && warp_all(skip) == 0
                            : warp_all(wk.width) >= kPieceCols || (warp_all(wk.dst_row) & (kPieceCols * 4 - 1)) == 0;
@@ -880,9 +879,9 @@ __device__ __forceinline__ void stage_search_block(uint32_t sbase, const FusedOp
 // the top.  With SEARCH the stage before the search writes the top level
 // into Pt instead.  Rows of the top level are nt apart in `out`; its columns
 // T0 + [lo, lim) are written.  GEN as for run_merge_stage; SCALE: the input
-// is multiplied by channel weights (float input only).
-template <class TI, class TB, class A, class TO, bool R16, bool FROM_INPUT, bool SEARCH, bool GEN = true,
-          bool SCALE = true>
+// is multiplied by channel weights (float input only); MOVES: some stage is
+// kStageMoves.
+template <class TI, class TB, class A, class TO, bool R16, bool FROM_INPUT, bool SEARCH, bool GEN, bool SCALE, bool MOVES>
 __device__ __forceinline__ void item_first_stage(uint32_t sbase, const Prog &prog, int n_stages,
                                                  const float *__restrict__ w, int warp, int lane,
                                                  TO *__restrict__ out, int64_t nt, int64_t T0, int lo, int lim) {
@@ -890,8 +889,9 @@ __device__ __forceinline__ void item_first_stage(uint32_t sbase, const Prog &pro
   const bool top = !SEARCH && n_stages == 1;
   if constexpr (FROM_INPUT) {
     constexpr bool kScale = SCALE && std::is_floating_point<A>::value;
-    const bool gen = GEN && (r.kind & kStageGeneral) != 0, moves = (r.kind & kStageMoves) != 0;
-    if (moves) walk_out<TI, A, TO, R16, kScale, GEN, true>(top, sbase, r, lane, w, out, nt, T0, lo, lim);
+    const bool gen = GEN && (r.kind & kStageGeneral) != 0;
+    if (MOVES && (r.kind & kStageMoves) != 0)
+      walk_out<TI, A, TO, R16, kScale, GEN, MOVES>(top, sbase, r, lane, w, out, nt, T0, lo, lim);
     else if (gen) walk_out<TI, A, TO, R16, kScale, GEN, false>(top, sbase, r, lane, w, out, nt, T0, lo, lim);
     else walk_out<TI, A, TO, R16, kScale, false, false>(top, sbase, r, lane, w, out, nt, T0, lo, lim);
   } else if constexpr (SEARCH) {

@@ -45,6 +45,9 @@ namespace fdmt {
 // GEN: the plan holds stages with passed-up or one-term halves (Nf not a
 // power of two); SCALE: channel weights multiply the input.  Each launch
 // takes the variant it needs, so a kernel carries only its own stage code.
+// MOVES: walks that move their upper sums as well (the code alone, not run,
+// cost the first launch of other plans up to a tenth: 2078 x 5536 x 2697
+// uint8, [0,4] 45 -> 49 us).
 // The register budget is set for two resident blocks per SM (a run keeps
 // four sources and two half sums of eight columns in registers).
 // Bound: the computing warps' instruction issue and latency (without copies
@@ -55,7 +58,7 @@ namespace fdmt {
 // us with the ops as runs; 139, 137 and 109 us with the walks' code
 // straightened as well; 105, 113 and 92 us with the programmes in shared
 // memory and a copying warp.
-template <class TI, class TB, class TO, class A, bool FROM_INPUT, bool R16, bool SEARCH, bool GEN, bool SCALE>
+template <class TI, class TB, class TO, class A, bool FROM_INPUT, bool R16, bool SEARCH, bool GEN, bool SCALE, bool MOVES>
 __global__ void __launch_bounds__(kFusedLaunchThreads, kFusedMinBlocks)
 fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t nt, int64_t pitch, int64_t first,
              int32_t W, int32_t tile0, int32_t ntiles, int64_t items, const FusedProg *__restrict__ progs,
@@ -87,7 +90,7 @@ fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t
     const int64_t tile = h.x, T0 = tile * W;
     const Prog prg{full + (uint32_t)(prog_off + (int)slot * prog_slot), prog_slot > 0 ? nullptr : prog + h.w};
     const int lo = first > T0 ? (int)(first - T0) : 0;
-    item_first_stage<TI, TB, A, TO, R16, FROM_INPUT, SEARCH, GEN, SCALE>(full, prg, n_stages, w, warp, lane, out,
+    item_first_stage<TI, TB, A, TO, R16, FROM_INPUT, SEARCH, GEN, SCALE, MOVES>(full, prg, n_stages, w, warp, lane, out,
                                                                          pitch, T0, lo, lim);
     __syncwarp();
     if (lane == 0) mbar_arrive(free_bar);  // this warp reads S no more
@@ -98,11 +101,11 @@ fused_kernel(const __grid_constant__ TmaMaps maps, TO *__restrict__ out, int64_t
 
 namespace {
 
-template <class TI, class TB, class TO, class A, bool FI, bool R16, bool SEARCH, bool GEN, bool SCALE>
+template <class TI, class TB, class TO, class A, bool FI, bool R16, bool SEARCH, bool GEN, bool SCALE, bool MOVES = false>
 cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const void *base, int64_t base_rows,
                            void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa,
                            int64_t tile0, const OutView *view) {
-  auto kern = fused_kernel<TI, TB, TO, A, FI, R16, SEARCH, GEN, SCALE>;
+  auto kern = fused_kernel<TI, TB, TO, A, FI, R16, SEARCH, GEN, SCALE, MOVES>;
   using TS = typename std::conditional<FI, TI, TB>::type;
   TmaMaps maps;
   int32_t cshift = 0;
@@ -127,13 +130,24 @@ cudaError_t launch_variant(const DeviceTables &dt, const FusedGroup &g, const vo
 }
 
 // The launch of one group, with the kernel variant the plan and the
-// arguments need: with or without pass-through stage code (GEN) and weights
-// (only for float input from the input).
+// arguments need: with or without pass-through stage code (GEN), moving walks
+// (from the input) and weights (only for float input from the input).
 template <class TI, class TB, class TO, class A, bool FI, bool R16, bool SEARCH = false>
 cudaError_t launch_group(const DeviceTables &dt, const FusedGroup &g, const void *base, int64_t base_rows,
                          void *dst, const float *w, int64_t nt, cudaStream_t s, const SearchArgs *sa, int64_t tile0,
                          const OutView *view) {
   const bool gen = dt.fused->general;
+  if constexpr (FI) {
+    if (g.moves) {  // (few channels, many delays: one variant for all of them)
+      if constexpr (std::is_floating_point<A>::value) {
+        if (w != nullptr)
+          return launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, true, true>(dt, g, base, base_rows, dst, w, nt, s,
+                                                                                  sa, tile0, view);
+      }
+      return launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, false, true>(dt, g, base, base_rows, dst, w, nt, s,
+                                                                               sa, tile0, view);
+    }
+  }
   if constexpr (FI && std::is_floating_point<A>::value) {
     if (w != nullptr)
       return gen ? launch_variant<TI, TB, TO, A, FI, R16, SEARCH, true, true>(dt, g, base, base_rows, dst, w, nt, s, sa,

@@ -335,22 +335,24 @@ double op_slots(int32_t kind, int32_t flags) {
 
 // The same of one walk: the first row's samples of both channels, then one
 // sample more per row, or, where the lower row grows, one and the upper
-// channel's j + 1 again or moved (walk_moves); and the rows' stores.
+// channel's j + 1 again or 9 shuffles and 8 selections of 8 columns each
+// (kWalkMoves); and the rows' stores.
 double walk_cost(const FusedWalk &wk) {
-  double n = wk.dl0 + 1 + (wk.flags & kWalkNoUpper ? 0 : wk.a - wk.dl0 + 1) + 1;
+  const bool upper = !(wk.flags & kWalkNoUpper), moves = (wk.flags & kWalkMoves) != 0;
+  double n = wk.dl0 + 1 + (upper ? wk.a - wk.dl0 + 1 : 0) + 1;
   int32_t j = wk.a - wk.dl0;
-  const bool moves = walk_moves(wk);
   for (int32_t r = 0; r < wk.e - wk.a; ++r) {
-    if (wk.flags & kWalkNoUpper) n += 2;
-    else if ((wk.bits >> r) & 1) n += 2 + (moves ? std::min(j + 1, 2) : j + 1);
+    if (!upper) n += 2;
+    else if ((wk.bits >> r) & 1) n += 2 + (moves ? 17.0 / 8 : j + 1);
     else n += 2, ++j;
   }
   return n;
 }
 
-// Rows ra .. re of level-1 node p as a walk: its row steps.
-FusedWalk walk_rows(const Tables &t, const Node &p, bool upper, int32_t ra, int32_t re) {
-  const std::vector<int32_t> &dl = t.dl[1][p.band];
+// Rows ra .. re of level-1 band `band` as a walk: its row steps, and with
+// `moves` whether its upper sums move.
+FusedWalk walk_rows(const Tables &t, int32_t band, bool upper, int32_t ra, int32_t re, bool moves) {
+  const std::vector<int32_t> &dl = t.dl[1][band];
   FusedWalk wk{};
   wk.a = ra;
   wk.e = re;
@@ -358,7 +360,35 @@ FusedWalk walk_rows(const Tables &t, const Node &p, bool upper, int32_t ra, int3
   for (int32_t r = ra + 1; r <= re; ++r)
     if (dl[r] > dl[r - 1]) wk.bits |= 1 << (r - ra - 1);
   wk.flags = upper ? 0 : kWalkNoUpper;
+  if (upper && moves) {
+    FusedWalk m = wk;
+    m.flags |= kWalkMoves;
+    if (walk_cost(m) < walk_cost(wk)) return m;
+  }
   return wk;
+}
+
+// Whether a plan's walks move their upper sums where that is less work: if it
+// saves enough of all walks (whole bands counted), since the launch's other
+// walks pay for the code.  Measured on a GB300, walks' cost without over with
+// moves and the first launch without / with them, us: 1024 x 65536 x 2048
+// float32 1.01, 185 / 193; 139 x 48444 x 541 float32 1.12, 46.0 / 47.1; 1024 x
+// 65536 x 4096 float32 1.13, 340 / 335; 366 x 8424 x 2258 fp16 state 1.31,
+// 43.3 / 41.3; 64 x 47828 x 847 float32 1.85, 72.5 / 57.7; 32 x 150000 x 4000
+// float32 5.4, 2516 / 505.
+constexpr double kMovesPay = 1.3;
+bool moves_pay(const Tables &t) {
+  if (t.levels < 1) return false;
+  double again = 0, least = 0;
+  for (int32_t b = 0; b < (int32_t)t.band_rows[1].size(); ++b) {
+    if (!has_upper(t, 1, b)) continue;
+    for (int32_t r = 0; r < t.band_rows[1][b]; r += 32) {
+      const int32_t e = std::min(t.band_rows[1][b], r + 32) - 1;
+      again += walk_cost(walk_rows(t, b, true, r, e, false));
+      least += walk_cost(walk_rows(t, b, true, r, e, true));
+    }
+  }
+  return again > kMovesPay * least;
 }
 
 // Cost model: the rows of one node of a single or pair stage.
@@ -459,7 +489,7 @@ void emit_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPl
         for (int32_t c0 = 0; c0 < wp; c0 += kPieceCols) {
           for (int32_t ra = p.a; ra <= p.e; ra += 32) {
             const int32_t re = std::min(p.e, ra + 31);
-            FusedWalk wk = walk_rows(t, p, upper, ra, re);
+            FusedWalk wk = walk_rows(t, p.band, upper, ra, re, fp.moves);
             wk.dst = top ? (t.band_row0[lt][p.band] + ra) : leaf(io, p, ra, c0);
             wk.dst_row = top ? 0 : p.stride * sA;
             wk.x_lo = clo.xsmem + (clo.xdelta + c0) * sI;
@@ -644,7 +674,7 @@ void count_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedP
       if (from_input && si == 0) {
         const double pieces = (wp + kPieceCols - 1) / kPieceCols;
         for (int32_t ra = p.a; ra <= p.e; ra += 32) {
-          const FusedWalk wk = walk_rows(t, p, upper, ra, std::min(p.e, ra + 31));
+          const FusedWalk wk = walk_rows(t, p.band, upper, ra, std::min(p.e, ra + 31), fp.moves);
           c.work += pieces * (walk_cost(wk) * kWalkSeconds + (top ? (wk.e - ra + 1) * kTopSeconds : 0));
         }
       } else {
@@ -931,7 +961,7 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
         if ((kinds[si] & kStageKindMask) == kStageWalk) {
           for (size_t i = (size_t)base; i < item.walks.size(); ++i) {
             general |= (item.walks[i].flags & kWalkNoUpper) != 0;
-            moves |= walk_moves(item.walks[i]);
+            moves |= (item.walks[i].flags & kWalkMoves) != 0;
           }
         } else {
           for (size_t i = (size_t)base; i < item.ops.size(); ++i)
@@ -1179,6 +1209,7 @@ bool append_group(FusedPlan &fp, GroupBuild &gb) {
     for (size_t i = 0; i < c.stages.size(); i += kStageWords) {
       const int32_t off = (c.stages[i] & kStageKindMask) == kStageWalk ? w0 : o0;
       fp.general |= (c.stages[i] & kStageGeneral) != 0;
+      g.moves |= (c.stages[i] & kStageMoves) != 0;
       fp.stages.push_back(c.stages[i]);
       for (int32_t w = 1; w < kStageWords; ++w) fp.stages.push_back(c.stages[i + w] + off);
       const int32_t kind = c.stages[i] & kStageKindMask;
@@ -1263,6 +1294,7 @@ std::string plan_fused(const Tables &t, int64_t nt, int32_t state_size, int32_t 
   // Short rows keep their length: their launches are not bound by copies.
   fp.state_nt = p.staging == 0 && nt >= kPadRows ? round_up(nt, 64) : nt;
   fp.acc_size = 4;
+  fp.moves = moves_pay(t);
   // Stored element size of each level at a launch boundary; the output
   // (level L) is 4 bytes.  With p.narrow (integer sums of uint8 samples), a
   // level whose sums stay below 2^16 is stored as uint16: row Dt of a band

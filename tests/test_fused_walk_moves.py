@@ -7,7 +7,7 @@ import pytest
 
 import paper_1411_5373_gb300 as FD
 
-MOVES = 2
+NO_UPPER, MOVES = 1, 2  # walk flags
 UNDER = 128  # bytes of slack below the staged rows, behind 128 of barriers
 
 
@@ -25,8 +25,9 @@ def test_sums_before_the_piece(nf, nt, nd, dtype, kw):
         grow = [(bits >> i) & 1 for i in range(e - a)]
         assert e - a < 32 and bits >> (e - a) == 0
         j, dl = a - dl0, dl0
-        if flags & 1 or j + len(grow) - sum(grow) < MOVES:
+        if not flags & MOVES:
             continue
+        assert not flags & NO_UPPER
         # (column, first sample, terms) of each lane's sum, as the kernel keeps
         # them: columns -32 .. -1, and of the piece its first one
         kept = [(c, c - dl, j + 1) for c in range(-32, 0)]

@@ -47,3 +47,14 @@ def test_weighted_equals_plain(nf, nt, nd):
     p = FD.Plan(1200.0, 1600.0, nf, nt, nd, "f32", schedule="fused")
     q = FD.Plan(1200.0, 1600.0, nf, nt, nd, "f32", schedule="plain")
     assert torch.equal(p.execute(x, weights=w), q.execute(x, weights=w))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "u8"])
+def test_batch_in_one_launch(dtype):
+    """Few channels and many delays beside an ordinary beam."""
+    beams = [(1200.0, 1600.0, 8, 2048, 600), (1200.0, 1600.0, 64, 1024, 64), (1200.0, 1600.0, 27, 4112, 900)]
+    xs = [fs.random_u8(i, b[2], b[3]) if dtype == "u8" else fs.random_f32(i, b[2], b[3]) for i, b in enumerate(beams)]
+    b = FD.BatchPlan(beams, dtype, schedule="fused")
+    outs = b.execute([torch.from_numpy(x).cuda() for x in xs], b.outputs())
+    for (f0, f1, nf, nt, nd), x, y in zip(beams, xs, outs):
+        assert np.array_equal(y.cpu().numpy(), oracle.fdmt(x, oracle.build_tables(f0, f1, nf, nd), MODE[dtype]))
