@@ -704,7 +704,9 @@ int fdmt_schedule_info(fdmt_plan_t plan, int32_t *groups, int32_t *bounds, int32
  * of its run of level-1 rows; else 0), first column relative to the tile
  * start), 14 stages (10 words: kind 1 gather / 2 initialisation transpose
  * / 3 initialisation transpose with the level 1 -> 0 gather folded in,
- * the first op of each warp, the end).  *count
+ * the first op of each warp, the end), 15 row lengths of the levels between
+ * launches (low and high word: forward, adjoint), then per adjoint launch the
+ * bytes of a programme slot (0: its programmes stay in global memory).  *count
  * receives the number of values; dst may be NULL to query.
  */
 int fdmt_fused_tables(fdmt_plan_t plan, int32_t kind, int32_t *dst, int64_t n, int64_t *count);

@@ -16,6 +16,7 @@ constexpr int32_t kAdjBarrierBytes = 128;  // mbarrier slot; regions stay 128-by
 constexpr int32_t kAdjBox = 64;            // provisional TMA box width of the staged rows (elements)
 constexpr int64_t kAdjPadRows = 4096;      // rows from this length on are padded between launches
 constexpr int64_t kAdjMaxSmem = 227 * 1024;
+constexpr int64_t kAdjTwoBlocks = 113 * 1024;  // a block's shared memory that leaves room for a second one on its SM
 constexpr int32_t kAdjChunk = 32;          // row blocks: chunks of 128 bytes
 
 int64_t rup(int64_t v, int64_t a) { return (v + a - 1) / a * a; }
@@ -462,49 +463,76 @@ std::string plan_group(const Tables &t, int64_t nt, int32_t lt, int32_t lb, int3
     const std::string err = build_subtree(t, lt, lb, B, st);
     if (!err.empty()) return err;
     subs.push_back(std::move(st));
-    const Subtree &s = subs.back();
-    const int32_t R = t.band_rows[lt][B];
-    // Split the top rows into ranges that fit the budget: the longest
-    // range from r0 whose cone fits (binary search; the size grows with r1).
-    for (int32_t r0 = 0; r0 < R;) {
-      Shape sh;
-      shape(t, s, lt, lb, init, fuse, r0, r0, W, pitch, box, sh);
-      if (shape_bytes(sh, far) > budget) {
-        // One row's cone can need most of its band (a band whose upper half
-        // is one channel: that channel's row reads every parent row); the
-        // launch then takes the shared memory it needs, if allowed.
-        if (!grow || shape_bytes(sh, far) > kAdjMaxSmem)
-          return "unsupported: one row of level " + std::to_string(lt) + " does not fit";
-        budget = (int32_t)shape_bytes(sh, far);
+  }
+  // Group-wide regions.
+  int64_t S = 0, Pa = 0, Pb = 0, slot = 0, total = 0;
+  // Splits every band's top rows into ranges whose cones fit the budget: the
+  // longest range from r0 whose cone fits (binary search; the size grows with
+  // r1).  With `grow` a row that does not fit raises it.
+  auto split = [&](int32_t limit, bool grow) -> std::string {
+    pieces.clear();
+    for (int32_t B = 0; B < nb; ++B) {
+      const Subtree &s = subs[B];
+      const int32_t R = t.band_rows[lt][B];
+      for (int32_t r0 = 0; r0 < R;) {
+        Shape sh;
+        shape(t, s, lt, lb, init, fuse, r0, r0, W, pitch, box, sh);
+        if (shape_bytes(sh, far) > limit) {
+          // One row's cone can need most of its band (a band whose upper half
+          // is one channel: that channel's row reads every parent row); the
+          // launch then takes the shared memory it needs, if allowed.
+          if (!grow || shape_bytes(sh, far) > kAdjMaxSmem)
+            return "unsupported: one row of level " + std::to_string(lt) + " does not fit";
+          limit = (int32_t)shape_bytes(sh, far);
+        }
+        int32_t lo = r0, hi = R - 1;
+        while (lo < hi) {
+          const int32_t mid = (lo + hi + 1) / 2;
+          shape(t, s, lt, lb, init, fuse, r0, mid, W, pitch, box, sh);
+          if (shape_bytes(sh, far) <= limit) lo = mid;
+          else hi = mid - 1;
+        }
+        shape(t, s, lt, lb, init, fuse, r0, lo, W, pitch, box, sh);
+        if (sh.any) pieces.push_back(Piece{B, r0, lo, std::move(sh)});
+        r0 = lo + 1;
       }
-      int32_t lo = r0, hi = R - 1;
-      while (lo < hi) {
-        const int32_t mid = (lo + hi + 1) / 2;
-        shape(t, s, lt, lb, init, fuse, r0, mid, W, pitch, box, sh);
-        if (shape_bytes(sh, far) <= budget) lo = mid;
-        else hi = mid - 1;
+    }
+    S = Pa = Pb = 0;
+    slot = far ? 0 : kProgMinBytes / 2;
+    for (const Piece &p : pieces) {
+      S = std::max(S, p.sh.s_bytes);
+      Pa = std::max(Pa, p.sh.pa_bytes);
+      Pb = std::max(Pb, p.sh.pb_bytes);
+      slot = std::max(slot, prog_slot_bytes(p.sh, far));
+    }
+    total = kAdjBarrierBytes + S + Pa + Pb + std::max<int64_t>(kProgMinBytes, 2 * slot) + kOverRead;
+    return "";
+  };
+  {
+    std::string err = split(budget, grow);
+    if (!err.empty()) return err;
+    // The maxima of different cones can leave room for one block per SM where
+    // every cone by itself leaves room for two: then smaller cones, down to
+    // three quarters of the budget.  Launches that held one block and hold two,
+    // on a GB300: 3334 x 65536 x 438, 12 -> 10 74 -> 51 us, 8 -> 6 70 -> 53; 256
+    // x 47696 x 1113, 8 -> 6 166 -> 111; 128 x 65536 x 827, 7 -> 4 232 -> 172.
+    if (budget <= kAdjTwoBlocks && total > kAdjTwoBlocks) {
+      int32_t limit = budget;
+      while (total > kAdjTwoBlocks && limit >= budget / 4 * 3 && err.empty()) {
+        limit -= (int32_t)(total - kAdjTwoBlocks);
+        err = split(limit, false);
       }
-      shape(t, s, lt, lb, init, fuse, r0, lo, W, pitch, box, sh);
-      if (sh.any) {
-        *widest = std::max(*widest, sh.nodes[0][0].need);
-        pieces.push_back(Piece{B, r0, lo, sh});
-      }
-      r0 = lo + 1;
+      if (!err.empty() || total > kAdjTwoBlocks) err = split(budget, grow);
+      if (!err.empty()) return err;
     }
   }
-  // Group-wide regions, tiles.
-  int64_t S = 0, Pa = 0, Pb = 0, slot = far ? 0 : kProgMinBytes / 2;
+  if (total > kAdjMaxSmem) return "unsupported: shared memory";
   int32_t omin = 0;
   for (const Piece &p : pieces) {
-    S = std::max(S, p.sh.s_bytes);
-    Pa = std::max(Pa, p.sh.pa_bytes);
-    Pb = std::max(Pb, p.sh.pb_bytes);
-    slot = std::max(slot, prog_slot_bytes(p.sh, far));
+    *widest = std::max(*widest, p.sh.nodes[0][0].need);
     for (const TNode &n : p.sh.nodes.back())
       if (!n.empty()) omin = std::min(omin, n.o);
   }
-  const int64_t total = kAdjBarrierBytes + S + Pa + Pb + std::max<int64_t>(kProgMinBytes, 2 * slot) + kOverRead;
-  if (total > kAdjMaxSmem) return "unsupported: shared memory";
   g.smem_bytes = (int32_t)total;
   g.prog_slot = (int32_t)slot;
   g.prog_off = (int32_t)(kAdjBarrierBytes + S + Pa + Pb);
@@ -559,18 +587,31 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
           !p.bounds.empty() && i - 1 < p.group_budget.size() && p.group_budget[i - 1] > 0 ? p.group_budget[i - 1]
                                                                                           : p.smem_budget;
       if (W < 64 || W % 64 != 0 || budget < 8 * 1024 || budget > 227 * 1024) return "bad launch parameters";
-      // (and where an item leaves no room for its programme, the programmes
-      // stay in global memory)
+      // Where an item leaves no room for its programme a somewhat narrower tile
+      // may (unless a tile is given); else the programmes stay in global memory.
+      // 512 x 65536 x 2717 on a GB300, launch 2 -> 0: 754 us with every op read
+      // ahead through its warp's slot, 914 at 256 columns with the programmes
+      // in global memory, 553 at 192 with them in shared memory; 32 x 65536 x
+      // 332: 153, 149 and 114 us.
+      const bool given = own || !p.grow_budget || !p.init_wide;
       bool far = false;
-      for (;; W /= 2) {
-        for (far = false;; far = true) {
-          err = plan_group(t, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, kAdjBox, far, out, g,
-                           &widest);
-          if (err.empty() || far) break;
-          rollback();
-        }
-        if (err.empty() || !p.grow_budget || W / 2 < 64 || (W / 2) % 64 != 0) break;
+      auto build = [&](int32_t w, bool f) {
         rollback();
+        far = f;
+        err = plan_group(t, out_nt, bounds[i], bounds[i - 1], w, budget, p.grow_budget, 0, 0, kAdjBox, f, out, g,
+                         &widest);
+        return err.empty();
+      };
+      for (;; W /= 2) {
+        if (build(W, false)) break;
+        if (build(W, true)) {
+          int32_t w = given ? 0 : W - 64;
+          while (w > W / 2 && !build(w, false)) w -= 64;
+          if (w > W / 2) W = w;
+          else build(W, true);
+          break;
+        }
+        if (!p.grow_budget || W / 2 < 64 || (W / 2) % 64 != 0) break;
       }
       if (!err.empty()) return err;
       const int32_t measured = widest;

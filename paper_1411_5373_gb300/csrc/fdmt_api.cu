@@ -745,6 +745,15 @@ int fdmt_fused_tables(fdmt_plan_t plan, int32_t kind, int32_t *dst, int64_t n, i
     case 14:
       v = plan->adj_fused.stages;
       break;
+    case 15: {
+      // row lengths of the levels between launches, low and high words:
+      // forward, adjoint; then the adjoint launches' programme slots
+      auto wide = [&](int64_t x) { v.insert(v.end(), {(int32_t)(uint32_t)x, (int32_t)(x >> 32)}); };
+      wide(f.state_nt);
+      wide(plan->adj_fused.state_nt);
+      for (const fdmt::AdjGroup &g : plan->adj_fused.groups) v.push_back(g.prog_slot);
+      break;
+    }
     default:
       return FDMT_ERR_INVALID_ARG;
   }

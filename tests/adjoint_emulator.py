@@ -50,6 +50,16 @@ def layout(plan):
     return tuple(int(v) for v in plan.fused_table(6)[4:6])
 
 
+def row_lengths(plan, groups):
+    """(samples per row read, samples per row written) of every launch: Nt for
+    the first launch's input and the last one's output, the padded length of
+    the levels between launches elsewhere."""
+    words = plan.fused_table(15).astype(np.int64)
+    state = int(words[2] & 0xffffffff) | int(words[3]) << 32
+    last = len(groups) - 1
+    return [(plan.nt if i == 0 else state, plan.nt if i == last else state) for i in range(len(groups))]
+
+
 def tables(plan):
     return (plan.fused_table(10).reshape(-1, 15), plan.fused_table(11).reshape(-1, 8),
             plan.fused_table(12).reshape(-1, 4), plan.fused_table(13).reshape(-1, 8), plan.fused_table(14))
@@ -62,17 +72,18 @@ def emulate_adjoint(plan, g_out, weights=None):
     if len(groups) == 0:
         raise AdjointTableError("the plan has no fused adjoint")
     over_read, desc = layout(plan)
-    nt = plan.nt
     L = plan.levels
     level_rows = [int(plan.band_rows(l).sum()) for l in range(L + 1)]
     cur = np.asarray(g_out, dtype=np.float32)
-    if cur.shape != (plan.nd, nt):
+    if cur.shape != (plan.nd, plan.nt):
         raise ValueError("g_out must be [nd, nt]")
+    lengths = row_lengths(plan, groups)
     w = None if weights is None else np.asarray(weights, dtype=np.float32)
     for gi, grp in enumerate(groups):
         lt, lb, init, W, box, tb, tc, smem_bytes, s_end, pa_end, ntiles, _, chunk, kchunks, max_p = (
             int(v) for v in grp)
-        if (box > 0) == (chunk > 0) or (chunk > 0 and (nt % chunk or not 1 <= kchunks <= 256 or max_p > 5)):
+        nt_in, nt = lengths[gi]
+        if (box > 0) == (chunk > 0) or (chunk > 0 and (nt_in % chunk or not 1 <= kchunks <= 256 or max_p > 5)):
             raise AdjointTableError("bad staging format")
         if cur.shape[0] != level_rows[lt]:
             raise AdjointTableError(f"launch {gi} stages level {lt} from a buffer of {cur.shape[0]} rows")
@@ -98,7 +109,7 @@ def emulate_adjoint(plan, g_out, weights=None):
                     if row < 0 or row + nrows > cur.shape[0]:
                         raise AdjointTableError("staged rows outside level lt")
                     cols = T0 + xoff + np.arange(n)
-                    ok = (cols >= 0) & (cols < nt)
+                    ok = (cols >= 0) & (cols < nt_in)
                     for r in range(nrows):
                         vals = np.zeros(n, dtype=np.float32)
                         vals[ok] = cur[row + r, cols[ok]]
@@ -164,17 +175,19 @@ def check_adjoint_tables(plan):
     once over the tiles).  Returns the number of ops checked."""
     groups, tpls, loads, ops, stages = tables(plan)
     over_read, desc = layout(plan)
-    nt = plan.nt
     L = plan.levels
     level_rows = [int(plan.band_rows(l).sum()) for l in range(L + 1)]
+    lengths = row_lengths(plan, groups)
     checked = 0
     for gi, grp in enumerate(groups):
         lt, lb, init, W, box, tb, tc, smem_bytes, s_end, pa_end, ntiles, _, chunk, kchunks, max_p = (
             int(v) for v in grp)
-        if (box > 0) == (chunk > 0) or (chunk > 0 and (nt % chunk or not 1 <= kchunks <= 256 or max_p > 5)):
+        nt_in, nt = lengths[gi]
+        if (box > 0) == (chunk > 0) or (chunk > 0 and (nt_in % chunk or not 1 <= kchunks <= 256 or max_p > 5)):
             raise AdjointTableError("bad staging format")
         owner = {}
         pieces = {}
+        parts = {}  # weight-gradient partials: (channel, piece) of a tile
         for tpl in range(tb, tb + tc):
             lb0, lc, _, _, sb, n_st, tx, _ = (int(v) for v in tpls[tpl])
             ld = loads[lb0:lb0 + lc]
@@ -226,6 +239,12 @@ def check_adjoint_tables(plan):
                     rows = plan.nf if init else level_rows[lb]
                     if (dst < 0).any() or (dst >= rows).any():
                         raise AdjointTableError("global row out of range")
+                    if init:
+                        for d, k in zip(dst.tolist(), op[:, 4].tolist()):
+                            if not 0 <= k < -(-W // PIECE) or parts.setdefault((d, k), tpl) != tpl:
+                                raise AdjointTableError(f"channel {d}: bad partial slot {k}")
+                        if len(set(zip(dst.tolist(), op[:, 4].tolist()))) != len(op):
+                            raise AdjointTableError("partial slot written twice")
                     for d, c, wd in zip(dst.tolist(), col.tolist(), width.tolist()):
                         if owner.setdefault(d, tpl) != tpl:
                             raise AdjointTableError(f"row {d} owned by two templates")
@@ -235,6 +254,8 @@ def check_adjoint_tables(plan):
                         raise AdjointTableError("op writes outside Pa / Pb")
                 checked += len(op)
         rows = plan.nf if init else level_rows[lb]
+        if init and len(parts) != rows * -(-W // PIECE):
+            raise AdjointTableError("partial slots missing")
         if len(owner) != rows:
             raise AdjointTableError(f"launch {gi}: {rows - len(owner)} output rows have no owner")
         for d, ps in pieces.items():
