@@ -130,6 +130,11 @@ int fdmt_stream_info(fdmt_stream_t s, int64_t *carry, int64_t *window) {
 int fdmt_stream_push(fdmt_stream_t s, const void *in, void *out, void *stream) {
   if (s == nullptr || in == nullptr || out == nullptr) return FDMT_ERR_INVALID_ARG;
   if ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) return FDMT_ERR_INVALID_ARG;
+  // (before the window's kernel is launched: the plan's own check comes later)
+  fdmt::PlanView view;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) return FDMT_ERR_CUDA;
+  if (!fdmt::plan_view(s->plan, &view) || dev != view.device) return FDMT_ERR_INVALID_ARG;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   const int nxt = s->cur ^ 1;
   void *dst = s->win[nxt];
