@@ -3,7 +3,9 @@
 // its work items, and for every item its TMA copies and gather ops.
 #include <algorithm>
 #include <cstdint>
+#include <map>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "fdmt_adjoint_fused.h"
@@ -427,10 +429,18 @@ void emit(const Tables &t, const Subtree &st, int32_t lt, int32_t lb, bool init,
   ++g.tpl_count;
 }
 
+// The subtrees of a level group's top bands, the row whose cone did not fit last
+// (the first to try another tile with), and why no tile fits, if none does.
+struct Forest {
+  std::vector<Subtree> bands;
+  int32_t bad_band = -1, bad_row = 0;
+  std::string err;
+};
+
 // pitch > 0: row blocks of `chunk` elements, every staged row `pitch` wide;
 // *widest receives the widest staged window of the launch's cones.
-std::string plan_group(const Tables &t, int64_t nt, int32_t lt, int32_t lb, int32_t W, int32_t budget, bool grow,
-                       int32_t pitch, int32_t chunk, int32_t box, bool far, AdjFusedPlan &out, AdjGroup &g, int32_t *widest) {
+std::string plan_group(const Tables &t, Forest &forest, int64_t nt, int32_t lt, int32_t lb,
+                       int32_t W, int32_t budget, bool grow, int32_t pitch, int32_t chunk, int32_t box, bool far, AdjFusedPlan &out, AdjGroup &g, int32_t *widest) {
   const bool init = (lb == 0);
   const bool fuse = init && lt - lb >= 2 && init_fusable(t);
   g = AdjGroup();
@@ -455,15 +465,9 @@ std::string plan_group(const Tables &t, int64_t nt, int32_t lt, int32_t lb, int3
     int32_t band, r0, r1;
     Shape sh;
   };
-  std::vector<Subtree> subs;
+  const std::vector<Subtree> &subs = forest.bands;
   std::vector<Piece> pieces;
   const int32_t nb = (int32_t)t.band_rows[lt].size();
-  for (int32_t B = 0; B < nb; ++B) {
-    Subtree st;
-    const std::string err = build_subtree(t, lt, lb, B, st);
-    if (!err.empty()) return err;
-    subs.push_back(std::move(st));
-  }
   // Group-wide regions.
   int64_t S = 0, Pa = 0, Pb = 0, slot = 0, total = 0;
   // Splits every band's top rows into ranges whose cones fit the budget: the
@@ -471,6 +475,12 @@ std::string plan_group(const Tables &t, int64_t nt, int32_t lt, int32_t lb, int3
   // r1).  With `grow` a row that does not fit raises it.
   auto split = [&](int32_t limit, bool grow) -> std::string {
     pieces.clear();
+    const std::string no = "unsupported: one row of level " + std::to_string(lt) + " does not fit";
+    if (forest.bad_band >= 0) {
+      Shape sh;
+      shape(t, subs[forest.bad_band], lt, lb, init, fuse, forest.bad_row, forest.bad_row, W, pitch, box, sh);
+      if (shape_bytes(sh, far) > (grow ? kAdjMaxSmem : limit)) return no;
+    }
     for (int32_t B = 0; B < nb; ++B) {
       const Subtree &s = subs[B];
       const int32_t R = t.band_rows[lt][B];
@@ -481,8 +491,11 @@ std::string plan_group(const Tables &t, int64_t nt, int32_t lt, int32_t lb, int3
           // One row's cone can need most of its band (a band whose upper half
           // is one channel: that channel's row reads every parent row); the
           // launch then takes the shared memory it needs, if allowed.
-          if (!grow || shape_bytes(sh, far) > kAdjMaxSmem)
-            return "unsupported: one row of level " + std::to_string(lt) + " does not fit";
+          if (!grow || shape_bytes(sh, far) > kAdjMaxSmem) {
+            forest.bad_band = B;
+            forest.bad_row = r0;
+            return no;
+          }
           limit = (int32_t)shape_bytes(sh, far);
         }
         int32_t lo = r0, hi = R - 1;
@@ -553,15 +566,28 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
   if (p.W < 64 || p.W % 64 != 0) return "tile must be a positive multiple of 64";
   if (p.smem_budget < 8 * 1024 || p.smem_budget > 227 * 1024) return "shared-memory budget out of range";
   const int64_t state_nt = nt >= kAdjPadRows ? rup(nt, kAdjChunk) : nt;
+  std::map<std::pair<int32_t, int32_t>, Forest> forests;  // of the level groups tried so far
   auto try_bounds = [&](const std::vector<int32_t> &bounds) -> std::string {
     out = AdjFusedPlan();
     out.state_nt = state_nt;
     if (bounds.size() < 2 || bounds.front() != 0 || bounds.back() != L) return "bounds must run from 0 to L";
     for (size_t i = 1; i < bounds.size(); ++i)
       if (bounds[i] <= bounds[i - 1]) return "bounds must increase";
+    for (size_t i = 1; i < bounds.size(); ++i) {
+      const std::string &known = forests[{bounds[i], bounds[i - 1]}].err;
+      if (!known.empty()) return known;
+    }
     for (size_t i = bounds.size() - 1; i >= 1; --i) {
       AdjGroup g;
       std::string err;
+      Forest &forest = forests[{bounds[i], bounds[i - 1]}];
+      std::vector<Subtree> &subs = forest.bands;
+      for (int32_t B = (int32_t)subs.size(); B < (int32_t)t.band_rows[bounds[i]].size(); ++B) {
+        Subtree st;
+        err = build_subtree(t, bounds[i], bounds[i - 1], B, st);
+        if (!err.empty()) return err;
+        subs.push_back(std::move(st));
+      }
       // Row lengths of what the launch reads and writes.
       const int64_t in_nt = bounds[i] == L ? nt : state_nt, out_nt = bounds[i - 1] == 0 ? nt : state_nt;
       const size_t tpls = out.tpls.size(), loads = out.loads.size(), ops = out.ops.size(),
@@ -598,7 +624,7 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
       auto build = [&](int32_t w, bool f) {
         rollback();
         far = f;
-        err = plan_group(t, out_nt, bounds[i], bounds[i - 1], w, budget, p.grow_budget, 0, 0, kAdjBox, f, out, g,
+        err = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], w, budget, p.grow_budget, 0, 0, kAdjBox, f, out, g,
                          &widest);
         return err.empty();
       };
@@ -613,7 +639,7 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
         }
         if (!p.grow_budget || W / 2 < 64 || (W / 2) % 64 != 0) break;
       }
-      if (!err.empty()) return err;
+      if (!err.empty()) return forest.err = err;
       const int32_t measured = widest;
       if (in_nt % kAdjChunk == 0) {
         // Row blocks: one TMA copy per 2^p staged rows, every row as wide as
@@ -624,7 +650,7 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
           if (k > 256 || (int64_t)k * kAdjChunk > in_nt) break;
           rollback();
           int32_t w2 = 0;
-          const std::string e2 = plan_group(t, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget,
+          const std::string e2 = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget,
                                             k * kAdjChunk, kAdjChunk, 0, far, out, gb, &w2);
           if (!e2.empty()) break;
           if (w2 <= k * kAdjChunk) {
@@ -640,10 +666,10 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
         // whole 128 bytes each.
         const int32_t n = (measured + 255) / 256, box = (int32_t)rup((measured + n - 1) / n, 32);
         rollback();
-        err = plan_group(t, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, box, far, out, g, &widest);
+        err = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, box, far, out, g, &widest);
         if (!err.empty()) {
           rollback();
-          err = plan_group(t, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, kAdjBox, far, out, g,
+          err = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, kAdjBox, far, out, g,
                            &widest);
         }
         if (!err.empty()) return err;

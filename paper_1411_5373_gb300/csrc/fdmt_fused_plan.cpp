@@ -87,6 +87,7 @@ struct ConeOut {
   FusedTemplate tpl{};
   std::vector<FusedLoad> loads;
   std::vector<FusedWalk> walks;                 // the first stage of a launch from the input
+  std::vector<double> walk_cost;                //   and what each costs (shared-memory pipe slots)
   std::vector<std::vector<FusedOp>> stage_ops;  // single / pair stages, in row order (before the warp split)
   std::vector<StageRows> stage_rows;            // the same by node (empty for the search)
   std::vector<int32_t> kinds;                   // stage kinds
@@ -333,38 +334,29 @@ double op_slots(int32_t kind, int32_t flags) {
   return lo + up + 1;
 }
 
-// The same of one walk: the first row's samples of both channels, then one
-// sample more per row, or, where the lower row grows, one and the upper
-// channel's j + 1 again or 9 shuffles and 8 selections of 8 columns each
-// (kWalkMoves); and the rows' stores.
-double walk_cost(const FusedWalk &wk) {
-  const bool upper = !(wk.flags & kWalkNoUpper), moves = (wk.flags & kWalkMoves) != 0;
-  double n = wk.dl0 + 1 + (upper ? wk.a - wk.dl0 + 1 : 0) + 1;
-  int32_t j = wk.a - wk.dl0;
-  for (int32_t r = 0; r < wk.e - wk.a; ++r) {
-    if (!upper) n += 2;
-    else if ((wk.bits >> r) & 1) n += 2 + (moves ? 17.0 / 8 : j + 1);
-    else n += 2, ++j;
-  }
-  return n;
-}
-
 // Rows ra .. re of level-1 band `band` as a walk: its row steps, and with
-// `moves` whether its upper sums move.
-FusedWalk walk_rows(const Tables &t, int32_t band, bool upper, int32_t ra, int32_t re, bool moves) {
+// `moves` whether its upper sums move.  *cost: the same slots of the walk: the
+// first row's samples of both channels, then one sample more per row, or,
+// where the lower row grows, one and the upper channel's j + 1 again or 9
+// shuffles and 8 selections of 8 columns each (kWalkMoves); and the rows'
+// stores.
+FusedWalk walk_rows(const Tables &t, int32_t band, bool upper, int32_t ra, int32_t re, bool moves, double *cost) {
   const std::vector<int32_t> &dl = t.dl[1][band];
   FusedWalk wk{};
   wk.a = ra;
   wk.e = re;
   wk.dl0 = dl[ra];
-  for (int32_t r = ra + 1; r <= re; ++r)
-    if (dl[r] > dl[r - 1]) wk.bits |= 1 << (r - ra - 1);
-  wk.flags = upper ? 0 : kWalkNoUpper;
-  if (upper && moves) {
-    FusedWalk m = wk;
-    m.flags |= kWalkMoves;
-    if (walk_cost(m) < walk_cost(wk)) return m;
+  int32_t j = ra - wk.dl0;
+  double again = wk.dl0 + 1 + (upper ? j + 1 : 0) + 1, moved = again;
+  for (int32_t r = ra + 1; r <= re; ++r) {
+    const bool grows = dl[r] > dl[r - 1];
+    if (grows) wk.bits |= 1 << (r - ra - 1);
+    again += upper && grows ? 2 + j + 1 : 2;
+    moved += upper && grows ? 2 + 17.0 / 8 : 2;
+    j += grows ? 0 : 1;
   }
+  wk.flags = !upper ? kWalkNoUpper : (moves && moved < again ? kWalkMoves : 0);
+  *cost = wk.flags & kWalkMoves ? moved : again;
   return wk;
 }
 
@@ -384,8 +376,11 @@ bool moves_pay(const Tables &t) {
     if (!has_upper(t, 1, b)) continue;
     for (int32_t r = 0; r < t.band_rows[1][b]; r += 32) {
       const int32_t e = std::min(t.band_rows[1][b], r + 32) - 1;
-      again += walk_cost(walk_rows(t, b, true, r, e, false));
-      least += walk_cost(walk_rows(t, b, true, r, e, true));
+      double cost = 0;
+      walk_rows(t, b, true, r, e, false, &cost);
+      again += cost;
+      walk_rows(t, b, true, r, e, true, &cost);
+      least += cost;
     }
   }
   return again > kMovesPay * least;
@@ -489,7 +484,8 @@ void emit_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPl
         for (int32_t c0 = 0; c0 < wp; c0 += kPieceCols) {
           for (int32_t ra = p.a; ra <= p.e; ra += 32) {
             const int32_t re = std::min(p.e, ra + 31);
-            FusedWalk wk = walk_rows(t, p.band, upper, ra, re, fp.moves);
+            double cost = 0;
+            FusedWalk wk = walk_rows(t, p.band, upper, ra, re, fp.moves, &cost);
             wk.dst = top ? (t.band_row0[lt][p.band] + ra) : leaf(io, p, ra, c0);
             wk.dst_row = top ? 0 : p.stride * sA;
             wk.x_lo = clo.xsmem + (clo.xdelta + c0) * sI;
@@ -498,8 +494,9 @@ void emit_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedPl
             wk.col = c0;
             wk.chan = clo.band;
             c.walks.push_back(wk);
-            c.slots += walk_cost(wk) * kLaneCols;
-            c.work += walk_cost(wk) * kWalkSeconds + (top ? (re - ra + 1) * kTopSeconds : 0);
+            c.walk_cost.push_back(cost);
+            c.slots += cost * kLaneCols;
+            c.work += cost * kWalkSeconds + (top ? (re - ra + 1) * kTopSeconds : 0);
             c.nops += 1;
             if (top) c.hbm += (double)std::min(kPieceCols, W - c0) * (re - ra + 1) * fp.level_size[lt];
           }
@@ -674,8 +671,9 @@ void count_cone(const Tables &t, int32_t lb, int32_t lt, int32_t W, const FusedP
       if (from_input && si == 0) {
         const double pieces = (wp + kPieceCols - 1) / kPieceCols;
         for (int32_t ra = p.a; ra <= p.e; ra += 32) {
-          const FusedWalk wk = walk_rows(t, p.band, upper, ra, std::min(p.e, ra + 31), fp.moves);
-          c.work += pieces * (walk_cost(wk) * kWalkSeconds + (top ? (wk.e - ra + 1) * kTopSeconds : 0));
+          double cost = 0;
+          const FusedWalk wk = walk_rows(t, p.band, upper, ra, std::min(p.e, ra + 31), fp.moves, &cost);
+          c.work += pieces * (cost * kWalkSeconds + (top ? (wk.e - ra + 1) * kTopSeconds : 0));
         }
       } else {
         c.work += stage_work(t, l1, p, wp, l1 - st[si] == 2, to_global);
@@ -924,11 +922,10 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
         int32_t base;
         if ((kinds[si] & kStageKindMask) == kStageWalk) {
           base = (int32_t)item.walks.size();
-          for (const ConeOut &c : cos)
-            for (const FusedWalk &wk : c.walks) {
-              item.walks.push_back(wk);
-              cost.push_back(walk_cost(wk));
-            }
+          for (const ConeOut &c : cos) {
+            item.walks.insert(item.walks.end(), c.walks.begin(), c.walks.end());
+            cost.insert(cost.end(), c.walk_cost.begin(), c.walk_cost.end());
+          }
         } else {
           base = (int32_t)item.ops.size();
           const size_t k = (lb == 0) ? si - 1 : si;
