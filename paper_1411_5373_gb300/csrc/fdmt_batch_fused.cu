@@ -105,28 +105,28 @@ __device__ __forceinline__ void batch_first_stage(bool from_input, bool i16, boo
     uint16_t *o_16 = static_cast<uint16_t *>(out);
     if (from_input) {
       if (o16)
-        item_first_stage<TI, TB, A, uint16_t, false, true, false, GEN, false, MOVES>(bar, prog, n_stages, nullptr, warp, lane,
-                                                                              o_16, nt, T0, lo, lim);
+        item_first_stage<TI, TB, A, uint16_t, false, true, false, GEN, false, MOVES>(
+            bar, prog, n_stages, nullptr, warp, lane, o_16, nt, T0, lo, lim);
       else
-        item_first_stage<TI, TB, A, TB, false, true, false, GEN, false, MOVES>(bar, prog, n_stages, nullptr, warp, lane, o,
-                                                                        nt, T0, lo, lim);
+        item_first_stage<TI, TB, A, TB, false, true, false, GEN, false, MOVES>(
+            bar, prog, n_stages, nullptr, warp, lane, o, nt, T0, lo, lim);
     } else if (i16 && o16) {
-      item_first_stage<TI, uint16_t, A, uint16_t, false, false, false, GEN, false, false>(bar, prog, n_stages, nullptr, warp,
-                                                                                   lane, o_16, nt, T0, lo, lim);
+      item_first_stage<TI, uint16_t, A, uint16_t, false, false, false, GEN, false, false>(
+          bar, prog, n_stages, nullptr, warp, lane, o_16, nt, T0, lo, lim);
     } else if (i16) {
-      item_first_stage<TI, uint16_t, A, TB, false, false, false, GEN, false, false>(bar, prog, n_stages, nullptr, warp, lane,
-                                                                             o, nt, T0, lo, lim);
+      item_first_stage<TI, uint16_t, A, TB, false, false, false, GEN, false, false>(
+          bar, prog, n_stages, nullptr, warp, lane, o, nt, T0, lo, lim);
     } else {
-      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
-                                                                       T0, lo, lim);
+      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false, false>(
+          bar, prog, n_stages, nullptr, warp, lane, o, nt, T0, lo, lim);
     }
   } else {
     if (from_input)
-      item_first_stage<TI, TB, A, TB, false, true, false, GEN, false, MOVES>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
-                                                                      T0, lo, lim);
+      item_first_stage<TI, TB, A, TB, false, true, false, GEN, false, MOVES>(
+          bar, prog, n_stages, nullptr, warp, lane, o, nt, T0, lo, lim);
     else
-      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false, false>(bar, prog, n_stages, nullptr, warp, lane, o, nt,
-                                                                       T0, lo, lim);
+      item_first_stage<TI, TB, A, TB, false, false, false, GEN, false, false>(
+          bar, prog, n_stages, nullptr, warp, lane, o, nt, T0, lo, lim);
   }
 }
 

@@ -88,8 +88,9 @@ constexpr int32_t kOverRead = kPieceCols * 4;
 // programmes stay in global memory).
 constexpr int32_t kProgMinBytes = 3712;
 
-// Reuse flags of an op, valid against the previous op of the same warp's
-// list (same column piece):
+// Reuse flags of an op against the op before it in the same warp's list (same
+// column piece).  No kernel reads them: they say what the runs (FusedRun) keep
+// in registers, for the tables that tests execute and the ops' share of work:
 //   kOpLoSame  the lower operand (single) or lower half sum (pair) is the
 //              previous op's (same lower row: the addition rule's dl did not
 //              change);

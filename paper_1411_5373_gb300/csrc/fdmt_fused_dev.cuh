@@ -929,20 +929,19 @@ __device__ __forceinline__ void item_later_stages(uint32_t sbase, const Prog &pr
   }
 }
 
-// Row copies of an item: T is FusedProg, or FusedTemplate for the adjoint.
-template <class T>
-__device__ __forceinline__ FusedLoad fetch_load(const T &tp, const FusedLoad *__restrict__ loads, int i) {
+// Row copies of an item.
+__device__ __forceinline__ FusedLoad fetch_load(const FusedProg &tp, const FusedLoad *__restrict__ loads, int i) {
   if (i < tp.load_count) return loads[tp.load_begin + i];
   return FusedLoad{0, 0, 0, 0};
 }
 
 // Stage the rows of a work item into region S: one warp; lane 0 announces
 // the bytes on the mbarrier, then the lanes issue the copies.  `first` is
-// load `lane` of the template, fetched ahead of time, so the copies go out
+// load `lane` of the item, fetched ahead of time, so the copies go out
 // without waiting on a descriptor read.  cshift > 0: row blocks of
 // 2^cshift-element chunks; else row boxes of `box` elements.
-template <class TS, class T>
-__device__ __forceinline__ void stage_item(unsigned char *smem, uint32_t bar, const CUtensorMap *maps, const T &tp,
+template <class TS>
+__device__ __forceinline__ void stage_item(unsigned char *smem, uint32_t bar, const CUtensorMap *maps, const FusedProg &tp,
                                            const FusedLoad *__restrict__ loads, const FusedLoad &first, int64_t T0,
                                            int32_t box, int32_t cshift, int lane) {
   // Order this block's earlier generic-proxy accesses of S before the
@@ -965,8 +964,8 @@ __device__ __forceinline__ void stage_item(unsigned char *smem, uint32_t bar, co
 
 // Ask for the rows of a work item to be brought into L2 (the same copies as
 // stage_item, without their shared memory).
-template <class TS, class T>
-__device__ __forceinline__ void prefetch_item(const CUtensorMap *maps, const T &tp,
+template <class TS>
+__device__ __forceinline__ void prefetch_item(const CUtensorMap *maps, const FusedProg &tp,
                                               const FusedLoad *__restrict__ loads, const FusedLoad &first, int64_t T0,
                                               int32_t box, int32_t cshift, int lane) {
   for (int i = lane; i < tp.load_count; i += 32) {
