@@ -137,10 +137,9 @@ def autotune(f_min, f_max, nf, nt, nd, dtype="f32", reps=10, use_cache=True, ver
             except (FdmtError, RuntimeError):
                 p.close()
                 continue
-            trials.append({"schedule": "fused", "tile": w, "smem_budget": kib * 1024,
-                           "bounds": bounds, "ms": ms})
+            trials.append(_trial(tile, kib, bounds, ms))
             if verbose:
-                print(f"autotune {key}: tile {w} budget {kib} KiB bounds {bounds}: {ms:.4f} ms")
+                print(f"autotune {key}: tile {tile or 'per launch'} budget {kib} KiB bounds {bounds}: {ms:.4f} ms")
             p.close()
     # Phase 2: per-launch tuning of the best groupings, and of a few regular
     # ones the cost model may rank too low.
@@ -199,6 +198,18 @@ def autotune(f_min, f_max, nf, nt, nd, dtype="f32", reps=10, use_cache=True, ver
         except OSError:
             pass
     return best
+
+
+def _trial(tile, kib, bounds, ms):
+    """The record of a plan made with `tile` (0: the planner's tile for every
+    launch) and a budget; _arguments makes the same plan again."""
+    return {"schedule": "fused", "tile": tile, "smem_budget": kib * 1024, "bounds": bounds, "ms": ms}
+
+
+def _arguments(trial):
+    """The Plan arguments that make a fused trial's plan."""
+    return dict(schedule="fused", tile=trial["tile"], smem_budget=trial["smem_budget"], bounds=trial["bounds"],
+                group_tiles=trial.get("group_tiles"), group_budgets=trial.get("group_budgets"))
 
 
 def _regular_groupings(levels, nf):
@@ -261,9 +272,7 @@ def tuned_plan(f_min, f_max, nf, nt, nd, dtype="f32", d_min=0, descending=False,
     m = dict(d_min=d_min, descending=descending)
     if best["schedule"] == "plain":
         return Plan(f_min, f_max, nf, nt, nd, dtype, schedule="plain", **m), best
-    return Plan(f_min, f_max, nf, nt, nd, dtype, schedule="fused", tile=best["tile"],
-                smem_budget=best["smem_budget"], bounds=best["bounds"],
-                group_tiles=best.get("group_tiles"), group_budgets=best.get("group_budgets"), **m), best
+    return Plan(f_min, f_max, nf, nt, nd, dtype, **_arguments(best), **m), best
 
 
 if __name__ == "__main__":
