@@ -109,6 +109,15 @@ struct ConeShape {
   int64_t prog_bytes = 0;  // at most this much of the item's programme (walks and runs)
   std::vector<std::pair<int32_t, int32_t>> needs;  // (window elements from the aligned start, rows) per staged node
   int32_t x_o = 0;  // row blocks, from input: the channels' common window starts at T0 - x_o
+  // Empty, for levels lb .. lb + m, in the memory it has (a plan shapes cones by
+  // the hundred thousand).
+  void reset(int32_t m) {
+    nodes.resize(m + 1);
+    for (std::vector<Node> &v : nodes) v.clear();
+    needs.clear();
+    s_bytes = pa_bytes = pb_bytes = pt_bytes = prog_bytes = 0;
+    top_rows = x_o = 0;
+  }
 };
 
 // Staging format of a launch.  chunk == 0: row boxes of `box` elements.
@@ -165,9 +174,8 @@ void shape_cone(const Tables &t, int32_t lb, int32_t lt, int32_t band, int32_t r
   const int32_t sA = fp.acc_size, sB = fp.level_size[lb], sI = fp.input_size;
   const int32_t alignB = f.chunk > 0 ? f.chunk : 16 / sB, alignI = f.chunk > 0 ? f.chunk : 16 / sI;
   const int32_t m = lt - lb;
-  cs = ConeShape();
+  cs.reset(m);
   std::vector<std::vector<Node>> &nodes = cs.nodes;
-  nodes.assign(m + 1, {});
   const int32_t hist = f.search_k > 0 ? search_hist(f.search_k) : 0;
   nodes[m].push_back(Node{band, r0, r1, hist, hist});
   for (int32_t l = lt; l > lb; --l) {
@@ -768,6 +776,7 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
   GroupBuild gb;
   const int32_t nb = bands_at(t.nf, lt);
   const int64_t nst = (int64_t)stored_levels(lb, lt).size() - 1 + (f.search_k > 0 ? 1 : 0);
+  ConeShape trial;
   for (int32_t cone_budget = budget; cone_budget >= 4096; cone_budget = cone_budget * 7 / 8) {
     std::vector<ConeShape> shapes;
     bool ok = true;
@@ -775,10 +784,9 @@ GroupBuild build_group_fmt(const Tables &t, int64_t nt, int32_t lb, int32_t lt, 
       const int32_t rows = t.band_rows[lt][b];
       auto fits = [&](int32_t per, std::vector<ConeShape> *keep) {
         for (int32_t r0 = 0; r0 < rows; r0 += per) {
-          ConeShape cs;
-          shape_cone(t, lb, lt, b, r0, std::min(rows, r0 + per) - 1, W, fp, f, cs);
-          if (cone_bytes(f, cs, nst) + search_q_bytes(f, cs.top_rows) > cone_budget) return false;
-          if (keep) keep->push_back(std::move(cs));
+          shape_cone(t, lb, lt, b, r0, std::min(rows, r0 + per) - 1, W, fp, f, trial);
+          if (cone_bytes(f, trial, nst) + search_q_bytes(f, trial.top_rows) > cone_budget) return false;
+          if (keep) keep->push_back(trial);
         }
         return true;
       };
