@@ -558,7 +558,8 @@ typedef struct fdmt_batch_params {
                               over 4 streams forked from the caller's stream, largest beam
                               first (no dependency waits; drop_level: UNSUPPORTED) */
   int32_t fused_tile;      /* fused: time tile, multiple of 64 (0 = chosen per level group) */
-  int32_t smem_budget;     /* fused: shared memory per block in bytes (0 = 104 KiB) */
+  int32_t smem_budget;     /* fused: shared memory per block in bytes (0 = 104 KiB; two blocks
+                              share an SM, so less leaves some of it unused) */
 } fdmt_batch_params;
 
 /*

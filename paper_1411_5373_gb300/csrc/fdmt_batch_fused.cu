@@ -50,6 +50,7 @@ struct BSeg {
   void *out;      // the group's top level: the beam's output or a workspace buffer
   int32_t beam, group, from_input, ntpl;
   int32_t ntiles, W, tpl_begin, box;  // tpl_begin: global template index
+  int32_t prog_off, prog_slot;        // byte offset of the first programme slot, bytes of one
   int32_t cshift, map, need, done_idx;
   int32_t dep_idx, in_size, out_size;  // bytes per staged / written sample
   int32_t s_end;  // end of the group's staging region in shared memory
@@ -134,9 +135,8 @@ template <class TI, class TB, class A, bool GEN, bool MOVES>
 __global__ void __launch_bounds__(kFusedThreads, kFusedMinBlocks)
 batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, const CUtensorMap *__restrict__ maps,
                    const FusedProg *__restrict__ tpls, const int4 *__restrict__ prog,
-                   const FusedLoad *__restrict__ loads, int prog_off, int prog_slot,
-                   unsigned long long *__restrict__ counter, int *__restrict__ done, int *__restrict__ status,
-                   uint64_t wait_ns) {
+                   const FusedLoad *__restrict__ loads, unsigned long long *__restrict__ counter,
+                   int *__restrict__ done, int *__restrict__ status, uint64_t wait_ns) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar = smem_u32(smem);
@@ -168,7 +168,7 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
   uint32_t phase = 0;
   bool staged = false;  // this item's copies were issued while the previous item computed
   uint32_t slot = 0;    // this item's programme slot
-  auto prog_at = [&](uint32_t k) { return bar + (uint32_t)(prog_off + (int)k * prog_slot); };
+  auto prog_at = [&](const BSeg *g, uint32_t k) { return bar + (uint32_t)(g->prog_off + (int)k * g->prog_slot); };
   // The previous item's completion, published off the critical path: by
   // thread 32 while the block waits for the next item's copies, or by
   // thread 0 before it waits for producers (so that it never waits on
@@ -195,14 +195,18 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     }
     // The next item's copies go out during this item when its producers are
     // done (always within the same segment; else its previous group's
-    // counter says so) and its staging region fits inside this item's,
-    // which is free once the first stage has run.
+    // counter says so), its staging region fits inside this item's, which is
+    // free once the first stage has run, and its programme's slot lies behind
+    // this item's regions, clear of the slot in use.
     if (threadIdx.x == 0) {
       int e = 0;
       if (next < total) {
         const BSeg &ns = segs[nsi];
+        const int32_t used = sg->prog_off + (int32_t)slot * sg->prog_slot;
+        const int32_t to = ns.prog_off + (int32_t)(slot ^ 1u) * ns.prog_slot;
+        const bool clear = tpn.far || (to >= sg->prog_off && (to + ns.prog_slot <= used || to >= used + sg->prog_slot));
         if (nsi == si) e = 1;
-        else if (ns.s_end <= sg->s_end && (ns.group == 0 || ld_acquire(done + ns.dep_idx) >= ns.need)) e = 1;
+        else if (ns.s_end <= sg->s_end && clear && (ns.group == 0 || ld_acquire(done + ns.dep_idx) >= ns.need)) e = 1;
       }
       *s_early = e;
     }
@@ -234,7 +238,7 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
       if (warp == 0) {
         // Rows written by other blocks with generic stores, read by TMA.
         asm volatile("fence.proxy.async.global;" ::: "memory");
-        stage_seg_item<TI, TB>(smem, bar, sg, maps, cur, prog, prog_at(slot), loads, fetch_load(cur, loads, lane), T0,
+        stage_seg_item<TI, TB>(smem, bar, sg, maps, cur, prog, prog_at(sg, slot), loads, fetch_load(cur, loads, lane), T0,
                                lane);
       }
     }
@@ -253,7 +257,7 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
     constexpr bool kNarrow = std::is_same<TB, int32_t>::value;
     const bool i16 = kNarrow && sg->in_size == 2, o16 = kNarrow && sg->out_size == 2;
     const int n_stages = cur.n_stages;
-    const Prog prg{prog_at(slot), cur.far ? prog + cur.prog : nullptr};
+    const Prog prg{prog_at(sg, slot), cur.far ? prog + cur.prog : nullptr};
     batch_first_stage<TI, TB, A, GEN, MOVES>(from_input, i16, o16, bar, prg, n_stages, warp, lane, sg->out, pitch,
                                       T0, 0, lim);
     __syncthreads();  // the staged rows are no longer read; s_early is visible
@@ -262,7 +266,7 @@ batch_fused_kernel(const BSeg *__restrict__ segs, int nsegs, int64_t total, cons
       const BSeg *nsg = segs + nsi;
       // rows written by other blocks with generic stores, read by TMA
       if (nsi != si) asm volatile("fence.proxy.async.global;" ::: "memory");
-      stage_seg_item<TI, TB>(smem, bar, nsg, maps, tpn, prog, prog_at(slot ^ 1u), loads, ldn,
+      stage_seg_item<TI, TB>(smem, bar, nsg, maps, tpn, prog, prog_at(nsg, slot ^ 1u), loads, ldn,
                              (int64_t)(nl % nsg->ntiles) * nsg->W, lane);
     }
     if (next < total) cur = tpn;
@@ -319,7 +323,8 @@ struct FusedBatch {
   size_t ws_bytes = 0;
   std::vector<BSeg> segs;
   int64_t total = 0;
-  int smem_bytes = 0, prog_off = 0, prog_slot = 0, grid = 0;
+  int smem_bytes = 0, grid = 0;
+  int prog_off = 0, prog_slot = 0;  // programme slots of every group (prog_off < 0: each group's own)
   bool general = false;  // some beam's plan has pass-through stages
   bool moves = false;    // or walks that move their upper sums
   // device
@@ -374,6 +379,8 @@ void build_segments(FusedBatch *fb, int drop_beam, int drop_group) {
       s.pitch = g + 1 == fp.groups.size() ? s.nt : fp.state_nt;
       s.beam = b;
       s.group = (int32_t)g;
+      s.prog_off = fb->prog_off < 0 ? gr.prog_off : fb->prog_off;
+      s.prog_slot = fb->prog_off < 0 ? gr.prog_slot : fb->prog_slot;
       s.from_input = gr.from_input ? 1 : 0;
       s.ntpl = gr.tpl_count;
       s.ntiles = (int32_t)gr.ntiles;
@@ -425,6 +432,7 @@ int fused_batch_create(const std::vector<fdmt_beam_desc> &desc, const std::vecto
   std::vector<FusedLoad> loads;
   std::vector<int32_t> prog;
   size_t ws = 0;
+  int own = 0;  // shared memory of the largest group by itself
   for (int b = 0; b < fb->n; ++b) {
     FusedPlan &fp = fb->plans[b];
     int same = -1;  // an earlier beam of the same shape: its programme is reused
@@ -456,24 +464,22 @@ int fused_batch_create(const std::vector<fdmt_beam_desc> &desc, const std::vecto
       // the programme slots lie behind the largest group's regions
       fb->prog_off = std::max(fb->prog_off, g.prog_off);
       fb->prog_slot = std::max(fb->prog_slot, g.prog_slot);
+      own = std::max(own, g.smem_bytes);
     }
     fb->ws_off[b] = ws;
     ws += (size_t)rup((int64_t)fp.ws_bytes, 256);
   }
   fb->ws_bytes = ws;
-  // One beam's regions and another's slots can exceed a block together (from
-  // budgets of 220 KiB on): programmes that the rest does not hold are then
-  // read in global memory.  (Each group by itself leaves its slots' room.)
-  const int32_t room = (227 * 1024 - kOverRead - fb->prog_off) / 2 / 128 * 128;
-  if (fb->prog_slot > room) {
-    fb->prog_slot = room;
-    for (FusedProg &tp : tpls) {
-      if (tp.far || tp.prog_bytes <= room) continue;
-      tp.far = 1;
-      tp.tx_bytes -= tp.prog_bytes;
-    }
-  }
-  fb->smem_bytes = fb->prog_off + 2 * fb->prog_slot + kOverRead;
+  // One place behind the largest group's regions for the largest slots, unless
+  // that costs the second block of an SM, or exceeds one, where every group by
+  // itself leaves its own slots' room: then each group keeps its place, and the
+  // next item's copies wait where it is in use.  64 beams, uint8, budget 112
+  // KiB, on a GB300: 66.8 ms with one place (one block per SM), 39.3 now; the
+  // default of 104 KiB, where one place fits, 40.5.
+  const int together = fb->prog_off + 2 * fb->prog_slot + kOverRead;
+  constexpr int kTwoBlocks = 113 * 1024;
+  if (own <= kTwoBlocks ? together > kTwoBlocks : together > 227 * 1024) fb->prog_off = -1;
+  fb->smem_bytes = fb->prog_off < 0 ? own : together;
   if (tpls.size() >= ((size_t)1 << 31) || prog.size() >= ((size_t)1 << 31)) {
     delete fb;
     return FDMT_ERR_UNSUPPORTED;
@@ -607,7 +613,7 @@ int fused_batch_execute(FusedBatch *fb, const void *const *in, void *const *out,
         const int nsegs = (int)fb->segs.size();
         const uint64_t wait_ns = (uint64_t)fb->prm.wait_ms * 1000000ull;
         void *args[] = {&fb->d_segs, (void *)&nsegs, &fb->total, &fb->d_maps, &fb->d_tpls, &fb->d_prog,
-                        &fb->d_loads, &fb->prog_off, &fb->prog_slot, &fb->d_counter, &fb->d_done, &fb->d_status,
+                        &fb->d_loads, &fb->d_counter, &fb->d_done, &fb->d_status,
                         (void *)&wait_ns};
         le = cudaLaunchKernel(kernel_for(fb->dtype, fb->general, fb->moves), dim3(fb->grid), dim3(kFusedThreads), args,
                               (size_t)fb->smem_bytes, cap);
