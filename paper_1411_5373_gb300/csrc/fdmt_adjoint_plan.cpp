@@ -439,8 +439,9 @@ struct Forest {
 
 // pitch > 0: row blocks of `chunk` elements, every staged row `pitch` wide;
 // *widest receives the widest staged window of the launch's cones.
-std::string plan_group(const Tables &t, Forest &forest, int64_t nt, int32_t lt, int32_t lb,
-                       int32_t W, int32_t budget, bool grow, int32_t pitch, int32_t chunk, int32_t box, bool far, AdjFusedPlan &out, AdjGroup &g, int32_t *widest) {
+std::string plan_group(const Tables &t, Forest &forest, int64_t nt, int32_t lt, int32_t lb, int32_t W, int32_t budget,
+                       bool grow, int32_t pitch, int32_t chunk, int32_t box, bool far, AdjFusedPlan &out, AdjGroup &g,
+                       int32_t *widest) {
   const bool init = (lb == 0);
   const bool fuse = init && lt - lb >= 2 && init_fusable(t);
   g = AdjGroup();
@@ -525,10 +526,12 @@ std::string plan_group(const Tables &t, Forest &forest, int64_t nt, int32_t lt, 
     std::string err = split(budget, grow);
     if (!err.empty()) return err;
     // The maxima of different cones can leave room for one block per SM where
-    // every cone by itself leaves room for two: then smaller cones, down to
-    // three quarters of the budget.  Launches that held one block and hold two,
-    // on a GB300: 3334 x 65536 x 438, 12 -> 10 74 -> 51 us, 8 -> 6 70 -> 53; 256
-    // x 47696 x 1113, 8 -> 6 166 -> 111; 128 x 65536 x 827, 7 -> 4 232 -> 172.
+    // every cone by itself leaves room for two: then smaller cones, by what the
+    // total exceeds, until the budget has lost a quarter.  Launches that held one
+    // block and hold two, on a GB300: 3334 x 65536 x 438, 12 -> 10 74 -> 51 us, 8
+    // -> 6 70 -> 53; 256 x 47696 x 1113, 8 -> 6 166 -> 111; 128 x 65536 x 827, 7
+    // -> 4 232 -> 172; 64 x 65536 x 2178, 6 -> 3 648 -> 526 with 1.7 times the
+    // cones.
     if (budget <= kAdjTwoBlocks && total > kAdjTwoBlocks) {
       int32_t limit = budget;
       while (total > kAdjTwoBlocks && limit >= budget / 4 * 3 && err.empty()) {
@@ -624,8 +627,8 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
       auto build = [&](int32_t w, bool f) {
         rollback();
         far = f;
-        err = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], w, budget, p.grow_budget, 0, 0, kAdjBox, f, out, g,
-                         &widest);
+        err = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], w, budget, p.grow_budget, 0, 0, kAdjBox, f, out,
+                         g, &widest);
         return err.empty();
       };
       for (;; W /= 2) {
@@ -666,11 +669,12 @@ std::string plan_adjoint_fused(const Tables &t, int64_t nt, const AdjParams &p, 
         // whole 128 bytes each.
         const int32_t n = (measured + 255) / 256, box = (int32_t)rup((measured + n - 1) / n, 32);
         rollback();
-        err = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, box, far, out, g, &widest);
+        err = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, box, far, out, g,
+                         &widest);
         if (!err.empty()) {
           rollback();
-          err = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, kAdjBox, far, out, g,
-                           &widest);
+          err = plan_group(t, forest, out_nt, bounds[i], bounds[i - 1], W, budget, p.grow_budget, 0, 0, kAdjBox, far,
+                           out, g, &widest);
         }
         if (!err.empty()) return err;
       }
