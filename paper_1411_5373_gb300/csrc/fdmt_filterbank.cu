@@ -13,7 +13,7 @@
 // global memory, a pass reads all its values before any is stored, so one
 // shared buffer serves every exchange, and the last pass stores squared
 // magnitudes.  Blocks are persistent: the twiddle table is made once per block.
-// Bound: instruction issue, then HBM.  64 M voltages into 1024 x 65536 on a
+// Bound: the shared-memory pipe, then HBM.  64 M voltages into 1024 x 65536 on a
 // GB300: 334 us with two exchange buffers (two blocks per SM), twiddles made
 // anew for every 4096 samples and the two parts of a complex sum added one
 // by one; 217 us now.
