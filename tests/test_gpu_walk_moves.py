@@ -58,3 +58,29 @@ def test_batch_in_one_launch(dtype):
     outs = b.execute([torch.from_numpy(x).cuda() for x in xs], b.outputs())
     for (f0, f1, nf, nt, nd), x, y in zip(beams, xs, outs):
         assert np.array_equal(y.cpu().numpy(), oracle.fdmt(x, oracle.build_tables(f0, f1, nf, nd), MODE[dtype]))
+
+
+@pytest.mark.parametrize("nf,nt,nd,k", [(8, 1920, 600, 5), (27, 4112, 900, 8), (64, 2048, 1935, 3)])
+@pytest.mark.parametrize("dtype", ["f32", "u8"])
+def test_search_in_the_last_launch(nf, nt, nd, k, dtype):
+    x = fs.random_u8(nt, nf, nt) if dtype == "u8" else fs.random_f32(nt, nf, nt)
+    p = FD.Plan(1200.0, 1600.0, nf, nt, nd, dtype, schedule="fused", search_widths=k)
+    out, peak, time = p.execute_search(torch.from_numpy(x).cuda(), k)
+    p.device_status()
+    want = oracle.fdmt(x, oracle.build_tables(1200.0, 1600.0, nf, nd), MODE[dtype])
+    assert np.array_equal(out.cpu().numpy(), want)
+    rp, rt = oracle.boxcar_search(want, k)
+    assert np.array_equal(peak.cpu().numpy(), rp) and np.array_equal(time.cpu().numpy(), rt)
+
+
+@pytest.mark.parametrize("nf,chunk,nd", [(2, 48, 70), (2, 512, 300), (8, 80, 600), (27, 1024, 900)])
+@pytest.mark.parametrize("dtype", ["f32", "u8"])
+def test_streams(nf, chunk, nd, dtype):
+    """A push writes only its chunk's columns: level 1 may be the top level."""
+    x = fs.random_u8(nf, nf, 4 * chunk) if dtype == "u8" else fs.random_f32(nf, nf, 4 * chunk)
+    want = oracle.fdmt(x, oracle.build_tables(1200.0, 1600.0, nf, nd), MODE[dtype])
+    s = FD.Stream(1200.0, 1600.0, nf, chunk, nd, dtype, "fused")
+    got = [s.push(torch.from_numpy(np.ascontiguousarray(x[:, i:i + chunk])).cuda()).cpu().numpy()
+           for i in range(0, 4 * chunk, chunk)]
+    s.close()
+    assert np.array_equal(np.concatenate(got, axis=1), want)
